@@ -169,18 +169,6 @@ __device__ inline float seg_finish_value(const SegOut<T> &o, int64_t s, int64_t 
     return v;
 }
 
-template <typename PtrT>
-__device__ inline int64_t seg_containing(const PtrT *__restrict__ ptr, int64_t n_seg, int64_t k)
-{
-    // largest s in [0, n_seg) with ptr[s] <= k   (k < ptr[n_seg])
-    int64_t lo = 0, hi = n_seg;
-    while (hi - lo > 1) {
-        const int64_t mid = (lo + hi) >> 1;
-        if ((int64_t)ptr[mid] <= k) lo = mid; else hi = mid;
-    }
-    return lo;
-}
-
 // Host side --------------------------------------------------------------------------------
 
 struct RowShape { int lpr, cpl; };

@@ -5,7 +5,7 @@
 // same reduction over the block's CSC with the two scales exchanged.
 #include <algorithm>
 
-#include "segreduce.cuh"
+#include "segwalk.cuh"
 
 namespace e2egrec {
 namespace {
@@ -136,14 +136,13 @@ int32_t forward_impl(const e2egrec_block *blocks, const LgPlan &p, const e2egrec
         const SegScratch sc = seg_scratch_carve(b.cap_edges, kLgRun, p.d, p.es, ctx + p.seg_off);
         bool ok;
         if (l == 0)     // H^(0) rows are read straight from the feature table through the global ids
-            ok = dispatch_seg_reduce<T, int32_t, true>(static_cast<const T *>(X->data), X->ld, b.indptr, b.nbr_global,
-                                                  &b.counts[CNT_DST], 0, b.cap_dst, inv_sqrt_deg, kLgRun, p.d, X->dtype, nullptr,
-                                                  sc, o, st);
+            ok = dispatch_seg_walk<T, int32_t, true>(static_cast<const T *>(X->data), X->ld, b.indptr, b.nbr_global,
+                                                     &b.counts[CNT_DST], 0, b.cap_dst, inv_sqrt_deg, kLgRun, p.d, X->dtype, sc, o, st);
         else
-            ok = dispatch_seg_reduce<T, int32_t, true>(reinterpret_cast<const T *>(ctx + p.h_off[l - 1]), p.d, b.indptr, b.col,
-                                                  &b.counts[CNT_DST], 0, b.cap_dst,
-                                                  reinterpret_cast<const float *>(ctx + p.s_off[L - 1 - l]), kLgRun, p.d,
-                                                  X->dtype, nullptr, sc, o, st);
+            ok = dispatch_seg_walk<T, int32_t, true>(reinterpret_cast<const T *>(ctx + p.h_off[l - 1]), p.d, b.indptr, b.col,
+                                                     &b.counts[CNT_DST], 0, b.cap_dst,
+                                                     reinterpret_cast<const float *>(ctx + p.s_off[L - 1 - l]), kLgRun, p.d,
+                                                     X->dtype, sc, o, st);
         if (!ok) {
             set_last_error("lightgcn_sampled_forward: no kernel for this row width");
             return E2EGREC_ERR_UNSUPPORTED;

@@ -2,8 +2,8 @@
 //
 //     out[s] = fin( sum_{k in [ptr[s], ptr[s+1])} w[idx[k]] * in[idx[k]] ),   fin as in SegOut.
 //
-// This is the transposed aggregation of the backward pass (segments = columns of the block CSC)
-// and the whole-graph aggregation in either direction (segments = CSR rows or CSC columns).
+// This is the transposed aggregation of the backward pass (segments = columns of the block CSC, with the column of every
+// entry at hand); where only the offsets exist (whole graph, CSR rows) segwalk.cuh does the first of the two launches.
 //
 // seg_run_kernel.  The entry stream is cut into runs of `run_len` consecutive entries and every group of
 //   LPR lanes owns one run.  The group streams through its run with several row loads in flight and closes
@@ -105,23 +105,6 @@ template <> __device__ inline void store4<__nv_bfloat16>(__nv_bfloat16 *p, const
 }
 
 // ------------------------------------------------------------------------------------ runs and windows
-// Advances the walk from segment s to the segment that holds entry k (k >= end of segment s): a few steps one
-// by one, then by bisection if a long stretch of empty segments is in the way.  Returns {segment, its end}; kept
-// out of line (the streaming loop stays short) and by value (nothing of the caller is forced into memory).
-struct SegStep { int64_t seg, end; };
-template <typename PtrT>
-__device__ __noinline__ SegStep seg_advance(const PtrT *__restrict__ ptr, int64_t n_seg, int64_t k, int64_t s)
-{
-    int64_t end;
-    int step = 0;
-    do { ++s; end = (int64_t)ptr[s + 1]; } while (end <= k && ++step < 4);
-    if (end <= k) {
-        s = seg_containing(ptr, n_seg, k);
-        end = (int64_t)ptr[s + 1];
-    }
-    return SegStep{s, end};
-}
-
 // Finishes segment `seg` whose entries (and self row) sum to acc: scale, round to the storage type, mask, store.
 template <typename T, int LPR, int CPL, int kExtra>
 __device__ __forceinline__ void seg_store_row(const SegOut<T> &o, int32_t seg, float inv, const float (&acc)[CPL][Chunk<T>::kElems],
@@ -211,25 +194,18 @@ __device__ __forceinline__ void seg_chain_arrive(int32_t sg, const int32_t *__re
 // With chain_cnt (sampled-block form, CPL = 1, no mean / scale) nothing is left for a second kernel: a group that has
 // written a window's part of a cut segment counts it in chain_cnt[first window of the segment]; the group whose part
 // completes the count adds all parts of the segment in window order and stores the row (seg_chain_arrive).
+// One run's share of the join: after the barrier behind the records in sh_info, by the LPR lanes of a group (c: lane in
+// the group).  n_runs: runs of the window.
 template <typename T, typename PtrT, int LPR, int CPL, int kExtra>
-__device__ __forceinline__ void seg_join_window(float *sh_head, float *sh_tail, int4 *sh_info, int32_t *sh_win, int rl, int c,
-                                                int n_chunks, int d, int32_t head_seg, int32_t head_ends, int32_t tail_seg,
-                                                const PtrT *__restrict__ ptr, float *__restrict__ head2, float *__restrict__ tail2,
-                                                int4 *__restrict__ win_info, const SegOut<T> &o, int32_t *chain_cnt = nullptr,
-                                                int run_len = 0)
+__device__ __forceinline__ void seg_join_run(const float *sh_head, const float *sh_tail, const int4 *sh_info, int32_t *sh_win, int rl,
+                                             int n_runs, int c, int n_chunks, int d, int32_t head_seg, int32_t head_ends, int32_t tail_seg,
+                                             const PtrT *__restrict__ ptr, float *__restrict__ head2, float *__restrict__ tail2,
+                                             const SegOut<T> &o, int32_t *chain_cnt, int run_len)
 {
     constexpr int E = Chunk<T>::kElems;
-    constexpr int RB = kAggThreads / LPR;
     constexpr int ROW = LPR * CPL * E;
-    if (c == 0) sh_info[rl] = make_int4(head_seg, head_ends, tail_seg, 0);
-    if (threadIdx.x < 4) sh_win[threadIdx.x] = threadIdx.x == 1 || threadIdx.x == 3 ? 0 : -1;
-    __syncthreads();
-
-    // ---- join the runs of the window.  The group of run rl acts where a chain of parts of one cut segment
-    // ends: at the run that holds the segment's end, or at the window's last run.  It walks back to the run in
-    // which the segment began (if that run is in the window) and adds the parts forward, in run order.
     {
-        const bool last_run = rl == RB - 1;
+        const bool last_run = rl == n_runs - 1;
         if (head_seg >= 0 && (head_ends || last_run)) {
             int first = rl - 1;                    // the run whose tail begins the chain, or -1: began before the window
             while (first >= 0 && sh_info[first].z != head_seg) --first;
@@ -299,6 +275,20 @@ __device__ __forceinline__ void seg_join_window(float *sh_head, float *sh_tail, 
                 if (chain_cnt) seg_chain_arrive<T, LPR, kExtra>(tail_seg, ptr, run_len, d, c, n_chunks, head2, tail2, chain_cnt, o);
         }
     }
+}
+
+template <typename T, typename PtrT, int LPR, int CPL, int kExtra>
+__device__ __forceinline__ void seg_join_window(float *sh_head, float *sh_tail, int4 *sh_info, int32_t *sh_win, int rl, int c,
+                                                int n_chunks, int d, int32_t head_seg, int32_t head_ends, int32_t tail_seg,
+                                                const PtrT *__restrict__ ptr, float *__restrict__ head2, float *__restrict__ tail2,
+                                                int4 *__restrict__ win_info, const SegOut<T> &o, int32_t *chain_cnt = nullptr,
+                                                int run_len = 0)
+{
+    if (c == 0) sh_info[rl] = make_int4(head_seg, head_ends, tail_seg, 0);
+    if (threadIdx.x < 4) sh_win[threadIdx.x] = threadIdx.x == 1 || threadIdx.x == 3 ? 0 : -1;
+    __syncthreads();
+    seg_join_run<T, PtrT, LPR, CPL, kExtra>(sh_head, sh_tail, sh_info, sh_win, rl, kAggThreads / LPR, c, n_chunks, d, head_seg, head_ends,
+                                            tail_seg, ptr, head2, tail2, o, chain_cnt, run_len);
     if (chain_cnt) return;                        // no record: nobody reads it
     __syncthreads();
     if (threadIdx.x == 0) win_info[blockIdx.x] = make_int4(sh_win[0], sh_win[1], sh_win[2], 0);
@@ -314,18 +304,17 @@ constexpr size_t seg_run_smem_bytes()
 
 // kExtra: 1 = the output has a self row per segment, 2 = a self row and / or a mask row (they are fetched together
 // with the segment's first gathered row); 0 = neither, and those registers and branches disappear.
-// kInFlight: gathered rows a lane group requests before it adds any.  Four suit the short streams of a sampled
-// block (few resident warps, latency hidden inside the thread); on streams that fill the machine two are faster,
-// because the smaller register footprint keeps five blocks resident per SM instead of three.
-template <typename T, typename PtrT, int LPR, int CPL, bool kWeight, int kExtra, int kInFlight>
-__global__ void __launch_bounds__(kAggThreads, (kInFlight <= 2 && !kExtra) ? 5 : 1)
+// Four gathered rows per lane group are requested before any is added (latency hidden inside the thread: the streams of
+// a sampled block keep few warps resident).
+template <typename T, typename PtrT, int LPR, int CPL, bool kWeight, int kExtra>
+__global__ void __launch_bounds__(kAggThreads)
 seg_run_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict__ ptr, const int32_t *__restrict__ idx,
                const int32_t *n_seg_dev, int64_t n_seg_host, const float *__restrict__ w, int run_len, int d,
                float *__restrict__ head2, float *__restrict__ tail2, int4 *__restrict__ win_info, int64_t cap_runs,
                const int32_t *__restrict__ seg_of, SegOut<T> o)
 {
     constexpr int E = Chunk<T>::kElems;
-    constexpr int U = CPL >= kInFlight ? 1 : kInFlight / CPL;
+    constexpr int U = CPL >= 4 ? 1 : 4 / CPL;
     constexpr int RB = kAggThreads / LPR;          // runs of this block = one window
     constexpr int ROW = LPR * CPL * E;             // floats per shared row (>= d)
     constexpr int kFar = 1 << 30;
@@ -373,27 +362,15 @@ seg_run_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict__
     if (run < cap_runs && k0 < total) {
         const int len = (int)min((int64_t)run_len, total - k0);   // entries of this run; positions below are relative to k0
         const int32_t *__restrict__ idx0 = idx + k0;
-        const int32_t *__restrict__ seg0 = seg_of ? seg_of + k0 : nullptr;
+        const int32_t *__restrict__ seg0 = seg_of + k0;
         const int64_t n_self = (kExtra && o.self) ? (o.n_self ? (int64_t)*o.n_self : n_seg) : 0;
 
-        // Segment boundaries are found one iteration ahead of the sums.  With an entry -> segment array a
-        // boundary is a change of that value; without it the offsets are walked.
-        int64_t ws;                    // segment of the entry classified last
-        int rel_end = kFar;            // its end (walk mode)
-        int first_beg_rel = 0;         // where the run's first segment begins (<= 0)
-        bool first_begins, last_ends = false;
-        if (seg0) {
-            ws = seg0[0];
-            first_begins = k0 == 0 || seg0[-1] != (int32_t)ws;
-            last_ends = k0 + len == total || seg0[len] != seg0[len - 1];
-            if (o.mean) first_beg_rel = (int)max((int64_t)ptr[ws] - k0, (int64_t)-kFar);
-        } else {
-            ws = seg_containing(ptr, n_seg, k0);
-            const int64_t wb = (int64_t)ptr[ws] - k0;
-            first_begins = wb >= 0;
-            first_beg_rel = (int)max(wb, (int64_t)-kFar);
-            rel_end = (int)min((int64_t)ptr[ws + 1] - k0, (int64_t)kFar);
-        }
+        // Segment boundaries are found one iteration ahead of the sums: changes of the entry -> segment array.
+        int32_t ws = seg0[0];          // segment of the entry classified last
+        const bool first_begins = k0 == 0 || seg0[-1] != ws;
+        const bool last_ends = k0 + len == total || seg0[len] != seg0[len - 1];
+        // where the run's first segment begins (<= 0)
+        const int first_beg_rel = o.mean ? (int)max((int64_t)ptr[ws] - k0, (int64_t)-kFar) : 0;
 
         int32_t seg_n[U], id_n[U];
         bool start_n[U];
@@ -405,19 +382,10 @@ seg_run_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict__
                 seg_n[u] = 0;
                 id_n[u] = 0;
                 if (r < len) {
-                    if (seg0) {
-                        const int32_t sg = seg0[r];
-                        start_n[u] = r == 0 || sg != (int32_t)ws;
-                        ws = sg;
-                    } else if (r == 0) {
-                        start_n[u] = true;
-                    } else if (r >= rel_end) {
-                        const SegStep nx = seg_advance(ptr, n_seg, k0 + r, ws);
-                        ws = nx.seg;
-                        rel_end = (int)min(nx.end - k0, (int64_t)kFar);
-                        start_n[u] = true;
-                    }
-                    seg_n[u] = (int32_t)ws;
+                    const int32_t sg = seg0[r];
+                    start_n[u] = r == 0 || sg != ws;
+                    ws = sg;
+                    seg_n[u] = ws;
                     id_n[u] = idx0[r];
                 }
             }
@@ -523,7 +491,7 @@ seg_run_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict__
                 }
             }
         }
-        emit(seg0 ? last_ends : rel_end <= len, len);
+        emit(last_ends, len);
     }
     seg_join_window<T, PtrT, LPR, CPL, kExtra>(sh_head, sh_tail, sh_info, sh_win, rl, c, n_chunks, d, head_seg, head_ends, tail_seg, ptr,
                                                head2, tail2, win_info, o);
@@ -1016,7 +984,22 @@ inline bool seg_stream_off()
     return v;
 }
 
-template <typename T, typename PtrT, int LPR, int CPL, bool kWeight, int kInFlight>
+// Chains across windows, segments without entries and padding rows, after a kernel that left its windows' records.
+template <typename T, typename PtrT>
+inline void launch_seg_final(const PtrT *ptr, const int32_t *n_seg_dev, int64_t n_seg_host, int64_t cap_seg, int run_len, int d,
+                             const SegScratch &sc, const SegOut<T> &o, cudaStream_t st)
+{
+    const int64_t window_blocks = std::min<int64_t>(ceil_div(sc.n_windows, kFinalWindows), 148 * 16);
+    const int64_t empty_blocks = std::min<int64_t>(ceil_div(cap_seg > 0 ? cap_seg : 1, kAggThreads), 148 * 8);
+    tap_begin(TAP_SEG_L3, st);
+    note_launch();
+    launch_pdl(seg_final_kernel<T, PtrT>, dim3((unsigned)(window_blocks + empty_blocks)), dim3(kAggThreads), 0, st, ptr, n_seg_dev,
+               n_seg_host, run_len, sc.runs_per_window, d, (const float *)sc.head2, (const float *)sc.tail2, (const int4 *)sc.win_info,
+               sc.n_windows, window_blocks, o);
+    tap_end(TAP_SEG_L3, st);
+}
+
+template <typename T, typename PtrT, int LPR, int CPL, bool kWeight>
 inline void launch_seg_reduce(const T *in, int64_t ld_in, const PtrT *ptr, const int32_t *idx, const int32_t *n_seg_dev,
                               int64_t n_seg_host, int64_t cap_seg, const float *w, int run_len, int d,
                               const int32_t *seg_of, const SegScratch &sc, const SegOut<T> &o, cudaStream_t st)
@@ -1037,7 +1020,7 @@ inline void launch_seg_reduce(const T *in, int64_t ld_in, const PtrT *ptr, const
             s1.tail2 = sc.tail2 + (size_t)r * sc.n_windows * d;
             s1.win_info = sc.win_info + (size_t)r * sc.n_windows;
             s1.chain_cnt = nullptr;
-            launch_seg_reduce<T, PtrT, LPR, CPL, kWeight, kInFlight>(in + r * o.rhs_in, ld_in, ptr, idx, n_seg_dev, n_seg_host, cap_seg, w,
+            launch_seg_reduce<T, PtrT, LPR, CPL, kWeight>(in + r * o.rhs_in, ld_in, ptr, idx, n_seg_dev, n_seg_host, cap_seg, w,
                                                                      run_len, d, seg_of, s1, o1, st);
         }
         return;
@@ -1094,35 +1077,28 @@ inline void launch_seg_reduce(const T *in, int64_t ld_in, const PtrT *ptr, const
     }
     if (block_form) {
     } else if (o.mask) {
-        auto kern = seg_run_kernel<T, PtrT, LPR, CPL, kWeight, 2, kInFlight>;
+        auto kern = seg_run_kernel<T, PtrT, LPR, CPL, kWeight, 2>;
         if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         launch_pdl(kern, dim3(grid1), dim3(kAggThreads), smem, st, in, ld_in, ptr, idx, n_seg_dev, n_seg_host, w, run_len, d, sc.head2,
                    sc.tail2, sc.win_info, sc.cap_runs, seg_of, o);
     } else if (o.self) {
-        auto kern = seg_run_kernel<T, PtrT, LPR, CPL, kWeight, 1, kInFlight>;
+        auto kern = seg_run_kernel<T, PtrT, LPR, CPL, kWeight, 1>;
         if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         launch_pdl(kern, dim3(grid1), dim3(kAggThreads), smem, st, in, ld_in, ptr, idx, n_seg_dev, n_seg_host, w, run_len, d, sc.head2,
                    sc.tail2, sc.win_info, sc.cap_runs, seg_of, o);
     } else {
-        auto kern = seg_run_kernel<T, PtrT, LPR, CPL, kWeight, 0, kInFlight>;
+        auto kern = seg_run_kernel<T, PtrT, LPR, CPL, kWeight, 0>;
         if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         launch_pdl(kern, dim3(grid1), dim3(kAggThreads), smem, st, in, ld_in, ptr, idx, n_seg_dev, n_seg_host, w, run_len, d, sc.head2,
                    sc.tail2, sc.win_info, sc.cap_runs, seg_of, o);
     }
     tap_end(TAP_SEG_L1, st);
-    const int64_t window_blocks = std::min<int64_t>(ceil_div(sc.n_windows, kFinalWindows), 148 * 16);
-    const int64_t empty_blocks = std::min<int64_t>(ceil_div(cap_seg > 0 ? cap_seg : 1, kAggThreads), 148 * 8);
-    tap_begin(TAP_SEG_L3, st);
-    note_launch();
-    launch_pdl(seg_final_kernel<T, PtrT>, dim3((unsigned)(window_blocks + empty_blocks)), dim3(kAggThreads), 0, st, ptr, n_seg_dev,
-               n_seg_host, run_len, sc.runs_per_window, d, (const float *)sc.head2, (const float *)sc.tail2, (const int4 *)sc.win_info,
-               sc.n_windows, window_blocks, o);
-    tap_end(TAP_SEG_L3, st);
+    launch_seg_final(ptr, n_seg_dev, n_seg_host, cap_seg, run_len, d, sc, o, st);
 }
 
 // Returns false (nothing enqueued) when no kernel is built for the row width; rows of up to 4096 bytes (kMaxDim fp32
 // values) are covered, so callers that checked dim <= kMaxDim never see it.
-template <typename T, typename PtrT, bool kWeight, int kInFlight = 4>
+template <typename T, typename PtrT, bool kWeight>
 inline bool dispatch_seg_reduce(const T *in, int64_t ld_in, const PtrT *ptr, const int32_t *idx, const int32_t *n_seg_dev,
                                 int64_t n_seg_host, int64_t cap_seg, const float *w, int run_len, int d, int32_t dtype,
                                 const int32_t *seg_of, const SegScratch &sc, const SegOut<T> &o, cudaStream_t st)
@@ -1130,7 +1106,7 @@ inline bool dispatch_seg_reduce(const T *in, int64_t ld_in, const PtrT *ptr, con
     const RowShape rs = row_shape(d, dtype);
 #define E2E_CASE(L, C)                                                                                                \
     if (rs.lpr == L && rs.cpl == C) {                                                                                 \
-        launch_seg_reduce<T, PtrT, L, C, kWeight, kInFlight>(in, ld_in, ptr, idx, n_seg_dev, n_seg_host, cap_seg, w, run_len, \
+        launch_seg_reduce<T, PtrT, L, C, kWeight>(in, ld_in, ptr, idx, n_seg_dev, n_seg_host, cap_seg, w, run_len, \
                                                          d, seg_of, sc, o, st);                                       \
         return true;                                                                                                  \
     }
