@@ -118,27 +118,6 @@ bce_kernel(const float *__restrict__ logits, const float *__restrict__ labels, i
     }
 }
 
-// dW3[j] = sum_p dt[p] a2[p, j]   (one block per 32 columns, rows in a fixed order)
-template <typename T>
-__global__ void __launch_bounds__(256)
-weighted_colsum_kernel(const T *__restrict__ a, int d, const float *__restrict__ wgt, int32_t P, int accumulate,
-                       float *__restrict__ out)
-{
-    __shared__ float red[8][32];
-    const int col = blockIdx.x * 32 + (threadIdx.x & 31);
-    const int rl = threadIdx.x >> 5;
-    float s = 0.f;
-    if (col < d)
-        for (int64_t r = rl; r < P; r += 8) s = fmaf(wgt[r], to_float<T>(a[r * d + col]), s);
-    red[rl][threadIdx.x & 31] = s;
-    __syncthreads();
-    if (rl == 0 && col < d) {
-        float t = accumulate ? out[col] : 0.f;
-        for (int w = 0; w < 8; ++w) t += red[w][threadIdx.x & 31];
-        out[col] = t;
-    }
-}
-
 // dZ2[p, j] = dt[p] * W3[j] where a2[p, j] > 0 (everywhere with the identity activation), stored in the feature dtype;
 // padding rows are zero.
 template <typename T>
@@ -218,10 +197,7 @@ void linear_backward_weight(const T *dY, int64_t rows, int n_out, const T *Xin, 
     const int64_t n = (int64_t)n_out * n_in;
     note_launch();
     splitk_reduce_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(part, n, kSplits, 0, dW, on_tc ? m_dev : nullptr);
-    if (db) {
-        note_launch();
-        colsum_kernel<T><<<(unsigned)ceil_div(n_out, 32), 256, 0, st>>>(dY, n_out, m_dev, n_out, 0, db);
-    }
+    if (db) launch_colsum<T>(dY, n_out, nullptr, m_dev, 0, n_out, 0, db, st);
 }
 
 // ------------------------------------------------------------------------------------------ gated fusion (Sec. 4.3.2)
@@ -333,10 +309,7 @@ void gate_backward_core(GMat<const T> dFused, GMat<const T> F, GMat<const T> gat
         gemm_simt_kernel<T, true, true, EpiPartial><<<grid, kGemmThreads, 0, st>>>(dpre, d, F.p, F.ld, d, d, rows, nullptr, meta, epi);
         note_launch();
         splitk_reduce_kernel<<<(unsigned)ceil_div((int64_t)d * d, 256), 256, 0, st>>>(part, (int64_t)d * d, kSplits, 0, dWg, nullptr);
-        if (dbg) {
-            note_launch();
-            colsum_kernel<T><<<(unsigned)ceil_div(d, 32), 256, 0, st>>>(dpre, d, meta, d, 0, dbg);
-        }
+        if (dbg) launch_colsum<T>(dpre, d, nullptr, meta, 0, d, 0, dbg, st);
     }
     if (use_tc<T>() && dF.rows >= rows && dFused.rows >= rows && gate.rows >= rows) {
         TcFuse fz{};
@@ -541,8 +514,6 @@ int32_t run_joint(const JointPlan &jp, const e2egrec_csr *graph, const e2egrec_m
     // 4. tower backward
     T *dz2 = tp(jp.dz2_off), *dz1 = tp(jp.dz1_off), *dz = tp(jp.dz_off), *wt = tp(jp.wt_off);
     float *part = reinterpret_cast<float *>(ws + jp.part_off);
-    note_launch();
-    weighted_colsum_kernel<T><<<(unsigned)ceil_div(jp.h2, 32), 256, 0, st>>>(a2, jp.h2, dt, jp.P, 0, dW_tower[2]);
     {
         const int64_t n = jp.rowsP * jp.h2;
         note_launch();
@@ -556,6 +527,7 @@ int32_t run_joint(const JointPlan &jp, const e2egrec_csr *graph, const e2egrec_m
         side->fork(st);
         ws_st = side->stream;
     }
+    launch_colsum<T>(a2, jp.h2, dt, nullptr, jp.P, jp.h2, 0, dW_tower[2], ws_st);                   // dW3 = dt^T a2
     linear_backward_weight<T>(dz2, jp.rowsP, jp.h2, a1, jp.h1, pmeta, part, dW_tower[1], db_tower ? db_tower[1] : nullptr, status, ws_st);
     linear_backward_input<T>(dz2, jp.rowsP, jp.h2, W2, jp.h1, relu ? a1 : nullptr, dz1, wt, pmeta, status, st);
     if (side) side->fork(st);

@@ -325,11 +325,9 @@ static int32_t backward_impl(const e2egrec_block *blocks, int32_t n_layers, cons
         }
         if (l == 0) tap_end(TAP_DW_OUTER, ws);
         if (dbias && dbias[l]) {
-            for (int r = 0; r < n_rhs; ++r) {
-                note_launch();
-                colsum_kernel<T><<<(unsigned)ceil_div(p.d_out, 32), 256, 0, ws>>>(dz + (int64_t)r * p.rows * p.d_out, p.d_out, n_dst,
-                                                                                 p.d_out, (accumulate || r > 0) ? 1 : 0, dbias[l]);
-            }
+            for (int r = 0; r < n_rhs; ++r)
+                launch_colsum<T>(dz + (int64_t)r * p.rows * p.d_out, p.d_out, nullptr, n_dst, 0, p.d_out, (accumulate || r > 0) ? 1 : 0,
+                                 dbias[l], ws);
         }
         if (dw_beside) {
             dz_free[l & 1] = side->event();
