@@ -1,19 +1,25 @@
 // Graph ingest on the device: canonical CSR from an edge list, and the CSC (transpose) of a CSR.
-// Both are two or three stable radix sorts plus offset look-ups, so the result depends only on the
-// multiset of edges: rows ordered by (row, col), columns by (col, CSR position), parallel edges kept.
+// Both are stable radix sorts plus offset look-ups, so the result depends only on the multiset of edges: rows ordered by
+// (row, col), columns by (col, CSR position), parallel edges kept.
+//
+// The CSR is the (col, row) pairs sorted by column and then, key and value exchanged, by row: the other id travels as the
+// value, so nothing is gathered between the sorts (entries equal in both ids need no order).  The transpose sorts
+// (col, position) and looks up the row of every position afterwards.  B200, 10^7 interactions (2 * 10^7 entries, 500 k nodes),
+// CSR and CSC together: 3.23 -> 1.52 ms.
 #include <algorithm>
 
 #include "radix.cuh"
+#include "segwalk.cuh"
 
 namespace e2egrec {
 namespace {
 
 struct IngestScratch {
-    int32_t *counts;                 // int32[4], counts[CNT_EDGES] = m
-    int32_t *a, *b, *c;              // three arrays of m
-    RadixScratch rs;
-    char *arena;
-    size_t arena_bytes, bytes;
+    int32_t *counts;                 // int32[4]: CNT_STATUS is the status word of the run
+    int32_t *a, *k0, *v0, *k1, *v1;  // arrays of m
+    SortState sort[2];
+    char *zero;                      // the part that has to be zero beforehand
+    size_t zero_bytes, bytes;
 };
 
 IngestScratch carve_ingest(int64_t m, void *base)
@@ -27,17 +33,16 @@ IngestScratch carve_ingest(int64_t m, void *base)
     };
     const size_t mm = (size_t)(m > 0 ? m : 1);
     s.counts = (int32_t *)take(256);
-    s.a = (int32_t *)take(mm * 4);
-    s.b = (int32_t *)take(mm * 4);
-    s.c = (int32_t *)take(mm * 4);
-    for (int i = 0; i < 2; ++i) s.rs.keys[i] = (int32_t *)take(mm * 4);
-    for (int i = 0; i < 2; ++i) s.rs.vals[i] = (int32_t *)take(mm * 4);
-    s.rs.tiles = ceil_div((int64_t)mm, kSortTile);
-    const size_t arena_begin = off;
-    s.arena = base ? static_cast<char *>(base) + off : nullptr;
-    s.rs.ghist = (unsigned *)take(sizeof(unsigned) * kMaxPasses * kMaxRadix);
-    s.arena_bytes = off - arena_begin;
-    s.rs.thist = (int32_t *)take(radix_thist_bytes(s.rs.tiles));
+    for (int32_t **p : {&s.a, &s.k0, &s.v0, &s.k1, &s.v1}) *p = (int32_t *)take(mm * 4);
+    const int64_t tiles = ceil_div((int64_t)mm, kSortTile);
+    const size_t begin = off;
+    s.zero = base ? static_cast<char *>(base) + off : nullptr;
+    for (SortState &ss : s.sort) {
+        ss.ghist = (unsigned *)take(kSortCountWords * sizeof(unsigned));
+        ss.tiles = tiles;
+        ss.state = (unsigned *)take(sort_state_bytes(tiles));
+    }
+    s.zero_bytes = off - begin;
     s.bytes = off;
     return s;
 }
@@ -50,31 +55,85 @@ __global__ void ingest_begin_kernel(int32_t *counts, int32_t m)
     counts[CNT_STATUS] = 0;
 }
 
-// ids outside [0, n) are flagged and clamped so that the sorts stay in range
-__global__ void clamp_ids_kernel(const int32_t *__restrict__ in, int64_t m, int64_t n, int32_t *__restrict__ out,
-                                 int32_t *counts)
+// Digit counts of one or two id arrays for every pass of their sorts.  Ids outside [0, n) are flagged here and count as
+// 0, which the first pass of a sort makes of them.
+__global__ void __launch_bounds__(256)
+id_hist_kernel(const int32_t *__restrict__ ids0, const int32_t *__restrict__ ids1, int64_t m, int64_t n, int bits, int passes,
+               unsigned *__restrict__ ghist0, unsigned *__restrict__ ghist1, int32_t *counts)
 {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-        int32_t v = in[i];
-        if ((uint32_t)v >= (uint64_t)n) {
-            atomicOr((unsigned *)&counts[CNT_STATUS], E2EGREC_DEV_RANGE);
-            v = 0;
+    extern __shared__ unsigned hist_sm[];                        // [arrays][passes][1 << bits]
+    const int R = 1 << bits, per = passes * R;
+    const int all = ids1 ? 2 * per : per;
+    for (int d = threadIdx.x; d < all; d += 256) hist_sm[d] = 0;
+    __syncthreads();
+    bool bad = false;
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < m; i += (int64_t)gridDim.x * 256) {
+        uint32_t v0 = (uint32_t)ids0[i], v1 = ids1 ? (uint32_t)ids1[i] : 0u;
+        if (v0 >= (uint64_t)n) { bad = true; v0 = 0; }
+        if (v1 >= (uint64_t)n) { bad = true; v1 = 0; }
+        for (int p = 0; p < passes; ++p) {
+            atomicAdd(&hist_sm[p * R + ((v0 >> (p * bits)) & (R - 1))], 1u);
+            if (ids1) atomicAdd(&hist_sm[per + p * R + ((v1 >> (p * bits)) & (R - 1))], 1u);
         }
-        out[i] = v;
+    }
+    if (bad) atomicOr((unsigned *)&counts[CNT_STATUS], E2EGREC_DEV_RANGE);
+    __syncthreads();
+    for (int d = threadIdx.x; d < all; d += 256) {
+        if (!hist_sm[d]) continue;
+        const int e = d % per;
+        atomicAdd(&(d < per ? ghist0 : ghist1)[(e / R) * kMaxRadix + e % R], hist_sm[d]);
     }
 }
 
-// out[i] = src[pos[i]], flagged and clamped like clamp_ids_kernel
-__global__ void gather_ids_kernel(const int32_t *__restrict__ src, const int32_t *__restrict__ pos, int64_t m, int64_t n,
-                                  int32_t *__restrict__ out, int32_t *counts)
+// row_of[e] = row of CSR position e.  A warp owns 1024 consecutive positions: it finds its first row by a search over the
+// offsets and then goes through them 32 rows at a time, lane i holding the end of row base + i; a position's row is the
+// number of ends at or before it, found by bisection across the lanes.
+__global__ void __launch_bounds__(256)
+expand_rows_kernel(const int64_t *__restrict__ indptr, int64_t n_rows, int64_t m, int32_t *__restrict__ row_of)
 {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-        int32_t v = src[pos[i]];
-        if ((uint32_t)v >= (uint64_t)n) {
-            atomicOr((unsigned *)&counts[CNT_STATUS], E2EGREC_DEV_RANGE);
-            v = 0;
+    constexpr int kSpan = 1024;
+    const int lane = threadIdx.x & 31;
+    const int64_t k0 = (((int64_t)blockIdx.x * 256 + threadIdx.x) >> 5) * kSpan;
+    if (k0 >= m) return;
+    const int len = (int)min((int64_t)kSpan, m - k0);
+    int64_t base = warp_seg_containing(indptr, n_rows, k0);
+    auto load_ends = [&](int64_t b) -> int { return b + lane < n_rows ? (int)min(indptr[b + lane + 1] - k0, (int64_t)kSpan) : kSpan; };
+    int ends = load_ends(base);
+    int quiet = 0;
+    for (int e0 = 0; e0 < len;) {
+        const int last = __shfl_sync(0xffffffffu, ends, 31);     // positions before it belong to this window of rows
+        if (last > e0) {
+            quiet = 0;
+            const int e = e0 + lane;
+            int r = 0;
+#pragma unroll
+            for (int step = 16; step > 0; step >>= 1)
+                if (__shfl_sync(0xffffffffu, ends, r + step - 1) <= e) r += step;
+            if (e < last && e < len) row_of[k0 + e] = (int32_t)max(min(base + r, n_rows - 1), (int64_t)0);
+            e0 = min(e0 + 32, last);
+            if (e0 < last) continue;
+            if (e0 >= len) break;
+        } else {
+            ++quiet;
         }
-        out[i] = v;
+        base = quiet < 4 ? base + 32 : warp_seg_containing(indptr, n_rows, k0 + e0);
+        ends = load_ends(base);
+    }
+}
+
+// csc_row[k] = row_of[csc_eid[k]], four scattered reads per thread in flight.  In a launch of its own row_of stays in L2
+// (80 MB at 2 * 10^7 entries); looked up by the sort's last pass, between its own 320 MB of output, it cost 160 us
+// against 59; the search over the offsets that came before took 360.
+__global__ void rows_of_kernel(const int64_t *__restrict__ eid, const int32_t *__restrict__ row_of, int64_t m, int32_t *__restrict__ csc_row)
+{
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < m; k += 4 * step) {
+        int32_t r[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) r[q] = k + q * step < m ? __ldg(row_of + __ldcs(eid + k + q * step)) : 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (k + q * step < m) __stcs(csc_row + k + q * step, r[q]);
     }
 }
 
@@ -91,33 +150,17 @@ __global__ void offsets_kernel(const int32_t *__restrict__ sorted, int64_t m, in
     }
 }
 
-// row and CSR position of every transposed entry
-__global__ void transpose_rows_kernel(const int32_t *__restrict__ eid32, int64_t m, const int64_t *__restrict__ indptr,
-                                      int64_t n_rows, int32_t *__restrict__ csc_row, int64_t *__restrict__ csc_eid)
-{
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < m; k += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t e = eid32[k];
-        int64_t lo = 0, hi = n_rows;                 // largest r with indptr[r] <= e
-        while (hi - lo > 1) {
-            const int64_t mid = (lo + hi) >> 1;
-            if (indptr[mid] <= e) lo = mid; else hi = mid;
-        }
-        csc_row[k] = (int32_t)lo;
-        csc_eid[k] = e;
-    }
-}
-
 unsigned wide_grid(int64_t n) { return (unsigned)std::min<int64_t>(ceil_div(n > 0 ? n : 1, 256), 148 * 16); }
 
-// stable sort of (keys, vals) by key; vals == nullptr: value = position
-void sort_stage(const int32_t *keys, const int32_t *vals, int32_t *keys_out, int32_t *vals_out, int64_t m, int64_t key_range,
-                IngestScratch &s, cudaStream_t st)
+SortPlan plan_for(int64_t key_range) { return sort_plan((int32_t)std::min<int64_t>(std::max<int64_t>(key_range, 2), 0x7fffffff)); }
+
+void id_hist(const int32_t *ids0, const int32_t *ids1, int64_t m, int64_t n, const SortPlan &sp, IngestScratch &s, cudaStream_t st)
 {
-    const SortPlan sp = sort_plan((int32_t)std::min<int64_t>(std::max<int64_t>(key_range, 2), 0x7fffffff));
-    cudaMemsetAsync(s.arena, 0, s.arena_bytes, st);
+    cudaMemsetAsync(s.zero, 0, s.zero_bytes, st);
+    const size_t smem = (size_t)(ids1 ? 2 : 1) * sp.passes * (1 << sp.bits) * sizeof(unsigned);
     note_launch();
-    key_hist_kernel<<<wide_grid(m), 256, 0, st>>>(keys, s.counts, sp.bits, sp.passes, s.rs.ghist);
-    radix_sort_pairs(keys, vals, s.counts, m, keys_out, vals_out, sp, s.rs, st);
+    id_hist_kernel<<<(unsigned)std::min<int64_t>(ceil_div(m, 2048), 148 * 8), 256, smem, st>>>(ids0, ids1, m, n, sp.bits, sp.passes,
+                                                                                             s.sort[0].ghist, s.sort[1].ghist, s.counts);
 }
 
 }  // namespace
@@ -142,16 +185,26 @@ extern "C" int32_t e2egrec_graph_from_coo(int64_t n_nodes, int64_t n_edges, cons
     note_launch();
     ingest_begin_kernel<<<1, 1, 0, st>>>(s.counts, (int32_t)m);
     if (m > 0) {
-        // 1. by column (value = position), 2. by row with the sorted columns as values: (row, col) order
-        note_launch();
-        clamp_ids_kernel<<<wide_grid(m), 256, 0, st>>>(col, m, n_nodes, s.a, s.counts);
-        sort_stage(s.a, nullptr, s.b, s.c, m, n_nodes, s, st);            // s.b = columns sorted, s.c = their positions
-        note_launch();
-        gather_ids_kernel<<<wide_grid(m), 256, 0, st>>>(row, s.c, m, n_nodes, s.a, s.counts);
-        sort_stage(s.a, s.b, s.c, indices, m, n_nodes, s, st);            // s.c = rows sorted
+        const SortPlan sp = plan_for(n_nodes);
+        const int32_t clamp = (int32_t)std::max<int64_t>(n_nodes, 1);
+        id_hist(col, row, m, n_nodes, sp, s, st);
+        // (col, row) by column, then (row, col) by row
+        const int32_t *k = col, *v = row;
+        int32_t *ka = s.k0, *va = s.v0, *kb = s.k1, *vb = s.v1;
+        for (int q = 0; q < 2 * sp.passes; ++q) {
+            const int sort = q / sp.passes, pass = q % sp.passes;
+            if (q == sp.passes) std::swap(k, v);
+            const bool last = q == 2 * sp.passes - 1;
+            sort_pass<int32_t>(sp, k, v, nullptr, m, q == 0 ? clamp : 0, q == 0 ? clamp : 0, pass, s.sort[sort], last ? s.a : ka,
+                               last ? indices : va, SortMap{}, &s.counts[CNT_STATUS], st);
+            k = ka;
+            v = va;
+            std::swap(ka, kb);
+            std::swap(va, vb);
+        }                                                        // s.a = rows sorted
     }
     note_launch();
-    offsets_kernel<<<wide_grid(n_nodes + 1), 256, 0, st>>>(s.c, m, n_nodes, indptr);
+    offsets_kernel<<<wide_grid(n_nodes + 1), 256, 0, st>>>(s.a, m, n_nodes, indptr);
     if (status) cudaMemcpyAsync(status, &s.counts[CNT_STATUS], sizeof(int32_t), cudaMemcpyDeviceToDevice, st);
     return check_launch("graph_from_coo");
 }
@@ -169,17 +222,33 @@ extern "C" int32_t e2egrec_csr_transpose(const e2egrec_csr *csr, int64_t n_cols,
     if (!csr->indptr || !csc_ptr || (csr->n_edges > 0 && (!csr->indices || !csc_row || !csc_eid))) return E2EGREC_ERR_NULL;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int64_t m = csr->n_edges;
+    const int32_t *sorted = s.k0;
     note_launch();
     ingest_begin_kernel<<<1, 1, 0, st>>>(s.counts, (int32_t)m);
     if (m > 0) {
+        const SortPlan sp = plan_for(n_cols);
+        id_hist(csr->indices, nullptr, m, n_cols, sp, s, st);
         note_launch();
-        clamp_ids_kernel<<<wide_grid(m), 256, 0, st>>>(csr->indices, m, n_cols, s.a, s.counts);
-        sort_stage(s.a, nullptr, s.b, s.c, m, n_cols, s, st);             // s.b = columns sorted, s.c = CSR positions
+        expand_rows_kernel<<<(unsigned)ceil_div(m, 8 * 1024), 256, 0, st>>>(csr->indptr, csr->n_nodes, m, s.a);
+        const int32_t *k = csr->indices, *v = nullptr;           // value = CSR position
+        int32_t *ka = s.k0, *va = s.v0, *kb = s.k1, *vb = s.v1;
+        for (int q = 0; q < sp.passes; ++q) {
+            const int32_t clamp = q == 0 ? (int32_t)std::max<int64_t>(n_cols, 1) : 0;
+            if (q == sp.passes - 1)
+                sort_pass<int64_t>(sp, k, v, nullptr, m, clamp, 0, q, s.sort[0], ka, csc_eid, SortMap{}, &s.counts[CNT_STATUS], st);
+            else
+                sort_pass<int32_t>(sp, k, v, nullptr, m, clamp, 0, q, s.sort[0], ka, va, SortMap{}, &s.counts[CNT_STATUS], st);
+            k = ka;
+            v = va;
+            std::swap(ka, kb);
+            std::swap(va, vb);
+        }
+        sorted = k;                                              // the columns in order
         note_launch();
-        transpose_rows_kernel<<<wide_grid(m), 256, 0, st>>>(s.c, m, csr->indptr, csr->n_nodes, csc_row, csc_eid);
+        rows_of_kernel<<<(unsigned)std::min<int64_t>(ceil_div(m, 1024), 148 * 16), 256, 0, st>>>(csc_eid, s.a, m, csc_row);
     }
     note_launch();
-    offsets_kernel<<<wide_grid(n_cols + 1), 256, 0, st>>>(s.b, m, n_cols, csc_ptr);
+    offsets_kernel<<<wide_grid(n_cols + 1), 256, 0, st>>>(sorted, m, n_cols, csc_ptr);
     if (status) cudaMemcpyAsync(status, &s.counts[CNT_STATUS], sizeof(int32_t), cudaMemcpyDeviceToDevice, st);
     return check_launch("csr_transpose");
 }

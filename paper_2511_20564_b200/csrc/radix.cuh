@@ -1,6 +1,5 @@
 // Building blocks shared by the sampler and the graph ingest: single-pass prefix sums across thread
-// blocks, and a stable least-significant-digit radix sort of (int32 key, int32 value) pairs (counts per
-// tile, scan over tiles, scatter: three launches per digit).
+// blocks, and a stable least-significant-digit radix sort of (int32 key, value) pairs, one launch per digit.
 #pragma once
 
 #include "common.cuh"
@@ -8,11 +7,11 @@
 
 namespace e2egrec {
 
-constexpr int kSortThreads = 256;
-constexpr int kSortItems = 16;
-constexpr int kSortTile = kSortThreads * kSortItems;
+constexpr int kSortItems = 16;          // elements per thread of a tile
+constexpr int kSortTile = 256 * kSortItems;        // the smaller of the two tile sizes: what scratch is sized for
 constexpr int kMaxRadix = 1024;
 constexpr int kMaxPasses = 4;
+constexpr int kPassWords = 2048;        // words of scan state per tile for all passes of a sort: two of 1024 digits or more of 256
 
 // ---------------------------------------------------------------------------------------
 // Single-pass prefix sums across thread blocks ("chained scan"): every tile publishes its own sum,
@@ -82,139 +81,230 @@ __device__ inline int chain_ticket(unsigned *ticket, int *bcast)
 
 
 // ---------------------------------------------------------------------------------------
-// Stable LSD radix sort of (key = col, value = block position), three launches per digit and no
-// waiting between thread blocks: (1) digit counts of every tile of kSortTile consecutive elements,
-// (2) per digit an exclusive scan of those counts over the tiles, (3) the scatter: a block ranks
-// the equal digits of its tile in element order (per warp by match_any, then across warps) and
-// places them at  start of the digit's bin (digit counts of the whole array, known beforehand)
-// + count of that digit in the tiles before it + rank.
+// Stable LSD radix sort, one launch per digit.  A block takes a tile of consecutive elements, ranks the equal digits in
+// element order (per warp by match_any, then across warps), publishes its digit counts and looks back over the tiles
+// before it, digit by digit, until it meets one whose full prefix is known -- the chained scan above with one chain per
+// digit.  The words of a chain tell their kind by themselves: 0 not there yet, count + 1 a tile's own count, top bit set
+// the position behind the tile's last element of that digit in the output.  Tile 0 begins the chains with the digits' bins
+// (digit counts of the whole array, known beforehand).  While the chains move, the tile is put into digit order in shared
+// memory, so that the elements leave in runs: with 1024 digits a warp's 32 scattered 4-byte stores touched 32 sectors and
+// the sectors, not the bytes, set the pace.
+//
+// The form before this one took three launches per digit (counts per tile, scan over the tiles, scatter straight from
+// registers).  B200, 2 * 10^7 pairs, 1024 digits, a pass: 500 and 345 us (random and half-sorted digits), now 238 and 169;
+// 2.9 * 10^5 entries of a sampled block: 24 us in three launches, now 16.  What bounds it now is the ranking's shared-memory
+// and match latency at 32 warps per SM; L2 and DRAM are at a quarter of their rates.
 // ---------------------------------------------------------------------------------------
-template <int BITS>
-__global__ void __launch_bounds__(kSortThreads)
-tile_hist_kernel(const int32_t *__restrict__ keys, const int32_t *__restrict__ counts, int shift,
-                 int32_t *__restrict__ thist)
+constexpr unsigned kPosFlag = 0x80000000u;
+
+// A sort's last launch may also look up where its values belong: row_out[pos] = row_of[value].
+struct SortMap { const int32_t *row_of; int32_t *row_out; };
+
+template <int BITS, int THREADS>
+constexpr size_t sort_smem_bytes()
 {
-    constexpr int R = 1 << BITS;
-    constexpr int W = kSortThreads / 32;
-    __shared__ int32_t h[W][R];                  // one histogram per warp: fewer colliding atomics
-    const int32_t n = counts[CNT_EDGES];
-    const int64_t n_live = ((int64_t)n + kSortTile - 1) / kSortTile;
-    const int warp = threadIdx.x >> 5;
-    for (int64_t tile = blockIdx.x; tile < n_live; tile += gridDim.x) {
-        for (int d = threadIdx.x; d < W * R; d += kSortThreads) (&h[0][0])[d] = 0;
-        __syncthreads();
-        const int64_t base = tile * kSortTile;
-#pragma unroll
-        for (int k = 0; k < kSortItems; ++k) {
-            const int64_t idx = base + k * kSortThreads + threadIdx.x;
-            if (idx < n) atomicAdd(&h[warp][(keys[idx] >> shift) & (R - 1)], 1);
-        }
-        __syncthreads();
-        for (int d = threadIdx.x; d < R; d += kSortThreads) {
-            int32_t c = 0;
-#pragma unroll
-            for (int w = 0; w < W; ++w) c += h[w][d];
-            thist[tile * R + d] = c;
-        }
-        __syncthreads();
-    }
+    return (size_t)(THREADS / 32) * (1 << BITS) * 2 + (size_t)2 * (1 << BITS) * 4 + (size_t)2 * THREADS * kSortItems * 4;
 }
 
-// thist[tile][d] <- sum of thist[tile'][d] over tile' < tile; one block per digit d
-template <int BITS>
-__global__ void __launch_bounds__(kSortThreads)
-tile_scan_kernel(const int32_t *__restrict__ counts, int32_t *__restrict__ thist)
+template <int BITS, int THREADS, typename ValT>
+__global__ void __launch_bounds__(THREADS, 2)
+sort_pass_kernel(const int32_t *__restrict__ keys_in, const int32_t *__restrict__ vals_in, const int32_t *n_dev, int32_t n_host,
+                 int32_t clamp_keys, int32_t clamp_vals, int shift, const unsigned *__restrict__ ghist, unsigned *ticket,
+                 unsigned *state, int32_t *__restrict__ keys_out, ValT *__restrict__ vals_out, SortMap map, int32_t *status)
 {
     constexpr int R = 1 << BITS;
-    __shared__ int32_t scan_sm[kSortThreads / 32 + 1];
-    const int32_t n = counts[CNT_EDGES];
-    const int64_t n_live = ((int64_t)n + kSortTile - 1) / kSortTile;
-    const int d = blockIdx.x;
-    int32_t carry = 0;
-    for (int64_t t0 = 0; t0 < n_live; t0 += kSortThreads) {
-        const int64_t t = t0 + threadIdx.x;
-        const int32_t v = t < n_live ? thist[t * R + d] : 0;
-        int32_t tot;
-        const int32_t ex = block_exclusive_scan<kSortThreads, int32_t>(v, tot, scan_sm);
-        if (t < n_live) thist[t * R + d] = carry + ex;
-        carry += tot;
-    }
-}
-
-template <int BITS>
-__global__ void __launch_bounds__(kSortThreads)
-sort_pass_kernel(const int32_t *__restrict__ keys_in, const int32_t *__restrict__ vals_in,
-                 const int32_t *__restrict__ counts, int shift, const unsigned *__restrict__ ghist,
-                 const int32_t *__restrict__ thist, int32_t *__restrict__ keys_out, int32_t *__restrict__ vals_out)
-{
-    constexpr int R = 1 << BITS;
-    constexpr int W = kSortThreads / 32;
-    __shared__ int32_t wc[W][R];                 // per-warp digit counts, then start offsets
-    __shared__ int32_t bin_base[R];
-    __shared__ int32_t scan_sm[kSortThreads / 32 + 1];
-    const int64_t tile = blockIdx.x;
-    const int32_t n = counts[CNT_EDGES];
-    if (tile * kSortTile >= n) return;
-    for (int d = threadIdx.x; d < W * R; d += kSortThreads) (&wc[0][0])[d] = 0;
-    // start of every digit's bin: exclusive scan of the global digit counts
-    {
-        int32_t carry = 0;
-        for (int d0 = 0; d0 < R; d0 += kSortThreads) {
-            const int d = d0 + threadIdx.x;
-            const int32_t v = d < R ? (int32_t)ghist[d] : 0;
-            int32_t tot;
-            const int32_t ex = block_exclusive_scan<kSortThreads, int32_t>(v, tot, scan_sm);
-            if (d < R) bin_base[d] = carry + ex;
-            carry += tot;
-        }
-    }
+    constexpr int W = THREADS / 32;
+    constexpr int TILE = THREADS * kSortItems;
+    constexpr int D = R >= THREADS ? R / THREADS : 1;            // consecutive digits per thread
+    extern __shared__ uint4 sort_smem[];
+    uint32_t *skey = reinterpret_cast<uint32_t *>(sort_smem);
+    uint32_t *sval = skey + TILE;
+    int32_t *start = reinterpret_cast<int32_t *>(sval + TILE);   // per digit: its first place in the tile's digit order
+    int32_t *gbase = start + R;                                  // per digit: output position minus place in the tile
+    uint16_t *wc = reinterpret_cast<uint16_t *>(gbase + R);      // [W][R] per warp: counts, then offsets within the digit
+    __shared__ int32_t scan_sm[W + 1];
+    __shared__ int tile_s;
+    const int32_t n = n_dev ? *n_dev : n_host;
+    const int tile = chain_ticket(ticket, &tile_s);
+    if ((int64_t)tile * TILE >= n) return;
+    for (int d = threadIdx.x; d < W * R / 2; d += THREADS) reinterpret_cast<uint32_t *>(wc)[d] = 0;
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t wbase = tile * kSortTile + (int64_t)warp * (32 * kSortItems);
-    int32_t key[kSortItems], val[kSortItems], rank[kSortItems];
-    // all loads first: the warp barrier inside the ranking loop would otherwise keep every round's load behind it
+    const int tile_n = (int)min((int64_t)TILE, n - (int64_t)tile * TILE);
+    const int w0 = warp * (32 * kSortItems);                     // the warp's first element of the tile
+    const int32_t *kin = keys_in + (int64_t)tile * TILE;
+    // every load of the tile is requested before the ranking, which then hides it
+    const int32_t *vin = vals_in ? vals_in + (int64_t)tile * TILE : nullptr;
+    uint32_t key[kSortItems], val[kSortItems];
+    int rank[kSortItems];
 #pragma unroll
     for (int k = 0; k < kSortItems; ++k) {
-        const int64_t idx = wbase + k * 32 + lane;
-        const bool ok = idx < n;
-        key[k] = ok ? keys_in[idx] : 0;
-        val[k] = ok ? (vals_in ? vals_in[idx] : (int32_t)idx) : 0;
+        const int i = w0 + k * 32 + lane;
+        key[k] = i < tile_n ? (uint32_t)__ldg(kin + i) : 0u;
+        if (clamp_keys && key[k] >= (uint32_t)clamp_keys) key[k] = 0;
     }
 #pragma unroll
     for (int k = 0; k < kSortItems; ++k) {
-        const int64_t idx = wbase + k * 32 + lane;
-        const bool ok = idx < n;
-        const uint32_t digit = ok ? (uint32_t)((key[k] >> shift) & (R - 1)) : 0xFFFFFFFFu;
+        const int i = w0 + k * 32 + lane;
+        val[k] = !vin ? (uint32_t)(tile * TILE + i) : i < tile_n ? (uint32_t)__ldg(vin + i) : 0u;
+        if (clamp_vals && val[k] >= (uint32_t)clamp_vals) val[k] = 0;
+    }
+#pragma unroll
+    for (int k = 0; k < kSortItems; ++k) {
+        const bool ok = w0 + k * 32 + lane < tile_n;
+        // (one ballot per bit instead: 240 and 231 us for the two passes over 2 * 10^7 pairs, against 238 and 169)
+        const uint32_t digit = ok ? (key[k] >> shift) & (R - 1) : 0xFFFFFFFFu;
         const uint32_t peers = __match_any_sync(0xffffffffu, digit);
         const int leader = __ffs(peers) - 1;
-        int32_t base = 0;
+        int base = 0;
         if (ok && lane == leader) {
-            base = wc[warp][digit];
-            wc[warp][digit] = base + __popc(peers);
+            base = wc[warp * R + digit];
+            wc[warp * R + digit] = (uint16_t)(base + __popc(peers));
         }
         base = __shfl_sync(0xffffffffu, base, leader);
         rank[k] = base + __popc(peers & ((1u << lane) - 1u));
         __syncwarp();
     }
     __syncthreads();
-    // per digit: where the elements of each warp start
-    for (int d = threadIdx.x; d < R; d += kSortThreads) {
-        int32_t run = bin_base[d] + thist[tile * R + d];
+    // the thread's digits: counts of the warps -> offsets, the tile's count, its place in the tile's digit order
+    const int d0 = threadIdx.x * D;
+    const bool owner = d0 < R;
+    int32_t cnt[D], sum = 0;
 #pragma unroll
-        for (int w = 0; w < W; ++w) {
-            const int32_t c2 = wc[w][d];
-            wc[w][d] = run;
-            run += c2;
+    for (int q = 0; q < D; ++q) {
+        cnt[q] = 0;
+        if (owner) {
+#pragma unroll
+            for (int w = 0; w < W; ++w) {
+                const int c = wc[w * R + d0 + q];
+                wc[w * R + d0 + q] = (uint16_t)cnt[q];
+                cnt[q] += c;
+            }
+            if (tile > 0) *reinterpret_cast<volatile unsigned *>(&state[(int64_t)tile * R + d0 + q]) = (unsigned)cnt[q] + 1u;
+        }
+        sum += cnt[q];
+    }
+    int32_t total;
+    int32_t place = block_exclusive_scan<THREADS, int32_t>(sum, total, scan_sm);
+    int32_t first[D];                                            // output position of the tile's first element of a digit
+    if (tile == 0) {
+        int32_t g = 0, gs[D];
+#pragma unroll
+        for (int q = 0; q < D; ++q) {
+            gs[q] = g;
+            g += owner ? (int32_t)ghist[d0 + q] : 0;
+        }
+        const int32_t bin = block_exclusive_scan<THREADS, int32_t>(g, total, scan_sm);
+#pragma unroll
+        for (int q = 0; q < D; ++q) first[q] = bin + gs[q];
+    }
+    if (owner) {
+        int32_t pl = place;
+#pragma unroll
+        for (int q = 0; q < D; ++q) {
+            start[d0 + q] = pl;
+            pl += cnt[q];
         }
     }
     __syncthreads();
+    // ---- the tile in digit order
 #pragma unroll
     for (int k = 0; k < kSortItems; ++k) {
-        const int64_t idx = wbase + k * 32 + lane;
-        if (idx < n) {
-            const int32_t pos = wc[warp][(key[k] >> shift) & (R - 1)] + rank[k];
-            keys_out[pos] = key[k];
-            vals_out[pos] = val[k];
+        const int i = w0 + k * 32 + lane;
+        if (i < tile_n) {
+            const uint32_t digit = (key[k] >> shift) & (R - 1);
+            const int pos = start[digit] + wc[warp * R + digit] + rank[k];
+            skey[pos] = key[k];
+            sval[pos] = val[k];
+        }
+    }
+    // ---- the chains of the thread's digits, the nearest tiles first
+    if (owner) {
+        if (tile > 0) {
+            int32_t before[D];
+            unsigned open = (1u << D) - 1;
+#pragma unroll
+            for (int q = 0; q < D; ++q) before[q] = 0;
+            constexpr int B = 8;                                 // tiles per round (16 and 32: no faster)
+            int spin = 0;
+            for (int p = tile - 1; open && p >= 0;) {
+                unsigned v[B][D];
+#pragma unroll
+                for (int b = 0; b < B; ++b) {
+                    const unsigned *src = state + (int64_t)max(p - b, 0) * R + d0;
+                    if constexpr (D == 4) {
+                        const uint4 x = __ldcv(reinterpret_cast<const uint4 *>(src));
+                        v[b][0] = x.x; v[b][1] = x.y; v[b][2] = x.z; v[b][3] = x.w;
+                    } else if constexpr (D == 2) {
+                        const uint2 x = __ldcv(reinterpret_cast<const uint2 *>(src));
+                        v[b][0] = x.x; v[b][1] = x.y;
+                    } else {
+                        v[b][0] = __ldcv(src);
+                    }
+                }
+                int went = 0;                                    // tiles of the batch that are behind us
+                bool ready = true;
+#pragma unroll
+                for (int b = 0; b < B; ++b) {
+#pragma unroll
+                    for (int q = 0; q < D; ++q) ready = ready && (v[b][q] != 0 || !((open >> q) & 1u));
+                    if (ready && open) {
+                        ++went;
+#pragma unroll
+                        for (int q = 0; q < D; ++q)
+                            if ((open >> q) & 1u) {
+                                if (v[b][q] & kPosFlag) {
+                                    before[q] += (int32_t)(v[b][q] & ~kPosFlag);
+                                    open &= ~(1u << q);
+                                } else {
+                                    before[q] += (int32_t)v[b][q] - 1;
+                                }
+                            }
+                    }
+                }
+                p -= went;
+                if (went) spin = 0;
+                else if (++spin > kChainSpinLimit) {
+                    if (status) atomicOr(reinterpret_cast<unsigned *>(status), E2EGREC_DEV_TIMEOUT);
+                    break;
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < D; ++q) first[q] = before[q];
+        }
+#pragma unroll
+        for (int q = 0; q < D; ++q)
+            *reinterpret_cast<volatile unsigned *>(&state[(int64_t)tile * R + d0 + q]) = kPosFlag | (unsigned)(first[q] + cnt[q]);
+        int32_t pl = place;
+#pragma unroll
+        for (int q = 0; q < D; ++q) {
+            gbase[d0 + q] = first[q] - pl;
+            pl += cnt[q];
+        }
+    }
+    __syncthreads();
+    constexpr int O = 8;                                         // elements per round: the look-ups of all are in flight
+    for (int i0 = threadIdx.x; i0 < tile_n; i0 += O * THREADS) {
+        uint32_t ky[O], v[O];
+        int32_t pos[O], row[O];
+#pragma unroll
+        for (int q = 0; q < O; ++q) {
+            const int i = i0 + q * THREADS;
+            pos[q] = -1;
+            row[q] = 0;
+            if (i < tile_n) {
+                ky[q] = skey[i];
+                v[q] = sval[i];
+                if (map.row_out) row[q] = __ldg(map.row_of + v[q]);
+                pos[q] = gbase[(ky[q] >> shift) & (R - 1)] + i;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < O; ++q) {
+            if ((uint32_t)pos[q] >= (uint32_t)n) continue;       // beyond the tile, or after a wait that ran out (flagged)
+            keys_out[pos[q]] = (int32_t)ky[q];
+            vals_out[pos[q]] = (ValT)v[q];
+            if (map.row_out) map.row_out[pos[q]] = row[q];
         }
     }
 }
@@ -231,75 +321,57 @@ static inline SortPlan sort_plan(int32_t cap_src)
     if (key_bits <= 16) return {8, 2};
     if (key_bits <= 20) return {10, 2};
     if (key_bits <= 24) return {8, 3};
-    if (key_bits <= 30) return {10, 3};
-    return {8, 4};
+    return {8, 4};                                // the scan state of a sort is kPassWords words per tile
 }
 
-// csc_col / csc_eid = columns and positions of the block entries ordered by (col, position).
+// Blocks of 512 threads where the array can fill the machine with their tiles (longer runs per digit on the way out),
+// of 256 below.  The line: 2 * 148 tiles of 8192.
+constexpr int64_t kSortWide = 2 * 148 * 512 * (int64_t)kSortItems;
 
-// Digit counts of a key array for every pass of the sort (what sort_pass_kernel needs beforehand).
-static __global__ void __launch_bounds__(256)
-key_hist_kernel(const int32_t *__restrict__ keys, const int32_t *__restrict__ counts, int bits, int passes,
-                unsigned *__restrict__ ghist)
-{
-    __shared__ unsigned h[kMaxPasses * kMaxRadix];
-    const int R = 1 << bits;
-    for (int d = threadIdx.x; d < passes * R; d += 256) h[d] = 0;
-    __syncthreads();
-    const int32_t n = counts[CNT_EDGES];
-    for (int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x; e < n; e += (int64_t)gridDim.x * 256) {
-        const int32_t c = keys[e];
-        for (int p = 0; p < passes; ++p) atomicAdd(&h[p * R + ((c >> (p * bits)) & (R - 1))], 1u);
-    }
-    __syncthreads();
-    for (int d = threadIdx.x; d < passes * R; d += 256)
-        if (h[d]) atomicAdd(&ghist[(d / R) * kMaxRadix + (d % R)], h[d]);
-}
-
-// Buffers of one sort: two ping-pong pairs, the digit counts of the whole array (filled before the sort) and
-// the per-tile digit counts (written before they are read: no zeroing needed).
-struct RadixScratch {
-    int32_t *keys[2], *vals[2];        // [n] each
-    unsigned *ghist;                   // [kMaxPasses x kMaxRadix]
-    int32_t *thist;                    // [tiles x radix], reused by every pass
-    int64_t tiles;
+// One sort's scratch in device memory: digit counts of the whole array per pass, one ticket per pass and the scan state
+// of every pass.  The counts and tickets must be zero before the kernel that fills the counts, the state of the live tiles
+// before the first pass.
+struct SortState {
+    unsigned *ghist;                   // [kMaxPasses x kMaxRadix], then kMaxPasses tickets
+    unsigned *state;                   // [passes][tiles][radix]
+    int64_t tiles;                     // tiles of kSortTile elements that the state was sized for
+    __host__ __device__ unsigned *tickets() const { return ghist + kMaxPasses * kMaxRadix; }
 };
+constexpr size_t kSortCountWords = kMaxPasses * kMaxRadix + 64;
+constexpr size_t sort_state_bytes(int64_t tiles) { return sizeof(unsigned) * (size_t)kPassWords * (size_t)tiles; }
 
-constexpr size_t radix_thist_bytes(int64_t tiles) { return sizeof(int32_t) * (size_t)kMaxRadix * (size_t)tiles; }
-
-template <int BITS>
-static inline void radix_pass(const int32_t *kin, const int32_t *vin, int32_t *counts, int n_tiles, int shift,
-                              const unsigned *ghist, int32_t *thist, int32_t *kout, int32_t *vout, cudaStream_t st)
+template <int BITS, int THREADS, typename ValT>
+static inline void launch_sort_pass(const int32_t *kin, const int32_t *vin, const int32_t *n_dev, int64_t cap, int32_t clamp_keys,
+                                    int32_t clamp_vals, int pass, const SortState &ss, int32_t *kout, ValT *vout, const SortMap &map,
+                                    int32_t *status, cudaStream_t st)
 {
-    const int hist_grid = n_tiles < 8 * 148 ? n_tiles : 8 * 148;
+    constexpr size_t smem = sort_smem_bytes<BITS, THREADS>();
+    auto kern = sort_pass_kernel<BITS, THREADS, ValT>;
+    if (smem > 48 * 1024) {
+        static bool set[64] = {};                                // per device; the attribute may be set twice by two threads
+        int dev = 0;
+        cudaGetDevice(&dev);
+        if (dev < 0 || dev >= 64 || !set[dev]) {
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (dev >= 0 && dev < 64) set[dev] = true;
+        }
+    }
+    const unsigned grid = (unsigned)ceil_div(cap > 0 ? cap : 1, (int64_t)THREADS * kSortItems);
     note_launch();
-    tile_hist_kernel<BITS><<<hist_grid, kSortThreads, 0, st>>>(kin, counts, shift, thist);
-    note_launch();
-    tile_scan_kernel<BITS><<<1 << BITS, kSortThreads, 0, st>>>(counts, thist);
-    note_launch();
-    sort_pass_kernel<BITS><<<n_tiles, kSortThreads, 0, st>>>(kin, vin, counts, shift, ghist, thist, kout, vout);
+    kern<<<grid, THREADS, smem, st>>>(kin, vin, n_dev, (int32_t)cap, clamp_keys, clamp_vals, pass * BITS, ss.ghist + pass * kMaxRadix,
+                                      ss.tickets() + pass, ss.state + (size_t)pass * ss.tiles * (1 << BITS), kout, vout, map, status);
 }
 
-// Sorts (keys, vals) by key, stable; vals == nullptr means "value = position".  counts[CNT_EDGES] holds the
-// number of elements (device).  ghist must already hold the digit counts.
-static inline void radix_sort_pairs(const int32_t *keys, const int32_t *vals, int32_t *counts, int64_t cap,
-                                    int32_t *keys_out, int32_t *vals_out, const SortPlan &sp, const RadixScratch &rs,
-                                    cudaStream_t st)
+template <typename ValT>
+static inline void sort_pass(const SortPlan &sp, const int32_t *kin, const int32_t *vin, const int32_t *n_dev, int64_t cap,
+                             int32_t clamp_keys, int32_t clamp_vals, int pass, const SortState &ss, int32_t *kout, ValT *vout,
+                             const SortMap &map, int32_t *status, cudaStream_t st)
 {
-    const int n_tiles = (int)ceil_div(cap > 0 ? cap : 1, kSortTile);
-    const int32_t *kin = keys;
-    const int32_t *vin = vals;
-    for (int p = 0; p < sp.passes; ++p) {
-        const bool last = p == sp.passes - 1;
-        int32_t *kout = last ? keys_out : rs.keys[p & 1];
-        int32_t *vout = last ? vals_out : rs.vals[p & 1];
-        if (sp.bits == 8)
-            radix_pass<8>(kin, vin, counts, n_tiles, p * sp.bits, rs.ghist + p * kMaxRadix, rs.thist, kout, vout, st);
-        else
-            radix_pass<10>(kin, vin, counts, n_tiles, p * sp.bits, rs.ghist + p * kMaxRadix, rs.thist, kout, vout, st);
-        kin = kout;
-        vin = vout;
-    }
+    const bool wide = cap >= kSortWide;
+    if (sp.bits == 8 && wide) launch_sort_pass<8, 512, ValT>(kin, vin, n_dev, cap, clamp_keys, clamp_vals, pass, ss, kout, vout, map, status, st);
+    else if (sp.bits == 8) launch_sort_pass<8, 256, ValT>(kin, vin, n_dev, cap, clamp_keys, clamp_vals, pass, ss, kout, vout, map, status, st);
+    else if (wide) launch_sort_pass<10, 512, ValT>(kin, vin, n_dev, cap, clamp_keys, clamp_vals, pass, ss, kout, vout, map, status, st);
+    else launch_sort_pass<10, 256, ValT>(kin, vin, n_dev, cap, clamp_keys, clamp_vals, pass, ss, kout, vout, map, status, st);
 }
 
 }  // namespace e2egrec

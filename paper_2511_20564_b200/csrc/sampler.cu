@@ -43,10 +43,8 @@ constexpr int kWordTile = 2048;        // bitmap words per block of the frontier
 // transposition of hop h can run beside the sampling of hop h+1.
 struct SortLane {
     int32_t  *edge_row;    // [max cap_edges]   destination of each block entry
-    int32_t  *keys[2];     // [max cap_edges]   radix sort ping-pong
-    int32_t  *vals[2];
-    unsigned *ghist;                   // [kMaxPasses x kMaxRadix] digit counts of the whole key array (zeroed before relabel)
-    int32_t  *thist;                   // [sort tiles x kMaxRadix] digit counts per tile of the pass that runs
+    int32_t  *key, *val;   // [max cap_edges]   the passes alternate between these and the block's arrays
+    SortState sort;        // counts and tickets zeroed before relabel, which zeroes the live tiles' scan state
 };
 
 struct SamplerScratch {
@@ -60,7 +58,6 @@ struct SamplerScratch {
     unsigned long long *state_dst;     // [dst tiles]
     unsigned long long *state_words;   // [word tiles]
     SortLane  lane[kMaxHops];
-    int64_t   sort_tiles;
     size_t    bytes;
     int64_t   n_words;
 };
@@ -76,7 +73,7 @@ static SamplerScratch carve(int64_t n_nodes, int64_t max_dst, int64_t max_src, i
         off += align_up(bytes, 256);
         return p;
     };
-    s.sort_tiles = ceil_div(max_edges > 0 ? max_edges : 1, kSortTile);
+    const int64_t sort_tiles = ceil_div(max_edges > 0 ? max_edges : 1, kSortTile);
     s.step_offset = (uint32_t *)take(256);
     s.local_id = (int32_t *)take(sizeof(int32_t) * (size_t)n_nodes);
     s.bitmap = (uint32_t *)take(sizeof(uint32_t) * (size_t)s.n_words);
@@ -89,10 +86,11 @@ static SamplerScratch carve(int64_t n_nodes, int64_t max_dst, int64_t max_src, i
     for (int h = 0; h < kMaxHops; ++h) {
         SortLane &l = s.lane[h];
         l.edge_row = (int32_t *)take(sizeof(int32_t) * (size_t)(max_edges + 1));
-        for (int i = 0; i < 2; ++i) l.keys[i] = (int32_t *)take(sizeof(int32_t) * (size_t)(max_edges + 1));
-        for (int i = 0; i < 2; ++i) l.vals[i] = (int32_t *)take(sizeof(int32_t) * (size_t)(max_edges + 1));
-        l.ghist = (unsigned *)take(sizeof(unsigned) * kMaxPasses * kMaxRadix);
-        l.thist = (int32_t *)take(radix_thist_bytes(s.sort_tiles));
+        l.key = (int32_t *)take(sizeof(int32_t) * (size_t)(max_edges + 1));
+        l.val = (int32_t *)take(sizeof(int32_t) * (size_t)(max_edges + 1));
+        l.sort.ghist = (unsigned *)take(sizeof(unsigned) * kSortCountWords);
+        l.sort.tiles = sort_tiles;
+        l.sort.state = (unsigned *)take(sort_state_bytes(sort_tiles));
     }
     s.bytes = off;
     return s;
@@ -317,12 +315,22 @@ frontier_kernel(uint32_t *__restrict__ bitmap, int64_t n_words, int32_t *__restr
     }
 }
 
-// col[e] = position of the sampled node in the frontier, and the digit counts of the whole col array
-// for every pass of the radix sort that follows.
+// Scan state of the tiles that a sort of n keys will use, zeroed by the whole grid.
+__device__ inline void zero_sort_state(const SortState &ss, int64_t n, int bits, int passes)
+{
+    const int64_t words = ((n + kSortTile - 1) / kSortTile) << bits;
+    for (int p = 0; p < passes; ++p) {
+        uint4 *dst = reinterpret_cast<uint4 *>(ss.state + ((size_t)p * ss.tiles << bits));
+        for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < words / 4; i += (int64_t)gridDim.x * blockDim.x)
+            dst[i] = make_uint4(0, 0, 0, 0);
+    }
+}
+
+// col[e] = position of the sampled node in the frontier, the digit counts of the whole col array for every pass of the
+// radix sort that follows, and that sort's scan state.
 __global__ void __launch_bounds__(256)
 relabel_kernel(const int32_t *__restrict__ nbr_global, const int32_t *__restrict__ local_id,
-               const int32_t *__restrict__ counts, int32_t *__restrict__ col, int bits, int passes,
-               unsigned *__restrict__ ghist)
+               const int32_t *__restrict__ counts, int32_t *__restrict__ col, int bits, int passes, SortState ss)
 {
     __shared__ unsigned h[kMaxPasses * kMaxRadix];
     const int R = 1 << bits;
@@ -338,7 +346,8 @@ relabel_kernel(const int32_t *__restrict__ nbr_global, const int32_t *__restrict
     }
     __syncthreads();
     for (int d = threadIdx.x; d < passes * R; d += 256)
-        if (h[d]) atomicAdd(&ghist[(d / R) * kMaxRadix + (d % R)], h[d]);
+        if (h[d]) atomicAdd(&ss.ghist[(d / R) * kMaxRadix + (d % R)], h[d]);
+    zero_sort_state(ss, n, bits, passes);
 }
 
 __global__ void frontier_release_kernel(const int32_t *__restrict__ src_nodes, const int32_t *__restrict__ counts,
@@ -348,22 +357,32 @@ __global__ void frontier_release_kernel(const int32_t *__restrict__ src_nodes, c
     if (i < counts[CNT_SRC]) local_id[src_nodes[i]] = -1;
 }
 
-// csc_ptr[s] = first position whose column is >= s (the columns are sorted), and the destination of
-// every transposed entry.
-__global__ void csc_finalize_kernel(const int32_t *__restrict__ csc_col, const int32_t *__restrict__ csc_eid,
-                                    const int32_t *__restrict__ edge_row, const int32_t *__restrict__ counts,
-                                    int32_t *__restrict__ csc_ptr, int32_t *__restrict__ csc_row)
+// csc_ptr[s] = first position whose column is >= s, from the steps of the sorted column array (a search per column cost 20
+// scattered reads each).  Leaves the sort's tickets and scan state
+// zero again, so that a block can be transposed any number of times.
+__global__ void csc_finalize_kernel(const int32_t *__restrict__ csc_col, const int32_t *__restrict__ counts,
+                                    int32_t *__restrict__ csc_ptr, SortState ss, int bits, int passes)
 {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    zero_sort_state(ss, counts[CNT_EDGES], bits, passes);
+    if (blockIdx.x == 0 && threadIdx.x < kMaxPasses) ss.tickets()[threadIdx.x] = 0;
     const int32_t n = counts[CNT_EDGES], n_src = counts[CNT_SRC];
-    if (t < n) csc_row[t] = edge_row[csc_eid[t]];
-    if (t <= n_src) {
-        int32_t lo = 0, hi = n;                      // lower bound of t in csc_col[0..n)
-        while (lo < hi) {
-            const int32_t mid = (lo + hi) >> 1;
-            if (csc_col[mid] < (int32_t)t) lo = mid + 1; else hi = mid;
+    const int lane = threadIdx.x & 31;
+    for (int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane; t0 <= n; t0 += (int64_t)gridDim.x * blockDim.x) {
+        // position t is the first one whose column is >= s for the columns s in (col[t - 1], col[t]]
+        const int32_t t = (int32_t)min(t0 + lane, (int64_t)n + 1);
+        int32_t a = n_src, b = n_src;
+        if (t <= n) {
+            a = t > 0 ? csc_col[t - 1] : -1;
+            b = t < n ? csc_col[t] : n_src;
         }
-        csc_ptr[t] = lo;
+        const bool wide = b - a > 4;                 // columns without entries: the warp fills long stretches together
+        if (!wide)
+            for (int32_t s = a + 1; s <= b; ++s) csc_ptr[s] = t;
+        for (unsigned m = __ballot_sync(0xffffffffu, wide); m; m &= m - 1) {
+            const int l = __ffs(m) - 1;
+            const int32_t wa = __shfl_sync(0xffffffffu, a, l), wb = __shfl_sync(0xffffffffu, b, l), wt = __shfl_sync(0xffffffffu, t, l);
+            for (int32_t s = wa + 1 + lane; s <= wb; s += 32) csc_ptr[s] = wt;
+        }
     }
 }
 
@@ -389,7 +408,7 @@ __global__ void __launch_bounds__(256)
 pair_local_kernel(const int32_t *__restrict__ user, const int32_t *__restrict__ item, int32_t n_pairs, int64_t n_nodes,
                   const int32_t *__restrict__ local_id, int32_t *__restrict__ pair_local,
                   int32_t *__restrict__ entry_unit, int units_per_row, int item_unit_off, int32_t *__restrict__ pcounts,
-                  int bits, int passes, unsigned *__restrict__ ghist)
+                  int bits, int passes, SortState ss)
 {
     __shared__ unsigned h[kMaxPasses * kMaxRadix];
     const int R = 1 << bits;
@@ -408,19 +427,26 @@ pair_local_kernel(const int32_t *__restrict__ user, const int32_t *__restrict__ 
     }
     __syncthreads();
     for (int d = threadIdx.x; d < passes * R; d += 256)
-        if (h[d]) atomicAdd(&ghist[(d / R) * kMaxRadix + (d % R)], h[d]);
+        if (h[d]) atomicAdd(&ss.ghist[(d / R) * kMaxRadix + (d % R)], h[d]);
+    zero_sort_state(ss, 2 * (int64_t)n_pairs, bits, passes);
 }
 
-static void sort_by_col(const int32_t *col, int32_t *counts, int32_t cap_edges, int32_t *csc_col, int32_t *csc_eid,
-                        const SortPlan &sp, const SortLane &l, int64_t sort_tiles, cudaStream_t st)
+// The transposed block: entries ordered by (column, position), the last pass looking up every entry's row, and the offsets.
+static void transpose_block(const int32_t *col, int32_t *counts, int32_t cap_edges, const int32_t *row_of,
+                            int32_t *csc_col, int32_t *csc_eid, int32_t *csc_row, int32_t *csc_ptr, const SortPlan &sp,
+                            const SortLane &l, cudaStream_t st)
 {
-    RadixScratch rs{};
-    rs.keys[0] = l.keys[0]; rs.keys[1] = l.keys[1];
-    rs.vals[0] = l.vals[0]; rs.vals[1] = l.vals[1];
-    rs.ghist = l.ghist;
-    rs.thist = l.thist;
-    rs.tiles = sort_tiles;
-    radix_sort_pairs(col, nullptr, counts, cap_edges, csc_col, csc_eid, sp, rs, st);
+    const int32_t *k = col, *v = nullptr;
+    for (int p = 0; p < sp.passes; ++p) {
+        const bool last = p == sp.passes - 1, own = (sp.passes - 1 - p) % 2 == 0;       // the last pass ends in the block's arrays
+        int32_t *ko = own ? csc_col : l.key, *vo = own ? csc_eid : l.val;
+        sort_pass<int32_t>(sp, k, v, &counts[CNT_EDGES], cap_edges, 0, 0, p, l.sort, ko, vo, last ? SortMap{row_of, csc_row} : SortMap{},
+                           &counts[CNT_STATUS], st);
+        k = ko;
+        v = vo;
+    }
+    note_launch();
+    csc_finalize_kernel<<<(unsigned)std::min<int64_t>(ceil_div((int64_t)cap_edges + 1, 256), 148 * 8), 256, 0, st>>>(csc_col, counts, csc_ptr, l.sort, sp.bits, sp.passes);
 }
 
 static inline unsigned grid_for(int64_t n, int threads) { return (unsigned)ceil_div(n > 0 ? n : 1, threads); }
@@ -580,6 +606,10 @@ int32_t e2egrec::sample_khop_impl(const e2egrec_csr *graph, const int32_t *seeds
 
     const int T = 256;
     const int64_t n = graph->n_nodes;
+    // The transposition of a hop (sort + offsets) is only needed by the backward pass, so it runs on the
+    // helper stream beside the sampling of the next hop; everything is joined before this call returns.
+    SideStream *side = SideStream::get(st);
+    if (side) side->join_pending(st);               // a transposition deferred by an earlier call still uses the lanes
     tap_begin(TAP_SAMPLE, st);
     const int32_t *dst_nodes = seeds;
     const int32_t *n_dst_ptr = &blocks[0].counts[CNT_DST];
@@ -600,22 +630,15 @@ int32_t e2egrec::sample_khop_impl(const e2egrec_csr *graph, const int32_t *seeds
                                                                         pi.seeds_out, s.tickets + 1, s.state_words);
         const SortPlan sp = sort_plan(P2 > 1 ? P2 : 2);
         const SortLane &l = s.lane[0];
-        cudaMemsetAsync(l.ghist, 0, sizeof(unsigned) * kMaxPasses * kMaxRadix, st);
+        cudaMemsetAsync(l.sort.ghist, 0, sizeof(unsigned) * kSortCountWords, st);
         note_launch();
         pair_local_kernel<<<(unsigned)std::min<int64_t>(grid_for(P2, T), 148 * 4), T, 0, st>>>(
             pi.user, pi.item, pi.n_pairs, n, s.local_id, pi.pair_local, pi.entry_unit, pi.units_per_row, pi.item_unit_off,
-            pi.pcounts, sp.bits, sp.passes, l.ghist);
-        sort_by_col(pi.pair_local, pi.pcounts, P2, pi.pcsc_col, pi.pcsc_eid, sp, l, s.sort_tiles, st);
-        note_launch();
-        csc_finalize_kernel<<<grid_for((int64_t)P2 + 1, T), T, 0, st>>>(pi.pcsc_col, pi.pcsc_eid, pi.entry_unit, pi.pcounts,
-                                                                       pi.pcsc_ptr, pi.pcsc_idx);
+            pi.pcounts, sp.bits, sp.passes, l.sort);
+        transpose_block(pi.pair_local, pi.pcounts, P2, pi.entry_unit, pi.pcsc_col, pi.pcsc_eid, pi.pcsc_idx, pi.pcsc_ptr, sp, l, st);
         dst_nodes = pi.seeds_out;
         n_dst_ptr = &pi.pcounts[CNT_SRC];
     }
-    // The transposition of a hop (sort + offsets) is only needed by the backward pass, so it runs on the
-    // helper stream beside the sampling of the next hop; everything is joined before this call returns.
-    SideStream *side = SideStream::get(st);
-    if (side) side->join_pending(st);               // a transposition deferred by an earlier call still uses the lanes
     for (int h = 0; h < n_hops; ++h) {
         const e2egrec_block &b = blocks[h];
         const int32_t f = fanouts[h];
@@ -631,20 +654,17 @@ int32_t e2egrec::sample_khop_impl(const e2egrec_csr *graph, const int32_t *seeds
         frontier_kernel<<<grid_for(s.n_words, kWordTile), 256, 0, st>>>(s.bitmap, s.n_words, b.counts, b.cap_src,
                                                                         s.local_id, b.src_nodes, s.tickets + 1,
                                                                         s.state_words);
-        cudaMemsetAsync(l.ghist, 0, sizeof(unsigned) * kMaxPasses * kMaxRadix, st);
+        cudaMemsetAsync(l.sort.ghist, 0, sizeof(unsigned) * kSortCountWords, st);
         note_launch();
         relabel_kernel<<<(unsigned)std::min<int64_t>(grid_for(b.cap_edges, T), 148 * 4), T, 0, st>>>(
-            b.nbr_global, s.local_id, b.counts, b.col, sp.bits, sp.passes, l.ghist);
+            b.nbr_global, s.local_id, b.counts, b.col, sp.bits, sp.passes, l.sort);
         if (!(flags & E2EGREC_SAMPLE_NO_TRANSPOSE)) {
             cudaStream_t ts = st;                    // stream of the transposition
             if (side) {
                 side->fork(st);
                 ts = side->stream;
             }
-            sort_by_col(b.col, b.counts, b.cap_edges, b.csc_col, b.csc_eid, sp, l, s.sort_tiles, ts);
-            note_launch();
-            csc_finalize_kernel<<<grid_for(std::max<int64_t>(b.cap_edges, (int64_t)b.cap_src + 1), T), T, 0, ts>>>(
-                b.csc_col, b.csc_eid, l.edge_row, b.counts, b.csc_ptr, b.csc_row);
+            transpose_block(b.col, b.counts, b.cap_edges, l.edge_row, b.csc_col, b.csc_eid, b.csc_row, b.csc_ptr, sp, l, ts);
         }
         dst_nodes = b.src_nodes;
         n_dst_ptr = &b.counts[CNT_SRC];
@@ -683,7 +703,6 @@ extern "C" int32_t e2egrec_blocks_transpose(int64_t n_nodes, int32_t n_hops, con
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     SideStream *side = SideStream::get(st);
     if (side) side->join_pending(st);
-    const int T = 256;
     const bool forked = side && n_hops > 1;
     if (forked) side->fork(st);
     for (int h = n_hops - 1; h >= 0; --h) {          // the largest block first, on the caller's stream
@@ -692,10 +711,7 @@ extern "C" int32_t e2egrec_blocks_transpose(int64_t n_nodes, int32_t n_hops, con
         const SortLane &l = s.lane[h];
         cudaStream_t ts = st;
         if (forked && ((n_hops - 1 - h) & 1)) ts = side->stream;
-        sort_by_col(b.col, b.counts, b.cap_edges, b.csc_col, b.csc_eid, sp, l, s.sort_tiles, ts);
-        note_launch();
-        csc_finalize_kernel<<<grid_for(std::max<int64_t>(b.cap_edges, (int64_t)b.cap_src + 1), T), T, 0, ts>>>(
-            b.csc_col, b.csc_eid, l.edge_row, b.counts, b.csc_ptr, b.csc_row);
+        transpose_block(b.col, b.counts, b.cap_edges, l.edge_row, b.csc_col, b.csc_eid, b.csc_row, b.csc_ptr, sp, l, ts);
     }
     if (forked) side->join(st);
     return check_launch("blocks_transpose");

@@ -1,0 +1,66 @@
+"""The radix sort behind graph ingest and block transposition at its edges: one element, tiles that are full, one short and
+one over, both tile sizes, every number of digits and passes, one key for all elements, keys out of range."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+import paper_2511_20564_b200 as E  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+def check_ingest(n, row, col):
+    ptr, idx, bad = E.graph_from_coo(n, torch.from_numpy(row).cuda(), torch.from_numpy(col).cuda())
+    order = np.lexsort((col, row))
+    want_ptr = np.zeros(n + 1, np.int64)
+    np.cumsum(np.bincount(row, minlength=n), out=want_ptr[1:])
+    assert int(bad) == 0
+    assert np.array_equal(ptr.cpu().numpy(), want_ptr) and np.array_equal(idx.cpu().numpy(), col[order])
+    cptr, crow, ceid, bad = E.csr_transpose(ptr, idx, n)
+    back = np.argsort(col[order], kind="stable")
+    np.cumsum(np.bincount(col, minlength=n), out=want_ptr[1:])
+    assert int(bad) == 0
+    assert np.array_equal(cptr.cpu().numpy(), want_ptr) and np.array_equal(ceid.cpu().numpy(), back)
+    assert np.array_equal(crow.cpu().numpy(), row[order][back])
+
+
+@pytest.mark.parametrize("m", [1, 31, 4095, 4096, 4097, 8193, 70_001])
+@pytest.mark.parametrize("n", [1, 200, 1024, 60_000, 1_000_000, 9_000_000, 20_000_000])
+def test_sizes(m, n):
+    rng = np.random.default_rng(m + n)
+    check_ingest(n, rng.integers(0, n, m).astype(np.int32), (n * rng.random(m) ** 4).astype(np.int32))
+
+
+@pytest.mark.parametrize("m", [2 * 148 * 8192 - 1, 2 * 148 * 8192 + 8191])
+def test_line_between_the_tile_sizes(m):
+    rng = np.random.default_rng(m)
+    row, col = rng.integers(0, 300_000, m).astype(np.int32), (300_000 * rng.random(m) ** 6).astype(np.int32)
+    check_ingest(300_000, row, col)
+    check_ingest(300_000, np.full(m, 299_999, np.int32), col)
+
+
+def test_ids_out_of_range_are_flagged_and_count_as_zero():
+    row, col = np.array([5, -1, 2, 7], np.int32), np.array([1, 2, 9, 3], np.int32)
+    ptr, idx, bad = E.graph_from_coo(8, torch.from_numpy(row).cuda(), torch.from_numpy(col).cuda())
+    assert int(bad) != 0
+    assert ptr.cpu().tolist() == [0, 1, 1, 2, 2, 2, 3, 3, 4] and idx.cpu().tolist() == [2, 0, 1, 3]
+
+
+def test_blocks_can_be_transposed_again():
+    rng = np.random.default_rng(3)
+    n, m = 50_000, 400_000
+    ids = [torch.from_numpy((n * rng.random(m) ** 3).astype(np.int32)).cuda() for _ in range(2)]
+    ptr, idx, _ = E.graph_from_coo(n, *ids)
+    seeds = torch.arange(0, 3000, dtype=torch.int32, device="cuda")
+    got = []
+    for again in (0, 1, 2):
+        b = E.Blocks(n, 3000, [12, 7], "cuda")
+        E.sample_khop(ptr, idx, seeds, b, 11, 4, transpose=again == 0)
+        for _ in range(again):
+            E.blocks_transpose(b)
+        torch.cuda.synchronize()
+        c = b.counts.cpu().numpy()
+        got.append([t[k][:e].cpu().numpy() for t, row in zip(b.t, c)
+                    for k, e in (("csc_ptr", row[1] + 1), ("csc_row", row[2]), ("csc_eid", row[2]), ("csc_col", row[2]))])
+    for other in got[1:]:
+        assert all(np.array_equal(a, b) for a, b in zip(got[0], other))
