@@ -474,6 +474,14 @@ int32_t run_joint(const JointPlan &jp, const e2egrec_csr *graph, const e2egrec_m
         if (phase == E2EGREC_JOINT_SAMPLE) return check_launch("joint_step(sample)");
     }
 
+    // the groups of the pairs' entries are ready on the helper stream (a whole step: nothing has been joined yet)
+    SideStream *side = SideStream::get(st);
+    cudaEvent_t grouped = nullptr;
+    if (side && phase == E2EGREC_JOINT_WHOLE) {
+        grouped = side->event();
+        cudaEventRecord(grouped, side->stream);
+    }
+
     // 2. encoder forward: embeddings of the seeds
     e2egrec_mat Hs{tp(jp.hseed_off), pad128(jp.cd[0]), jp.dL, jp.dL, X->dtype};
     size_t ctx_bytes = jp.ctx_bytes;
@@ -521,7 +529,6 @@ int32_t run_joint(const JointPlan &jp, const e2egrec_csr *graph, const e2egrec_m
     }
     // the weight gradients feed nothing later in the step: they go to the helper stream (behind the block
     // transposition that the sampler left there); the encoder backward waits for that stream before its first launch
-    SideStream *side = SideStream::get(st);
     cudaStream_t ws_st = st;
     if (side) {
         side->fork(st);
@@ -549,6 +556,7 @@ int32_t run_joint(const JointPlan &jp, const e2egrec_csr *graph, const e2egrec_m
 
     // 5. gradient of every seed embedding: the rows of dz that belong to it, added in pair order
     {
+        if (grouped) cudaStreamWaitEvent(st, grouped, 0);
         SegOut<T> o{};
         o.out = tp(jp.dhseed_off);
         o.ld_out = jp.dL;

@@ -28,40 +28,46 @@ __device__ inline unsigned long long chain_read(const unsigned long long *slot)
     return *reinterpret_cast<const volatile unsigned long long *>(slot);
 }
 
-// Called by all threads of the block.  Returns the sum of the aggregates of tiles 0 .. tile-1.
+// One thread of the block publishes the tile's own sum as soon as it is known ...
+__device__ inline void chain_publish(unsigned long long *state, int tile, long long aggregate)
+{
+    atomicExch(&state[tile], (tile == 0 ? kChainPrefix : kChainAgg) | (unsigned long long)aggregate);
+}
+
+// ... and later all threads of the block ask for the sum of the tiles before it.  A round of the first warp reads
+// 4 x 32 tiles: where all tiles of a launch start together none has its prefix yet, and rounds are what the far ones pay.
 __device__ inline long long chain_lookback(unsigned long long *state, int tile, long long aggregate, int32_t *status,
                                            long long *bcast)
 {
     if (threadIdx.x < 32) {
         const int lane = threadIdx.x;
         long long excl = 0;
-        if (lane == 0) atomicExch(&state[tile], (tile == 0 ? kChainPrefix : kChainAgg) | (unsigned long long)aggregate);
         if (tile > 0) {
-            int p = tile - 1;
             bool done = false;
-            while (!done) {
-                const int idx = p - lane;
-                unsigned long long v = kChainPrefix;                 // before tile 0: an empty prefix
-                bool timed_out = false;
-                for (int spin = 0;; ++spin) {
-                    if (idx >= 0) v = chain_read(&state[idx]);
-                    if (__all_sync(0xffffffffu, (v >> 62) != 0)) break;
-                    if (spin >= kChainSpinLimit) { timed_out = true; break; }
-                }
-                timed_out = __any_sync(0xffffffffu, timed_out);
-                const unsigned pref = __ballot_sync(0xffffffffu, (v >> 62) == 2);
-                const int first = pref ? __ffs(pref) - 1 : 31;
-                long long c = lane <= first ? (long long)(v & kChainMask) : 0;
+            for (int p = tile - 1; !done; p -= 128) {
+                unsigned long long v[4];
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-                excl += c;
-                if (timed_out) {
-                    if (lane == 0) atomicOr(reinterpret_cast<unsigned *>(status), E2EGREC_DEV_TIMEOUT);
-                    done = true;
-                } else if (pref) {
-                    done = true;
-                } else {
-                    p -= 32;
+                for (int j = 0; j < 4; ++j) {
+                    const int idx = p - 32 * j - lane;
+                    v[j] = idx >= 0 ? chain_read(&state[idx]) : kChainPrefix;    // before tile 0: an empty prefix
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (done) break;
+                    const int idx = p - 32 * j - lane;
+                    bool timed_out = false;
+                    for (int spin = 0; !__all_sync(0xffffffffu, (v[j] >> 62) != 0); ++spin) {
+                        if (spin >= kChainSpinLimit) { timed_out = true; break; }
+                        if (idx >= 0) v[j] = chain_read(&state[idx]);
+                    }
+                    const unsigned pref = __ballot_sync(0xffffffffu, (v[j] >> 62) == 2);
+                    const int first = pref ? __ffs(pref) - 1 : 31;
+                    long long c = lane <= first ? (long long)(v[j] & kChainMask) : 0;
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+                    excl += c;
+                    if (timed_out && lane == 0) atomicOr(reinterpret_cast<unsigned *>(status), E2EGREC_DEV_TIMEOUT);
+                    done = timed_out || pref != 0;
                 }
             }
             if (lane == 0) atomicExch(&state[tile], kChainPrefix | (unsigned long long)(excl + aggregate));

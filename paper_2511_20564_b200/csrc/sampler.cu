@@ -35,9 +35,21 @@ __device__ inline uint4 philox4x32_10(uint4 c, uint2 k)
 // ---------------------------------------------------------------------------------------
 // Scratch layout (host and device agree through this struct).
 // ---------------------------------------------------------------------------------------
-constexpr int kDstTile = 64;           // destinations per block of the sampling kernel
+constexpr int kDstTile = 64;           // most destinations per block of the sampling kernel
+constexpr int kDstTileMin = 4;
 constexpr int kDstThreads = 256;       // its threads: one per destination for the counts, then all of them draw
-constexpr int kWordTile = 2048;        // bitmap words per block of the frontier kernel
+constexpr int kWordTile = 512;         // bitmap words per block of the frontier kernel (2048: 8 blocks on 500 k nodes)
+
+// Destinations per block: about 1024 slots, four per thread, where that gives two blocks per SM and more; about 256 below,
+// where the time is that of one block's chain of loads.  With 64 destinations whatever the fanout, 4096 seeds at fanout
+// 100 were 64 blocks of 25 slots per thread.
+static inline int dst_tile(int32_t cap_dst, int32_t fanout)
+{
+    const int64_t slots = (int64_t)cap_dst * fanout >= 2 * 148 * 1024 ? 1024 : 256;
+    int t = kDstTileMin;
+    while (t < kDstTile && 2ll * t * fanout <= slots) t *= 2;
+    return t;
+}
 
 // Everything one block transposition (radix sort by column + offsets) needs; one lane per hop, so that the
 // transposition of hop h can run beside the sampling of hop h+1.
@@ -51,12 +63,12 @@ struct SamplerScratch {
     uint32_t *step_offset; // [1]         added to the `step` argument of every call (see e2egrec_sampler_set_step)
     int32_t  *local_id;    // [n_nodes]   -1 when idle, else position in the current frontier
     uint32_t *bitmap;      // [n_words]   newly reached nodes of the hop in progress; 0 when idle
-    // chain arena of the sampling / frontier kernels, zeroed at the start of every hop
-    char     *arena;
-    size_t    arena_bytes;
-    unsigned *tickets;                 // [2]
-    unsigned long long *state_dst;     // [dst tiles]
-    unsigned long long *state_words;   // [word tiles]
+    // everything from here to the chain states' used end is zeroed by the first kernel of a call
+    char     *zero;
+    unsigned *tickets;                 // [2 per hop, 1 for the seeds of a joint step]
+    unsigned *ghist[kMaxHops];         // digit counts and tickets of the lanes' sorts
+    unsigned long long *chain;         // per frontier (seeds of a joint step, hops): word tiles; then per hop: dst tiles
+    int64_t   word_tiles;
     SortLane  lane[kMaxHops];
     size_t    bytes;
     int64_t   n_words;
@@ -77,18 +89,18 @@ static SamplerScratch carve(int64_t n_nodes, int64_t max_dst, int64_t max_src, i
     s.step_offset = (uint32_t *)take(256);
     s.local_id = (int32_t *)take(sizeof(int32_t) * (size_t)n_nodes);
     s.bitmap = (uint32_t *)take(sizeof(uint32_t) * (size_t)s.n_words);
-    size_t begin = off;
-    s.arena = base ? static_cast<char *>(base) + off : nullptr;
+    s.word_tiles = ceil_div(s.n_words > 0 ? s.n_words : 1, kWordTile);
+    s.zero = base ? static_cast<char *>(base) + off : nullptr;
     s.tickets = (unsigned *)take(256);
-    s.state_dst = (unsigned long long *)take(8 * (size_t)(ceil_div(max_dst > 0 ? max_dst : 1, kDstTile) + 1));
-    s.state_words = (unsigned long long *)take(8 * (size_t)(ceil_div(s.n_words > 0 ? s.n_words : 1, kWordTile) + 1));
-    s.arena_bytes = off - begin;
+    for (int h = 0; h < kMaxHops; ++h) s.ghist[h] = (unsigned *)take(sizeof(unsigned) * kSortCountWords);
+    s.chain = (unsigned long long *)take(
+        8 * (size_t)((kMaxHops + 1) * s.word_tiles + kMaxHops * (ceil_div(max_dst > 0 ? max_dst : 1, kDstTileMin) + 1)));
     for (int h = 0; h < kMaxHops; ++h) {
         SortLane &l = s.lane[h];
         l.edge_row = (int32_t *)take(sizeof(int32_t) * (size_t)(max_edges + 1));
         l.key = (int32_t *)take(sizeof(int32_t) * (size_t)(max_edges + 1));
         l.val = (int32_t *)take(sizeof(int32_t) * (size_t)(max_edges + 1));
-        l.sort.ghist = (unsigned *)take(sizeof(unsigned) * kSortCountWords);
+        l.sort.ghist = s.ghist[h];
         l.sort.tiles = sort_tiles;
         l.sort.state = (unsigned *)take(sort_state_bytes(sort_tiles));
     }
@@ -105,32 +117,45 @@ __global__ void fill_i32_kernel(int32_t *p, int64_t n, int32_t v)
         p[i] = v;
 }
 
-// Seeds become the first frontier: local id = position in the batch.
-__global__ void seed_init_kernel(const int32_t *__restrict__ seeds, int32_t n_seeds, int64_t n_nodes,
-                                 int32_t *__restrict__ local_id, int32_t *counts0)
+// First kernel of a call: clears the tickets, digit counts and chain states of all hops (one launch instead of two memsets
+// per hop) and, with seeds, makes them the first frontier: local id = position in the batch.  counts1 (joint step): a second
+// set of counters to clear.
+__global__ void __launch_bounds__(256)
+sample_begin_kernel(uint4 *__restrict__ zero, int64_t zero16, const int32_t *__restrict__ seeds, int32_t n_seeds, int64_t n_nodes,
+                    int32_t *__restrict__ local_id, int32_t *counts0, int32_t *counts1)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, all = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t k = i; k < zero16; k += all) zero[k] = make_uint4(0, 0, 0, 0);
     if (i == 0) {
-        counts0[CNT_DST] = n_seeds;
+        counts0[CNT_DST] = seeds ? n_seeds : 0;
         counts0[CNT_STATUS] = 0;
+        if (counts1) *reinterpret_cast<int4 *>(counts1) = make_int4(0, 0, 0, 0);
     }
-    if (i >= n_seeds) return;
-    const int32_t u = seeds[i];
-    if ((uint32_t)u < (uint64_t)n_nodes) local_id[u] = i;
+    if (!seeds) return;
+    for (int64_t k = i; k < n_seeds; k += all) {
+        const int32_t u = seeds[k];
+        if ((uint32_t)u < (uint64_t)n_nodes) local_id[u] = (int32_t)k;
+    }
 }
 
-// One hop of sampling in one launch.  A block owns kDstTile destinations: |S(u)| = min(deg, fanout) per
+// One hop of sampling in one launch.  A block owns `tile_dst` destinations: |S(u)| = min(deg, fanout) per
 // destination, a chained scan for the block's offset into the entry arrays, then one thread per
 // (destination, slot).  Slot j of node u at hop h draws with the counter (j/2, u, (1<<8)|h, step) and
 // key (seed lo, seed hi); words 2(j%2), 2(j%2)+1 form r and the picked row position is
 // floor(r * deg / 2^64); with running sums of integer edge weights (g_cum) it is the first entry of the row
 // whose running sum exceeds floor(r * total / 2^64).  deg <= fanout copies the row instead.  Sampled nodes
 // that are not yet in the frontier are marked in the bitmap.
+//
+// Latency is what it costs: a dozen dependent loads per block.  The block's sum is published before the draws and the
+// offset asked for after them, so that the chain moves meanwhile; four slots per thread keep their loads in flight together,
+// and a weighted draw narrows its row to a quarter per step with the three probes of all four slots in flight (one slot
+// after the other by halves: 154 us for 4096 seeds x 100, now 28).
+template <bool kWeighted>
 __global__ void __launch_bounds__(kDstThreads)
 hop_sample_kernel(const int64_t *__restrict__ g_indptr, const int32_t *__restrict__ g_indices,
                   const uint64_t *__restrict__ g_cum, int64_t n_nodes,
                   const int32_t *__restrict__ dst_nodes, const int32_t *n_dst_ptr, int32_t cap_dst, int32_t cap_edges,
-                  int32_t fanout, int32_t hop, uint32_t seed_lo, uint32_t seed_hi, uint32_t step_arg,
+                  int32_t fanout, int32_t tile_dst, int32_t hop, uint32_t seed_lo, uint32_t seed_hi, uint32_t step_arg,
                   const uint32_t *__restrict__ step_offset, int first_hop, int32_t *__restrict__ counts,
                   int32_t *__restrict__ blk_indptr, float *__restrict__ inv_cnt, int32_t *__restrict__ src_nodes,
                   int32_t *__restrict__ nbr_global, int32_t *__restrict__ edge_row,
@@ -144,8 +169,9 @@ hop_sample_kernel(const int64_t *__restrict__ g_indptr, const int32_t *__restric
     __shared__ int32_t scan_sm[kDstThreads / 32 + 1];
     __shared__ long long bcast;
     __shared__ int tile_s;
+    int32_t n_dst = *n_dst_ptr;                      // on their way while the ticket is
+    const uint32_t step = step_arg + *step_offset;
     const int tile = chain_ticket(ticket, &tile_s);
-    int32_t n_dst = *n_dst_ptr;
     const bool over = n_dst > cap_dst;
     if (over) n_dst = cap_dst;
     if (tile == 0 && threadIdx.x == 0) {
@@ -153,14 +179,14 @@ hop_sample_kernel(const int64_t *__restrict__ g_indptr, const int32_t *__restric
         if (!first_hop) counts[CNT_STATUS] = 0;
         if (over) atomicOr((unsigned *)&counts[CNT_STATUS], E2EGREC_DEV_CAPACITY);
     }
-    const int64_t i0 = (int64_t)tile * kDstTile;
+    const int64_t i0 = (int64_t)tile * tile_dst;
     if (i0 >= n_dst) {
         if (n_dst == 0 && tile == 0 && threadIdx.x == 0) { blk_indptr[0] = 0; counts[CNT_EDGES] = 0; }
         return;
     }
     const int64_t i = i0 + threadIdx.x;
     int32_t c = 0;
-    if (threadIdx.x < kDstTile && i < n_dst) {
+    if (threadIdx.x < tile_dst && i < n_dst) {
         int32_t u = dst_nodes[i];
         int64_t gb = 0, deg = 0;
         if ((uint32_t)u < (uint64_t)n_nodes) {
@@ -179,65 +205,80 @@ hop_sample_kernel(const int64_t *__restrict__ g_indptr, const int32_t *__restric
     }
     int32_t tile_total;
     const int32_t ex = block_exclusive_scan<kDstThreads, int32_t>(c, tile_total, scan_sm);
-    if (threadIdx.x < kDstTile) off[threadIdx.x] = ex;
-    if (threadIdx.x == 0) off[kDstTile] = tile_total;
-    const long long base = chain_lookback(state, tile, tile_total, &counts[CNT_STATUS], &bcast);   // syncs the block
-    if (threadIdx.x < kDstTile && i < n_dst) blk_indptr[i] = (int32_t)(base + ex);
-    const bool last_tile = i0 + kDstTile >= n_dst;
-    if (last_tile && threadIdx.x == 0) {
-        const long long total = base + tile_total;
-        blk_indptr[n_dst] = (int32_t)total;
-        counts[CNT_EDGES] = total > cap_edges ? cap_edges : (int32_t)total;
-        if (total > cap_edges) atomicOr((unsigned *)&counts[CNT_STATUS], E2EGREC_DEV_CAPACITY);
+    if (threadIdx.x < tile_dst) off[threadIdx.x] = ex;
+    if (threadIdx.x == 0) {
+        off[tile_dst] = tile_total;
+        chain_publish(state, tile, tile_total);
     }
-    const uint32_t step = step_arg + *step_offset;
-    // four slots per thread and round, so that the loads of the graph entry, of the frontier position and of
-    // the bitmap word are in flight for all four before any of them is needed
+    __syncthreads();
+    long long base = -1;
     constexpr int S = 4;
-    for (int32_t sl0 = threadIdx.x; sl0 < tile_total; sl0 += kDstThreads * S) {
+    for (int32_t sl0 = threadIdx.x; sl0 - (int32_t)threadIdx.x < tile_total || base < 0; sl0 += kDstThreads * S) {
         int rr[S];
-        long long e[S];
-        int64_t src[S];
+        int64_t src[S], rbeg[S];
+        uint64_t target[S];
+        int64_t a[S], b[S];
         bool ok[S];
 #pragma unroll
         for (int q = 0; q < S; ++q) {
             const int32_t sl = sl0 + q * kDstThreads;
             ok[q] = sl < tile_total;
             rr[q] = 0;
-            e[q] = 0;
-            src[q] = 0;
+            src[q] = rbeg[q] = 0;
+            a[q] = b[q] = 0;
+            target[q] = 0;
             if (!ok[q]) continue;
-            int lo = 0, hi = kDstTile;               // largest r with off[r] <= sl
+            int lo = 0, hi = tile_dst;               // largest r with off[r] <= sl
             while (hi - lo > 1) {
                 const int mid = (lo + hi) >> 1;
                 if (off[mid] <= sl) lo = mid; else hi = mid;
             }
             rr[q] = lo;
             const int32_t j = sl - off[lo];
-            e[q] = base + sl;
-            if (e[q] >= cap_edges) { ok[q] = false; continue; }
             const int64_t deg = deg_s[lo];
             int64_t pos = j;
+            rbeg[q] = gbeg_s[lo];
             if (deg > fanout) {
                 const uint4 r4 = philox4x32_10(make_uint4((uint32_t)(j >> 1), (uint32_t)node[lo], (1u << 8) | (uint32_t)hop, step),
                                                make_uint2(seed_lo, seed_hi));
                 const uint64_t rnd = (j & 1) ? (((uint64_t)r4.w << 32) | r4.z) : (((uint64_t)r4.y << 32) | r4.x);
-                const uint64_t *cum = g_cum ? g_cum + gbeg_s[lo] : nullptr;
-                const uint64_t total = cum ? cum[deg - 1] : 0;
-                if (total > 0) {
-                    // weighted draw: the first entry of the row whose running sum exceeds t
-                    const uint64_t t = __umul64hi(rnd, total);
-                    int64_t a = 0, b = deg - 1;                 // cum[b] > t always
-                    while (a < b) {
-                        const int64_t mid = (a + b) >> 1;
-                        if (cum[mid] > t) b = mid; else a = mid + 1;
-                    }
-                    pos = a;
+                const uint64_t total = kWeighted ? g_cum[rbeg[q] + deg - 1] : 0;
+                if (kWeighted && total > 0) {
+                    target[q] = __umul64hi(rnd, total);
+                    b[q] = deg - 1;                  // its running sum is `total`, above every target
                 } else {
                     pos = (int64_t)__umul64hi(rnd, (uint64_t)deg);
                 }
             }
-            src[q] = gbeg_s[lo] + pos;
+            src[q] = rbeg[q] + pos;
+        }
+        if constexpr (kWeighted) {
+            // the first entry in [a, b] whose running sum exceeds the target
+            while (true) {
+                uint64_t c1[S], c2[S], c3[S];
+                bool any = false;
+#pragma unroll
+                for (int q = 0; q < S; ++q) {
+                    if (a[q] >= b[q]) continue;
+                    any = true;
+                    const uint64_t *cum = g_cum + rbeg[q] + a[q];
+                    const int64_t w = b[q] - a[q];
+                    c1[q] = __ldg(cum + w / 4);
+                    c2[q] = __ldg(cum + w / 2);
+                    c3[q] = __ldg(cum + w / 2 + (w - w / 2) / 2);
+                }
+                if (!any) break;
+#pragma unroll
+                for (int q = 0; q < S; ++q) {
+                    if (a[q] >= b[q]) continue;
+                    const int64_t w = b[q] - a[q], m1 = a[q] + w / 4, m2 = a[q] + w / 2, m3 = m2 + (w - w / 2) / 2;
+                    if (c1[q] > target[q]) b[q] = m1;
+                    else if (c2[q] > target[q]) { a[q] = m1 + 1; b[q] = m2; }
+                    else if (c3[q] > target[q]) { a[q] = m2 + 1; b[q] = m3; }
+                    else a[q] = m3 + 1;
+                    if (a[q] >= b[q]) src[q] = rbeg[q] + b[q];
+                }
+            }
         }
         int32_t v[S];
 #pragma unroll
@@ -255,11 +296,22 @@ hop_sample_kernel(const int64_t *__restrict__ g_indptr, const int32_t *__restric
 #pragma unroll
         for (int q = 0; q < S; ++q)   // hubs are sampled thousands of times per hop: look before the atomic
             word[q] = (ok[q] && lid[q] < 0) ? *reinterpret_cast<volatile uint32_t *>(&bitmap[v[q] >> 5]) : 0xFFFFFFFFu;
+        if (base < 0) {                                  // the same for all threads: after the first round's loads
+            base = chain_lookback(state, tile, tile_total, &counts[CNT_STATUS], &bcast);   // syncs the block
+            if (threadIdx.x < tile_dst && i < n_dst) blk_indptr[i] = (int32_t)(base + ex);
+            if (i0 + tile_dst >= n_dst && threadIdx.x == 0) {
+                const long long total = base + tile_total;
+                blk_indptr[n_dst] = (int32_t)total;
+                counts[CNT_EDGES] = total > cap_edges ? cap_edges : (int32_t)total;
+                if (total > cap_edges) atomicOr((unsigned *)&counts[CNT_STATUS], E2EGREC_DEV_CAPACITY);
+            }
+        }
 #pragma unroll
         for (int q = 0; q < S; ++q) {
-            if (!ok[q]) continue;
-            nbr_global[e[q]] = v[q];
-            edge_row[e[q]] = (int32_t)(i0 + rr[q]);
+            const long long e = base + sl0 + q * kDstThreads;
+            if (!ok[q] || e >= cap_edges) continue;
+            nbr_global[e] = v[q];
+            edge_row[e] = (int32_t)(i0 + rr[q]);
             if (lid[q] < 0 && !(word[q] & (1u << (v[q] & 31)))) atomicOr(&bitmap[v[q] >> 5], 1u << (v[q] & 31));
         }
     }
@@ -288,6 +340,7 @@ frontier_kernel(uint32_t *__restrict__ bitmap, int64_t n_words, int32_t *__restr
     }
     int32_t tile_total;
     const int32_t ex = block_exclusive_scan<256, int32_t>(c, tile_total, scan_sm);
+    if (threadIdx.x == 0) chain_publish(state, tile, tile_total);
     const long long base = chain_lookback(state, tile, tile_total, &counts[CNT_STATUS], &bcast);
     const int32_t n_dst = counts[CNT_DST];
     const bool last_tile = (int64_t)(tile + 1) * kWordTile >= n_words;
@@ -361,8 +414,12 @@ __global__ void frontier_release_kernel(const int32_t *__restrict__ src_nodes, c
 // scattered reads each).  Leaves the sort's tickets and scan state
 // zero again, so that a block can be transposed any number of times.
 __global__ void csc_finalize_kernel(const int32_t *__restrict__ csc_col, const int32_t *__restrict__ counts,
-                                    int32_t *__restrict__ csc_ptr, SortState ss, int bits, int passes)
+                                    int32_t *__restrict__ csc_ptr, SortState ss, int bits, int passes,
+                                    const int32_t *__restrict__ release_nodes, int32_t *__restrict__ local_id)
 {
+    if (release_nodes)                               // the last block of a sample also gives the local ids back
+        for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < counts[CNT_SRC]; k += (int64_t)gridDim.x * blockDim.x)
+            local_id[release_nodes[k]] = -1;
     zero_sort_state(ss, counts[CNT_EDGES], bits, passes);
     if (blockIdx.x == 0 && threadIdx.x < kMaxPasses) ss.tickets()[threadIdx.x] = 0;
     const int32_t n = counts[CNT_EDGES], n_src = counts[CNT_SRC];
@@ -434,7 +491,7 @@ pair_local_kernel(const int32_t *__restrict__ user, const int32_t *__restrict__ 
 // The transposed block: entries ordered by (column, position), the last pass looking up every entry's row, and the offsets.
 static void transpose_block(const int32_t *col, int32_t *counts, int32_t cap_edges, const int32_t *row_of,
                             int32_t *csc_col, int32_t *csc_eid, int32_t *csc_row, int32_t *csc_ptr, const SortPlan &sp,
-                            const SortLane &l, cudaStream_t st)
+                            const SortLane &l, cudaStream_t st, const int32_t *release_nodes = nullptr, int32_t *local_id = nullptr)
 {
     const int32_t *k = col, *v = nullptr;
     for (int p = 0; p < sp.passes; ++p) {
@@ -446,7 +503,8 @@ static void transpose_block(const int32_t *col, int32_t *counts, int32_t cap_edg
         v = vo;
     }
     note_launch();
-    csc_finalize_kernel<<<(unsigned)std::min<int64_t>(ceil_div((int64_t)cap_edges + 1, 256), 148 * 8), 256, 0, st>>>(csc_col, counts, csc_ptr, l.sort, sp.bits, sp.passes);
+    csc_finalize_kernel<<<(unsigned)std::min<int64_t>(ceil_div((int64_t)cap_edges + 1, 256), 148 * 8), 256, 0, st>>>(csc_col, counts, csc_ptr, l.sort, sp.bits, sp.passes,
+                                                                                                                release_nodes, local_id);
 }
 
 static inline unsigned grid_for(int64_t n, int threads) { return (unsigned)ceil_div(n > 0 ? n : 1, threads); }
@@ -613,69 +671,79 @@ int32_t e2egrec::sample_khop_impl(const e2egrec_csr *graph, const int32_t *seeds
     tap_begin(TAP_SAMPLE, st);
     const int32_t *dst_nodes = seeds;
     const int32_t *n_dst_ptr = &blocks[0].counts[CNT_DST];
-    if (!pairs) {
-        note_launch();
-        seed_init_kernel<<<grid_for(n_seeds, T), T, 0, st>>>(seeds, n_seeds, n, s.local_id, blocks[0].counts);
-    } else {
-        // seeds = ascending distinct endpoints of the pairs; entries (pair, side) grouped by seed
+    // chain states of this call: one run of word tiles per frontier, then the destination tiles of every hop
+    unsigned long long *words[kMaxHops + 1], *tiles[kMaxHops], *chain = s.chain;
+    for (int f = 0; f <= n_hops; ++f, chain += s.word_tiles) words[f] = chain;
+    for (int h = 0; h < n_hops; ++h) {
+        tiles[h] = chain;
+        chain += ceil_div(blocks[h].cap_dst > 0 ? blocks[h].cap_dst : 1, dst_tile(blocks[h].cap_dst, fanouts[h]));
+    }
+    const int64_t zero16 = ceil_div(reinterpret_cast<char *>(chain) - s.zero, 16);
+    note_launch();
+    sample_begin_kernel<<<(unsigned)std::min<int64_t>(std::max<int64_t>(ceil_div(zero16, 256 * 2), grid_for(pairs ? 0 : n_seeds, 256)), 148 * 8), 256, 0, st>>>(
+        reinterpret_cast<uint4 *>(s.zero), zero16, pairs ? nullptr : seeds, n_seeds, n, s.local_id, blocks[0].counts,
+        pairs ? pairs->pcounts : nullptr);
+    cudaStream_t ts = side ? side->stream : st;          // stream of the transpositions
+    if (pairs) {
+        // seeds = ascending distinct endpoints of the pairs; entries (pair, side) grouped by seed.  Nobody reads the groups
+        // before the backward pass: they are sorted on the helper stream, in a lane that no hop uses if there is one.
         const PairInput &pi = *pairs;
         const int32_t P2 = 2 * pi.n_pairs;
-        cudaMemsetAsync(s.arena, 0, s.arena_bytes, st);
-        cudaMemsetAsync(pi.pcounts, 0, 4 * sizeof(int32_t), st);
-        cudaMemsetAsync(blocks[0].counts, 0, 4 * sizeof(int32_t), st);
         note_launch();
         pair_mark_kernel<<<grid_for(pi.n_pairs, T), T, 0, st>>>(pi.user, pi.item, pi.n_pairs, n, s.bitmap, blocks[0].counts);
         note_launch();
-        frontier_kernel<<<grid_for(s.n_words, kWordTile), 256, 0, st>>>(s.bitmap, s.n_words, pi.pcounts, P2, s.local_id,
-                                                                        pi.seeds_out, s.tickets + 1, s.state_words);
+        frontier_kernel<<<(unsigned)s.word_tiles, 256, 0, st>>>(s.bitmap, s.n_words, pi.pcounts, P2, s.local_id, pi.seeds_out,
+                                                                s.tickets + 2 * kMaxHops, words[n_hops]);
         const SortPlan sp = sort_plan(P2 > 1 ? P2 : 2);
-        const SortLane &l = s.lane[0];
-        cudaMemsetAsync(l.sort.ghist, 0, sizeof(unsigned) * kSortCountWords, st);
+        const bool own_lane = n_hops < kMaxHops;
+        const SortLane &l = s.lane[own_lane ? kMaxHops - 1 : 0];
         note_launch();
         pair_local_kernel<<<(unsigned)std::min<int64_t>(grid_for(P2, T), 148 * 4), T, 0, st>>>(
             pi.user, pi.item, pi.n_pairs, n, s.local_id, pi.pair_local, pi.entry_unit, pi.units_per_row, pi.item_unit_off,
             pi.pcounts, sp.bits, sp.passes, l.sort);
-        transpose_block(pi.pair_local, pi.pcounts, P2, pi.entry_unit, pi.pcsc_col, pi.pcsc_eid, pi.pcsc_idx, pi.pcsc_ptr, sp, l, st);
+        if (side && own_lane) side->fork(st);
+        transpose_block(pi.pair_local, pi.pcounts, P2, pi.entry_unit, pi.pcsc_col, pi.pcsc_eid, pi.pcsc_idx, pi.pcsc_ptr, sp, l,
+                        own_lane ? ts : st);
+        if (!own_lane) cudaMemsetAsync(l.sort.ghist, 0, sizeof(unsigned) * kSortCountWords, st);
         dst_nodes = pi.seeds_out;
         n_dst_ptr = &pi.pcounts[CNT_SRC];
     }
+    const bool transpose = !(flags & E2EGREC_SAMPLE_NO_TRANSPOSE);
+    const e2egrec_block &last = blocks[n_hops - 1];
     for (int h = 0; h < n_hops; ++h) {
         const e2egrec_block &b = blocks[h];
-        const int32_t f = fanouts[h];
         const SortPlan sp = sort_plan(b.cap_src);
         const SortLane &l = s.lane[h];
-        cudaMemsetAsync(s.arena, 0, s.arena_bytes, st);
+        const int tile = dst_tile(b.cap_dst, fanouts[h]);
+        auto sample = graph->edge_cum ? hop_sample_kernel<true> : hop_sample_kernel<false>;
         note_launch();
-        hop_sample_kernel<<<grid_for(b.cap_dst, kDstTile), kDstThreads, 0, st>>>(
-            graph->indptr, graph->indices, graph->edge_cum, n, dst_nodes, n_dst_ptr, b.cap_dst, b.cap_edges, f, h + 1,
+        sample<<<grid_for(b.cap_dst, tile), kDstThreads, 0, st>>>(
+            graph->indptr, graph->indices, graph->edge_cum, n, dst_nodes, n_dst_ptr, b.cap_dst, b.cap_edges, fanouts[h], tile, h + 1,
             (uint32_t)(seed & 0xFFFFFFFFu), (uint32_t)(seed >> 32), step, s.step_offset, h == 0, b.counts, b.indptr,
-            b.inv_cnt, b.src_nodes, b.nbr_global, l.edge_row, s.local_id, s.bitmap, s.tickets + 0, s.state_dst);
+            b.inv_cnt, b.src_nodes, b.nbr_global, l.edge_row, s.local_id, s.bitmap, s.tickets + 2 * h, tiles[h]);
         note_launch();
-        frontier_kernel<<<grid_for(s.n_words, kWordTile), 256, 0, st>>>(s.bitmap, s.n_words, b.counts, b.cap_src,
-                                                                        s.local_id, b.src_nodes, s.tickets + 1,
-                                                                        s.state_words);
-        cudaMemsetAsync(l.sort.ghist, 0, sizeof(unsigned) * kSortCountWords, st);
+        frontier_kernel<<<(unsigned)s.word_tiles, 256, 0, st>>>(s.bitmap, s.n_words, b.counts, b.cap_src, s.local_id, b.src_nodes,
+                                                                s.tickets + 2 * h + 1, words[h]);
         note_launch();
         relabel_kernel<<<(unsigned)std::min<int64_t>(grid_for(b.cap_edges, T), 148 * 4), T, 0, st>>>(
             b.nbr_global, s.local_id, b.counts, b.col, sp.bits, sp.passes, l.sort);
-        if (!(flags & E2EGREC_SAMPLE_NO_TRANSPOSE)) {
-            cudaStream_t ts = st;                    // stream of the transposition
-            if (side) {
-                side->fork(st);
-                ts = side->stream;
-            }
-            transpose_block(b.col, b.counts, b.cap_edges, l.edge_row, b.csc_col, b.csc_eid, b.csc_row, b.csc_ptr, sp, l, ts);
+        if (transpose) {
+            if (side) side->fork(st);
+            const bool release = h == n_hops - 1;        // every relabelling is done: the last block's offsets release the ids
+            transpose_block(b.col, b.counts, b.cap_edges, l.edge_row, b.csc_col, b.csc_eid, b.csc_row, b.csc_ptr, sp, l, ts,
+                            release ? last.src_nodes : nullptr, s.local_id);
         }
         dst_nodes = b.src_nodes;
         n_dst_ptr = &b.counts[CNT_SRC];
     }
-    if (side && !(flags & E2EGREC_SAMPLE_NO_TRANSPOSE)) {
+    if (!transpose) {
+        note_launch();
+        frontier_release_kernel<<<grid_for(last.cap_src, T), T, 0, st>>>(last.src_nodes, last.counts, s.local_id);
+    }
+    if (side && (transpose || (pairs && n_hops < kMaxHops))) {
         if (flags & E2EGREC_SAMPLE_DEFER_TRANSPOSE) side->defer();
         else side->join(st);
     }
-    const e2egrec_block &last = blocks[n_hops - 1];
-    note_launch();
-    frontier_release_kernel<<<grid_for(last.cap_src, T), T, 0, st>>>(last.src_nodes, last.counts, s.local_id);
     tap_end(TAP_SAMPLE, st);
     return check_launch("sample_khop");
 }
