@@ -31,9 +31,8 @@ sage_aggregate_kernel(const T *__restrict__ Hsrc, int64_t ld, const int32_t *__r
     const int lane = threadIdx.x & 31;
     const int g = lane / LPR, c = lane % LPR;
     const int n_chunks = d / E;
-    pdl_launch_dependents();
     pdl_wait();                                    // the kernel before this one in the stream has completed
-    const int32_t n_dst = counts[CNT_DST];
+    const int32_t n_dst = __ldcg(counts + CNT_DST);
     int64_t pad_end = ((int64_t)n_dst + 127) / 128 * 128;
     if (pad_end > cap_dst) pad_end = cap_dst;
     // The grid is sized for the machine, not for the capacity: every warp walks over destinations
@@ -47,10 +46,10 @@ sage_aggregate_kernel(const T *__restrict__ Hsrc, int64_t ld, const int32_t *__r
         b = e = m = 0;
         sr = ii;
         if (ii < n_dst) {
-            b = indptr[ii];
-            e = indptr[ii + 1];
-            if (lane < e - b) m = nbr[b + lane];
-            if (self_ids) sr = (int64_t)self_ids[ii];
+            b = __ldcg(indptr + ii);
+            e = __ldcg(indptr + ii + 1);
+            if (lane < e - b) m = __ldcg(nbr + b + lane);
+            if (self_ids) sr = (int64_t)__ldcg(self_ids + ii);
         }
     };
     fetch(i, beg, end, mine, self_row);

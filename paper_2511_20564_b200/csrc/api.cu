@@ -30,15 +30,6 @@ int32_t check_launch(const char *what)
     return E2EGREC_ERR_CUDA;
 }
 
-bool pdl_enabled()
-{
-    static const bool on = []() {
-        const char *v = getenv("E2EGREC_PDL");
-        return v && *v && strcmp(v, "0") != 0;
-    }();
-    return on;
-}
-
 static bool helper_streams_enabled()
 {
     static const bool on = []() {

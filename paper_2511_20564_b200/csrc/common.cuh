@@ -47,19 +47,23 @@ struct SideStream {
 };
 // host side: every kernel launch is counted (e2egrec_launch_count)
 void note_launch();
-// host side: true when the environment variable E2EGREC_PDL is set to a non-empty value other than "0"
-bool pdl_enabled();
 
-// Launch, optionally (E2EGREC_PDL=1) with programmatic stream serialization: the kernel's blocks may then become
-// resident while the kernel before it in the stream is still finishing, so that its set-up (and the launch latency)
-// overlaps that kernel's tail.  Off by default: measured on B200 inside a step whose three legs run on three streams,
-// the early-resident blocks (a persistent product holds ~200 KB of shared memory per SM while it waits) keep the
-// other legs' kernels off the SMs and the step gets slower (0.126 -> 0.148 ms on the 20 M-entry workload).  Only for
-// kernels that call pdl_wait() in every thread before they touch global memory: the wait returns once the
-// preceding kernel has completed and its writes are visible, which makes the pair behave like an ordinary dependent
-// launch.  Kernels launched this way call pdl_launch_dependents() first, so that their own successor is admitted early.
+// Launch with programmatic stream serialization when `chain` is set: the kernel's blocks may become resident once every
+// block of the kernel before it in the stream has finished, so that its launch and set-up overlap that kernel's draining.
+// Only for kernels that call pdl_wait() in every thread before they touch global memory (the wait returns once the
+// preceding kernel has completed and its writes are visible) and that read what such a kernel leaves with loads that the
+// compiler cannot move above the wait or take from a cache of constant data: __ldcg for everything whose address is known
+// beforehand (plain loads of const __restrict__ arrays gave stale frontiers), any load for what depends on those.
+//
+// Who sets `chain`: the small kernels of a sample, an encoder pass or a ranking tower, where the gaps between launches are
+// a fifth of the time -- samples all of whose blocks stay below kChainEdges entries of capacity.  B200, us a pass without and with: serving 64 users
+// 69.7 / 55.2, tiny fp32 step 136 / 122, medium step 176 / 164, joint step 316 / 293; the large step, whose kernels fill the
+// machine and whose legs run on two streams, loses: 1357 / 1370 with its samples' sorts
+// and first hops launched this way, 1385 with the small kernels of its top layer as well.  Admitting the next kernel while this one still runs
+// (griddepcontrol.launch_dependents at its beginning) keeps the other stream's kernels off the SMs: 182 for the medium step.
+constexpr int64_t kChainEdges = 1ll << 20, kChainRows = 1ll << 17;
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args &&...args)
+inline cudaError_t launch_pdl(bool chain, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args &&...args)
 {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
@@ -70,11 +74,10 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = pdl_enabled() ? 1 : 0;
+    cfg.numAttrs = chain ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
-__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // host side: timing taps (e2egrec_profile_tap).  tap_begin/tap_end record the armed events around
 // kernel group `which` and disarm the tap.

@@ -113,18 +113,17 @@ struct EpiPartial {
 static __global__ void splitk_reduce_kernel(const float *__restrict__ partial, int64_t n, int splits, int accumulate,
                                             float *__restrict__ out, const int32_t *rows_dev, int n_rhs = 1)
 {
-    pdl_launch_dependents();
     pdl_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     int active = splits;
     if (rows_dev) {
-        const int64_t total = (((int64_t)*rows_dev + 63) / 64) * n_rhs;
+        const int64_t total = (((int64_t)__ldcg(rows_dev) + 63) / 64) * n_rhs;
         const int64_t per = max((int64_t)8, (total + splits - 1) / splits);
         active = (int)max((int64_t)1, (total + per - 1) / per);
     }
     float s = accumulate ? out[i] : 0.f;
-    for (int z = 0; z < active; ++z) s += partial[(int64_t)z * n + i];
+    for (int z = 0; z < active; ++z) s += __ldcg(partial + (int64_t)z * n + i);
     out[i] = s;
 }
 
@@ -136,7 +135,6 @@ __global__ void relu_mask_kernel(const T *__restrict__ dH, int64_t ld_dh, const 
                                  const int32_t *n_dev, int64_t rows_alloc, int d, int relu, T *__restrict__ dZ,
                                  const T *__restrict__ dH1 = nullptr, int64_t ld_dh1 = 0)
 {
-    pdl_launch_dependents();
     pdl_wait();
     if (blockIdx.y == 1) {
         dH = dH1;
@@ -148,9 +146,9 @@ __global__ void relu_mask_kernel(const T *__restrict__ dH, int64_t ld_dh, const 
     const int k = (int)(i - r * d);
     if (r >= rows_alloc) return;
     T v = from_float<T>(0.f);
-    if (r < *n_dev) {
-        v = dH[r * ld_dh + k];
-        if (relu && !(to_float<T>(H[r * ld_h + k]) > 0.f)) v = from_float<T>(0.f);
+    if (r < __ldcg(n_dev)) {
+        v = __ldcg(dH + r * ld_dh + k);
+        if (relu && !(to_float<T>(__ldcg(H + r * ld_h + k)) > 0.f)) v = from_float<T>(0.f);
     }
     dZ[r * d + k] = v;
 }

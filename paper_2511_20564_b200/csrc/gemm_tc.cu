@@ -184,6 +184,7 @@ struct TcEpilogue {
     const __nv_bfloat16 *mask; // optional [rows x ld_mask]: outputs are zeroed where mask <= 0 (ReLU derivative)
     int64_t ld_mask;
     const int32_t *m_dev;      // rows at and beyond *m_dev are written as zeros
+    bool chain;                // host side: launch_pdl's `chain` for small products
     __nv_bfloat16 *out2;       // optional second copy of the output: rows below rows2, leading dimension ldo2
     int64_t ldo2, rows2;
     int32_t *status;           // device status word (E2EGREC_DEV_TIMEOUT)
@@ -365,7 +366,6 @@ tc_gemm_tn_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     __shared__ int abort_flag;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    pdl_launch_dependents();                    // (with programmatic launches) the next kernel may set itself up beside this one
     uint8_t *tiles = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t a_bytes = kTileM * kTileK * 2, b_bytes = (uint32_t)nt * kTileK * 2;
     uint8_t *a_tiles = tiles;
@@ -398,7 +398,7 @@ tc_gemm_tn_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
     const uint32_t buf_stride = tmem_cols >> 1;
     // barriers and tensor memory are set up; global memory is touched only once the preceding kernel has completed
     pdl_wait();
-    const int32_t m_valid = *ep.m_dev;
+    const int32_t m_valid = __ldcg(ep.m_dev);
     const int64_t live_tiles = ((int64_t)m_valid + kTileM - 1) / kTileM;    // per block of rows; tiles wholly beyond *m_dev stay as they are
     const int64_t n_work = live_tiles * n_tiles_n * ep.n_rhs;
     // tile t of the list: column tile t % n_tiles_n of live row tile (t / n_tiles_n) % live_tiles of block (t / n_tiles_n) / live_tiles
@@ -748,10 +748,10 @@ bool launch_tn(const __nv_bfloat16 *A, int64_t rows, int k, int64_t lda, const _
     const unsigned grid = (unsigned)std::min<int64_t>(tiles_cap, sm_count());
     note_launch();
     if (fused)
-        launch_pdl(tc_gemm_tn_kernel<true>, dim3(grid), dim3(kTnThreads), smem, st, ma, mb, mo, k_blocks, stages, nt, n_tiles_n, tmem_cols,
+        launch_pdl(ep.chain && rows * n_rhs < kChainRows, tc_gemm_tn_kernel<true>, dim3(grid), dim3(kTnThreads), smem, st, ma, mb, mo, k_blocks, stages, nt, n_tiles_n, tmem_cols,
                    b_mn ? 1 : 0, ep);
     else
-        launch_pdl(tc_gemm_tn_kernel<false>, dim3(grid), dim3(kTnThreads), smem, st, ma, mb, mo, k_blocks, stages, nt, n_tiles_n, tmem_cols,
+        launch_pdl(ep.chain && rows * n_rhs < kChainRows, tc_gemm_tn_kernel<false>, dim3(grid), dim3(kTnThreads), smem, st, ma, mb, mo, k_blocks, stages, nt, n_tiles_n, tmem_cols,
                    b_mn ? 1 : 0, ep);
     return true;
 }
@@ -775,9 +775,8 @@ tc_gemm_rows_kernel(const __grid_constant__ CUtensorMap map_y, const __grid_cons
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int m0 = blockIdx.x * kTileM, n0 = blockIdx.y * nt;
-    pdl_launch_dependents();
     pdl_wait();                                 // the preceding kernel of the stream has completed
-    const int64_t m_valid = *m_dev;
+    const int64_t m_valid = __ldcg(m_dev);
     // Y may hold n_rhs blocks of rhs_rows rows (the first *m_dev of each live) that all meet the same rows of X: the
     // k-blocks of the blocks of rows form one list, and the sum runs over all of them
     const int64_t blocks_per_rhs = (m_valid + kTileK - 1) / kTileK;
@@ -1184,7 +1183,7 @@ bool launch_fused(const CUtensorMap &mb, const __nv_bfloat16 *Hsrc, int64_t ld, 
 
 bool tc_update_forward(const __nv_bfloat16 *cat, int64_t rows, int k, const __nv_bfloat16 *W, int n, const float *bias,
                        int relu, __nv_bfloat16 *out, const int32_t *m_dev, int32_t *status, cudaStream_t st,
-                       __nv_bfloat16 *out2, int64_t ldo2, int64_t rows2)
+                       __nv_bfloat16 *out2, int64_t ldo2, int64_t rows2, bool chain)
 {
     if (out2 && (reinterpret_cast<uintptr_t>(out2) % 16 || (ldo2 * 2) % 16 || ldo2 < n)) return false;
     TcEpilogue ep{};
@@ -1199,6 +1198,7 @@ bool tc_update_forward(const __nv_bfloat16 *cat, int64_t rows, int k, const __nv
     ep.scale_from = 0;
     ep.m_dev = m_dev;
     ep.status = status;
+    ep.chain = chain;
     return launch_tn(cat, rows, k, k, W, n, k, ep, st);
 }
 
@@ -1223,12 +1223,13 @@ bool tc_linear(const __nv_bfloat16 *A, int64_t rows, int k, const __nv_bfloat16 
     ep.ld_mask = ld_mask;
     ep.m_dev = m_dev;
     ep.status = status;
+    ep.chain = true;
     return b_is_k_by_n ? launch_tn(A, rows, k, k, B, n, n, ep, st, true) : launch_tn(A, rows, k, k, B, n, k, ep, st);
 }
 
 bool tc_dcat_backward(const __nv_bfloat16 *dz, int64_t rows, int d_out, const __nv_bfloat16 *W, int two_d_in,
                       const float *inv_cnt, __nv_bfloat16 *dcat, const int32_t *m_dev, int32_t *status, cudaStream_t st,
-                      int n_rhs)
+                      int n_rhs, bool chain)
 {
     TcEpilogue ep{};
     ep.out = dcat;
@@ -1239,6 +1240,7 @@ bool tc_dcat_backward(const __nv_bfloat16 *dz, int64_t rows, int d_out, const __
     ep.scale_from = two_d_in / 2;
     ep.m_dev = m_dev;
     ep.status = status;
+    ep.chain = chain;
     return launch_tn(dz, rows, d_out, d_out, W, two_d_in, two_d_in, ep, st, true, n_rhs);
 }
 
@@ -1261,7 +1263,7 @@ int tc_weight_grad_tiles(int m, int n)
 }
 
 bool tc_weight_grad(const __nv_bfloat16 *dY, int64_t rows, int m, const __nv_bfloat16 *Xin, int n, const int32_t *m_dev,
-                    float *part, int splits, int32_t *status, cudaStream_t st, int n_rhs)
+                    float *part, int splits, int32_t *status, cudaStream_t st, int n_rhs, bool chain)
 {
     if (rows <= 0 || rows % kTileK || m % kTileM || n % 64 || n_rhs < 1 || splits < 1) return false;
     const int nt = weight_grad_nt(n);
@@ -1277,7 +1279,7 @@ bool tc_weight_grad(const __nv_bfloat16 *dY, int64_t rows, int m, const __nv_bfl
     if (!raise_smem_limit(tc_gemm_rows_kernel, attr_set)) return false;
     dim3 grid((unsigned)(m / kTileM), (unsigned)(n / nt), (unsigned)splits);
     note_launch();
-    launch_pdl(tc_gemm_rows_kernel, grid, dim3(kThreads), smem, st, my, mx, nt, tmem_cols, stages, m_dev, part, (int64_t)n,
+    launch_pdl(chain && rows * n_rhs < kChainRows, tc_gemm_rows_kernel, grid, dim3(kThreads), smem, st, my, mx, nt, tmem_cols, stages, m_dev, part, (int64_t)n,
                (int64_t)m * n, status, n_rhs, rows);
     return true;
 }

@@ -195,7 +195,7 @@ extern "C" int32_t e2egrec_graph_from_coo(int64_t n_nodes, int64_t n_edges, cons
             const int sort = q / sp.passes, pass = q % sp.passes;
             if (q == sp.passes) std::swap(k, v);
             const bool last = q == 2 * sp.passes - 1;
-            sort_pass<int32_t>(sp, k, v, nullptr, m, q == 0 ? clamp : 0, q == 0 ? clamp : 0, pass, s.sort[sort], last ? s.a : ka,
+            sort_pass<int32_t>(sp, k, v, nullptr, m, q == 0 ? clamp : 0, q == 0 ? clamp : 0, pass, s.sort[sort], false, last ? s.a : ka,
                                last ? indices : va, SortMap{}, &s.counts[CNT_STATUS], st);
             k = ka;
             v = va;
@@ -235,9 +235,9 @@ extern "C" int32_t e2egrec_csr_transpose(const e2egrec_csr *csr, int64_t n_cols,
         for (int q = 0; q < sp.passes; ++q) {
             const int32_t clamp = q == 0 ? (int32_t)std::max<int64_t>(n_cols, 1) : 0;
             if (q == sp.passes - 1)
-                sort_pass<int64_t>(sp, k, v, nullptr, m, clamp, 0, q, s.sort[0], ka, csc_eid, SortMap{}, &s.counts[CNT_STATUS], st);
+                sort_pass<int64_t>(sp, k, v, nullptr, m, clamp, 0, q, s.sort[0], false, ka, csc_eid, SortMap{}, &s.counts[CNT_STATUS], st);
             else
-                sort_pass<int32_t>(sp, k, v, nullptr, m, clamp, 0, q, s.sort[0], ka, va, SortMap{}, &s.counts[CNT_STATUS], st);
+                sort_pass<int32_t>(sp, k, v, nullptr, m, clamp, 0, q, s.sort[0], false, ka, va, SortMap{}, &s.counts[CNT_STATUS], st);
             k = ka;
             v = va;
             std::swap(ka, kb);

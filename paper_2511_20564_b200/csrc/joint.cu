@@ -49,24 +49,35 @@ void fill_blocks(const JointPlan &jp, char *ws, e2egrec_block *blocks)
 // ------------------------------------------------------------------------------------------ kernels
 __global__ void joint_meta_kernel(int32_t *pmeta, int32_t n_pairs) { pmeta[0] = n_pairs; }
 
-// z[p] = [ h[user seed] | h[item seed] | dense[p] ] in the feature dtype; rows P .. rows_alloc-1 are zero.
+// z[p] = [ h[user seed] | h[item seed] | dense[p] ] in the feature dtype; rows P .. rows_alloc-1 are zero.  A thread writes
+// 16 bytes of a row (the widths are multiples of that); one value per thread with its divisions took 6.4 us for 4096 rows.
 template <typename T>
-__global__ void build_z_kernel(const T *__restrict__ H, int dL, const int32_t *__restrict__ pair_local,
-                               const float *__restrict__ dense, int dense_dim, int32_t P, int64_t rows_alloc,
-                               T *__restrict__ z)
+__global__ void __launch_bounds__(256)
+build_z_kernel(const T *__restrict__ H, int dL, const int32_t *__restrict__ pair_local, const float *__restrict__ dense, int dense_dim,
+               int32_t P, int64_t rows_alloc, T *__restrict__ z)
 {
-    const int zdim = 2 * dL + dense_dim;
+    constexpr int E = Chunk<T>::kElems;
+    pdl_wait();
+    const int zdim = 2 * dL + dense_dim, chunks = zdim / E;
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t p = t / zdim;
-    const int k = (int)(t - p * zdim);
+    const int64_t p = t / chunks;
     if (p >= rows_alloc) return;
-    T v = from_float<T>(0.f);
+    const int k = (int)(t - p * chunks) * E;
+    uint4 v = make_uint4(0, 0, 0, 0);
     if (p < P) {
-        if (k < dL) v = H[(int64_t)pair_local[p] * dL + k];
-        else if (k < 2 * dL) v = H[(int64_t)pair_local[P + p] * dL + (k - dL)];
-        else v = from_float<T>(dense[p * (int64_t)dense_dim + (k - 2 * dL)]);
+        if (k < 2 * dL) {
+            const int side = k >= dL;
+            v = __ldcg(reinterpret_cast<const uint4 *>(H + (int64_t)__ldcg(pair_local + side * P + p) * dL + (k - side * dL)));
+        } else {
+            float x[E];
+            const float *src = dense + p * (int64_t)dense_dim + (k - 2 * dL);
+#pragma unroll
+            for (int e = 0; e < E; ++e) x[e] = __ldcg(src + e);
+            Chunk<T>::store(z + p * zdim + k, x);
+            return;
+        }
     }
-    z[t] = v;
+    *reinterpret_cast<uint4 *>(z + p * zdim + k) = v;
 }
 
 // logits t[p] = b + <a[p], w>, fp32, one warp per pair
@@ -75,11 +86,12 @@ __global__ void __launch_bounds__(256)
 logit_kernel(const T *__restrict__ a, int d, const T *__restrict__ w, const float *__restrict__ b, int32_t P,
              float *__restrict__ logits)
 {
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const int64_t p = ((int64_t)blockIdx.x * 256 + threadIdx.x) >> 5;
     if (p >= P) return;
     float s = 0.f;
-    for (int k = lane; k < d; k += 32) s = fmaf(to_float<T>(a[p * d + k]), to_float<T>(w[k]), s);
+    for (int k = lane; k < d; k += 32) s = fmaf(to_float<T>(__ldcg(a + p * d + k)), to_float<T>(w[k]), s);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) logits[p] = s + (b ? b[0] : 0.f);
@@ -92,10 +104,11 @@ bce_kernel(const float *__restrict__ logits, const float *__restrict__ labels, i
            float *__restrict__ dt, float *__restrict__ db3, int accumulate)
 {
     __shared__ float red[2][1024];
+    pdl_wait();
     float ls = 0.f, ds = 0.f;
     const float invP = 1.0f / (float)P;
     for (int p = threadIdx.x; p < P; p += 1024) {
-        const float t = logits[p], y = labels[p];
+        const float t = __ldcg(logits + p), y = __ldcg(labels + p);
         ls += fmaxf(t, 0.f) - y * t + log1pf(expf(-fabsf(t)));
         const float sg = t >= 0.f ? 1.0f / (1.0f + expf(-t)) : expf(t) / (1.0f + expf(t));
         const float g = (sg - y) * invP;
@@ -119,18 +132,31 @@ bce_kernel(const float *__restrict__ logits, const float *__restrict__ labels, i
 }
 
 // dZ2[p, j] = dt[p] * W3[j] where a2[p, j] > 0 (everywhere with the identity activation), stored in the feature dtype;
-// padding rows are zero.
+// padding rows are zero.  16 bytes of a row per thread.
 template <typename T>
-__global__ void dz_top_kernel(const float *__restrict__ dt, const T *__restrict__ w3, const T *__restrict__ a2, int d,
-                              int32_t P, int64_t rows_alloc, int relu, T *__restrict__ dz2)
+__global__ void __launch_bounds__(256)
+dz_top_kernel(const float *__restrict__ dt, const T *__restrict__ w3, const T *__restrict__ a2, int d, int32_t P, int64_t rows_alloc,
+              int relu, T *__restrict__ dz2)
 {
+    constexpr int E = Chunk<T>::kElems;
+    pdl_wait();
+    const int chunks = d / E;
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t p = t / d;
-    const int j = (int)(t - p * d);
+    const int64_t p = t / chunks;
     if (p >= rows_alloc) return;
-    float v = 0.f;
-    if (p < P && (!relu || to_float<T>(a2[t]) > 0.f)) v = dt[p] * to_float<T>(w3[j]);
-    dz2[t] = from_float<T>(v);
+    const int j = (int)(t - p * chunks) * E;
+    float v[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[e] = 0.f;
+    if (p < P) {
+        const float g = __ldcg(dt + p);
+        float a[E];
+        Chunk<T>::unpack(__ldcg(reinterpret_cast<const uint4 *>(a2 + p * d + j)), a);
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            if (!relu || a[e] > 0.f) v[e] = g * to_float<T>(w3[j + e]);
+    }
+    Chunk<T>::store(dz2 + p * d + j, v);
 }
 
 // ------------------------------------------------------------------------------------------ dense helpers
@@ -196,7 +222,8 @@ void linear_backward_weight(const T *dY, int64_t rows, int n_out, const T *Xin, 
     }
     const int64_t n = (int64_t)n_out * n_in;
     note_launch();
-    splitk_reduce_kernel<<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(part, n, kSplits, 0, dW, on_tc ? m_dev : nullptr);
+    launch_pdl(rows < kChainRows, splitk_reduce_kernel, dim3((unsigned)ceil_div(n, 256)), dim3(256), 0, st, (const float *)part, n, kSplits, 0, dW,
+               on_tc ? m_dev : (const int32_t *)nullptr, 1);
     if (db) launch_colsum<T>(dY, n_out, nullptr, m_dev, 0, n_out, 0, db, st);
 }
 
@@ -489,6 +516,7 @@ int32_t run_joint(const JointPlan &jp, const e2egrec_csr *graph, const e2egrec_m
     if (rc != E2EGREC_OK) return rc;
 
     // 3. tower forward and loss
+    const bool small = jp.rowsP < kChainRows;
     T *z = tp(jp.z_off), *a1 = tp(jp.a1_off), *a2 = tp(jp.a2_off);
     const T *W1 = static_cast<const T *>(W_tower[0].data), *W2 = static_cast<const T *>(W_tower[1].data),
             *W3 = static_cast<const T *>(W_tower[2].data);
@@ -496,10 +524,10 @@ int32_t run_joint(const JointPlan &jp, const e2egrec_csr *graph, const e2egrec_m
                 *b3 = b_tower ? b_tower[2] : nullptr;
     float *dt = reinterpret_cast<float *>(ws + jp.dt_off);
     {
-        const int64_t n = jp.rowsP * jp.zdim;
+        const int64_t n = jp.rowsP * (jp.zdim / jp.unit);
         note_launch();
-        build_z_kernel<T><<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(tp(jp.hseed_off), jp.dL, pi.pair_local, dense, jp.dense_dim,
-                                                                     jp.P, jp.rowsP, z);
+        launch_pdl(small, build_z_kernel<T>, dim3((unsigned)ceil_div(n, 256)), dim3(256), 0, st, (const T *)tp(jp.hseed_off), jp.dL,
+                   (const int32_t *)pi.pair_local, dense, jp.dense_dim, jp.P, jp.rowsP, z);
     }
     // gating fusion (Sec. 4.3.2): the tower reads z_fused = sigmoid(W_g z + b_g) * z instead of z
     const T *tin = z;
@@ -515,17 +543,19 @@ int32_t run_joint(const JointPlan &jp, const e2egrec_csr *graph, const e2egrec_m
     linear_forward<T>(tin, jp.rowsP, jp.zdim, W1, jp.h1, b1, relu, a1, pmeta, status, st);
     linear_forward<T>(a1, jp.rowsP, jp.h1, W2, jp.h2, b2, relu, a2, pmeta, status, st);
     note_launch();
-    logit_kernel<T><<<(unsigned)ceil_div((int64_t)jp.P * 32, 256), 256, 0, st>>>(a2, jp.h2, W3, b3, jp.P, logits);
+    launch_pdl(small, logit_kernel<T>, dim3((unsigned)ceil_div((int64_t)jp.P * 32, 256)), dim3(256), 0, st, (const T *)a2, jp.h2, W3, b3,
+               jp.P, logits);
     note_launch();
-    bce_kernel<<<1, 1024, 0, st>>>(logits, labels, jp.P, loss, dt, db_tower ? db_tower[2] : nullptr, 0);
+    launch_pdl(small, bce_kernel, dim3(1), dim3(1024), 0, st, (const float *)logits, labels, jp.P, loss, dt, db_tower ? db_tower[2] : nullptr, 0);
 
     // 4. tower backward
     T *dz2 = tp(jp.dz2_off), *dz1 = tp(jp.dz1_off), *dz = tp(jp.dz_off), *wt = tp(jp.wt_off);
     float *part = reinterpret_cast<float *>(ws + jp.part_off);
     {
-        const int64_t n = jp.rowsP * jp.h2;
+        const int64_t n = jp.rowsP * (jp.h2 / jp.unit);
         note_launch();
-        dz_top_kernel<T><<<(unsigned)ceil_div(n, 256), 256, 0, st>>>(dt, W3, a2, jp.h2, jp.P, jp.rowsP, relu, dz2);
+        launch_pdl(small, dz_top_kernel<T>, dim3((unsigned)ceil_div(n, 256)), dim3(256), 0, st, (const float *)dt, W3, (const T *)a2, jp.h2,
+                   jp.P, jp.rowsP, relu, dz2);
     }
     // the weight gradients feed nothing later in the step: they go to the helper stream (behind the block
     // transposition that the sampler left there); the encoder backward waits for that stream before its first launch

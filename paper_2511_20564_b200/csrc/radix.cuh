@@ -130,7 +130,8 @@ sort_pass_kernel(const int32_t *__restrict__ keys_in, const int32_t *__restrict_
     uint16_t *wc = reinterpret_cast<uint16_t *>(gbase + R);      // [W][R] per warp: counts, then offsets within the digit
     __shared__ int32_t scan_sm[W + 1];
     __shared__ int tile_s;
-    const int32_t n = n_dev ? *n_dev : n_host;
+    pdl_wait();
+    const int32_t n = n_dev ? __ldcg(n_dev) : n_host;
     const int tile = chain_ticket(ticket, &tile_s);
     if ((int64_t)tile * TILE >= n) return;
     for (int d = threadIdx.x; d < W * R / 2; d += THREADS) reinterpret_cast<uint32_t *>(wc)[d] = 0;
@@ -146,13 +147,13 @@ sort_pass_kernel(const int32_t *__restrict__ keys_in, const int32_t *__restrict_
 #pragma unroll
     for (int k = 0; k < kSortItems; ++k) {
         const int i = w0 + k * 32 + lane;
-        key[k] = i < tile_n ? (uint32_t)__ldg(kin + i) : 0u;
+        key[k] = i < tile_n ? (uint32_t)__ldcg(kin + i) : 0u;
         if (clamp_keys && key[k] >= (uint32_t)clamp_keys) key[k] = 0;
     }
 #pragma unroll
     for (int k = 0; k < kSortItems; ++k) {
         const int i = w0 + k * 32 + lane;
-        val[k] = !vin ? (uint32_t)(tile * TILE + i) : i < tile_n ? (uint32_t)__ldg(vin + i) : 0u;
+        val[k] = !vin ? (uint32_t)(tile * TILE + i) : i < tile_n ? (uint32_t)__ldcg(vin + i) : 0u;
         if (clamp_vals && val[k] >= (uint32_t)clamp_vals) val[k] = 0;
     }
 #pragma unroll
@@ -198,7 +199,7 @@ sort_pass_kernel(const int32_t *__restrict__ keys_in, const int32_t *__restrict_
 #pragma unroll
         for (int q = 0; q < D; ++q) {
             gs[q] = g;
-            g += owner ? (int32_t)ghist[d0 + q] : 0;
+            g += owner ? (int32_t)__ldcg(ghist + d0 + q) : 0;
         }
         const int32_t bin = block_exclusive_scan<THREADS, int32_t>(g, total, scan_sm);
 #pragma unroll
@@ -301,7 +302,7 @@ sort_pass_kernel(const int32_t *__restrict__ keys_in, const int32_t *__restrict_
             if (i < tile_n) {
                 ky[q] = skey[i];
                 v[q] = sval[i];
-                if (map.row_out) row[q] = __ldg(map.row_of + v[q]);
+                if (map.row_out) row[q] = __ldcg(map.row_of + v[q]);
                 pos[q] = gbase[(ky[q] >> shift) & (R - 1)] + i;
             }
         }
@@ -348,7 +349,7 @@ constexpr size_t sort_state_bytes(int64_t tiles) { return sizeof(unsigned) * (si
 
 template <int BITS, int THREADS, typename ValT>
 static inline void launch_sort_pass(const int32_t *kin, const int32_t *vin, const int32_t *n_dev, int64_t cap, int32_t clamp_keys,
-                                    int32_t clamp_vals, int pass, const SortState &ss, int32_t *kout, ValT *vout, const SortMap &map,
+                                    int32_t clamp_vals, int pass, const SortState &ss, bool chain, int32_t *kout, ValT *vout, const SortMap &map,
                                     int32_t *status, cudaStream_t st)
 {
     constexpr size_t smem = sort_smem_bytes<BITS, THREADS>();
@@ -364,20 +365,20 @@ static inline void launch_sort_pass(const int32_t *kin, const int32_t *vin, cons
     }
     const unsigned grid = (unsigned)ceil_div(cap > 0 ? cap : 1, (int64_t)THREADS * kSortItems);
     note_launch();
-    kern<<<grid, THREADS, smem, st>>>(kin, vin, n_dev, (int32_t)cap, clamp_keys, clamp_vals, pass * BITS, ss.ghist + pass * kMaxRadix,
+    launch_pdl(chain, kern, dim3(grid), dim3(THREADS), smem, st, kin, vin, n_dev, (int32_t)cap, clamp_keys, clamp_vals, pass * BITS, ss.ghist + pass * kMaxRadix,
                                       ss.tickets() + pass, ss.state + (size_t)pass * ss.tiles * (1 << BITS), kout, vout, map, status);
 }
 
 template <typename ValT>
 static inline void sort_pass(const SortPlan &sp, const int32_t *kin, const int32_t *vin, const int32_t *n_dev, int64_t cap,
-                             int32_t clamp_keys, int32_t clamp_vals, int pass, const SortState &ss, int32_t *kout, ValT *vout,
+                             int32_t clamp_keys, int32_t clamp_vals, int pass, const SortState &ss, bool chain, int32_t *kout, ValT *vout,
                              const SortMap &map, int32_t *status, cudaStream_t st)
 {
     const bool wide = cap >= kSortWide;
-    if (sp.bits == 8 && wide) launch_sort_pass<8, 512, ValT>(kin, vin, n_dev, cap, clamp_keys, clamp_vals, pass, ss, kout, vout, map, status, st);
-    else if (sp.bits == 8) launch_sort_pass<8, 256, ValT>(kin, vin, n_dev, cap, clamp_keys, clamp_vals, pass, ss, kout, vout, map, status, st);
-    else if (wide) launch_sort_pass<10, 512, ValT>(kin, vin, n_dev, cap, clamp_keys, clamp_vals, pass, ss, kout, vout, map, status, st);
-    else launch_sort_pass<10, 256, ValT>(kin, vin, n_dev, cap, clamp_keys, clamp_vals, pass, ss, kout, vout, map, status, st);
+    if (sp.bits == 8 && wide) launch_sort_pass<8, 512, ValT>(kin, vin, n_dev, cap, clamp_keys, clamp_vals, pass, ss, chain, kout, vout, map, status, st);
+    else if (sp.bits == 8) launch_sort_pass<8, 256, ValT>(kin, vin, n_dev, cap, clamp_keys, clamp_vals, pass, ss, chain, kout, vout, map, status, st);
+    else if (wide) launch_sort_pass<10, 512, ValT>(kin, vin, n_dev, cap, clamp_keys, clamp_vals, pass, ss, chain, kout, vout, map, status, st);
+    else launch_sort_pass<10, 256, ValT>(kin, vin, n_dev, cap, clamp_keys, clamp_vals, pass, ss, chain, kout, vout, map, status, st);
 }
 
 }  // namespace e2egrec

@@ -57,27 +57,35 @@ static int32_t plan_layers(const e2egrec_block *blocks, int32_t n_layers, const 
 }
 
 // ------------------------------------------------------------------------------ launch helpers
+// launch_pdl's `chain` for the kernels of an encoder pass
+static bool chain_blocks(const e2egrec_block *blocks, int32_t n_layers)
+{
+    for (int l = 0; l < n_layers; ++l)
+        if (blocks[l].cap_edges >= kChainEdges) return false;
+    return true;
+}
+
 template <typename T, int LPR, int CPL>
 static void launch_sage_aggregate(const T *Hsrc, int64_t ld, const int32_t *nbr, const int32_t *self_ids,
-                                  const e2egrec_block &b, T *cat, int d, int64_t rows, cudaStream_t st)
+                                  const e2egrec_block &b, T *cat, int d, int64_t rows, bool chain, cudaStream_t st)
 {
     // one warp per destination at a time, the warps stride over the destinations: at most eight blocks per SM for the
     // capacities of small batches (most of such a grid finds no destination), 32 where a block can hold a million rows
     const int64_t per_sm = rows >= (1ll << 20) ? 32 : 8;
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(ceil_div(rows * 32, kAggThreads), 148 * per_sm));
     note_launch();
-    launch_pdl(sage_aggregate_kernel<T, LPR, CPL>, dim3(grid), dim3(kAggThreads), 0, st, Hsrc, ld, nbr, self_ids, b.indptr,
+    launch_pdl(chain, sage_aggregate_kernel<T, LPR, CPL>, dim3(grid), dim3(kAggThreads), 0, st, Hsrc, ld, nbr, self_ids, b.indptr,
                b.counts, cat, d, (int32_t)rows);
 }
 
 template <typename T>
 static bool dispatch_sage_aggregate(const T *Hsrc, int64_t ld, const int32_t *nbr, const int32_t *self_ids,
-                                    const e2egrec_block &b, T *cat, int d, int64_t rows, int32_t dtype, cudaStream_t st)
+                                    const e2egrec_block &b, T *cat, int d, int64_t rows, int32_t dtype, bool chain, cudaStream_t st)
 {
     const RowShape rs = row_shape(d, dtype);
 #define E2E_CASE(L, C)                                                                           \
     if (rs.lpr == L && rs.cpl == C) {                                                            \
-        launch_sage_aggregate<T, L, C>(Hsrc, ld, nbr, self_ids, b, cat, d, rows, st);            \
+        launch_sage_aggregate<T, L, C>(Hsrc, ld, nbr, self_ids, b, cat, d, rows, chain, st);     \
         return true;                                                                             \
     }
     E2E_CASE(4, 1) E2E_CASE(8, 1) E2E_CASE(16, 1) E2E_CASE(32, 1) E2E_CASE(32, 2) E2E_CASE(32, 4)
@@ -144,6 +152,7 @@ static int32_t forward_impl(const e2egrec_block *blocks, int32_t n_layers, const
     const size_t es = sizeof(T);
     const int64_t out_rows = blocks[0].cap_dst < H_out->rows ? blocks[0].cap_dst : H_out->rows;
     bool top_stored = false;
+    const bool chain = chain_blocks(blocks, n_layers);
     for (int l = 0; l < n_layers; ++l) {
         const LayerPlan &p = plan[l];
         const e2egrec_block &b = blocks[p.block];
@@ -178,11 +187,11 @@ static int32_t forward_impl(const e2egrec_block *blocks, int32_t n_layers, const
             if (l == 0) tap_end(TAP_AGG_FWD_OUTER, st);
         } else if (l == 0) {  // h^(0) rows are read straight from the feature table through the global ids
             agg_ok = dispatch_sage_aggregate<T>(static_cast<const T *>(X->data), X->ld, b.nbr_global, b.src_nodes, b, cat,
-                                                p.d_in, p.rows, X->dtype, st);
+                                                p.d_in, p.rows, X->dtype, chain, st);
             tap_end(TAP_AGG_FWD_OUTER, st);
         } else
             agg_ok = dispatch_sage_aggregate<T>(reinterpret_cast<const T *>(ctx + plan[l - 1].h_off), p.d_in, b.col, nullptr, b,
-                                                cat, p.d_in, p.rows, X->dtype, st);
+                                                cat, p.d_in, p.rows, X->dtype, chain, st);
         if (!agg_ok) {
             set_last_error("sage_forward: no aggregation kernel for this row width");
             return E2EGREC_ERR_UNSUPPORTED;
@@ -197,7 +206,7 @@ static int32_t forward_impl(const e2egrec_block *blocks, int32_t n_layers, const
             done = tc_update_forward(reinterpret_cast<const __nv_bfloat16 *>(cat), p.rows, 2 * p.d_in,
                                      static_cast<const __nv_bfloat16 *>(W[l].data), p.d_out, bl, relu,
                                      reinterpret_cast<__nv_bfloat16 *>(hn), &b.counts[CNT_DST], &b.counts[CNT_STATUS], st,
-                                     top ? static_cast<__nv_bfloat16 *>(H_out->data) : nullptr, H_out->ld, out_rows);
+                                     top ? static_cast<__nv_bfloat16 *>(H_out->data) : nullptr, H_out->ld, out_rows, chain);
             top_stored = done && top;
         }
         if (!done) {
@@ -263,6 +272,7 @@ static int32_t backward_impl(const e2egrec_block *blocks, int32_t n_layers, cons
     T *dz_buf[2] = {reinterpret_cast<T *>(scratch + bs.dz_off[0]), reinterpret_cast<T *>(scratch + bs.dz_off[1])};
     T *dcat = reinterpret_cast<T *>(scratch + bs.dcat_off);
     float *part = reinterpret_cast<float *>(scratch + bs.part_off);
+    const bool chain = chain_blocks(blocks, n_layers);
 
     // counters of the transposed aggregation (one per window of a block's entry stream); every launch leaves them zero
     cudaMemsetAsync(scratch + bs.chain_off, 0, bs.chain_bytes, st);
@@ -272,7 +282,7 @@ static int32_t backward_impl(const e2egrec_block *blocks, int32_t n_layers, cons
         const e2egrec_block &b = blocks[p.block];
         const int64_t total = p.rows * p.d_out;
         note_launch();
-        launch_pdl(relu_mask_kernel<T>, dim3((unsigned)std::max<int64_t>(1, ceil_div(total, 256)), (unsigned)n_rhs), dim3(256), 0, st,
+        launch_pdl(chain, relu_mask_kernel<T>, dim3((unsigned)std::max<int64_t>(1, ceil_div(total, 256)), (unsigned)n_rhs), dim3(256), 0, st,
                    static_cast<const T *>(dH_out[0].data), dH_out[0].ld, reinterpret_cast<const T *>(ctx + p.h_off), (int64_t)p.d_out,
                    &b.counts[CNT_DST], p.rows, p.d_out, act ? act[n_layers - 1] : 1, dz_buf[(n_layers - 1) & 1],
                    static_cast<const T *>(dH_out[n_rhs - 1].data), dH_out[n_rhs - 1].ld);
@@ -305,11 +315,11 @@ static int32_t backward_impl(const e2egrec_block *blocks, int32_t n_layers, cons
         if (X->dtype == E2EGREC_BF16)
             dw_done = tc_weight_grad(reinterpret_cast<const __nv_bfloat16 *>(dz), p.rows, p.d_out,
                                      reinterpret_cast<const __nv_bfloat16 *>(cat), two_d, n_dst, part, tc_splits,
-                                     &b.counts[CNT_STATUS], ws, n_rhs);
+                                     &b.counts[CNT_STATUS], ws, n_rhs, chain);
         const int64_t n_w = (int64_t)p.d_out * two_d;
         if (dw_done) {
             note_launch();
-            launch_pdl(splitk_reduce_kernel, dim3((unsigned)ceil_div(n_w, 256)), dim3(256), 0, ws, part, n_w, tc_splits, accumulate,
+            launch_pdl(chain, splitk_reduce_kernel, dim3((unsigned)ceil_div(n_w, 256)), dim3(256), 0, ws, part, n_w, tc_splits, accumulate,
                        dW[l], n_dst, n_rhs);
         } else {
             for (int r = 0; r < n_rhs; ++r) {             // fp32-FMA product: one right-hand side per pass, added up
@@ -319,7 +329,7 @@ static int32_t backward_impl(const e2egrec_block *blocks, int32_t n_layers, cons
                 gemm_simt_kernel<T, true, true, EpiPartial><<<grid, kGemmThreads, 0, ws>>>(
                     dz + (int64_t)r * p.rows * p.d_out, p.d_out, cat, two_d, p.d_out, two_d, p.rows, nullptr, n_dst, epi);
                 note_launch();
-                launch_pdl(splitk_reduce_kernel, dim3((unsigned)ceil_div(n_w, 256)), dim3(256), 0, ws, part, n_w, kDwSplits,
+                launch_pdl(chain, splitk_reduce_kernel, dim3((unsigned)ceil_div(n_w, 256)), dim3(256), 0, ws, part, n_w, kDwSplits,
                            (accumulate || r > 0) ? 1 : 0, dW[l], (const int32_t *)nullptr, 1);
             }
         }
@@ -340,7 +350,7 @@ static int32_t backward_impl(const e2egrec_block *blocks, int32_t n_layers, cons
             if (W[l].ld == two_d)               // W as stored: the product reads it with its N index contiguous
                 dcat_done = tc_dcat_backward(reinterpret_cast<const __nv_bfloat16 *>(dz), p.rows, p.d_out,
                                              static_cast<const __nv_bfloat16 *>(W[l].data), two_d, b.inv_cnt,
-                                             reinterpret_cast<__nv_bfloat16 *>(dcat), n_dst, &b.counts[CNT_STATUS], st, n_rhs);
+                                             reinterpret_cast<__nv_bfloat16 *>(dcat), n_dst, &b.counts[CNT_STATUS], st, n_rhs, chain);
         }
         if (!dcat_done) {
             for (int r = 0; r < n_rhs; ++r) {
@@ -385,6 +395,7 @@ static int32_t backward_impl(const e2egrec_block *blocks, int32_t n_layers, cons
         }
         if (l == 0) tap_begin(TAP_AGG_BWD_OUTER, st);
         SegScratch sc = seg_scratch_carve(b.cap_edges, block_run_len(b.cap_edges, p.d_in, dtype_size(X->dtype)), p.d_in, dtype_size(X->dtype), scratch + bs.seg_off, n_rhs);
+        sc.chain = chain;
         sc.chain_cnt = reinterpret_cast<int32_t *>(scratch + bs.chain_off);
         const bool seg_ok = dispatch_seg_reduce<T, int32_t, false>(dcat + p.d_in, two_d, b.csc_ptr, b.csc_row, &b.counts[CNT_SRC], 0,
                                                                    b.cap_src, nullptr, block_run_len(b.cap_edges, p.d_in, dtype_size(X->dtype)), p.d_in, X->dtype,

@@ -169,8 +169,9 @@ hop_sample_kernel(const int64_t *__restrict__ g_indptr, const int32_t *__restric
     __shared__ int32_t scan_sm[kDstThreads / 32 + 1];
     __shared__ long long bcast;
     __shared__ int tile_s;
-    int32_t n_dst = *n_dst_ptr;                      // on their way while the ticket is
-    const uint32_t step = step_arg + *step_offset;
+    pdl_wait();
+    int32_t n_dst = __ldcg(n_dst_ptr);               // on their way while the ticket is
+    const uint32_t step = step_arg + __ldcg(step_offset);
     const int tile = chain_ticket(ticket, &tile_s);
     const bool over = n_dst > cap_dst;
     if (over) n_dst = cap_dst;
@@ -187,7 +188,7 @@ hop_sample_kernel(const int64_t *__restrict__ g_indptr, const int32_t *__restric
     const int64_t i = i0 + threadIdx.x;
     int32_t c = 0;
     if (threadIdx.x < tile_dst && i < n_dst) {
-        int32_t u = dst_nodes[i];
+        int32_t u = __ldcg(dst_nodes + i);
         int64_t gb = 0, deg = 0;
         if ((uint32_t)u < (uint64_t)n_nodes) {
             gb = g_indptr[u];
@@ -290,7 +291,7 @@ hop_sample_kernel(const int64_t *__restrict__ g_indptr, const int32_t *__restric
                 atomicOr((unsigned *)&counts[CNT_STATUS], E2EGREC_DEV_RANGE);
                 v[q] = node[rr[q]];
             }
-            lid[q] = ok[q] ? local_id[v[q]] : 0;
+            lid[q] = ok[q] ? __ldcg(local_id + v[q]) : 0;
         }
         uint32_t word[S];
 #pragma unroll
@@ -329,20 +330,21 @@ frontier_kernel(uint32_t *__restrict__ bitmap, int64_t n_words, int32_t *__restr
     __shared__ int32_t scan_sm[256 / 32 + 1];
     __shared__ long long bcast;
     __shared__ int tile_s;
+    pdl_wait();
     const int tile = chain_ticket(ticket, &tile_s);
     const int64_t w0 = (int64_t)tile * kWordTile + (int64_t)threadIdx.x * WPT;
     uint32_t bits[WPT];
     int32_t c = 0;
 #pragma unroll
     for (int k = 0; k < WPT; ++k) {
-        bits[k] = w0 + k < n_words ? bitmap[w0 + k] : 0u;
+        bits[k] = w0 + k < n_words ? __ldcg(bitmap + w0 + k) : 0u;
         c += __popc(bits[k]);
     }
     int32_t tile_total;
     const int32_t ex = block_exclusive_scan<256, int32_t>(c, tile_total, scan_sm);
     if (threadIdx.x == 0) chain_publish(state, tile, tile_total);
     const long long base = chain_lookback(state, tile, tile_total, &counts[CNT_STATUS], &bcast);
-    const int32_t n_dst = counts[CNT_DST];
+    const int32_t n_dst = __ldcg(counts + CNT_DST);
     const bool last_tile = (int64_t)(tile + 1) * kWordTile >= n_words;
     if (last_tile && threadIdx.x == 0) {
         long long n_src = (long long)n_dst + base + tile_total;
@@ -386,13 +388,14 @@ relabel_kernel(const int32_t *__restrict__ nbr_global, const int32_t *__restrict
                const int32_t *__restrict__ counts, int32_t *__restrict__ col, int bits, int passes, SortState ss)
 {
     __shared__ unsigned h[kMaxPasses * kMaxRadix];
+    pdl_wait();
     const int R = 1 << bits;
     for (int d = threadIdx.x; d < passes * R; d += 256) h[d] = 0;
     __syncthreads();
-    const int32_t n = counts[CNT_EDGES];
-    const int32_t n_src = counts[CNT_SRC];
+    const int32_t n = __ldcg(counts + CNT_EDGES);
+    const int32_t n_src = __ldcg(counts + CNT_SRC);
     for (int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x; e < n; e += (int64_t)gridDim.x * 256) {
-        int32_t c = local_id[nbr_global[e]];
+        int32_t c = __ldcg(local_id + __ldcg(nbr_global + e));
         if (c < 0 || c >= n_src) c = 0;              // only after a capacity overrun, which is flagged
         col[e] = c;
         for (int p = 0; p < passes; ++p) atomicAdd(&h[p * R + ((c >> (p * bits)) & (R - 1))], 1u);
@@ -406,8 +409,9 @@ relabel_kernel(const int32_t *__restrict__ nbr_global, const int32_t *__restrict
 __global__ void frontier_release_kernel(const int32_t *__restrict__ src_nodes, const int32_t *__restrict__ counts,
                                         int32_t *__restrict__ local_id)
 {
+    pdl_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < counts[CNT_SRC]) local_id[src_nodes[i]] = -1;
+    if (i < __ldcg(counts + CNT_SRC)) local_id[__ldcg(src_nodes + i)] = -1;
 }
 
 // csc_ptr[s] = first position whose column is >= s, from the steps of the sorted column array (a search per column cost 20
@@ -417,20 +421,21 @@ __global__ void csc_finalize_kernel(const int32_t *__restrict__ csc_col, const i
                                     int32_t *__restrict__ csc_ptr, SortState ss, int bits, int passes,
                                     const int32_t *__restrict__ release_nodes, int32_t *__restrict__ local_id)
 {
+    pdl_wait();
     if (release_nodes)                               // the last block of a sample also gives the local ids back
-        for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < counts[CNT_SRC]; k += (int64_t)gridDim.x * blockDim.x)
-            local_id[release_nodes[k]] = -1;
-    zero_sort_state(ss, counts[CNT_EDGES], bits, passes);
+        for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < __ldcg(counts + CNT_SRC); k += (int64_t)gridDim.x * blockDim.x)
+            local_id[__ldcg(release_nodes + k)] = -1;
+    zero_sort_state(ss, __ldcg(counts + CNT_EDGES), bits, passes);
     if (blockIdx.x == 0 && threadIdx.x < kMaxPasses) ss.tickets()[threadIdx.x] = 0;
-    const int32_t n = counts[CNT_EDGES], n_src = counts[CNT_SRC];
+    const int32_t n = __ldcg(counts + CNT_EDGES), n_src = __ldcg(counts + CNT_SRC);
     const int lane = threadIdx.x & 31;
     for (int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane; t0 <= n; t0 += (int64_t)gridDim.x * blockDim.x) {
         // position t is the first one whose column is >= s for the columns s in (col[t - 1], col[t]]
         const int32_t t = (int32_t)min(t0 + lane, (int64_t)n + 1);
         int32_t a = n_src, b = n_src;
         if (t <= n) {
-            a = t > 0 ? csc_col[t - 1] : -1;
-            b = t < n ? csc_col[t] : n_src;
+            a = t > 0 ? __ldcg(csc_col + t - 1) : -1;
+            b = t < n ? __ldcg(csc_col + t) : n_src;
         }
         const bool wide = b - a > 4;                 // columns without entries: the warp fills long stretches together
         if (!wide)
@@ -448,6 +453,7 @@ __global__ void csc_finalize_kernel(const int32_t *__restrict__ csc_col, const i
 __global__ void pair_mark_kernel(const int32_t *__restrict__ user, const int32_t *__restrict__ item, int32_t n_pairs,
                                  int64_t n_nodes, uint32_t *__restrict__ bitmap, int32_t *__restrict__ counts)
 {
+    pdl_wait();
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n_pairs) return;
     const int32_t ids[2] = {user[p], item[p]};
@@ -468,6 +474,7 @@ pair_local_kernel(const int32_t *__restrict__ user, const int32_t *__restrict__ 
                   int bits, int passes, SortState ss)
 {
     __shared__ unsigned h[kMaxPasses * kMaxRadix];
+    pdl_wait();
     const int R = 1 << bits;
     for (int d = threadIdx.x; d < passes * R; d += 256) h[d] = 0;
     __syncthreads();
@@ -476,7 +483,7 @@ pair_local_kernel(const int32_t *__restrict__ user, const int32_t *__restrict__ 
         const bool is_item = e >= n_pairs;
         const int32_t pr = (int32_t)(is_item ? e - n_pairs : e);
         const int32_t id = is_item ? item[pr] : user[pr];
-        int32_t c = (uint32_t)id < (uint64_t)n_nodes ? local_id[id] : 0;
+        int32_t c = (uint32_t)id < (uint64_t)n_nodes ? __ldcg(local_id + id) : 0;
         if (c < 0) c = 0;
         pair_local[e] = c;
         entry_unit[e] = pr * units_per_row + (is_item ? item_unit_off : 0);
@@ -491,19 +498,19 @@ pair_local_kernel(const int32_t *__restrict__ user, const int32_t *__restrict__ 
 // The transposed block: entries ordered by (column, position), the last pass looking up every entry's row, and the offsets.
 static void transpose_block(const int32_t *col, int32_t *counts, int32_t cap_edges, const int32_t *row_of,
                             int32_t *csc_col, int32_t *csc_eid, int32_t *csc_row, int32_t *csc_ptr, const SortPlan &sp,
-                            const SortLane &l, cudaStream_t st, const int32_t *release_nodes = nullptr, int32_t *local_id = nullptr)
+                            const SortLane &l, bool chain, cudaStream_t st, const int32_t *release_nodes = nullptr, int32_t *local_id = nullptr)
 {
     const int32_t *k = col, *v = nullptr;
     for (int p = 0; p < sp.passes; ++p) {
         const bool last = p == sp.passes - 1, own = (sp.passes - 1 - p) % 2 == 0;       // the last pass ends in the block's arrays
         int32_t *ko = own ? csc_col : l.key, *vo = own ? csc_eid : l.val;
-        sort_pass<int32_t>(sp, k, v, &counts[CNT_EDGES], cap_edges, 0, 0, p, l.sort, ko, vo, last ? SortMap{row_of, csc_row} : SortMap{},
+        sort_pass<int32_t>(sp, k, v, &counts[CNT_EDGES], cap_edges, 0, 0, p, l.sort, chain, ko, vo, last ? SortMap{row_of, csc_row} : SortMap{},
                            &counts[CNT_STATUS], st);
         k = ko;
         v = vo;
     }
     note_launch();
-    csc_finalize_kernel<<<(unsigned)std::min<int64_t>(ceil_div((int64_t)cap_edges + 1, 256), 148 * 8), 256, 0, st>>>(csc_col, counts, csc_ptr, l.sort, sp.bits, sp.passes,
+    launch_pdl(chain, csc_finalize_kernel, dim3((unsigned)std::min<int64_t>(ceil_div((int64_t)cap_edges + 1, 256), 148 * 8)), dim3(256), 0, st, csc_col, counts, csc_ptr, l.sort, sp.bits, sp.passes,
                                                                                                                 release_nodes, local_id);
 }
 
@@ -680,29 +687,28 @@ int32_t e2egrec::sample_khop_impl(const e2egrec_csr *graph, const int32_t *seeds
     }
     const int64_t zero16 = ceil_div(reinterpret_cast<char *>(chain) - s.zero, 16);
     note_launch();
-    sample_begin_kernel<<<(unsigned)std::min<int64_t>(std::max<int64_t>(ceil_div(zero16, 256 * 2), grid_for(pairs ? 0 : n_seeds, 256)), 148 * 8), 256, 0, st>>>(
-        reinterpret_cast<uint4 *>(s.zero), zero16, pairs ? nullptr : seeds, n_seeds, n, s.local_id, blocks[0].counts,
+    sample_begin_kernel<<<(unsigned)std::min<int64_t>(std::max<int64_t>(ceil_div(zero16, 256 * 2), grid_for(pairs ? 0 : n_seeds, 256)), 148 * 8), 256, 0, st>>>(reinterpret_cast<uint4 *>(s.zero), zero16, pairs ? nullptr : seeds, n_seeds, n, s.local_id, blocks[0].counts,
         pairs ? pairs->pcounts : nullptr);
     cudaStream_t ts = side ? side->stream : st;          // stream of the transpositions
+    const bool chained = me < kChainEdges;
     if (pairs) {
         // seeds = ascending distinct endpoints of the pairs; entries (pair, side) grouped by seed.  Nobody reads the groups
         // before the backward pass: they are sorted on the helper stream, in a lane that no hop uses if there is one.
         const PairInput &pi = *pairs;
         const int32_t P2 = 2 * pi.n_pairs;
         note_launch();
-        pair_mark_kernel<<<grid_for(pi.n_pairs, T), T, 0, st>>>(pi.user, pi.item, pi.n_pairs, n, s.bitmap, blocks[0].counts);
+        launch_pdl(chained, pair_mark_kernel, dim3(grid_for(pi.n_pairs, T)), dim3(T), 0, st, pi.user, pi.item, pi.n_pairs, n, s.bitmap, blocks[0].counts);
         note_launch();
-        frontier_kernel<<<(unsigned)s.word_tiles, 256, 0, st>>>(s.bitmap, s.n_words, pi.pcounts, P2, s.local_id, pi.seeds_out,
+        launch_pdl(chained, frontier_kernel, dim3((unsigned)s.word_tiles), dim3(256), 0, st, s.bitmap, s.n_words, pi.pcounts, P2, s.local_id, pi.seeds_out,
                                                                 s.tickets + 2 * kMaxHops, words[n_hops]);
         const SortPlan sp = sort_plan(P2 > 1 ? P2 : 2);
         const bool own_lane = n_hops < kMaxHops;
         const SortLane &l = s.lane[own_lane ? kMaxHops - 1 : 0];
         note_launch();
-        pair_local_kernel<<<(unsigned)std::min<int64_t>(grid_for(P2, T), 148 * 4), T, 0, st>>>(
-            pi.user, pi.item, pi.n_pairs, n, s.local_id, pi.pair_local, pi.entry_unit, pi.units_per_row, pi.item_unit_off,
+        launch_pdl(chained, pair_local_kernel, dim3((unsigned)std::min<int64_t>(grid_for(P2, T), 148 * 4)), dim3(T), 0, st, pi.user, pi.item, pi.n_pairs, n, s.local_id, pi.pair_local, pi.entry_unit, pi.units_per_row, pi.item_unit_off,
             pi.pcounts, sp.bits, sp.passes, l.sort);
         if (side && own_lane) side->fork(st);
-        transpose_block(pi.pair_local, pi.pcounts, P2, pi.entry_unit, pi.pcsc_col, pi.pcsc_eid, pi.pcsc_idx, pi.pcsc_ptr, sp, l,
+        transpose_block(pi.pair_local, pi.pcounts, P2, pi.entry_unit, pi.pcsc_col, pi.pcsc_eid, pi.pcsc_idx, pi.pcsc_ptr, sp, l, chained,
                         own_lane ? ts : st);
         if (!own_lane) cudaMemsetAsync(l.sort.ghist, 0, sizeof(unsigned) * kSortCountWords, st);
         dst_nodes = pi.seeds_out;
@@ -717,20 +723,18 @@ int32_t e2egrec::sample_khop_impl(const e2egrec_csr *graph, const int32_t *seeds
         const int tile = dst_tile(b.cap_dst, fanouts[h]);
         auto sample = graph->edge_cum ? hop_sample_kernel<true> : hop_sample_kernel<false>;
         note_launch();
-        sample<<<grid_for(b.cap_dst, tile), kDstThreads, 0, st>>>(
-            graph->indptr, graph->indices, graph->edge_cum, n, dst_nodes, n_dst_ptr, b.cap_dst, b.cap_edges, fanouts[h], tile, h + 1,
+        launch_pdl(chained, sample, dim3(grid_for(b.cap_dst, tile)), dim3(kDstThreads), 0, st, graph->indptr, graph->indices, graph->edge_cum, n, dst_nodes, n_dst_ptr, b.cap_dst, b.cap_edges, fanouts[h], tile, h + 1,
             (uint32_t)(seed & 0xFFFFFFFFu), (uint32_t)(seed >> 32), step, s.step_offset, h == 0, b.counts, b.indptr,
             b.inv_cnt, b.src_nodes, b.nbr_global, l.edge_row, s.local_id, s.bitmap, s.tickets + 2 * h, tiles[h]);
         note_launch();
-        frontier_kernel<<<(unsigned)s.word_tiles, 256, 0, st>>>(s.bitmap, s.n_words, b.counts, b.cap_src, s.local_id, b.src_nodes,
+        launch_pdl(chained, frontier_kernel, dim3((unsigned)s.word_tiles), dim3(256), 0, st, s.bitmap, s.n_words, b.counts, b.cap_src, s.local_id, b.src_nodes,
                                                                 s.tickets + 2 * h + 1, words[h]);
         note_launch();
-        relabel_kernel<<<(unsigned)std::min<int64_t>(grid_for(b.cap_edges, T), 148 * 4), T, 0, st>>>(
-            b.nbr_global, s.local_id, b.counts, b.col, sp.bits, sp.passes, l.sort);
+        launch_pdl(chained, relabel_kernel, dim3((unsigned)std::min<int64_t>(grid_for(b.cap_edges, T), 148 * 4)), dim3(T), 0, st, b.nbr_global, s.local_id, b.counts, b.col, sp.bits, sp.passes, l.sort);
         if (transpose) {
             if (side) side->fork(st);
             const bool release = h == n_hops - 1;        // every relabelling is done: the last block's offsets release the ids
-            transpose_block(b.col, b.counts, b.cap_edges, l.edge_row, b.csc_col, b.csc_eid, b.csc_row, b.csc_ptr, sp, l, ts,
+            transpose_block(b.col, b.counts, b.cap_edges, l.edge_row, b.csc_col, b.csc_eid, b.csc_row, b.csc_ptr, sp, l, chained, ts,
                             release ? last.src_nodes : nullptr, s.local_id);
         }
         dst_nodes = b.src_nodes;
@@ -738,7 +742,7 @@ int32_t e2egrec::sample_khop_impl(const e2egrec_csr *graph, const int32_t *seeds
     }
     if (!transpose) {
         note_launch();
-        frontier_release_kernel<<<grid_for(last.cap_src, T), T, 0, st>>>(last.src_nodes, last.counts, s.local_id);
+        launch_pdl(chained, frontier_release_kernel, dim3(grid_for(last.cap_src, T)), dim3(T), 0, st, last.src_nodes, last.counts, s.local_id);
     }
     if (side && (transpose || (pairs && n_hops < kMaxHops))) {
         if (flags & E2EGREC_SAMPLE_DEFER_TRANSPOSE) side->defer();
@@ -779,7 +783,7 @@ extern "C" int32_t e2egrec_blocks_transpose(int64_t n_nodes, int32_t n_hops, con
         const SortLane &l = s.lane[h];
         cudaStream_t ts = st;
         if (forked && ((n_hops - 1 - h) & 1)) ts = side->stream;
-        transpose_block(b.col, b.counts, b.cap_edges, l.edge_row, b.csc_col, b.csc_eid, b.csc_row, b.csc_ptr, sp, l, ts);
+        transpose_block(b.col, b.counts, b.cap_edges, l.edge_row, b.csc_col, b.csc_eid, b.csc_row, b.csc_ptr, sp, l, me < kChainEdges, ts);
     }
     if (forked) side->join(st);
     return check_launch("blocks_transpose");

@@ -45,6 +45,7 @@ struct SegScratch {
     // The caller sets it to n_windows zeroed int32 (seg_chain_bytes) before the first launch that uses them; every
     // launch leaves them zero again.
     int32_t *chain_cnt;
+    bool chain;                    // launch_pdl's `chain` for small streams (sampled blocks)
 };
 
 inline size_t seg_chain_bytes(int64_t cap_entries, int run_len, int d, size_t elem_size, int n_rhs = 1)
@@ -71,6 +72,7 @@ inline SegScratch seg_scratch_carve(int64_t cap_entries, int run_len, int d, siz
     s.tail2 = (float *)take((size_t)n_rhs * s.n_windows * d * sizeof(float));
     s.win_info = (int4 *)take((size_t)n_rhs * s.n_windows * sizeof(int4));
     s.bytes = off;
+    s.chain = true;
     return s;
 }
 
@@ -328,10 +330,9 @@ seg_run_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict__
     const int rl = threadIdx.x / LPR;              // run within the block
     const int n_chunks = d / E;
     const int64_t run = (int64_t)blockIdx.x * RB + rl;
-    pdl_launch_dependents();
     pdl_wait();                                    // the kernel before this one in the stream has completed
-    const int64_t n_seg = n_seg_dev ? (int64_t)*n_seg_dev : n_seg_host;
-    const int64_t total = n_seg > 0 ? (int64_t)ptr[n_seg] : 0;
+    const int64_t n_seg = n_seg_dev ? (int64_t)__ldcg(n_seg_dev) : n_seg_host;
+    const int64_t total = n_seg > 0 ? (int64_t)__ldcg(ptr + n_seg) : 0;
     const int64_t k0 = run * run_len;
     // a window that lies wholly beyond the stream (grids are sized for capacities) has nothing to do, not even a
     // record: seg_final_kernel only looks at the windows that hold entries
@@ -363,7 +364,7 @@ seg_run_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict__
         const int len = (int)min((int64_t)run_len, total - k0);   // entries of this run; positions below are relative to k0
         const int32_t *__restrict__ idx0 = idx + k0;
         const int32_t *__restrict__ seg0 = seg_of + k0;
-        const int64_t n_self = (kExtra && o.self) ? (o.n_self ? (int64_t)*o.n_self : n_seg) : 0;
+        const int64_t n_self = (kExtra && o.self) ? (o.n_self ? (int64_t)__ldcg(o.n_self) : n_seg) : 0;
 
         // Segment boundaries are found one iteration ahead of the sums: changes of the entry -> segment array.
         int32_t ws = seg0[0];          // segment of the entry classified last
@@ -549,7 +550,6 @@ seg_run_block_kernel(const __grid_constant__ CUtensorMap in_map, const T *__rest
         }
         __syncwarp();
     }
-    pdl_launch_dependents();
     pdl_wait();                                    // the kernel before this one in the stream has completed
     if (blockIdx.y) {                              // the second right-hand side: other rows, same segments
         const int64_t r = blockIdx.y, nw = gridDim.x;
@@ -561,8 +561,8 @@ seg_run_block_kernel(const __grid_constant__ CUtensorMap in_map, const T *__rest
         tail2 += r * nw * d;
         if (chain_cnt) chain_cnt += r * nw;
     }
-    const int32_t n_seg = *n_seg_dev;
-    const int32_t total = n_seg > 0 ? ptr[n_seg] : 0;
+    const int32_t n_seg = __ldcg(n_seg_dev);
+    const int32_t total = n_seg > 0 ? __ldcg(ptr + n_seg) : 0;
     const int64_t k0 = run * run_len;
     int32_t head_seg = -1, head_ends = 0, tail_seg = -1;
     // a window that lies wholly beyond the stream (grids are sized for capacities) has no run work and no join, but
@@ -573,7 +573,7 @@ seg_run_block_kernel(const __grid_constant__ CUtensorMap in_map, const T *__rest
         const int len = (int)min((int64_t)run_len, (int64_t)total - k0);
         const int32_t *__restrict__ idx0 = idx + k0;
         const int32_t *__restrict__ seg0 = seg_of + k0;
-        const int32_t n_self = o.n_self ? *o.n_self : n_seg;
+        const int32_t n_self = o.n_self ? __ldcg(o.n_self) : n_seg;
         const bool lane_on = c < n_chunks;
         const T *__restrict__ in_c = in + c * E;
         const T *__restrict__ self_c = o.self + c * E;
@@ -767,7 +767,7 @@ seg_run_block_kernel(const __grid_constant__ CUtensorMap in_map, const T *__rest
     // ---- segments without entries (their row is the self row, masked, or zero) and the zero rows up to the next
     // multiple of 128: every block of the grid takes a slice, one lane group per segment
     {
-        const int32_t n_self = o.n_self ? *o.n_self : n_seg;
+        const int32_t n_self = o.n_self ? __ldcg(o.n_self) : n_seg;
         const int32_t per = (n_seg + (int32_t)gridDim.x - 1) / (int32_t)gridDim.x;
         const int32_t s1 = min(n_seg, ((int32_t)blockIdx.x + 1) * per);
         for (int32_t sg = (int32_t)blockIdx.x * per + rl; sg < s1; sg += RB) {
@@ -804,11 +804,10 @@ seg_final_kernel(const PtrT *__restrict__ ptr, const int32_t *n_seg_dev, int64_t
     __shared__ int32_t sh_seg[kFinalWindows];
     __shared__ int sh_long[kFinalWindows];
     __shared__ int sh_n_long;
-    pdl_launch_dependents();
     pdl_wait();
-    const int64_t n_seg = n_seg_dev ? (int64_t)*n_seg_dev : n_seg_host;
+    const int64_t n_seg = n_seg_dev ? (int64_t)__ldcg(n_seg_dev) : n_seg_host;
     if (n_seg < 0) return;
-    const int64_t n_self = o.self ? (o.n_self ? (int64_t)*o.n_self : n_seg) : 0;
+    const int64_t n_self = o.self ? (o.n_self ? (int64_t)__ldcg(o.n_self) : n_seg) : 0;
 
     if ((int64_t)blockIdx.x >= n_window_blocks) {
         // segments without entries, the extra blocks stride over all segments
@@ -993,7 +992,7 @@ inline void launch_seg_final(const PtrT *ptr, const int32_t *n_seg_dev, int64_t 
     const int64_t empty_blocks = std::min<int64_t>(ceil_div(cap_seg > 0 ? cap_seg : 1, kAggThreads), 148 * 8);
     tap_begin(TAP_SEG_L3, st);
     note_launch();
-    launch_pdl(seg_final_kernel<T, PtrT>, dim3((unsigned)(window_blocks + empty_blocks)), dim3(kAggThreads), 0, st, ptr, n_seg_dev,
+    launch_pdl(sc.chain && n_seg_dev && sc.cap_runs * run_len < kChainEdges, seg_final_kernel<T, PtrT>, dim3((unsigned)(window_blocks + empty_blocks)), dim3(kAggThreads), 0, st, ptr, n_seg_dev,
                n_seg_host, run_len, sc.runs_per_window, d, (const float *)sc.head2, (const float *)sc.tail2, (const int4 *)sc.win_info,
                sc.n_windows, window_blocks, o);
     tap_end(TAP_SEG_L3, st);
@@ -1025,6 +1024,7 @@ inline void launch_seg_reduce(const T *in, int64_t ld_in, const PtrT *ptr, const
         }
         return;
     }
+    const bool chain = sc.chain && n_seg_dev && sc.cap_runs * run_len < kChainEdges;
     tap_begin(TAP_SEG_L1, st);
     note_launch();
     const unsigned grid1 = (unsigned)sc.n_windows;
@@ -1052,20 +1052,20 @@ inline void launch_seg_reduce(const T *in, int64_t ld_in, const PtrT *ptr, const
                     if (dev >= 0 && dev < 64 && attr_set[mk][dev]) {
                         streamed = true;
                         if (o.mask)
-                            launch_pdl(seg_run_block_kernel<T, LPR, true, 4, 3, true>, grid_b, dim3(kAggThreads), smem_s, st, in_map, in, ld_in, ptr,
+                            launch_pdl(chain, seg_run_block_kernel<T, LPR, true, 4, 3, true>, grid_b, dim3(kAggThreads), smem_s, st, in_map, in, ld_in, ptr,
                                        idx, seg_of, n_seg_dev, run_len, d, sc.head2, sc.tail2, sc.win_info, sc.cap_runs, sc.chain_cnt, o);
                         else
-                            launch_pdl(seg_run_block_kernel<T, LPR, false, 4, 4, true>, grid_b, dim3(kAggThreads), smem_s, st, in_map, in, ld_in, ptr,
+                            launch_pdl(chain, seg_run_block_kernel<T, LPR, false, 4, 4, true>, grid_b, dim3(kAggThreads), smem_s, st, in_map, in, ld_in, ptr,
                                        idx, seg_of, n_seg_dev, run_len, d, sc.head2, sc.tail2, sc.win_info, sc.cap_runs, sc.chain_cnt, o);
                     }
                 }
             }
             if (streamed) {
             } else if (o.mask)
-                launch_pdl(seg_run_block_kernel<T, LPR, true>, grid_b, dim3(kAggThreads), smem, st, in_map, in, ld_in, ptr, idx, seg_of,
+                launch_pdl(chain, seg_run_block_kernel<T, LPR, true>, grid_b, dim3(kAggThreads), smem, st, in_map, in, ld_in, ptr, idx, seg_of,
                            n_seg_dev, run_len, d, sc.head2, sc.tail2, sc.win_info, sc.cap_runs, sc.chain_cnt, o);
             else
-                launch_pdl(seg_run_block_kernel<T, LPR, false>, grid_b, dim3(kAggThreads), smem, st, in_map, in, ld_in, ptr, idx, seg_of,
+                launch_pdl(chain, seg_run_block_kernel<T, LPR, false>, grid_b, dim3(kAggThreads), smem, st, in_map, in, ld_in, ptr, idx, seg_of,
                            n_seg_dev, run_len, d, sc.head2, sc.tail2, sc.win_info, sc.cap_runs, sc.chain_cnt, o);
             if (sc.chain_cnt) {                   // chains, empty segments and padding were all done in that launch
                 tap_end(TAP_SEG_L1, st);
@@ -1079,17 +1079,17 @@ inline void launch_seg_reduce(const T *in, int64_t ld_in, const PtrT *ptr, const
     } else if (o.mask) {
         auto kern = seg_run_kernel<T, PtrT, LPR, CPL, kWeight, 2>;
         if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        launch_pdl(kern, dim3(grid1), dim3(kAggThreads), smem, st, in, ld_in, ptr, idx, n_seg_dev, n_seg_host, w, run_len, d, sc.head2,
+        launch_pdl(chain, kern, dim3(grid1), dim3(kAggThreads), smem, st, in, ld_in, ptr, idx, n_seg_dev, n_seg_host, w, run_len, d, sc.head2,
                    sc.tail2, sc.win_info, sc.cap_runs, seg_of, o);
     } else if (o.self) {
         auto kern = seg_run_kernel<T, PtrT, LPR, CPL, kWeight, 1>;
         if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        launch_pdl(kern, dim3(grid1), dim3(kAggThreads), smem, st, in, ld_in, ptr, idx, n_seg_dev, n_seg_host, w, run_len, d, sc.head2,
+        launch_pdl(chain, kern, dim3(grid1), dim3(kAggThreads), smem, st, in, ld_in, ptr, idx, n_seg_dev, n_seg_host, w, run_len, d, sc.head2,
                    sc.tail2, sc.win_info, sc.cap_runs, seg_of, o);
     } else {
         auto kern = seg_run_kernel<T, PtrT, LPR, CPL, kWeight, 0>;
         if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        launch_pdl(kern, dim3(grid1), dim3(kAggThreads), smem, st, in, ld_in, ptr, idx, n_seg_dev, n_seg_host, w, run_len, d, sc.head2,
+        launch_pdl(chain, kern, dim3(grid1), dim3(kAggThreads), smem, st, in, ld_in, ptr, idx, n_seg_dev, n_seg_host, w, run_len, d, sc.head2,
                    sc.tail2, sc.win_info, sc.cap_runs, seg_of, o);
     }
     tap_end(TAP_SEG_L1, st);

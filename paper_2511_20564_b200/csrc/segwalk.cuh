@@ -135,8 +135,9 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
     __shared__ int32_t sh_win[4];
 
     const int n_chunks = d / E;
-    const int64_t n_seg = n_seg_dev ? (int64_t)*n_seg_dev : n_seg_host;
-    const int64_t total = n_seg > 0 ? min((int64_t)ptr[n_seg], cap) : 0;
+    pdl_wait();
+    const int64_t n_seg = n_seg_dev ? (int64_t)__ldcg(n_seg_dev) : n_seg_host;
+    const int64_t total = n_seg > 0 ? min((int64_t)__ldcg(ptr + n_seg), cap) : 0;
     if ((int64_t)blockIdx.x * win_len >= total) return;          // a window beyond the stream leaves no record
     const int stretch = win_len / kWalkWarps;
     if (threadIdx.x < 4) sh_win[threadIdx.x] = threadIdx.x == 1 || threadIdx.x == 3 ? 0 : -1;
@@ -356,9 +357,9 @@ inline void launch_seg_walk(const T *in, int64_t ld_in, const PtrT *ptr, const i
     if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     tap_begin(TAP_SEG_L1, st);
     note_launch();
-    kern<<<(unsigned)sc.n_windows, kAggThreads, smem, st>>>(in, ld_in, ptr, idx, n_seg_dev, n_seg_host, w,
-                                                            run_len * sc.runs_per_window, sc.cap_runs * run_len, d, sc.head2, sc.tail2,
-                                                            sc.win_info, o);
+    launch_pdl(n_seg_dev && sc.cap_runs * run_len < kChainEdges, kern, dim3((unsigned)sc.n_windows), dim3(kAggThreads), smem, st, in, ld_in,
+               ptr, idx, n_seg_dev, n_seg_host, w, run_len * sc.runs_per_window, sc.cap_runs * run_len, d, sc.head2, sc.tail2,
+               sc.win_info, o);
     tap_end(TAP_SEG_L1, st);
     launch_seg_final(ptr, n_seg_dev, n_seg_host, cap_seg, run_len, d, sc, o, st);
 }
