@@ -61,7 +61,7 @@ void note_launch();
 // machine and whose legs run on two streams, loses: 1357 / 1370 with its samples' sorts
 // and first hops launched this way, 1385 with the small kernels of its top layer as well.  Admitting the next kernel while this one still runs
 // (griddepcontrol.launch_dependents at its beginning) keeps the other stream's kernels off the SMs: 182 for the medium step.
-constexpr int64_t kChainEdges = 1ll << 20, kChainRows = 1ll << 17;
+constexpr int64_t kChainEdges = 1ll << 21, kChainRows = 1ll << 17;
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(bool chain, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args &&...args)
 {

@@ -10,21 +10,90 @@
 #include <cooperative_groups.h>
 #include <string.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace e2egrec {
 
-constexpr int kGemmBM = 64, kGemmBN = 64, kGemmBK = 16, kGemmThreads = 256;
+// At the sizes of a batch the time is the K loop's chain of loads, not its arithmetic: the next 64 x 32 tiles are loaded
+// into registers (four values at a time where rows are aligned) while the current ones are multiplied out of shared memory,
+// two buffers, one barrier per step.  Loading, storing and multiplying in turn with steps of 16 took 1.7 us a step; B200,
+// 10 k x 72 x 200 fp32 29 -> 22 us, 777 x 72 x 144 16 -> 12.
+constexpr int kGemmBM = 64, kGemmBN = 64, kGemmBK = 32, kGemmThreads = 256;
+
+// four values from p on, `n` of them there
+template <typename T> __device__ __forceinline__ float4 gemm_load4(const T *p, int n, bool vec)
+{
+    if (vec && n >= 4) {
+        if constexpr (sizeof(T) == 4) {
+            return *reinterpret_cast<const float4 *>(p);
+        } else {
+            const uint2 r = *reinterpret_cast<const uint2 *>(p);
+            return make_float4(__uint_as_float(r.x << 16), __uint_as_float(r.x & 0xFFFF0000u), __uint_as_float(r.y << 16),
+                               __uint_as_float(r.y & 0xFFFF0000u));
+        }
+    }
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (n > 0) v.x = to_float<T>(p[0]);
+    if (n > 1) v.y = to_float<T>(p[1]);
+    if (n > 2) v.z = to_float<T>(p[2]);
+    if (n > 3) v.w = to_float<T>(p[3]);
+    return v;
+}
+
+// One operand's 64 x kGemmBK tile: two groups of four values per thread, along k (rows of the matrix are rows of the tile)
+// or along the tile's rows (KM: rows of the matrix are lines of k).
+template <typename T, bool KM>
+struct GemmTile {
+    static constexpr int kLd = 64 + 4;
+    const T *p;
+    int64_t ld, rows, r0;
+    bool vec;
+    __device__ GemmTile(const T *p_, int64_t ld_, int64_t rows_, int64_t r0_) : p(p_), ld(ld_), rows(rows_), r0(r0_)
+    {
+        vec = (ld * (int64_t)sizeof(T)) % (4 * sizeof(T)) == 0 && reinterpret_cast<uintptr_t>(p) % (4 * sizeof(T)) == 0;
+    }
+    __device__ __forceinline__ void load(float4 (&v)[2], int64_t k0, int64_t ke) const
+    {
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            const int id = threadIdx.x + t * kGemmThreads;
+            v[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (KM) {
+                const int64_t k = k0 + (id >> 4), r = r0 + (id & 15) * 4;
+                if (k < ke && r < rows) v[t] = gemm_load4(p + k * ld + r, (int)min((int64_t)4, rows - r), vec);
+            } else {
+                const int64_t r = r0 + (id >> 3), k = k0 + (id & 7) * 4;
+                if (r < rows && k < ke) v[t] = gemm_load4(p + r * ld + k, (int)min((int64_t)4, ke - k), vec);
+            }
+        }
+    }
+    __device__ __forceinline__ void store(const float4 (&v)[2], float (*s)[kLd]) const
+    {
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            const int id = threadIdx.x + t * kGemmThreads;
+            if (KM) {
+                *reinterpret_cast<float4 *>(&s[id >> 4][(id & 15) * 4]) = v[t];
+            } else {
+                const int r = id >> 3, k = (id & 7) * 4;
+                s[k][r] = v[t].x; s[k + 1][r] = v[t].y; s[k + 2][r] = v[t].z; s[k + 3][r] = v[t].w;
+            }
+        }
+    }
+};
 
 template <typename T, bool A_KM, bool B_KN, class Epi>
 __global__ void __launch_bounds__(kGemmThreads)
-gemm_simt_kernel(const T *__restrict__ A, int64_t lda, const T *__restrict__ B, int64_t ldb, int64_t M_host,
-                 int N, int64_t K_host, const int32_t *m_dev, const int32_t *k_dev, Epi epi)
+gemm_simt_kernel(const T *A, int64_t lda, const T *B, int64_t ldb, int64_t M_host, int N, int64_t K_host, const int32_t *m_dev,
+                 const int32_t *k_dev, Epi epi)
 {
-    __shared__ float As[kGemmBK][kGemmBM + 4];
-    __shared__ float Bs[kGemmBK][kGemmBN + 4];
-    const int64_t M = m_dev ? min((int64_t)*m_dev, M_host) : M_host;
-    const int64_t K = k_dev ? min((int64_t)*k_dev, K_host) : K_host;
+    __shared__ __align__(16) float As[2][kGemmBK][kGemmBM + 4];
+    __shared__ __align__(16) float Bs[2][kGemmBK][kGemmBN + 4];
+    pdl_wait();
+    const int64_t M = m_dev ? min((int64_t)__ldcg(m_dev), M_host) : M_host;
+    const int64_t K = k_dev ? min((int64_t)__ldcg(k_dev), K_host) : K_host;
     const int64_t m0 = (int64_t)blockIdx.x * kGemmBM;
     const int n0 = blockIdx.y * kGemmBN;
     if (m0 >= M) return;
@@ -39,34 +108,36 @@ gemm_simt_kernel(const T *__restrict__ A, int64_t lda, const T *__restrict__ B, 
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
 
-    for (int64_t k0 = kb; k0 < ke; k0 += kGemmBK) {
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const int id = threadIdx.x + t * kGemmThreads;
-            int r, kk;
-            if (A_KM) { r = id & 63; kk = id >> 6; } else { r = id >> 4; kk = id & 15; }
-            const int64_t m = m0 + r, k = k0 + kk;
-            float v = 0.f;
-            if (m < M && k < ke) v = to_float<T>(A_KM ? A[k * lda + m] : A[m * lda + k]);
-            As[kk][r] = v;
-            if (B_KN) { r = id & 63; kk = id >> 6; } else { r = id >> 4; kk = id & 15; }
-            const int64_t n = n0 + r;
-            v = 0.f;
-            if (n < N && k0 + kk < ke) v = to_float<T>(B_KN ? B[(k0 + kk) * ldb + n] : B[n * ldb + k0 + kk]);
-            Bs[kk][r] = v;
+    const GemmTile<T, A_KM> ta(A, lda, M, m0);
+    const GemmTile<T, B_KN> tb(B, ldb, N, n0);
+    float4 va[2], vb[2];
+    if (kb < ke) {
+        ta.load(va, kb, ke);
+        tb.load(vb, kb, ke);
+        ta.store(va, As[0]);
+        tb.store(vb, Bs[0]);
+    }
+    __syncthreads();
+    int cur = 0;
+    for (int64_t k0 = kb; k0 < ke; k0 += kGemmBK, cur ^= 1) {
+        const bool more = k0 + kGemmBK < ke;
+        if (more) {
+            ta.load(va, k0 + kGemmBK, ke);
+            tb.load(vb, k0 + kGemmBK, ke);
         }
-        __syncthreads();
-#pragma unroll
+#pragma unroll 8
         for (int kk = 0; kk < kGemmBK; ++kk) {
-            float a[4], b[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = As[kk][ty * 4 + i];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx * 4 + j];
+            const float4 a4 = *reinterpret_cast<const float4 *>(&As[cur][kk][ty * 4]);
+            const float4 b4 = *reinterpret_cast<const float4 *>(&Bs[cur][kk][tx * 4]);
+            const float a[4] = {a4.x, a4.y, a4.z, a4.w}, b[4] = {b4.x, b4.y, b4.z, b4.w};
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+        }
+        if (more) {
+            ta.store(va, As[cur ^ 1]);
+            tb.store(vb, Bs[cur ^ 1]);
         }
         __syncthreads();
     }
@@ -78,6 +149,23 @@ gemm_simt_kernel(const T *__restrict__ A, int64_t lda, const T *__restrict__ B, 
             const int n = n0 + tx * 4 + j;
             if (m < M && n < N) epi(m, n, acc[i][j], blockIdx.z);
         }
+}
+
+template <typename T, bool A_KM, bool B_KN, class Epi>
+inline void launch_gemm_simt(bool chain, dim3 grid, cudaStream_t st, const T *A, int64_t lda, const T *B, int64_t ldb, int64_t M, int N,
+                             int64_t K, const int32_t *m_dev, const int32_t *k_dev, const Epi &epi)
+{
+    note_launch();
+    launch_pdl(chain, gemm_simt_kernel<T, A_KM, B_KN, Epi>, grid, dim3(kGemmThreads), 0, st, A, lda, B, ldb, M, N, K, m_dev, k_dev, epi);
+}
+
+// Splits over `rows` (a capacity) of an m x n weight gradient on this kernel, at most `most`: two blocks per SM over all
+// output tiles and at least 64 rows each.  With 148 splits whatever the shape, a 320 x 320 result was 3700 blocks of at
+// most 16 rows and 60 MB of partial sums (24 + 12 us; the gated joint step 331 -> 273 us with this and the narrower products).
+inline int simt_splits(int64_t rows, int m, int n, int most)
+{
+    const int64_t tiles = ceil_div(m, kGemmBM) * ceil_div(n, kGemmBN);
+    return (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)most, ceil_div(2 * 148, tiles), ceil_div(rows, 64)}));
 }
 
 // h' = act(z + b), stored in the feature dtype
@@ -123,6 +211,8 @@ static __global__ void splitk_reduce_kernel(const float *__restrict__ partial, i
         active = (int)max((int64_t)1, (total + per - 1) / per);
     }
     float s = accumulate ? out[i] : 0.f;
+    // eight loads in flight, added in order
+#pragma unroll 8
     for (int z = 0; z < active; ++z) s += __ldcg(partial + (int64_t)z * n + i);
     out[i] = s;
 }

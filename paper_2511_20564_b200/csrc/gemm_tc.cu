@@ -708,8 +708,15 @@ bool launch_tn(const __nv_bfloat16 *A, int64_t rows, int k, int64_t lda, const _
     ep.rhs_rows = rows;
     int nt = 0;                                 // widest tile <= 256 columns that divides n (a multiple of 32, or of 64 for b_mn)
     const int unit = b_mn ? 64 : 32;
-    for (int c = 256; c >= unit; c -= unit)
-        if (n % c == 0) { nt = c; break; }
+    // ... or, where such tiles would leave more than half of the SMs without one, the widest of 64 columns and more that does
+    // not, else the narrowest of those: one tile's chain of loads, products and stores is what a small product costs, and
+    // half the columns are half of its stores (B200, 4096 x 320 x 512: 13.3 us with 64 tiles of 256 columns, 10.2 with 128
+    // of 128; 1000 x 320 x 320 gated: 27 us with 16 tiles of 160 before)
+    for (int c = 256; c >= unit; c -= unit) {
+        if (n % c || (nt && c < 64)) continue;
+        nt = c;
+        if ((rows / kTileM) * (n / c) * n_rhs >= sm_count() / 2) break;
+    }
     if (!nt) return false;
     if (reinterpret_cast<uintptr_t>(A) % 16 || reinterpret_cast<uintptr_t>(B) % 16 || (lda * 2) % 16 || (ldb * 2) % 16 ||
         reinterpret_cast<uintptr_t>(ep.out) % 16 || (ep.ldo * 2) % 16)

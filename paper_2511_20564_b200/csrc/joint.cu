@@ -174,8 +174,7 @@ void linear_forward(const T *A, int64_t rows, int k, const T *W, int n, const fl
         return;
     EpiUpdate<T> epi{out, n, bias, relu};
     dim3 grid((unsigned)ceil_div(rows, kGemmBM), (unsigned)ceil_div(n, kGemmBN), 1);
-    note_launch();
-    gemm_simt_kernel<T, false, false, EpiUpdate<T>><<<grid, kGemmThreads, 0, st>>>(A, k, W, k, rows, n, k, m_dev, nullptr, epi);
+    launch_gemm_simt<T, false, false>(rows < kChainRows, grid, st, A, k, W, k, rows, n, k, m_dev, nullptr, epi);
 }
 
 // dX = mask * (dY W), dY [rows x n_out], W [n_out x n_in] -> dX [rows x n_in]; wt is scratch for W^T
@@ -200,9 +199,7 @@ void linear_backward_input(const T *dY, int64_t rows, int n_out, const T *W, int
     }
     EpiMasked<T> epi{dX, n_in, mask, n_in};
     dim3 grid((unsigned)ceil_div(rows, kGemmBM), (unsigned)ceil_div(n_in, kGemmBN), 1);
-    note_launch();
-    gemm_simt_kernel<T, false, true, EpiMasked<T>><<<grid, kGemmThreads, 0, st>>>(dY, n_out, W, n_in, rows, n_in, n_out, m_dev,
-                                                                                 nullptr, epi);
+    launch_gemm_simt<T, false, true>(rows < kChainRows, grid, st, dY, n_out, W, n_in, rows, n_in, n_out, m_dev, nullptr, epi);
 }
 
 // dW = dY^T X (fp32, rows split kSplits ways and added in order), db = column sums of dY
@@ -213,16 +210,15 @@ void linear_backward_weight(const T *dY, int64_t rows, int n_out, const T *Xin, 
     const bool on_tc = use_tc<T>() && tc_weight_grad(reinterpret_cast<const __nv_bfloat16 *>(dY), rows, n_out,
                                                      reinterpret_cast<const __nv_bfloat16 *>(Xin), n_in, m_dev, part, kSplits,
                                                      status, st);
+    const int splits = on_tc ? kSplits : simt_splits(rows, n_out, n_in, kSplits);
     if (!on_tc) {
         EpiPartial epi{part, n_in, (int64_t)n_out * n_in};
-        dim3 grid((unsigned)ceil_div(n_out, kGemmBM), (unsigned)ceil_div(n_in, kGemmBN), kSplits);
-        note_launch();
-        gemm_simt_kernel<T, true, true, EpiPartial><<<grid, kGemmThreads, 0, st>>>(dY, n_out, Xin, n_in, n_out, n_in, rows,
-                                                                                  nullptr, m_dev, epi);
+        dim3 grid((unsigned)ceil_div(n_out, kGemmBM), (unsigned)ceil_div(n_in, kGemmBN), (unsigned)splits);
+        launch_gemm_simt<T, true, true>(rows < kChainRows, grid, st, dY, n_out, Xin, n_in, n_out, n_in, rows, nullptr, m_dev, epi);
     }
     const int64_t n = (int64_t)n_out * n_in;
     note_launch();
-    launch_pdl(rows < kChainRows, splitk_reduce_kernel, dim3((unsigned)ceil_div(n, 256)), dim3(256), 0, st, (const float *)part, n, kSplits, 0, dW,
+    launch_pdl(rows < kChainRows, splitk_reduce_kernel, dim3((unsigned)ceil_div(n, 256)), dim3(256), 0, st, (const float *)part, n, splits, 0, dW,
                on_tc ? m_dev : (const int32_t *)nullptr, 1);
     if (db) launch_colsum<T>(dY, n_out, nullptr, m_dev, 0, n_out, 0, db, st);
 }
@@ -310,8 +306,7 @@ void gate_forward_core(GMat<const T> F, int64_t rows, int32_t n_rows, int d, con
     } else {
         EpiUpdate<T> epi{pre, d, bg, 0};
         dim3 grid((unsigned)ceil_div(rows, kGemmBM), (unsigned)ceil_div(d, kGemmBN), 1);
-        note_launch();
-        gemm_simt_kernel<T, false, false, EpiUpdate<T>><<<grid, kGemmThreads, 0, st>>>(F.p, F.ld, Wg, d, rows, d, d, meta, nullptr, epi);
+        launch_gemm_simt<T, false, false>(rows < kChainRows, grid, st, F.p, F.ld, Wg, d, rows, d, d, meta, nullptr, epi);
     }
     note_launch();
     gate_apply_kernel<T><<<cells_grid(rows, d), 256, 0, st>>>(pre, F.p, F.ld, d, n_rows,
@@ -331,11 +326,11 @@ void gate_backward_core(GMat<const T> dFused, GMat<const T> F, GMat<const T> gat
         linear_backward_weight<T>(dpre, rows, d, F.p, d, meta, part, dWg, dbg, status, st);
     } else {                                                             // strided F: fp32-FMA product
         EpiPartial epi{part, d, (int64_t)d * d};
-        dim3 grid((unsigned)ceil_div(d, kGemmBM), (unsigned)ceil_div(d, kGemmBN), kSplits);
+        const int splits = simt_splits(rows, d, d, kSplits);
+        dim3 grid((unsigned)ceil_div(d, kGemmBM), (unsigned)ceil_div(d, kGemmBN), (unsigned)splits);
+        launch_gemm_simt<T, true, true>(rows < kChainRows, grid, st, dpre, d, F.p, F.ld, d, d, rows, nullptr, meta, epi);
         note_launch();
-        gemm_simt_kernel<T, true, true, EpiPartial><<<grid, kGemmThreads, 0, st>>>(dpre, d, F.p, F.ld, d, d, rows, nullptr, meta, epi);
-        note_launch();
-        splitk_reduce_kernel<<<(unsigned)ceil_div((int64_t)d * d, 256), 256, 0, st>>>(part, (int64_t)d * d, kSplits, 0, dWg, nullptr);
+        splitk_reduce_kernel<<<(unsigned)ceil_div((int64_t)d * d, 256), 256, 0, st>>>(part, (int64_t)d * d, splits, 0, dWg, nullptr);
         if (dbg) launch_colsum<T>(dpre, d, nullptr, meta, 0, d, 0, dbg, st);
     }
     if (use_tc<T>() && dF.rows >= rows && dFused.rows >= rows && gate.rows >= rows) {

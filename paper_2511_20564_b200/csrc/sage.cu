@@ -212,10 +212,8 @@ static int32_t forward_impl(const e2egrec_block *blocks, int32_t n_layers, const
         if (!done) {
             EpiUpdate<T> epi{hn, p.d_out, bl, relu};
             dim3 grid((unsigned)std::max<int64_t>(1, ceil_div(p.rows, kGemmBM)), (unsigned)ceil_div(p.d_out, kGemmBN), 1);
-            note_launch();
-            gemm_simt_kernel<T, false, false, EpiUpdate<T>><<<grid, kGemmThreads, 0, st>>>(
-                cat, 2 * p.d_in, static_cast<const T *>(W[l].data), 2 * p.d_in, p.rows, p.d_out, 2 * p.d_in,
-                &b.counts[CNT_DST], nullptr, epi);
+            launch_gemm_simt<T, false, false>(chain, grid, st, (const T *)cat, 2 * p.d_in, static_cast<const T *>(W[l].data), 2 * p.d_in,
+                                              p.rows, p.d_out, 2 * p.d_in, &b.counts[CNT_DST], nullptr, epi);
         }
         if (l == 0) tap_end(TAP_UPDATE_FWD_OUTER, st);
     }
@@ -322,14 +320,14 @@ static int32_t backward_impl(const e2egrec_block *blocks, int32_t n_layers, cons
             launch_pdl(chain, splitk_reduce_kernel, dim3((unsigned)ceil_div(n_w, 256)), dim3(256), 0, ws, part, n_w, tc_splits, accumulate,
                        dW[l], n_dst, n_rhs);
         } else {
+            const int splits = simt_splits(p.rows, p.d_out, two_d, kDwSplits);
             for (int r = 0; r < n_rhs; ++r) {             // fp32-FMA product: one right-hand side per pass, added up
                 EpiPartial epi{part, two_d, n_w};
-                dim3 grid((unsigned)ceil_div(p.d_out, kGemmBM), (unsigned)ceil_div(two_d, kGemmBN), kDwSplits);
+                dim3 grid((unsigned)ceil_div(p.d_out, kGemmBM), (unsigned)ceil_div(two_d, kGemmBN), (unsigned)splits);
+                launch_gemm_simt<T, true, true>(chain, grid, ws, dz + (int64_t)r * p.rows * p.d_out, p.d_out, cat, two_d, p.d_out, two_d,
+                                                p.rows, nullptr, n_dst, epi);
                 note_launch();
-                gemm_simt_kernel<T, true, true, EpiPartial><<<grid, kGemmThreads, 0, ws>>>(
-                    dz + (int64_t)r * p.rows * p.d_out, p.d_out, cat, two_d, p.d_out, two_d, p.rows, nullptr, n_dst, epi);
-                note_launch();
-                launch_pdl(chain, splitk_reduce_kernel, dim3((unsigned)ceil_div(n_w, 256)), dim3(256), 0, ws, part, n_w, kDwSplits,
+                launch_pdl(chain, splitk_reduce_kernel, dim3((unsigned)ceil_div(n_w, 256)), dim3(256), 0, ws, part, n_w, splits,
                            (accumulate || r > 0) ? 1 : 0, dW[l], (const int32_t *)nullptr, 1);
             }
         }
@@ -356,10 +354,8 @@ static int32_t backward_impl(const e2egrec_block *blocks, int32_t n_layers, cons
             for (int r = 0; r < n_rhs; ++r) {
                 EpiDCat<T> epi{dcat + (int64_t)r * p.rows * two_d, two_d, p.d_in, b.inv_cnt};
                 dim3 grid((unsigned)std::max<int64_t>(1, ceil_div(p.rows, kGemmBM)), (unsigned)ceil_div(two_d, kGemmBN), 1);
-                note_launch();
-                gemm_simt_kernel<T, false, true, EpiDCat<T>><<<grid, kGemmThreads, 0, st>>>(
-                    dz + (int64_t)r * p.rows * p.d_out, p.d_out, static_cast<const T *>(W[l].data), two_d, p.rows, two_d, p.d_out,
-                    n_dst, nullptr, epi);
+                launch_gemm_simt<T, false, true>(chain, grid, st, dz + (int64_t)r * p.rows * p.d_out, p.d_out,
+                                                 static_cast<const T *>(W[l].data), two_d, p.rows, two_d, p.d_out, n_dst, nullptr, epi);
             }
         }
         if (l == 0) tap_end(TAP_DCAT_OUTER, st);

@@ -35,7 +35,7 @@ __device__ inline uint4 philox4x32_10(uint4 c, uint2 k)
 // ---------------------------------------------------------------------------------------
 // Scratch layout (host and device agree through this struct).
 // ---------------------------------------------------------------------------------------
-constexpr int kDstTile = 64;           // most destinations per block of the sampling kernel
+constexpr int kDstTile = 128;          // most destinations per block of the sampling kernel
 constexpr int kDstTileMin = 4;
 constexpr int kDstThreads = 256;       // its threads: one per destination for the counts, then all of them draw
 constexpr int kWordTile = 512;         // bitmap words per block of the frontier kernel (2048: 8 blocks on 500 k nodes)
