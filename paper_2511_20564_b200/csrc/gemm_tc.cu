@@ -711,7 +711,7 @@ bool launch_tn(const __nv_bfloat16 *A, int64_t rows, int k, int64_t lda, const _
     // ... or, where such tiles would leave more than half of the SMs without one, the widest of 64 columns and more that does
     // not, else the narrowest of those: one tile's chain of loads, products and stores is what a small product costs, and
     // half the columns are half of its stores (B200, 4096 x 320 x 512: 13.3 us with 64 tiles of 256 columns, 10.2 with 128
-    // of 128; 1000 x 320 x 320 gated: 27 us with 16 tiles of 160 before)
+    // of 128; 1000 x 320 x 320 gated: 27 us with 16 tiles of 160, 14 with 40 of 64)
     for (int c = 256; c >= unit; c -= unit) {
         if (n % c || (nt && c < 64)) continue;
         nt = c;

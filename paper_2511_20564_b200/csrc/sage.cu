@@ -98,12 +98,10 @@ static bool dispatch_sage_aggregate(const T *Hsrc, int64_t ld, const int32_t *nb
 
 // transposed-block entries per lane group: 16, or 128 where the block can hold a million entries or more (the longer run's
 // lower overhead per entry wins there; measured on the 2 * 10^9-entry workload: 0.69 -> 0.63 ms)
-// (longer runs were measured with the streamed rows as well: 256 entries 0.422 ms, 512 0.461, 1024 0.777 against 0.421)
-// A block that can hold two million entries gets runs of 128 entries.  Where the rows can be streamed through shared
-// memory (512-byte bf16 rows) the long runs and the streaming start at a million (2 * 10^9-entry workload: the outer
-// block alone 2.207 ms per step, the middle block as well 2.168; with 2^17 the top block joins and its 0.065 ms become
-// 0.127).  Capacities, not sizes, are what the host knows: a small batch in large buffers pays for the long runs (a
-// 71 k-entry block in a 1.2 M-entry buffer: 0.327 -> 0.362 ms per joint step), hence no lower than this.
+// A block that can hold two million entries gets runs of 128 entries; with 512-byte bf16 rows (whose forward aggregation is
+// streamed from the same size on) a million.  Capacities, not sizes, are what the host knows: a small batch in large
+// buffers pays for the long runs (a 71 k-entry block in a 1.2 M-entry buffer: 0.327 -> 0.362 ms per joint step), hence no
+// lower than this.
 static inline bool streamable_rows(int d, size_t es) { return es == 2 && d == 256; }
 static inline int64_t big_block_edges(int d, size_t es) { return streamable_rows(d, es) ? (1ll << 20) : (1ll << 21); }
 static inline int block_run_len(int64_t cap_edges, int d, size_t es) { return cap_edges >= big_block_edges(d, es) ? 128 : 16; }
@@ -368,8 +366,6 @@ static int32_t backward_impl(const e2egrec_block *blocks, int32_t n_layers, cons
         o.mean = 0;
         o.n_rhs = n_rhs;
         o.rhs_in = o.rhs_self = (int64_t)p.rows * two_d;
-        o.in_rows = (int64_t)p.rows * n_rhs;
-        o.status = &b.counts[CNT_STATUS];
         if (l > 0) {
             // the buffer that receives dZ of the layer below may still be read by the helper stream (layer l+1)
             if (side && dz_free[(l - 1) & 1]) {
