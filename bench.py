@@ -1170,7 +1170,7 @@ def run_fullgraph(args):
     big, big_d = ("fwd", fwd_d) if t_f >= t_b else ("bwd", bwd_d)
     roof = dict(bound="hbm", achieved=big_d["no_reuse"]["gbs"], peak=peaks["hbm_gbs"], unit="GB/s",
                 traffic=big_d["dram_counter"]["bytes"] if big_d["dram_counter"] else None,
-                kernel=f"seg_run_kernel+seg_final_kernel ({big})", ms_per_launch=big_d["ms"],
+                kernel=f"seg_walk_kernel+seg_final_kernel ({big})", ms_per_launch=big_d["ms"],
                 algorithmic_units_per_launch=big_d["no_reuse"]["bytes"], peak_source=peaks["source"],
                 frac_of_nominal_8tbs=big_d["no_reuse"]["frac_of_nominal_8tbs"],
                 compulsory_frac=big_d["compulsory"]["frac_of_measured_copy"],
