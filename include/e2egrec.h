@@ -194,9 +194,12 @@ int32_t e2egrec_sampler_set_step(void *scratch, uint32_t step_offset, void *stre
  * E2EGREC_SAMPLE_DEFER_TRANSPOSE it does not: indptr / col / nbr_global / src_nodes / inv_cnt / counts are valid in
  * stream order as always, but the csc_* arrays are only complete after the next e2egrec_sage_backward,
  * e2egrec_lightgcn_sampled_backward, e2egrec_sample_khop or e2egrec_sample_join that the host issues on any stream
- * of the same device: that call makes its stream wait for every transposition deferred on the device so far
- * (e2egrec_sage_forward does not need the csc_* arrays, so the forward pass overlaps the transposition).  Inside a
- * stream capture the deferring call and the joining call must belong to the same capture.  Calls that share a
+ * of the same device: that call makes its stream wait for every transposition deferred on the device so far, also for
+ * those that another stream has waited for (e2egrec_sage_forward does not need the csc_* arrays, so the forward pass
+ * overlaps the transposition).  Until then the deferred work goes on using the scratch and all arrays of the blocks:
+ * neither may be freed, written or handed to a stream that has not joined.  Inside a
+ * stream capture the deferring call and the joining call must belong to the same capture: a capture holds no wait for
+ * work deferred before it.  Calls that share a
  * caller stream must not be issued from two host threads at once. */
 int32_t e2egrec_sample_khop(const e2egrec_csr *graph, const int32_t *seeds, int32_t n_seeds,
                             int32_t n_hops, const int32_t *fanouts, uint64_t seed, uint32_t step,

@@ -23,7 +23,7 @@ def sources():
 
 
 def _headers():
-    return glob.glob(os.path.join(HERE, "csrc", "*.cuh")) + glob.glob(os.path.join(HERE, "..", "include", "*.h"))
+    return [f for d, e in (("csrc", "*.cuh"), ("csrc", "*.h"), ("../include", "*.h")) for f in glob.glob(os.path.join(HERE, d, e))]
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

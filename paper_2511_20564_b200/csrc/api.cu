@@ -9,6 +9,7 @@
 #include <string.h>
 
 #include "common.cuh"
+#include "deferral.h"
 
 namespace e2egrec {
 
@@ -41,9 +42,9 @@ static bool helper_streams_enabled()
 
 // Helper streams: one per (device, caller's stream), created on first use and kept until the process ends, so calls
 // made on different streams (a sampling leg beside a compute leg, say) never meet on a common helper stream.
-// Deferred work (a block transposition left running by e2egrec_sample_khop) is tracked per device: whichever stream
-// of that device asks next (e2egrec_sage_backward, e2egrec_sample_join, the next e2egrec_sample_khop) waits for all of
-// it.  The table and the pending lists are guarded by one mutex; the event ring of a helper stream is touched only by
+// Deferred work (a block transposition left running by e2egrec_sample_khop) is tracked per device: every stream of that
+// device that asks (e2egrec_sage_backward, e2egrec_sample_join, the next e2egrec_sample_khop) waits for all of it, once.
+// The table and the ledgers are guarded by one mutex; the event ring of a helper stream is touched only by
 // calls issued on its caller's stream, which the caller must not issue from two host threads at once.
 static std::mutex g_side_mutex;
 struct SideKey {
@@ -55,7 +56,8 @@ struct SideKeyHash {
     size_t operator()(const SideKey &k) const { return std::hash<const void *>()(k.stream) * 31u + (size_t)k.dev; }
 };
 static std::unordered_map<SideKey, SideStream *, SideKeyHash> g_side;
-static std::vector<SideStream *> g_pending[64];          // per device: helper streams whose `pending` event is unjoined
+static std::vector<SideStream *> g_helpers[64];          // per device, by SideStream::index
+static DeferralLedger g_deferred[64];
 
 SideStream *SideStream::get(cudaStream_t caller)
 {
@@ -75,7 +77,8 @@ SideStream *SideStream::get(cudaStream_t caller)
     for (int i = 0; i < 32; ++i)
         if (cudaEventCreateWithFlags(&s->ev[i], cudaEventDisableTiming) != cudaSuccess) { delete s; cudaGetLastError(); return nullptr; }
     if (cudaEventCreateWithFlags(&s->pending, cudaEventDisableTiming) != cudaSuccess) { delete s; cudaGetLastError(); return nullptr; }
-    s->has_pending = false;
+    s->index = g_helpers[dev].size();
+    g_helpers[dev].push_back(s);
     g_side.emplace(SideKey{dev, caller}, s);
     return s;
 }
@@ -96,22 +99,30 @@ void SideStream::join(cudaStream_t into)
     cudaStreamWaitEvent(into, e, 0);
 }
 
+// the capture that a stream is part of, 0 for none
+static uint64_t capture_of(cudaStream_t st)
+{
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    if (cudaStreamGetCaptureInfo(st, &status, &id) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return status == cudaStreamCaptureStatusActive ? (uint64_t)id : 0;
+}
+
 void SideStream::defer()
 {
     std::lock_guard<std::mutex> lock(g_side_mutex);
     cudaEventRecord(pending, stream);
-    if (!has_pending) g_pending[device].push_back(this);
-    has_pending = true;
+    g_deferred[device].defer(index, capture_of(stream));
 }
 
-void SideStream::join_pending(cudaStream_t into)
+void SideStream::join_pending()
 {
     std::lock_guard<std::mutex> lock(g_side_mutex);
-    for (SideStream *s : g_pending[device]) {
-        cudaStreamWaitEvent(into, s->pending, 0);
-        s->has_pending = false;
-    }
-    g_pending[device].clear();
+    g_deferred[device].join(index, [&] { return capture_of(owner); },
+                            [&](size_t h) { cudaStreamWaitEvent(owner, g_helpers[device][h]->pending, 0); });
 }
 
 static std::atomic<uint64_t> g_launches{0};
@@ -136,8 +147,7 @@ void tap_end(int which, cudaStream_t st)
 
 extern "C" int32_t e2egrec_sample_join(void *stream)
 {
-    e2egrec::SideStream *side = e2egrec::SideStream::get(static_cast<cudaStream_t>(stream));
-    if (side) side->join_pending(static_cast<cudaStream_t>(stream));
+    if (e2egrec::SideStream *side = e2egrec::SideStream::get(static_cast<cudaStream_t>(stream))) side->join_pending();
     return e2egrec::check_launch("sample_join");
 }
 

@@ -234,7 +234,7 @@ extern "C" int32_t e2egrec_lightgcn_sampled_backward(const e2egrec_block *blocks
         return E2EGREC_ERR_ARG;
     if ((dX_rows->ld * fp.es) % 16 || reinterpret_cast<uintptr_t>(dX_rows->data) % 16) return E2EGREC_ERR_ALIGN;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (SideStream *side = SideStream::get(st)) side->join_pending(st);     // a deferred block transposition
+    if (SideStream *side = SideStream::get(st)) side->join_pending();     // a deferred block transposition
     if (dY->dtype == E2EGREC_BF16)
         return backward_impl<__nv_bfloat16>(blocks, fp, bp, dY->dtype, static_cast<const char *>(ctx), dY, dX_rows,
                                             static_cast<char *>(scratch), st);

@@ -472,7 +472,7 @@ static int32_t sage_backward_entry(const e2egrec_block *blocks, int32_t n_layers
         if (dX_rows[r].ld != dX_rows[0].ld) return E2EGREC_ERR_ARG;       // the results share one leading dimension
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (SideStream *side = SideStream::get(st)) side->join_pending(st);     // a deferred block transposition
+    if (SideStream *side = SideStream::get(st)) side->join_pending();     // a deferred block transposition
     if (X->dtype == E2EGREC_BF16)
         return backward_impl<__nv_bfloat16>(blocks, n_layers, X, W, act, plan, static_cast<const char *>(ctx), dH_out, n_rhs, dW,
                                             dbias, dX_rows, static_cast<char *>(scratch), bs, flags, st);

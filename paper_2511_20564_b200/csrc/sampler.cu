@@ -674,7 +674,7 @@ int32_t e2egrec::sample_khop_impl(const e2egrec_csr *graph, const int32_t *seeds
     // The transposition of a hop (sort + offsets) is only needed by the backward pass, so it runs on the
     // helper stream beside the sampling of the next hop; everything is joined before this call returns.
     SideStream *side = SideStream::get(st);
-    if (side) side->join_pending(st);               // a transposition deferred by an earlier call still uses the lanes
+    if (side) side->join_pending();               // a transposition deferred by an earlier call still uses the lanes
     tap_begin(TAP_SAMPLE, st);
     const int32_t *dst_nodes = seeds;
     const int32_t *n_dst_ptr = &blocks[0].counts[CNT_DST];
@@ -774,7 +774,7 @@ extern "C" int32_t e2egrec_blocks_transpose(int64_t n_nodes, int32_t n_hops, con
     if (scratch_bytes < s.bytes) return E2EGREC_ERR_WORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     SideStream *side = SideStream::get(st);
-    if (side) side->join_pending(st);
+    if (side) side->join_pending();
     const bool forked = side && n_hops > 1;
     if (forked) side->fork(st);
     for (int h = n_hops - 1; h >= 0; --h) {          // the largest block first, on the caller's stream

@@ -1,0 +1,66 @@
+"""Host-side bookkeeping of the library, compiled from its headers with the host compiler (no GPU needed)."""
+import os
+import subprocess
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2511_20564_b200", "csrc")
+
+
+def run_cpp(tmp_path, body, *headers):
+    """Compiles and runs `body` as main(); it returns 0 when all is well, else the number of the check that failed."""
+    src = tmp_path / "t.cpp"
+    src.write_text("".join(f'#include "{h}"\n' for h in headers) + "#include <string>\nusing namespace e2egrec;\n"
+                   "int main() {\n" + body + "\nreturn 0;\n}\n")
+    exe = tmp_path / "t"
+    subprocess.check_call(["g++", "-std=c++17", "-Wall", "-Werror", "-I", CSRC, str(src), "-o", str(exe)])
+    assert subprocess.call([str(exe)], timeout=60) == 0
+
+
+LEDGER = """
+DeferralLedger led;
+std::string log;
+uint64_t capture = 0;
+auto join = [&](size_t who) {
+    log.clear();
+    led.join(who, [&] { return capture; }, [&](size_t h) { log += char('A' + h); });
+    return log;
+};
+enum : size_t { A, B, C };
+"""
+
+
+def test_every_stream_waits_once_for_every_deferral(tmp_path):
+    run_cpp(tmp_path, LEDGER + """
+if (join(A) != "") return 1;
+led.defer(A, 0);
+if (join(B) != "A") return 2;          // an unrelated stream asks first ...
+if (join(A) != "A") return 3;          // ... and the owner, about to use the scratch again, still waits
+if (join(A) != "" || join(B) != "") return 4;
+if (join(C) != "A") return 5;
+led.defer(A, 0);                       // two callers, each with its own sample
+led.defer(B, 0);
+if (join(A) != "AB" || join(B) != "AB" || join(A) != "") return 6;
+led.defer(A, 0);
+led.defer(A, 0);
+if (join(A) != "A" || join(A) != "") return 7;
+""", "deferral.h")
+
+
+def test_waits_and_stream_captures(tmp_path):
+    run_cpp(tmp_path, LEDGER + """
+capture = 7;                           // deferred and joined inside one capture, by two of its streams
+led.defer(A, 7);
+if (join(B) != "A" || join(A) != "A") return 1;
+led.defer(A, 7);
+if (join(B) != "A") return 2;
+capture = 0;                           // the capture has ended: its events are no longer to be waited for
+if (join(A) != "") return 3;
+led.defer(A, 0);
+if (join(B) != "A") return 4;
+capture = 8;                           // no wait for outside work inside a capture, unless nobody has waited for it
+if (join(A) != "") return 5;
+capture = 0;                           // the owner's next call outside makes up for it
+if (join(A) != "A" || join(A) != "") return 6;
+led.defer(A, 0);
+capture = 9;
+if (join(A) != "A") return 7;          // refused by CUDA, as a join of another capture's work always was
+""", "deferral.h")
