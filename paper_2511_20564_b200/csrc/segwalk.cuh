@@ -192,8 +192,8 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
         // Segments come in windows of 32, lane i holding where segment s_base + i begins and ends; the ends of the window
         // after it are on their way.
         auto rel = [&](int64_t p) -> int { return (int)max(min(p - k0, (int64_t)kFar), (int64_t)-kFar); };
-        auto load_ends = [&](int32_t b) -> int { return (int64_t)b + lane < n_seg ? rel((int64_t)__ldg(&ptr[(int64_t)b + lane + 1])) : kFar; };
-        int32_t s_base = (int32_t)warp_seg_containing(ptr, n_seg, k0);
+        auto load_ends = [&](uint32_t b) -> int { return (int64_t)b + lane < n_seg ? rel((int64_t)__ldg(&ptr[(int64_t)b + lane + 1])) : kFar; };
+        uint32_t s_base = (uint32_t)warp_seg_containing(ptr, n_seg, k0);       // unsigned: windows reach beyond the last segment, 2^31 and on
         int ends = load_ends(s_base), ends_ahead = load_ends(s_base + 32);
         int carry = rel((int64_t)__ldg(&ptr[s_base]));           // where the window's first segment begins
         int quiet = 0;                                           // windows without an entry in a row
@@ -246,7 +246,7 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
                             if (j0 + u < longest) add_row(v[u], wt[u], true);
                     }
                     if (live) {
-                        const int32_t seg = s_base + i;
+                        const int32_t seg = (int32_t)(s_base + i);
                         const float inv = scale_of(seg, sn);
 #pragma unroll
                         for (int q = 0; q < CPL; ++q) {
@@ -263,7 +263,7 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
             while (big_m) {
                 const int i = __ffs(big_m) - 1;
                 big_m &= big_m - 1;
-                const int32_t seg = s_base + i;
+                const int32_t seg = (int32_t)(s_base + i);
                 const int sbeg = __shfl_sync(0xffffffffu, beg, i), send = __shfl_sync(0xffffffffu, ends, i);
                 const int first = max(sbeg, 0), sn = min(send, len) - first;
                 const int32_t *__restrict__ ids = idx0 + first;
@@ -329,7 +329,7 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
                 s_base += 32;
                 ends = ends_ahead;
             } else {                                             // a long stretch of empty segments
-                s_base = (int32_t)warp_seg_containing(ptr, n_seg, k0 + carry);
+                s_base = (uint32_t)warp_seg_containing(ptr, n_seg, k0 + carry);
                 ends = load_ends(s_base);
                 quiet = 0;
             }

@@ -55,3 +55,27 @@ def test_walk(lengths, dtype, d):
     dX, _ = E.aggregate_backward(pd, ix, torch.from_numpy(w).cuda(), Xd)
     wr = rows * w.astype(np.float64)[idx][:, None]
     check(dX, sums(wr), sums(np.abs(wr)))
+
+
+def test_as_many_segments_as_the_entry_point_takes():
+    """2^31 - 1 segments, with entries in the first and the last ones: windows of 32 segments that begin among the last and
+    reach beyond 2^31.  52 GB of offsets and rows."""
+    if torch.cuda.mem_get_info()[0] < 70 << 30:
+        pytest.skip("needs 70 GB of device memory")
+    n, d = (1 << 31) - 1, 4
+    tail = torch.tensor([3, 0, 40, 1, 300, 0, 10_000], dtype=torch.int64)
+    ptr = torch.zeros(n + 1, dtype=torch.int64, device="cuda")
+    ptr[1:] = 2                                              # segment 0: two entries
+    ptr[n + 1 - tail.numel():] += torch.cumsum(tail, 0).cuda()
+    m = 2 + int(tail.sum())
+    rng = np.random.default_rng(9)
+    X = torch.from_numpy(rng.integers(-8, 9, (50, d)).astype(np.float32))       # sums of whole numbers: exact in any order
+    idx = torch.from_numpy(rng.integers(0, 50, m).astype(np.int32))
+    out = torch.empty(n, d, device="cuda")
+    E.aggregate_forward(ptr, idx.cuda(), X.cuda(), out=out, sum_only=True)
+    rows = X[idx.long()]
+    cuts = [0, 2] + (2 + torch.cumsum(tail, 0)).tolist()
+    want = torch.stack([rows[a:b].sum(0) for a, b in zip(cuts, cuts[1:])])
+    assert torch.equal(out[0].cpu(), want[0]) and torch.equal(out[n - tail.numel():].cpu(), want[1:])
+    for a in range(1, n - tail.numel(), 1 << 28):            # everything between is empty
+        assert not bool(out[a:min(a + (1 << 28), n - tail.numel())].any())
