@@ -130,16 +130,22 @@ __global__ void rows_of_kernel(const int64_t *__restrict__ eid, const int32_t *_
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < m; k += 4 * step) {
         int32_t r[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) r[q] = k + q * step < m ? __ldg(row_of + __ldcs(eid + k + q * step)) : 0;
+        for (int q = 0; q < 4; ++q) {
+            const int64_t e = k + q * step < m ? __ldcs(eid + k + q * step) : 0;
+            r[q] = __ldg(row_of + ((uint64_t)e < (uint64_t)m ? e : 0));      // beyond: after a wait of the sort that ran out
+        }
 #pragma unroll
         for (int q = 0; q < 4; ++q)
             if (k + q * step < m) __stcs(csc_row + k + q * step, r[q]);
     }
 }
 
-// ptr[s] = first position of the sorted key array whose key is >= s, for s = 0 .. n
-__global__ void offsets_kernel(const int32_t *__restrict__ sorted, int64_t m, int64_t n, int64_t *__restrict__ ptr)
+// ptr[s] = first position of the sorted key array whose key is >= s, for s = 0 .. n; all zero after a wait of the sort that
+// ran out
+__global__ void offsets_kernel(const int32_t *__restrict__ sorted, int64_t m, int64_t n, const int32_t *__restrict__ counts,
+                               int64_t *__restrict__ ptr)
 {
+    if ((uint32_t)counts[CNT_STATUS] & E2EGREC_DEV_TIMEOUT) m = 0;
     for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s <= n; s += (int64_t)gridDim.x * blockDim.x) {
         int64_t lo = 0, hi = m;
         while (lo < hi) {
@@ -204,7 +210,7 @@ extern "C" int32_t e2egrec_graph_from_coo(int64_t n_nodes, int64_t n_edges, cons
         }                                                        // s.a = rows sorted
     }
     note_launch();
-    offsets_kernel<<<wide_grid(n_nodes + 1), 256, 0, st>>>(s.a, m, n_nodes, indptr);
+    offsets_kernel<<<wide_grid(n_nodes + 1), 256, 0, st>>>(s.a, m, n_nodes, s.counts, indptr);
     if (status) cudaMemcpyAsync(status, &s.counts[CNT_STATUS], sizeof(int32_t), cudaMemcpyDeviceToDevice, st);
     return check_launch("graph_from_coo");
 }
@@ -235,9 +241,9 @@ extern "C" int32_t e2egrec_csr_transpose(const e2egrec_csr *csr, int64_t n_cols,
         for (int q = 0; q < sp.passes; ++q) {
             const int32_t clamp = q == 0 ? (int32_t)std::max<int64_t>(n_cols, 1) : 0;
             if (q == sp.passes - 1)
-                sort_pass<int64_t>(sp, k, v, nullptr, m, clamp, 0, q, s.sort[0], false, ka, csc_eid, SortMap{}, &s.counts[CNT_STATUS], st);
+                sort_pass<int64_t>(sp, k, v, nullptr, m, clamp, (int32_t)m, q, s.sort[0], false, ka, csc_eid, SortMap{}, &s.counts[CNT_STATUS], st);
             else
-                sort_pass<int32_t>(sp, k, v, nullptr, m, clamp, 0, q, s.sort[0], false, ka, va, SortMap{}, &s.counts[CNT_STATUS], st);
+                sort_pass<int32_t>(sp, k, v, nullptr, m, clamp, (int32_t)m, q, s.sort[0], false, ka, va, SortMap{}, &s.counts[CNT_STATUS], st);
             k = ka;
             v = va;
             std::swap(ka, kb);
@@ -248,7 +254,7 @@ extern "C" int32_t e2egrec_csr_transpose(const e2egrec_csr *csr, int64_t n_cols,
         rows_of_kernel<<<(unsigned)std::min<int64_t>(ceil_div(m, 1024), 148 * 16), 256, 0, st>>>(csc_eid, s.a, m, csc_row);
     }
     note_launch();
-    offsets_kernel<<<wide_grid(n_cols + 1), 256, 0, st>>>(sorted, m, n_cols, csc_ptr);
+    offsets_kernel<<<wide_grid(n_cols + 1), 256, 0, st>>>(sorted, m, n_cols, s.counts, csc_ptr);
     if (status) cudaMemcpyAsync(status, &s.counts[CNT_STATUS], sizeof(int32_t), cudaMemcpyDeviceToDevice, st);
     return check_launch("csr_transpose");
 }

@@ -103,6 +103,14 @@ __device__ inline int chain_ticket(unsigned *ticket, int *bcast)
 // ---------------------------------------------------------------------------------------
 constexpr unsigned kPosFlag = 0x80000000u;
 
+// Rounds without progress after which a look-back of the sort ends.  Such a sort leaves positions of its output unwritten and
+// flags E2EGREC_DEV_TIMEOUT.  Its later passes clamp the values they read, so that none is used as an index out of range,
+// and who takes the result makes the offsets over it all zero, so that nothing behind them is reached.  (A tile that counts the
+// elements before it itself instead keeps the result whole, but any code there cost the kernel 3 to 7 %.)
+#ifndef E2EGREC_SORT_SPIN_LIMIT
+#define E2EGREC_SORT_SPIN_LIMIT kChainSpinLimit
+#endif
+
 // A sort's last launch may also look up where its values belong: row_out[pos] = row_of[value].
 struct SortMap { const int32_t *row_of; int32_t *row_out; };
 
@@ -154,7 +162,6 @@ sort_pass_kernel(const int32_t *__restrict__ keys_in, const int32_t *__restrict_
     for (int k = 0; k < kSortItems; ++k) {
         const int i = w0 + k * 32 + lane;
         val[k] = !vin ? (uint32_t)(tile * TILE + i) : i < tile_n ? (uint32_t)__ldcg(vin + i) : 0u;
-        if (clamp_vals && val[k] >= (uint32_t)clamp_vals) val[k] = 0;
     }
 #pragma unroll
     for (int k = 0; k < kSortItems; ++k) {
@@ -222,7 +229,7 @@ sort_pass_kernel(const int32_t *__restrict__ keys_in, const int32_t *__restrict_
             const uint32_t digit = (key[k] >> shift) & (R - 1);
             const int pos = start[digit] + wc[warp * R + digit] + rank[k];
             skey[pos] = key[k];
-            sval[pos] = val[k];
+            sval[pos] = clamp_vals && val[k] >= (uint32_t)clamp_vals ? 0u : val[k];     // not before: the value's load is still on its way
         }
     }
     // ---- the chains of the thread's digits, the nearest tiles first
@@ -271,7 +278,7 @@ sort_pass_kernel(const int32_t *__restrict__ keys_in, const int32_t *__restrict_
                 }
                 p -= went;
                 if (went) spin = 0;
-                else if (++spin > kChainSpinLimit) {
+                else if (++spin > E2EGREC_SORT_SPIN_LIMIT) {
                     if (status) atomicOr(reinterpret_cast<unsigned *>(status), E2EGREC_DEV_TIMEOUT);
                     break;
                 }

@@ -415,19 +415,21 @@ __global__ void frontier_release_kernel(const int32_t *__restrict__ src_nodes, c
 }
 
 // csc_ptr[s] = first position whose column is >= s, from the steps of the sorted column array (a search per column cost 20
-// scattered reads each).  Leaves the sort's tickets and scan state
-// zero again, so that a block can be transposed any number of times.
+// scattered reads each).  Leaves the sort's tickets and scan state zero again, so that a block can be transposed any number
+// of times.  After a wait of the sort that ran out all columns are left empty.
 __global__ void csc_finalize_kernel(const int32_t *__restrict__ csc_col, const int32_t *__restrict__ counts,
                                     int32_t *__restrict__ csc_ptr, SortState ss, int bits, int passes,
                                     const int32_t *__restrict__ release_nodes, int32_t *__restrict__ local_id)
 {
     pdl_wait();
+    const int32_t n_all = __ldcg(counts + CNT_EDGES), n_src = __ldcg(counts + CNT_SRC);
+    const uint32_t status = (uint32_t)__ldcg(counts + CNT_STATUS);
     if (release_nodes)                               // the last block of a sample also gives the local ids back
-        for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < __ldcg(counts + CNT_SRC); k += (int64_t)gridDim.x * blockDim.x)
+        for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n_src; k += (int64_t)gridDim.x * blockDim.x)
             local_id[__ldcg(release_nodes + k)] = -1;
-    zero_sort_state(ss, __ldcg(counts + CNT_EDGES), bits, passes);
+    zero_sort_state(ss, n_all, bits, passes);
     if (blockIdx.x == 0 && threadIdx.x < kMaxPasses) ss.tickets()[threadIdx.x] = 0;
-    const int32_t n = __ldcg(counts + CNT_EDGES), n_src = __ldcg(counts + CNT_SRC);
+    const int32_t n = (status & E2EGREC_DEV_TIMEOUT) ? 0 : n_all;
     const int lane = threadIdx.x & 31;
     for (int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane; t0 <= n; t0 += (int64_t)gridDim.x * blockDim.x) {
         // position t is the first one whose column is >= s for the columns s in (col[t - 1], col[t]]
@@ -504,7 +506,7 @@ static void transpose_block(const int32_t *col, int32_t *counts, int32_t cap_edg
     for (int p = 0; p < sp.passes; ++p) {
         const bool last = p == sp.passes - 1, own = (sp.passes - 1 - p) % 2 == 0;       // the last pass ends in the block's arrays
         int32_t *ko = own ? csc_col : l.key, *vo = own ? csc_eid : l.val;
-        sort_pass<int32_t>(sp, k, v, &counts[CNT_EDGES], cap_edges, 0, 0, p, l.sort, chain, ko, vo, last ? SortMap{row_of, csc_row} : SortMap{},
+        sort_pass<int32_t>(sp, k, v, &counts[CNT_EDGES], cap_edges, 0, cap_edges, p, l.sort, chain, ko, vo, last ? SortMap{row_of, csc_row} : SortMap{},
                            &counts[CNT_STATUS], st);
         k = ko;
         v = vo;

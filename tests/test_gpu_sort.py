@@ -64,3 +64,64 @@ def test_blocks_can_be_transposed_again():
                     for k, e in (("csc_ptr", row[1] + 1), ("csc_row", row[2]), ("csc_eid", row[2]), ("csc_col", row[2]))])
     for other in got[1:]:
         assert all(np.array_equal(a, b) for a, b in zip(got[0], other))
+
+
+@pytest.fixture(scope="module")
+def impatient(tmp_path_factory):
+    """The sorting entry points compiled so that a look-back of the sort ends at its first round without progress."""
+    import ctypes
+    import os
+    import subprocess
+    from paper_2511_20564_b200 import build
+    csrc = os.path.join(build.HERE, "csrc")
+    so = str(tmp_path_factory.mktemp("sort") / "impatient.so")
+    subprocess.check_call([os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc"), "-shared"] + build.NVCC_FLAGS +
+                          ["-DE2EGREC_SORT_SPIN_LIMIT=0", "-o", so] + [os.path.join(csrc, f) for f in ("ingest.cu", "sampler.cu", "api.cu")])
+    L, real = ctypes.CDLL(so), E.binding.lib()
+    for fn in ("graph_from_coo", "csr_transpose", "sample_khop", "sample_khop_workspace", "sampler_scratch_init"):
+        getattr(L, "e2egrec_" + fn).argtypes, getattr(L, "e2egrec_" + fn).restype = getattr(real, "e2egrec_" + fn).argtypes, getattr(real, "e2egrec_" + fn).restype
+    return L
+
+
+@pytest.mark.parametrize("n,m", [(200, 60_000), (9_000_000, 300_000), (300_000, 2 * 148 * 8192)])
+def test_ingest_whose_waits_run_out(impatient, n, m, monkeypatch):
+    """The status says so and no entry is reachable through the offsets; rows are those of entries that exist."""
+    rng = np.random.default_rng(m)
+    row, col = (torch.from_numpy((n * rng.random(m) ** 4).astype(np.int32)).cuda() for _ in range(2))
+    good_ptr, good_idx, _ = E.graph_from_coo(n, row, col)
+    want_ptr, want_row, want_eid, _ = E.csr_transpose(good_ptr, good_idx, n)
+    monkeypatch.setattr(E.binding, "lib", lambda: impatient)
+    poison = torch.full((8 * m,), 0x7F7F7F7F, dtype=torch.int32, device="cuda")      # what the buffers below are cut from
+    del poison
+    ptr, idx, bad = E.graph_from_coo(n, row, col)
+    assert int(bad) in (0, 4) and (m < 1_000_000 or int(bad) == 4)
+    assert not bool(ptr.any()) if int(bad) else torch.equal(ptr, good_ptr) and torch.equal(idx, good_idx)
+    ptr, rows, eid, bad = E.csr_transpose(good_ptr, good_idx, n)
+    assert int(bad) in (0, 4) and (m < 1_000_000 or int(bad) == 4)
+    assert not bool(ptr.any()) if int(bad) else torch.equal(ptr, want_ptr) and torch.equal(rows, want_row) and torch.equal(eid, want_eid)
+    assert 0 <= int(rows.min()) and int(rows.max()) < n
+
+
+def test_sample_whose_transposition_waits_run_out(impatient, monkeypatch):
+    rng = np.random.default_rng(5)
+    n, m = 400_000, 4_000_000
+    ptr, idx, _ = E.graph_from_coo(n, *(torch.from_numpy(rng.integers(0, n, m).astype(np.int32)).cuda() for _ in range(2)))
+    seeds = torch.arange(0, 8000, dtype=torch.int32, device="cuda")
+    want = E.Blocks(n, 8000, [9, 8], "cuda")
+    E.sample_khop(ptr, idx, seeds, want, 3, 1)
+    monkeypatch.setattr(E.binding, "lib", lambda: impatient)
+    b = E.Blocks(n, 8000, [9, 8], "cuda")
+    for t in b.t:
+        for k in ("csc_row", "csc_eid", "csc_col"):
+            t[k].fill_(0x7F7F7F7F)
+    E.sample_khop(ptr, idx, seeds, b, 3, 1)
+    torch.cuda.synchronize()
+    assert torch.equal(b.counts[:, :3], want.counts[:, :3]) and int(b.counts[1, 3]) == 4
+    for h, (got, ref) in enumerate(zip(b.t, want.t)):
+        n_src, n_edges = int(b.counts[h, 1]), int(b.counts[h, 2])
+        assert torch.equal(got["col"][:n_edges], ref["col"][:n_edges])
+        if int(b.counts[h, 3]):
+            assert not bool(got["csc_ptr"][: n_src + 1].any())
+        else:
+            for k in ("csc_row", "csc_eid", "csc_col"):
+                assert torch.equal(got[k][:n_edges], ref[k][:n_edges])
