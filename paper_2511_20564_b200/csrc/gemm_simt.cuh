@@ -102,11 +102,17 @@ gemm_simt_kernel(const T *A, int64_t lda, const T *B, int64_t ldb, int64_t M_hos
     const int64_t kb = (int64_t)blockIdx.z * k_per;
     const int64_t ke = min(K, kb + k_per);
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    float acc[4][4];
+    // kFold (products that contract over the rows of a batch, thousands of terms): every K step is summed by itself and added
+    // to `total`, so that a chain of additions is 32 + K / 32 long and not K
+    constexpr bool kFold = A_KM && B_KN;
+    float acc[4][4], total[kFold ? 4 : 1][4];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+        for (int j = 0; j < 4; ++j) {
+            acc[i][j] = 0.f;
+            if (kFold) total[i][j] = 0.f;
+        }
 
     const GemmTile<T, A_KM> ta(A, lda, M, m0);
     const GemmTile<T, B_KN> tb(B, ldb, N, n0);
@@ -135,6 +141,15 @@ gemm_simt_kernel(const T *A, int64_t lda, const T *B, int64_t ldb, int64_t M_hos
 #pragma unroll
                 for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
         }
+        if (kFold) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    total[i][j] += acc[i][j];
+                    acc[i][j] = 0.f;
+                }
+        }
         if (more) {
             ta.store(va, As[cur ^ 1]);
             tb.store(vb, Bs[cur ^ 1]);
@@ -147,7 +162,7 @@ gemm_simt_kernel(const T *A, int64_t lda, const T *B, int64_t ldb, int64_t M_hos
         for (int j = 0; j < 4; ++j) {
             const int64_t m = m0 + ty * 4 + i;
             const int n = n0 + tx * 4 + j;
-            if (m < M && n < N) epi(m, n, acc[i][j], blockIdx.z);
+            if (m < M && n < N) epi(m, n, kFold ? total[kFold ? i : 0][j] : acc[i][j], blockIdx.z);
         }
 }
 
@@ -159,13 +174,18 @@ inline void launch_gemm_simt(bool chain, dim3 grid, cudaStream_t st, const T *A,
     launch_pdl(chain, gemm_simt_kernel<T, A_KM, B_KN, Epi>, grid, dim3(kGemmThreads), 0, st, A, lda, B, ldb, M, N, K, m_dev, k_dev, epi);
 }
 
-// Splits over `rows` (a capacity) of an m x n weight gradient on this kernel, at most `most`: two blocks per SM over all
+// Splits over `rows` (a capacity) of an m x n weight gradient on this kernel, at most `most` (148): two blocks per SM over all
 // output tiles and at least 64 rows each.  With 148 splits whatever the shape, a 320 x 320 result was 3700 blocks of at
 // most 16 rows and 60 MB of partial sums (24 + 12 us; the gated joint step 331 -> 273 us with this and the narrower products).
+// Wide results get more, up to five, at 4096 rows each: a sum's rounding error goes with the square root of its longest chain
+// of additions, K / 32 / splits + 32 + splits here and K / 148 + 148 before, and K / 160 is below K / 148 for every K.
+// Relative error of 256 x 512 weights over 12 k, 50 k and 200 k rows: 2.8e-7, 4.2e-7 and 7.1e-7 with 148 splits, 1.6e-7, 2.8e-7
+// and 4.7e-7 now (6.5e-7, 1.3e-6 and 2.8e-6 with ten splits and no folding).
 inline int simt_splits(int64_t rows, int m, int n, int most)
 {
     const int64_t tiles = ceil_div(m, kGemmBM) * ceil_div(n, kGemmBN);
-    return (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)most, ceil_div(2 * 148, tiles), ceil_div(rows, 64)}));
+    const int64_t wanted = std::max<int64_t>(ceil_div(2 * 148, tiles), std::min<int64_t>(5, ceil_div(rows, 4096)));
+    return (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)most, wanted, ceil_div(rows, 64)}));
 }
 
 // h' = act(z + b), stored in the feature dtype

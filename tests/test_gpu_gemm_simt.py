@@ -34,3 +34,24 @@ def test_gate_in_fp32(rows, d):
     assert (np.abs(dbg.double().cpu().numpy() - dpre.sum(0)) <= (rows + 8) * EPS * mass.sum(0) + 1e-30).all()
     bound = (d + 10) * EPS * (mass @ np.abs(w)) + 4 * EPS * np.abs(df * g)
     assert (np.abs(dF[:rows].double().cpu().numpy() - (dpre @ w + df * g)) <= bound + 1e-30).all()
+
+
+@pytest.mark.parametrize("rows,d,hidden", [(50_000, 256, 256), (12_000, 256, 256), (6_000, 1024, 1024), (35_000, 256, 64), (4_096, 160, 320),
+                                           (150, 64, 64)])
+def test_weight_gradients_over_many_rows(rows, d, hidden):
+    """Weight gradients contract over all rows of a batch.  The error of a sum of independent terms, relative to the sums'
+    norm, is below half a unit times the square root of the longest chain of additions, which is that of 148 splits of
+    the rows at most: 148 + rows / 148.  A chain over a tenth of 50 k rows misses it by a factor of two."""
+    g = torch.Generator(device="cuda").manual_seed(rows + d)
+    mk = lambda *s: torch.randn(*s, device="cuda", generator=g)
+    ptr = torch.arange(rows + 1, device="cuda", dtype=torch.int64)
+    idx = torch.randint(0, rows, (rows,), device="cuda", generator=g, dtype=torch.int32)
+    blocks = E.Blocks(rows, rows, [1], "cuda")
+    E.sample_khop(ptr, idx, torch.arange(rows, dtype=torch.int32, device="cuda"), blocks, 1, 1)
+    X, W, dH = mk(rows, d), mk(hidden, 2 * d) * 0.05, mk(rows, hidden)
+    _, ctx = E.sage_forward(blocks, X, [W], acts=[0])
+    dWs, _ = E.sage_backward(blocks, X, [W], ctx, dH, acts=[0])
+    cat = E.sage_ctx_views(blocks, X, [W], ctx)[0][0][:rows]
+    want = dH.double().T @ cat.double()
+    err = float((dWs[0].double() - want).norm() / want.norm())
+    assert err <= 0.5 * EPS * (148 + rows / 148) ** 0.5 + EPS, err
