@@ -117,18 +117,22 @@ __global__ void fill_i32_kernel(int32_t *p, int64_t n, int32_t v)
         p[i] = v;
 }
 
-// First kernel of a call: clears the tickets, digit counts and chain states of all hops (one launch instead of two memsets
-// per hop) and, with seeds, makes them the first frontier: local id = position in the batch.  counts1 (joint step): a second
-// set of counters to clear.
+struct HopCounts { int32_t *of[kMaxHops]; };
+
+// First kernel of a call: clears the tickets, digit counts, chain states and status words of all hops (one launch instead of
+// two memsets per hop; a tile of a hop that cleared its status word raced with what other tiles flagged) and, with seeds,
+// makes them the first frontier: local id = position in the batch.  counts1 (joint step): a second set of counters to clear.
 __global__ void __launch_bounds__(256)
 sample_begin_kernel(uint4 *__restrict__ zero, int64_t zero16, const int32_t *__restrict__ seeds, int32_t n_seeds, int64_t n_nodes,
-                    int32_t *__restrict__ local_id, int32_t *counts0, int32_t *counts1)
+                    int32_t *__restrict__ local_id, HopCounts counts, int n_hops, int32_t *counts1)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, all = (int64_t)gridDim.x * blockDim.x;
     for (int64_t k = i; k < zero16; k += all) zero[k] = make_uint4(0, 0, 0, 0);
     if (i == 0) {
-        counts0[CNT_DST] = seeds ? n_seeds : 0;
-        counts0[CNT_STATUS] = 0;
+        counts.of[0][CNT_DST] = seeds ? n_seeds : 0;
+#pragma unroll
+        for (int h = 0; h < kMaxHops; ++h)
+            if (h < n_hops) counts.of[h][CNT_STATUS] = 0;
         if (counts1) *reinterpret_cast<int4 *>(counts1) = make_int4(0, 0, 0, 0);
     }
     if (!seeds) return;
@@ -156,7 +160,7 @@ hop_sample_kernel(const int64_t *__restrict__ g_indptr, const int32_t *__restric
                   const uint64_t *__restrict__ g_cum, int64_t n_nodes,
                   const int32_t *__restrict__ dst_nodes, const int32_t *n_dst_ptr, int32_t cap_dst, int32_t cap_edges,
                   int32_t fanout, int32_t tile_dst, int32_t hop, uint32_t seed_lo, uint32_t seed_hi, uint32_t step_arg,
-                  const uint32_t *__restrict__ step_offset, int first_hop, int32_t *__restrict__ counts,
+                  const uint32_t *__restrict__ step_offset, int32_t *__restrict__ counts,
                   int32_t *__restrict__ blk_indptr, float *__restrict__ inv_cnt, int32_t *__restrict__ src_nodes,
                   int32_t *__restrict__ nbr_global, int32_t *__restrict__ edge_row,
                   const int32_t *__restrict__ local_id, uint32_t *__restrict__ bitmap, unsigned *ticket,
@@ -177,7 +181,6 @@ hop_sample_kernel(const int64_t *__restrict__ g_indptr, const int32_t *__restric
     if (over) n_dst = cap_dst;
     if (tile == 0 && threadIdx.x == 0) {
         counts[CNT_DST] = n_dst;
-        if (!first_hop) counts[CNT_STATUS] = 0;
         if (over) atomicOr((unsigned *)&counts[CNT_STATUS], E2EGREC_DEV_CAPACITY);
     }
     const int64_t i0 = (int64_t)tile * tile_dst;
@@ -688,8 +691,12 @@ int32_t e2egrec::sample_khop_impl(const e2egrec_csr *graph, const int32_t *seeds
         chain += ceil_div(blocks[h].cap_dst > 0 ? blocks[h].cap_dst : 1, dst_tile(blocks[h].cap_dst, fanouts[h]));
     }
     const int64_t zero16 = ceil_div(reinterpret_cast<char *>(chain) - s.zero, 16);
+    HopCounts counts{};
+    for (int h = 0; h < n_hops; ++h) counts.of[h] = blocks[h].counts;
+    const int64_t begin_blocks = std::max<int64_t>(ceil_div(zero16, T * 2), grid_for(pairs ? 0 : n_seeds, T));
     note_launch();
-    sample_begin_kernel<<<(unsigned)std::min<int64_t>(std::max<int64_t>(ceil_div(zero16, 256 * 2), grid_for(pairs ? 0 : n_seeds, 256)), 148 * 8), 256, 0, st>>>(reinterpret_cast<uint4 *>(s.zero), zero16, pairs ? nullptr : seeds, n_seeds, n, s.local_id, blocks[0].counts,
+    sample_begin_kernel<<<(unsigned)std::min<int64_t>(begin_blocks, 148 * 8), T, 0, st>>>(
+        reinterpret_cast<uint4 *>(s.zero), zero16, pairs ? nullptr : seeds, n_seeds, n, s.local_id, counts, n_hops,
         pairs ? pairs->pcounts : nullptr);
     cudaStream_t ts = side ? side->stream : st;          // stream of the transpositions
     const bool chained = me < kChainEdges;
@@ -726,7 +733,7 @@ int32_t e2egrec::sample_khop_impl(const e2egrec_csr *graph, const int32_t *seeds
         auto sample = graph->edge_cum ? hop_sample_kernel<true> : hop_sample_kernel<false>;
         note_launch();
         launch_pdl(chained, sample, dim3(grid_for(b.cap_dst, tile)), dim3(kDstThreads), 0, st, graph->indptr, graph->indices, graph->edge_cum, n, dst_nodes, n_dst_ptr, b.cap_dst, b.cap_edges, fanouts[h], tile, h + 1,
-            (uint32_t)(seed & 0xFFFFFFFFu), (uint32_t)(seed >> 32), step, s.step_offset, h == 0, b.counts, b.indptr,
+            (uint32_t)(seed & 0xFFFFFFFFu), (uint32_t)(seed >> 32), step, s.step_offset, b.counts, b.indptr,
             b.inv_cnt, b.src_nodes, b.nbr_global, l.edge_row, s.local_id, s.bitmap, s.tickets + 2 * h, tiles[h]);
         note_launch();
         launch_pdl(chained, frontier_kernel, dim3((unsigned)s.word_tiles), dim3(256), 0, st, s.bitmap, s.n_words, b.counts, b.cap_src, s.local_id, b.src_nodes,

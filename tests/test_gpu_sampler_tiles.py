@@ -45,3 +45,35 @@ def test_blocks(graph, batch, fanouts, weighted):
         want = oracle.sample_khop(indptr, indices, seeds, fanouts, 77, step, edge_cum=want_cum)
         torch.cuda.synchronize()
         assert_blocks_equal(blocks.to_host(), want)
+
+
+@pytest.mark.parametrize("batch,fanouts", [(3000, [4, 3]), (40, [5, 100, 2])])
+def test_ids_out_of_range_are_flagged_at_the_hop_that_meets_them(graph, batch, fanouts):
+    """One entry of one node beyond the graph: the status of the hops that draw from that node's row has the bit in every
+    sample, whichever tile of the hop flags it and however early, and no other hop's has; the entry becomes its row's node."""
+    n, _, _, _ = graph
+    rng = np.random.default_rng(batch)
+    deg = np.full(n, 2)
+    indptr = np.r_[0, np.cumsum(deg)].astype(np.int64)
+    indices = rng.integers(0, n, 2 * n).astype(np.int32)
+    seeds = rng.permutation(n)[:batch].astype(np.int32)
+    clean = oracle.sample_khop(indptr, indices, seeds, fanouts, 3, 0)
+    new = clean[1]["src_nodes"][clean[0]["n_src"]:]          # met by the second hop first: the third one draws from it
+    late = clean[0]["src_nodes"][-1]                         # the second hop's last destination
+    ip = torch.from_numpy(indptr).cuda()
+    blocks = E.Blocks(n, batch, fanouts, "cuda")
+    sd = torch.from_numpy(seeds).cuda()
+    for node, first_hop in ((late, 1), (new[len(new) // 2], 2)):
+        if first_hop >= len(fanouts):
+            continue
+        bad = indices.copy()
+        bad[indptr[node]] = n + 7
+        ix = torch.from_numpy(bad).cuda()
+        for step in range(20):
+            E.sample_khop(ip, ix, sd, blocks, 3, step)
+            assert [int(s) & 1 for s in blocks.counts[:, 3].tolist()] == [int(h >= first_hop) for h in range(len(fanouts))]
+        b = blocks.to_host()[first_hop]
+        at = b["indptr"][np.flatnonzero(b["src_nodes"][: b["n_dst"]] == node)[0]]
+        assert b["nbr_global"][at] == node
+    E.sample_khop(ip, torch.from_numpy(indices).cuda(), sd, blocks, 3, 0)
+    assert_blocks_equal(blocks.to_host(), clean)
