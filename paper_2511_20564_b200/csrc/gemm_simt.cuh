@@ -141,7 +141,12 @@ gemm_simt_kernel(const T *A, int64_t lda, const T *B, int64_t ldb, int64_t M_hos
 #pragma unroll
                 for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
         }
-        if (kFold) {
+        if (more) {
+            ta.store(va, As[cur ^ 1]);
+            tb.store(vb, Bs[cur ^ 1]);
+        }
+        __syncthreads();
+        if (kFold) {                           // behind the barrier: before it, the stores waited (35.3 and 36.9 us, 1000 x 320 x 320 gate)
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -150,11 +155,6 @@ gemm_simt_kernel(const T *A, int64_t lda, const T *B, int64_t ldb, int64_t M_hos
                     acc[i][j] = 0.f;
                 }
         }
-        if (more) {
-            ta.store(va, As[cur ^ 1]);
-            tb.store(vb, Bs[cur ^ 1]);
-        }
-        __syncthreads();
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i)
