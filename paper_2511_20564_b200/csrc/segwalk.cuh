@@ -14,7 +14,10 @@
 //     steps of 32 / LPR rows with no test per entry, and one sum across the lane groups per segment that halves the row at
 //     every exchange, so that every lane stores its own share of the finished row;
 //   - short ones (in a power-law graph nine tenths of the segments and a tenth of the entries) by one lane group each,
-//     32 / LPR segments side by side, with no exchange.
+//     32 / LPR segments side by side, with no exchange; where a row takes the whole warp, as one stream of entries, so that
+//     ids and weights come 32 at a time and four rows are in flight whatever the segments' lengths (one after another,
+//     2 M segments of two entries on average took 719 and, weighted, 857 us with 256 bf16 values, 824 with 100 fp32 values;
+//     now 578, 655 and 577).
 // Together 11 warp instructions per row.  Tried and slower: rows through a cp.async ring in shared memory (4.57 ms
 // against 3.74: the copies and the reads of the ring load the L1 path to 86 %), two groups of rows in registers (5.18),
 // all segments by the whole warp (4.57), stretches handed out by a counter (3.76 to 3.88: less waiting at the join's
@@ -99,7 +102,7 @@ template <typename T, int N> __device__ __forceinline__ void store_share(T *p, c
     }
 }
 
-// Steps (of 32 / LPR rows) whose loads a warp has in flight, and the longest segment that a single lane group sums.
+// Steps (of 32 / LPR rows) whose loads a warp has in flight, and the longest segment that counts as short.
 // Measured on whole_mean / three LightGCN layers (see launch_seg_walk), ms: 4 steps at four blocks per SM 3.74 / 3.03,
 // 4 steps at three blocks 4.40 / 3.42, 8 steps at three 4.10 / 3.31; short segments up to 4, 8, 16 entries: 3.89 / 3.10,
 // 3.74 / 3.03, 3.74 / 3.04.
@@ -125,7 +128,6 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
     constexpr int S = walk_share<LPR, E>();
     constexpr int ROW = LPR * CPL * E;
     constexpr int kFar = 1 << 30;
-    constexpr int kSmall = G >= 2 ? kWalkSmall : 0;              // one group per warp: nothing to put side by side
     static_assert(32 % C == 0, "a group takes its ids from one window of 32");
     extern __shared__ float4 seg_smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -202,11 +204,11 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
             int beg = __shfl_up_sync(0xffffffffu, ends, 1);
             if (lane == 0) beg = carry;
             const int n = min(ends, len) - max(beg, 0);          // entries of the segment in this stretch
-            const bool small = n > 0 && n <= kSmall && beg >= 0 && ends <= len;
+            const bool small = n > 0 && n <= kWalkSmall && beg >= 0 && ends <= len;
             unsigned small_m = __ballot_sync(0xffffffffu, small), big_m = __ballot_sync(0xffffffffu, n > 0 && !small);
 
             // ---- short segments: one lane group each
-            if constexpr (kSmall > 0) {
+            if constexpr (G >= 2) {
                 while (small_m) {
                     // the group's segment: the (sub + 1)-th lane that is set
                     unsigned m = small_m;
@@ -255,6 +257,54 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
 #pragma unroll
                             for (int e = 0; e < E; ++e) acc[q][e] *= inv;
                             if (ch < n_chunks) Chunk<T>::store(o.out + (int64_t)seg * o.ld_out + ch * E, acc[q]);
+                        }
+                    }
+                }
+            }
+
+            // ---- short segments whose rows take the whole warp: their entries in one stream, 32 ids and weights at a time, a row
+            // stored where a segment's last entry has been added
+            if constexpr (G == 1) {
+                int upto = small ? n : 0;                        // entries of the short segments up to and with the lane's
+#pragma unroll
+                for (int k = 1; k < 32; k <<= 1) {
+                    const int t = __shfl_up_sync(0xffffffffu, upto, k);
+                    if (lane >= k) upto += t;
+                }
+                const int all = __shfl_sync(0xffffffffu, upto, 31);
+                clear();
+                for (int e0 = 0; e0 < all; e0 += 32) {
+                    const int e = min(e0 + lane, all - 1);
+                    int i = 0;                                   // the lane of entry e's segment
+#pragma unroll
+                    for (int step = 16; step > 0; step >>= 1)
+                        if (__shfl_sync(0xffffffffu, upto, i + step - 1) <= e) i += step;
+                    const int after = __shfl_sync(0xffffffffu, upto, i) - e;             // entries of the segment from e on
+                    const int32_t id = __ldg(idx0 + __shfl_sync(0xffffffffu, ends, i) - after);
+                    const float wt = kWeight ? __ldg(w + id) : 1.f;
+                    const unsigned last = __ballot_sync(0xffffffffu, after == 1 && e0 + lane < all);
+                    const int cnt = min(32, all - e0);
+#pragma unroll 1
+                    for (int c0 = 0; c0 < cnt; c0 += U) {
+                        uint4 v[U][CPL];
+#pragma unroll
+                        for (int u = 0; u < U; ++u) load_row(row_of(__shfl_sync(0xffffffffu, id, c0 + u)), v[u]);
+#pragma unroll
+                        for (int u = 0; u < U; ++u) {
+                            if (c0 + u >= cnt) break;            // uniform over the warp, as is the next condition
+                            add_row(v[u], kWeight ? __shfl_sync(0xffffffffu, wt, c0 + u) : 1.f, true);
+                            if (!((last >> (c0 + u)) & 1u)) continue;
+                            const int j = __shfl_sync(0xffffffffu, i, c0 + u);
+                            const int32_t seg = (int32_t)(s_base + j);
+                            const float inv = scale_of(seg, __shfl_sync(0xffffffffu, n, j));
+#pragma unroll
+                            for (int q = 0; q < CPL; ++q) {
+                                const int ch = c + q * LPR;
+#pragma unroll
+                                for (int k = 0; k < E; ++k) acc[q][k] *= inv;
+                                if (ch < n_chunks) Chunk<T>::store(o.out + (int64_t)seg * o.ld_out + ch * E, acc[q]);
+                            }
+                            clear();
                         }
                     }
                 }
