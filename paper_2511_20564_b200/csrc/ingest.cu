@@ -116,7 +116,7 @@ expand_rows_kernel(const int64_t *__restrict__ indptr, int64_t n_rows, int64_t m
         } else {
             ++quiet;
         }
-        base = next_window(base, quiet, [&]() { return warp_seg_containing(indptr, n_rows, k0 + e0); });
+        base = quiet < kQuietWindows ? base + 32 : window_found(base, warp_seg_containing(indptr, n_rows, k0 + e0));
         ends = load_ends(base);
     }
 }

@@ -376,10 +376,11 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
             carry = __shfl_sync(0xffffffffu, ends, 31);          // the offsets do not decrease: the window's last end
             if (carry >= len) break;
             quiet = __any_sync(0xffffffffu, n > 0) ? 0 : quiet + 1;
-            s_base = next_window(s_base, quiet, [&]() { return (uint32_t)warp_seg_containing(ptr, n_seg, k0 + carry); });
             if (quiet < kQuietWindows) {
+                s_base += 32;
                 ends = ends_ahead;
             } else {                                             // a long stretch of empty segments
+                s_base = window_found(s_base, (uint32_t)warp_seg_containing(ptr, n_seg, k0 + carry));
                 ends = load_ends(s_base);
                 quiet = 0;
             }

@@ -11,15 +11,13 @@ namespace e2egrec {
 
 constexpr int kQuietWindows = 4;
 
-// First segment of the window of 32 that a walk looks at after the one that begins at `base`.  `quiet`: windows without an
-// entry in a row; from the fourth on the walk asks find() where the next entry's segment is.  Never the same window again:
-// offsets that decrease, which no entry point accepts but none can refuse, could make find() go back, and the walk ends
-// nevertheless, after one window per 32 segments at most.
-template <typename T, class Find> E2EGREC_HD T next_window(T base, int quiet, Find find)
+// A walk looks at windows of 32 segments.  After kQuietWindows windows without an entry it asks a search where the next
+// entry's segment is; this is where it goes on from the window at `base` when the search says `found`.  Never the same window
+// again: offsets that decrease, which no entry point accepts but none can refuse, could make a search go back, and the walk
+// ends nevertheless, after one window per 32 segments at most.
+template <typename T> E2EGREC_HD T window_found(T base, T found)
 {
     const T next = base + 32;
-    if (quiet < kQuietWindows) return next;
-    const T found = find();
     return found > next ? found : next;
 }
 
