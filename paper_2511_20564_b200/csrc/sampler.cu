@@ -43,11 +43,17 @@ constexpr int kWordTile = 512;         // bitmap words per block of the frontier
 // Destinations per block: about 1024 slots, four per thread, where that gives two blocks per SM and more; about 256 below,
 // where the time is that of one block's chain of loads.  With 64 destinations whatever the fanout, 4096 seeds at fanout
 // 100 were 64 blocks of 25 slots per thread.
+//
+// At most kDstBlocks blocks, three times what the machine holds, up to 64 destinations each: the host knows capacities, rows are
+// shorter, and a block of eight destinations with ten entries each costs what one with a hundred each does (B200,
+// 100 k seeds at fanout 128 on rows of 40 entries on average: 127 us with 12 500 blocks, 73 with 1563; on rows of 130 289 and 283).
+constexpr int64_t kDstBlocks = 148 * 16;
 static inline int dst_tile(int32_t cap_dst, int32_t fanout)
 {
     const int64_t slots = (int64_t)cap_dst * fanout >= 2 * 148 * 1024 ? 1024 : 256;
     int t = kDstTileMin;
     while (t < kDstTile && 2ll * t * fanout <= slots) t *= 2;
+    while (t < 64 && ceil_div(cap_dst, t) > kDstBlocks) t *= 2;
     return t;
 }
 
