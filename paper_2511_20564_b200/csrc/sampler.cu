@@ -157,11 +157,18 @@ sample_begin_kernel(uint4 *__restrict__ zero, int64_t zero16, const int32_t *__r
 // that are not yet in the frontier are marked in the bitmap.
 //
 // Latency is what it costs: a dozen dependent loads per block.  The block's sum is published before the draws and the
-// offset asked for after them, so that the chain moves meanwhile; four slots per thread keep their loads in flight together,
-// and a weighted draw narrows its row to a quarter per step with the three probes of all four slots in flight (one slot
-// after the other by halves: 154 us for 4096 seeds x 100, now 28).
-template <bool kWeighted>
-__global__ void __launch_bounds__(kDstThreads)
+// offset asked for after them, so that the chain moves meanwhile; four slots per thread keep their loads in flight together.
+// Weighted draws: with up to kQuarterBlocks blocks a draw narrows its row to a quarter per step with the three probes of all
+// four slots in flight (kDrawQuarters: 110 registers, two blocks per SM); with more, other blocks hide the latency and what
+// counts are probes and registers: one slot after the other by halves, six blocks per SM (kDrawHalves).  B200, us for a
+// sample whose table of running sums is not in L2, by quarters / by halves / by halves with four slots' loads behind a common
+// look-back as before: seeds by activity (rows of up to a million entries), 64 x 100 33 / 41 / 207, 4096 x 100 57 / 66 / 229,
+// 4096 x 15 x 10 68 / 88 / 125, 16 000 x 100 107 / 76 / 231; rows of 130 entries, 8192 x 20 x 10 x 5 416 / 315 / 401,
+// 100 000 x 128 647 / 426 / 467.
+constexpr int64_t kQuarterBlocks = 148 * 8;
+enum { kDrawUniform, kDrawQuarters, kDrawHalves };
+template <int kDraw>
+__global__ void __launch_bounds__(kDstThreads, kDraw == kDrawUniform ? 5 : kDraw == kDrawHalves ? 6 : 2)
 hop_sample_kernel(const int64_t *__restrict__ g_indptr, const int32_t *__restrict__ g_indices,
                   const uint64_t *__restrict__ g_cum, int64_t n_nodes,
                   const int32_t *__restrict__ dst_nodes, const int32_t *n_dst_ptr, int32_t cap_dst, int32_t cap_edges,
@@ -252,17 +259,26 @@ hop_sample_kernel(const int64_t *__restrict__ g_indptr, const int32_t *__restric
                 const uint4 r4 = philox4x32_10(make_uint4((uint32_t)(j >> 1), (uint32_t)node[lo], (1u << 8) | (uint32_t)hop, step),
                                                make_uint2(seed_lo, seed_hi));
                 const uint64_t rnd = (j & 1) ? (((uint64_t)r4.w << 32) | r4.z) : (((uint64_t)r4.y << 32) | r4.x);
-                const uint64_t total = kWeighted ? g_cum[rbeg[q] + deg - 1] : 0;
-                if (kWeighted && total > 0) {
+                const uint64_t total = kDraw != kDrawUniform ? g_cum[rbeg[q] + deg - 1] : 0;
+                if (kDraw == kDrawQuarters && total > 0) {
                     target[q] = __umul64hi(rnd, total);
                     b[q] = deg - 1;                  // its running sum is `total`, above every target
+                } else if (kDraw == kDrawHalves && total > 0) {
+                    const uint64_t *cum = g_cum + rbeg[q];
+                    const uint64_t t = __umul64hi(rnd, total);
+                    int64_t hi_pos = deg - 1;        // its running sum is `total`, above every target
+                    pos = 0;
+                    while (pos < hi_pos) {
+                        const int64_t mid = (pos + hi_pos) >> 1;
+                        if (__ldg(cum + mid) > t) hi_pos = mid; else pos = mid + 1;
+                    }
                 } else {
                     pos = (int64_t)__umul64hi(rnd, (uint64_t)deg);
                 }
             }
             src[q] = rbeg[q] + pos;
         }
-        if constexpr (kWeighted) {
+        if constexpr (kDraw == kDrawQuarters) {
             // the first entry in [a, b] whose running sum exceeds the target
             while (true) {
                 uint64_t c1[S], c2[S], c3[S];
@@ -736,9 +752,11 @@ int32_t e2egrec::sample_khop_impl(const e2egrec_csr *graph, const int32_t *seeds
         const SortPlan sp = sort_plan(b.cap_src);
         const SortLane &l = s.lane[h];
         const int tile = dst_tile(b.cap_dst, fanouts[h]);
-        auto sample = graph->edge_cum ? hop_sample_kernel<true> : hop_sample_kernel<false>;
+        const unsigned grid = grid_for(b.cap_dst, tile);
+        auto sample = !graph->edge_cum ? hop_sample_kernel<kDrawUniform>
+                      : grid <= kQuarterBlocks ? hop_sample_kernel<kDrawQuarters> : hop_sample_kernel<kDrawHalves>;
         note_launch();
-        launch_pdl(chained, sample, dim3(grid_for(b.cap_dst, tile)), dim3(kDstThreads), 0, st, graph->indptr, graph->indices, graph->edge_cum, n, dst_nodes, n_dst_ptr, b.cap_dst, b.cap_edges, fanouts[h], tile, h + 1,
+        launch_pdl(chained, sample, dim3(grid), dim3(kDstThreads), 0, st, graph->indptr, graph->indices, graph->edge_cum, n, dst_nodes, n_dst_ptr, b.cap_dst, b.cap_edges, fanouts[h], tile, h + 1,
             (uint32_t)(seed & 0xFFFFFFFFu), (uint32_t)(seed >> 32), step, s.step_offset, b.counts, b.indptr,
             b.inv_cnt, b.src_nodes, b.nbr_global, l.edge_row, s.local_id, s.bitmap, s.tickets + 2 * h, tiles[h]);
         note_launch();
