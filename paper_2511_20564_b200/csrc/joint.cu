@@ -49,6 +49,18 @@ void fill_blocks(const JointPlan &jp, char *ws, e2egrec_block *blocks)
 // ------------------------------------------------------------------------------------------ kernels
 __global__ void joint_meta_kernel(int32_t *pmeta, int32_t n_pairs) { pmeta[0] = n_pairs; }
 
+// out = {gradient rows, status bits of all hops and of the pairs' grouping}
+struct StatusWords { const int32_t *counts[kMaxHops + 1]; };
+__global__ void joint_result_kernel(StatusWords words, int n_words, const int32_t *outer, int32_t *out)
+{
+    int32_t status = 0;
+#pragma unroll
+    for (int k = 0; k <= kMaxHops; ++k)
+        if (k < n_words) status |= words.counts[k][CNT_STATUS];
+    out[0] = outer[CNT_SRC];
+    out[1] = status;
+}
+
 // z[p] = [ h[user seed] | h[item seed] | dense[p] ] in the feature dtype; rows P .. rows_alloc-1 are zero.  A thread writes
 // 16 bytes of a row (the widths are multiples of that); one value per thread with its divisions took 6.4 us for 4096 rows.
 template <typename T>
@@ -601,8 +613,11 @@ int32_t run_joint(const JointPlan &jp, const e2egrec_csr *graph, const e2egrec_m
     if (rc != E2EGREC_OK) return rc;
     const e2egrec_block &outer = blocks[jp.n_hops - 1];
     cudaMemcpyAsync(dX_ids, outer.src_nodes, sizeof(int32_t) * (size_t)outer.cap_src, cudaMemcpyDeviceToDevice, st);
-    cudaMemcpyAsync(n_dX_rows, &outer.counts[CNT_SRC], sizeof(int32_t), cudaMemcpyDeviceToDevice, st);
-    cudaMemcpyAsync(n_dX_rows + 1, status, sizeof(int32_t), cudaMemcpyDeviceToDevice, st);
+    StatusWords words{};
+    for (int h = 0; h < jp.n_hops; ++h) words.counts[h] = blocks[h].counts;
+    words.counts[jp.n_hops] = pcounts;
+    note_launch();
+    joint_result_kernel<<<1, 1, 0, st>>>(words, jp.n_hops + 1, outer.counts, n_dX_rows);
     return check_launch("joint_step");
 }
 

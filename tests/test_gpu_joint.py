@@ -149,3 +149,20 @@ def test_joint_step_in_two_phases_equals_the_whole_step():
     assert torch.equal(js.dX_ids[:n_rows], whole.dX_ids[:n_rows]) and torch.equal(js.dX_rows[:n_rows], whole.dX_rows[:n_rows])
     for a, b in zip(js.dW_gnn + js.dW_tower + js.db_tower, whole.dW_gnn + whole.dW_tower + whole.db_tower):
         assert torch.equal(a, b)
+
+
+def test_status_of_every_hop_reaches_the_caller():
+    """An id out of range in the rows of a node that only the second hop draws from: the step's status has the bit."""
+    import paper_2511_20564_b200 as E
+    w = S.WORKLOADS["tiny"]
+    indptr, indices, X, W_gnn, pu, pi, dense, labels, W_t, b_t = args = _inputs(w, 96, 8, 48, 24, 13)
+    js = _run_gpu(w, *args, 3)
+    assert js.n_rows.tolist()[1] == 0
+    seeds = np.unique(np.r_[pu, pi]).astype(np.int32)
+    first = oracle.sample_khop(indptr, indices, seeds, w.fanouts, w.seed, 3)[0]
+    node = first["src_nodes"][first["n_dst"]]                # reached by the first hop, no seed
+    bad = indices.copy()
+    bad[indptr[node]: indptr[node + 1]] = w.n_nodes + 3
+    js = _run_gpu(w, indptr, bad, X, W_gnn, pu, pi, dense, labels, W_t, b_t, 3)
+    hops = [int(c[3]) for c in js.activations()["counts"]]
+    assert hops[0] == 0 and hops[1] & 1 and js.n_rows.tolist()[1] & 1
