@@ -57,11 +57,12 @@ void note_launch();
 // beforehand (plain loads of const __restrict__ arrays gave stale frontiers), any load for what depends on those.
 //
 // Who sets `chain`: the small kernels of a sample, an encoder pass or a ranking tower, where the gaps between launches are
-// a fifth of the time -- samples all of whose blocks stay below kChainEdges entries of capacity.  B200, us a pass without and with: serving 64 users
-// 69.7 / 55.2, tiny fp32 step 136 / 122, medium step 176 / 164, joint step 316 / 293; the large step, whose kernels fill the
-// machine and whose legs run on two streams, loses: 1357 / 1370 with its samples' sorts
-// and first hops launched this way, 1385 with the small kernels of its top layer as well.  Admitting the next kernel while this one still runs
-// (griddepcontrol.launch_dependents at its beginning) keeps the other stream's kernels off the SMs: 182 for the medium step.
+// a fifth of the time -- samples all of whose blocks stay below kChainEdges entries of capacity.  B200, us a pass without and
+// with: serving 64 users 69.7 / 55.2, tiny fp32 step 136 / 122, medium step 176 / 164, joint step 316 / 293; the large step,
+// whose kernels fill the machine and whose legs run on two streams, loses: 1357 / 1370 with its samples' sorts and first hops
+// launched this way, 1385 with the small kernels of its top layer as well.  Admitting the next kernel while this one still
+// runs (griddepcontrol.launch_dependents at its beginning) keeps the other stream's kernels off the SMs: 182 for the medium
+// step.
 constexpr int64_t kChainEdges = 1ll << 21, kChainRows = 1ll << 17;
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(bool chain, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args &&...args)

@@ -754,12 +754,8 @@ bool launch_tn(const __nv_bfloat16 *A, int64_t rows, int k, int64_t lda, const _
     const int64_t tiles_cap = (rows / kTileM) * n_tiles_n * n_rhs;
     const unsigned grid = (unsigned)std::min<int64_t>(tiles_cap, sm_count());
     note_launch();
-    if (fused)
-        launch_pdl(ep.chain && rows * n_rhs < kChainRows, tc_gemm_tn_kernel<true>, dim3(grid), dim3(kTnThreads), smem, st, ma, mb, mo, k_blocks, stages, nt, n_tiles_n, tmem_cols,
-                   b_mn ? 1 : 0, ep);
-    else
-        launch_pdl(ep.chain && rows * n_rhs < kChainRows, tc_gemm_tn_kernel<false>, dim3(grid), dim3(kTnThreads), smem, st, ma, mb, mo, k_blocks, stages, nt, n_tiles_n, tmem_cols,
-                   b_mn ? 1 : 0, ep);
+    launch_pdl(ep.chain && rows * n_rhs < kChainRows, fused ? tc_gemm_tn_kernel<true> : tc_gemm_tn_kernel<false>, dim3(grid),
+               dim3(kTnThreads), smem, st, ma, mb, mo, k_blocks, stages, nt, n_tiles_n, tmem_cols, b_mn ? 1 : 0, ep);
     return true;
 }
 
@@ -1286,8 +1282,8 @@ bool tc_weight_grad(const __nv_bfloat16 *dY, int64_t rows, int m, const __nv_bfl
     if (!raise_smem_limit(tc_gemm_rows_kernel, attr_set)) return false;
     dim3 grid((unsigned)(m / kTileM), (unsigned)(n / nt), (unsigned)splits);
     note_launch();
-    launch_pdl(chain && rows * n_rhs < kChainRows, tc_gemm_rows_kernel, grid, dim3(kThreads), smem, st, my, mx, nt, tmem_cols, stages, m_dev, part, (int64_t)n,
-               (int64_t)m * n, status, n_rhs, rows);
+    launch_pdl(chain && rows * n_rhs < kChainRows, tc_gemm_rows_kernel, grid, dim3(kThreads), smem, st, my, mx, nt, tmem_cols, stages,
+               m_dev, part, (int64_t)n, (int64_t)m * n, status, n_rhs, rows);
     return true;
 }
 

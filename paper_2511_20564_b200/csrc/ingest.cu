@@ -241,9 +241,11 @@ extern "C" int32_t e2egrec_csr_transpose(const e2egrec_csr *csr, int64_t n_cols,
         for (int q = 0; q < sp.passes; ++q) {
             const int32_t clamp = q == 0 ? (int32_t)std::max<int64_t>(n_cols, 1) : 0;
             if (q == sp.passes - 1)
-                sort_pass<int64_t>(sp, k, v, nullptr, m, clamp, (int32_t)m, q, s.sort[0], false, ka, csc_eid, SortMap{}, &s.counts[CNT_STATUS], st);
+                sort_pass<int64_t>(sp, k, v, nullptr, m, clamp, (int32_t)m, q, s.sort[0], false, ka, csc_eid, SortMap{},
+                                   &s.counts[CNT_STATUS], st);
             else
-                sort_pass<int32_t>(sp, k, v, nullptr, m, clamp, (int32_t)m, q, s.sort[0], false, ka, va, SortMap{}, &s.counts[CNT_STATUS], st);
+                sort_pass<int32_t>(sp, k, v, nullptr, m, clamp, (int32_t)m, q, s.sort[0], false, ka, va, SortMap{},
+                                   &s.counts[CNT_STATUS], st);
             k = ka;
             v = va;
             std::swap(ka, kb);

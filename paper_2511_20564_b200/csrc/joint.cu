@@ -553,7 +553,8 @@ int32_t run_joint(const JointPlan &jp, const e2egrec_csr *graph, const e2egrec_m
     launch_pdl(small, logit_kernel<T>, dim3((unsigned)ceil_div((int64_t)jp.P * 32, 256)), dim3(256), 0, st, (const T *)a2, jp.h2, W3, b3,
                jp.P, logits);
     note_launch();
-    launch_pdl(small, bce_kernel, dim3(1), dim3(1024), 0, st, (const float *)logits, labels, jp.P, loss, dt, db_tower ? db_tower[2] : nullptr, 0);
+    launch_pdl(small, bce_kernel, dim3(1), dim3(1024), 0, st, (const float *)logits, labels, jp.P, loss, dt,
+               db_tower ? db_tower[2] : nullptr, 0);
 
     // 4. tower backward
     T *dz2 = tp(jp.dz2_off), *dz1 = tp(jp.dz1_off), *dz = tp(jp.dz_off), *wt = tp(jp.wt_off);
@@ -572,7 +573,8 @@ int32_t run_joint(const JointPlan &jp, const e2egrec_csr *graph, const e2egrec_m
         ws_st = side->stream;
     }
     launch_colsum<T>(a2, jp.h2, dt, nullptr, jp.P, jp.h2, 0, dW_tower[2], ws_st);                   // dW3 = dt^T a2
-    linear_backward_weight<T>(dz2, jp.rowsP, jp.h2, a1, jp.h1, pmeta, part, dW_tower[1], db_tower ? db_tower[1] : nullptr, status, ws_st);
+    linear_backward_weight<T>(dz2, jp.rowsP, jp.h2, a1, jp.h1, pmeta, part, dW_tower[1], db_tower ? db_tower[1] : nullptr, status,
+                              ws_st);
     linear_backward_input<T>(dz2, jp.rowsP, jp.h2, W2, jp.h1, relu ? a1 : nullptr, dz1, wt, pmeta, status, st);
     if (side) side->fork(st);
     linear_backward_weight<T>(dz1, jp.rowsP, jp.h1, tin, jp.zdim, pmeta, part, dW_tower[0], db_tower ? db_tower[0] : nullptr, status, ws_st);
@@ -598,8 +600,8 @@ int32_t run_joint(const JointPlan &jp, const e2egrec_csr *graph, const e2egrec_m
         o.out = tp(jp.dhseed_off);
         o.ld_out = jp.dL;
         const SegScratch sc = seg_scratch_carve(jp.P2, kPairRun, jp.dL, dtype_size(X->dtype), ws + jp.seg_off);
-        if (!dispatch_seg_reduce<T, int32_t, false>(dz, jp.unit, pi.pcsc_ptr, pi.pcsc_idx, &pcounts[CNT_SRC], 0, jp.P2, nullptr,
-                                                    kPairRun, jp.dL, X->dtype, pi.pcsc_col, sc, o, st)) {
+        if (!dispatch_seg_reduce<T, false>(dz, jp.unit, pi.pcsc_ptr, pi.pcsc_idx, &pcounts[CNT_SRC], 0, jp.P2, nullptr, kPairRun,
+                                           jp.dL, X->dtype, pi.pcsc_col, sc, o, st)) {
             set_last_error("joint_step: no reduction kernel for this embedding width");
             return E2EGREC_ERR_UNSUPPORTED;
         }

@@ -177,9 +177,9 @@ int32_t backward_impl(const e2egrec_block *blocks, const LgPlan &fp, const LgPla
         o.ld_out = ld_out;
         o.seg_scale = reinterpret_cast<const float *>(ctx + fp.s_off[L - 1 - l]);
         const SegScratch sc = seg_scratch_carve(b.cap_edges, kLgRun, d, fp.es, scratch + bp.seg_off);
-        if (!dispatch_seg_reduce<T, int32_t, true>(g_in, d, b.csc_ptr, b.csc_row, &b.counts[CNT_SRC], 0, b.cap_src,
-                                                   reinterpret_cast<const float *>(ctx + fp.t_off[L - 1 - l]), kLgRun, d, dtype,
-                                                   b.csc_col, sc, o, st)) {
+        if (!dispatch_seg_reduce<T, true>(g_in, d, b.csc_ptr, b.csc_row, &b.counts[CNT_SRC], 0, b.cap_src,
+                                          reinterpret_cast<const float *>(ctx + fp.t_off[L - 1 - l]), kLgRun, d, dtype, b.csc_col, sc,
+                                          o, st)) {
             set_last_error("lightgcn_sampled_backward: no kernel for this row width");
             return E2EGREC_ERR_UNSUPPORTED;
         }

@@ -372,8 +372,8 @@ static inline void launch_sort_pass(const int32_t *kin, const int32_t *vin, cons
     }
     const unsigned grid = (unsigned)ceil_div(cap > 0 ? cap : 1, (int64_t)THREADS * kSortItems);
     note_launch();
-    launch_pdl(chain, kern, dim3(grid), dim3(THREADS), smem, st, kin, vin, n_dev, (int32_t)cap, clamp_keys, clamp_vals, pass * BITS, ss.ghist + pass * kMaxRadix,
-                                      ss.tickets() + pass, ss.state + (size_t)pass * ss.tiles * (1 << BITS), kout, vout, map, status);
+    launch_pdl(chain, kern, dim3(grid), dim3(THREADS), smem, st, kin, vin, n_dev, (int32_t)cap, clamp_keys, clamp_vals, pass * BITS,
+               ss.ghist + pass * kMaxRadix, ss.tickets() + pass, ss.state + (size_t)pass * ss.tiles * (1 << BITS), kout, vout, map, status);
 }
 
 template <typename ValT>
@@ -382,10 +382,9 @@ static inline void sort_pass(const SortPlan &sp, const int32_t *kin, const int32
                              const SortMap &map, int32_t *status, cudaStream_t st)
 {
     const bool wide = cap >= kSortWide;
-    if (sp.bits == 8 && wide) launch_sort_pass<8, 512, ValT>(kin, vin, n_dev, cap, clamp_keys, clamp_vals, pass, ss, chain, kout, vout, map, status, st);
-    else if (sp.bits == 8) launch_sort_pass<8, 256, ValT>(kin, vin, n_dev, cap, clamp_keys, clamp_vals, pass, ss, chain, kout, vout, map, status, st);
-    else if (wide) launch_sort_pass<10, 512, ValT>(kin, vin, n_dev, cap, clamp_keys, clamp_vals, pass, ss, chain, kout, vout, map, status, st);
-    else launch_sort_pass<10, 256, ValT>(kin, vin, n_dev, cap, clamp_keys, clamp_vals, pass, ss, chain, kout, vout, map, status, st);
+    auto launch = sp.bits == 8 ? (wide ? launch_sort_pass<8, 512, ValT> : launch_sort_pass<8, 256, ValT>)
+                               : (wide ? launch_sort_pass<10, 512, ValT> : launch_sort_pass<10, 256, ValT>);
+    launch(kin, vin, n_dev, cap, clamp_keys, clamp_vals, pass, ss, chain, kout, vout, map, status, st);
 }
 
 }  // namespace e2egrec

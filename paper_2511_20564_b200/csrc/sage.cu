@@ -99,7 +99,8 @@ static bool dispatch_sage_aggregate(const T *Hsrc, int64_t ld, const int32_t *nb
 // transposed-block entries per lane group: 16, or 128 where the block can hold a million entries or more (the longer run's
 // lower overhead per entry wins there; measured on the 2 * 10^9-entry workload: 0.69 -> 0.63 ms)
 // A block that can hold two million entries gets runs of 128 entries; with 512-byte bf16 rows (whose forward aggregation is
-// streamed from the same size on) a million.  Capacities, not sizes, are what the host knows: a small batch in large
+// streamed from the same size on) a million: a large step whose middle block holds 1.7 million takes 1236 us with runs of 128 in
+// that block and 1272 with runs of 16 (B200).  Capacities, not sizes, are what the host knows: a small batch in large
 // buffers pays for the long runs (a 71 k-entry block in a 1.2 M-entry buffer: 0.327 -> 0.362 ms per joint step), hence no
 // lower than this.
 static inline bool streamable_rows(int d, size_t es) { return es == 2 && d == 256; }
@@ -175,7 +176,8 @@ static int32_t forward_impl(const e2egrec_block *blocks, int32_t n_layers, const
         }
         bool agg_ok = false;
         if (l == 0) tap_begin(TAP_AGG_FWD_OUTER, st);
-        if (X->dtype == E2EGREC_BF16 && streamable_rows(p.d_in, sizeof(T)) && b.cap_edges >= big_block_edges(p.d_in, sizeof(T)) && stream_gather_enabled())
+        if (X->dtype == E2EGREC_BF16 && streamable_rows(p.d_in, sizeof(T)) &&
+            b.cap_edges >= big_block_edges(p.d_in, sizeof(T)) && stream_gather_enabled())
             agg_ok = stream_sage_aggregate(l == 0 ? static_cast<const __nv_bfloat16 *>(X->data)
                                                   : reinterpret_cast<const __nv_bfloat16 *>(ctx + plan[l - 1].h_off),
                                            l == 0 ? X->rows : plan[l - 1].rows, l == 0 ? X->ld : p.d_in,
@@ -238,8 +240,10 @@ static BackwardScratch plan_backward(const e2egrec_block *blocks, int32_t n_laye
         dcat = std::max(dcat, (size_t)n_rhs * p.rows * 2 * p.d_in * es);
         part = std::max(part, (size_t)kDwSplits * p.d_out * 2 * p.d_in * sizeof(float));
         wt = std::max(wt, (size_t)p.d_out * 2 * p.d_in * es);
-        ht = std::max(ht, seg_scratch_carve(blocks[p.block].cap_edges, block_run_len(blocks[p.block].cap_edges, p.d_in, es), p.d_in, es, nullptr, n_rhs).bytes);
-        chain = std::max(chain, seg_chain_bytes(blocks[p.block].cap_edges, block_run_len(blocks[p.block].cap_edges, p.d_in, es), p.d_in, es, n_rhs));
+        const int64_t edges = blocks[p.block].cap_edges;
+        const int run_len = block_run_len(edges, p.d_in, es);
+        ht = std::max(ht, seg_scratch_carve(edges, run_len, p.d_in, es, nullptr, n_rhs).bytes);
+        chain = std::max(chain, seg_chain_bytes(edges, run_len, p.d_in, es, n_rhs));
     }
     size_t off = 0;
     auto take = [&](size_t b) { size_t o = off; off += align_up(b, 256); return o; };
@@ -386,12 +390,12 @@ static int32_t backward_impl(const e2egrec_block *blocks, int32_t n_layers, cons
             o.rhs_out = static_cast<T *>(dX_rows[n_rhs - 1].data) - static_cast<T *>(dX_rows[0].data);
         }
         if (l == 0) tap_begin(TAP_AGG_BWD_OUTER, st);
-        SegScratch sc = seg_scratch_carve(b.cap_edges, block_run_len(b.cap_edges, p.d_in, dtype_size(X->dtype)), p.d_in, dtype_size(X->dtype), scratch + bs.seg_off, n_rhs);
+        const int run_len = block_run_len(b.cap_edges, p.d_in, sizeof(T));
+        SegScratch sc = seg_scratch_carve(b.cap_edges, run_len, p.d_in, sizeof(T), scratch + bs.seg_off, n_rhs);
         sc.chain = chain;
         sc.chain_cnt = reinterpret_cast<int32_t *>(scratch + bs.chain_off);
-        const bool seg_ok = dispatch_seg_reduce<T, int32_t, false>(dcat + p.d_in, two_d, b.csc_ptr, b.csc_row, &b.counts[CNT_SRC], 0,
-                                                                   b.cap_src, nullptr, block_run_len(b.cap_edges, p.d_in, dtype_size(X->dtype)), p.d_in, X->dtype,
-                                                                   b.csc_col, sc, o, st);
+        const bool seg_ok = dispatch_seg_reduce<T, false>(dcat + p.d_in, two_d, b.csc_ptr, b.csc_row, &b.counts[CNT_SRC], 0, b.cap_src,
+                                                          nullptr, run_len, p.d_in, X->dtype, b.csc_col, sc, o, st);
         if (l == 0) tap_end(TAP_AGG_BWD_OUTER, st);
         if (!seg_ok) {
             if (side) side->join(st);

@@ -525,20 +525,21 @@ pair_local_kernel(const int32_t *__restrict__ user, const int32_t *__restrict__ 
 // The transposed block: entries ordered by (column, position), the last pass looking up every entry's row, and the offsets.
 static void transpose_block(const int32_t *col, int32_t *counts, int32_t cap_edges, const int32_t *row_of,
                             int32_t *csc_col, int32_t *csc_eid, int32_t *csc_row, int32_t *csc_ptr, const SortPlan &sp,
-                            const SortLane &l, bool chain, cudaStream_t st, const int32_t *release_nodes = nullptr, int32_t *local_id = nullptr)
+                            const SortLane &l, bool chain, cudaStream_t st, const int32_t *release_nodes = nullptr,
+                            int32_t *local_id = nullptr)
 {
     const int32_t *k = col, *v = nullptr;
     for (int p = 0; p < sp.passes; ++p) {
         const bool last = p == sp.passes - 1, own = (sp.passes - 1 - p) % 2 == 0;       // the last pass ends in the block's arrays
         int32_t *ko = own ? csc_col : l.key, *vo = own ? csc_eid : l.val;
-        sort_pass<int32_t>(sp, k, v, &counts[CNT_EDGES], cap_edges, 0, cap_edges, p, l.sort, chain, ko, vo, last ? SortMap{row_of, csc_row} : SortMap{},
-                           &counts[CNT_STATUS], st);
+        sort_pass<int32_t>(sp, k, v, &counts[CNT_EDGES], cap_edges, 0, cap_edges, p, l.sort, chain, ko, vo,
+                           last ? SortMap{row_of, csc_row} : SortMap{}, &counts[CNT_STATUS], st);
         k = ko;
         v = vo;
     }
     note_launch();
-    launch_pdl(chain, csc_finalize_kernel, dim3((unsigned)std::min<int64_t>(ceil_div((int64_t)cap_edges + 1, 256), 148 * 8)), dim3(256), 0, st, csc_col, counts, csc_ptr, l.sort, sp.bits, sp.passes,
-                                                                                                                release_nodes, local_id);
+    launch_pdl(chain, csc_finalize_kernel, dim3((unsigned)std::min<int64_t>(ceil_div((int64_t)cap_edges + 1, 256), 148 * 8)), dim3(256),
+               0, st, csc_col, counts, csc_ptr, l.sort, sp.bits, sp.passes, release_nodes, local_id);
 }
 
 static inline unsigned grid_for(int64_t n, int threads) { return (unsigned)ceil_div(n > 0 ? n : 1, threads); }
@@ -728,16 +729,18 @@ int32_t e2egrec::sample_khop_impl(const e2egrec_csr *graph, const int32_t *seeds
         const PairInput &pi = *pairs;
         const int32_t P2 = 2 * pi.n_pairs;
         note_launch();
-        launch_pdl(chained, pair_mark_kernel, dim3(grid_for(pi.n_pairs, T)), dim3(T), 0, st, pi.user, pi.item, pi.n_pairs, n, s.bitmap, blocks[0].counts);
+        launch_pdl(chained, pair_mark_kernel, dim3(grid_for(pi.n_pairs, T)), dim3(T), 0, st, pi.user, pi.item, pi.n_pairs, n, s.bitmap,
+                   blocks[0].counts);
         note_launch();
-        launch_pdl(chained, frontier_kernel, dim3((unsigned)s.word_tiles), dim3(256), 0, st, s.bitmap, s.n_words, pi.pcounts, P2, s.local_id, pi.seeds_out,
-                                                                s.tickets + 2 * kMaxHops, words[n_hops]);
+        launch_pdl(chained, frontier_kernel, dim3((unsigned)s.word_tiles), dim3(256), 0, st, s.bitmap, s.n_words, pi.pcounts, P2,
+                   s.local_id, pi.seeds_out, s.tickets + 2 * kMaxHops, words[n_hops]);
         const SortPlan sp = sort_plan(P2 > 1 ? P2 : 2);
         const bool own_lane = n_hops < kMaxHops;
         const SortLane &l = s.lane[own_lane ? kMaxHops - 1 : 0];
         note_launch();
-        launch_pdl(chained, pair_local_kernel, dim3((unsigned)std::min<int64_t>(grid_for(P2, T), 148 * 4)), dim3(T), 0, st, pi.user, pi.item, pi.n_pairs, n, s.local_id, pi.pair_local, pi.entry_unit, pi.units_per_row, pi.item_unit_off,
-            pi.pcounts, sp.bits, sp.passes, l.sort);
+        launch_pdl(chained, pair_local_kernel, dim3((unsigned)std::min<int64_t>(grid_for(P2, T), 148 * 4)), dim3(T), 0, st, pi.user,
+                   pi.item, pi.n_pairs, n, s.local_id, pi.pair_local, pi.entry_unit, pi.units_per_row, pi.item_unit_off, pi.pcounts,
+                   sp.bits, sp.passes, l.sort);
         if (side && own_lane) side->fork(st);
         transpose_block(pi.pair_local, pi.pcounts, P2, pi.entry_unit, pi.pcsc_col, pi.pcsc_eid, pi.pcsc_idx, pi.pcsc_ptr, sp, l, chained,
                         own_lane ? ts : st);
@@ -756,14 +759,16 @@ int32_t e2egrec::sample_khop_impl(const e2egrec_csr *graph, const int32_t *seeds
         auto sample = !graph->edge_cum ? hop_sample_kernel<kDrawUniform>
                       : grid <= kQuarterBlocks ? hop_sample_kernel<kDrawQuarters> : hop_sample_kernel<kDrawHalves>;
         note_launch();
-        launch_pdl(chained, sample, dim3(grid), dim3(kDstThreads), 0, st, graph->indptr, graph->indices, graph->edge_cum, n, dst_nodes, n_dst_ptr, b.cap_dst, b.cap_edges, fanouts[h], tile, h + 1,
-            (uint32_t)(seed & 0xFFFFFFFFu), (uint32_t)(seed >> 32), step, s.step_offset, b.counts, b.indptr,
-            b.inv_cnt, b.src_nodes, b.nbr_global, l.edge_row, s.local_id, s.bitmap, s.tickets + 2 * h, tiles[h]);
+        launch_pdl(chained, sample, dim3(grid), dim3(kDstThreads), 0, st, graph->indptr, graph->indices, graph->edge_cum, n, dst_nodes,
+                   n_dst_ptr, b.cap_dst, b.cap_edges, fanouts[h], tile, h + 1, (uint32_t)(seed & 0xFFFFFFFFu), (uint32_t)(seed >> 32),
+                   step, s.step_offset, b.counts, b.indptr, b.inv_cnt, b.src_nodes, b.nbr_global, l.edge_row, s.local_id, s.bitmap,
+                   s.tickets + 2 * h, tiles[h]);
         note_launch();
-        launch_pdl(chained, frontier_kernel, dim3((unsigned)s.word_tiles), dim3(256), 0, st, s.bitmap, s.n_words, b.counts, b.cap_src, s.local_id, b.src_nodes,
-                                                                s.tickets + 2 * h + 1, words[h]);
+        launch_pdl(chained, frontier_kernel, dim3((unsigned)s.word_tiles), dim3(256), 0, st, s.bitmap, s.n_words, b.counts, b.cap_src,
+                   s.local_id, b.src_nodes, s.tickets + 2 * h + 1, words[h]);
         note_launch();
-        launch_pdl(chained, relabel_kernel, dim3((unsigned)std::min<int64_t>(grid_for(b.cap_edges, T), 148 * 4)), dim3(T), 0, st, b.nbr_global, s.local_id, b.counts, b.col, sp.bits, sp.passes, l.sort);
+        launch_pdl(chained, relabel_kernel, dim3((unsigned)std::min<int64_t>(grid_for(b.cap_edges, T), 148 * 4)), dim3(T), 0, st,
+                   b.nbr_global, s.local_id, b.counts, b.col, sp.bits, sp.passes, l.sort);
         if (transpose) {
             if (side) side->fork(st);
             const bool release = h == n_hops - 1;        // every relabelling is done: the last block's offsets release the ids
@@ -775,7 +780,8 @@ int32_t e2egrec::sample_khop_impl(const e2egrec_csr *graph, const int32_t *seeds
     }
     if (!transpose) {
         note_launch();
-        launch_pdl(chained, frontier_release_kernel, dim3(grid_for(last.cap_src, T)), dim3(T), 0, st, last.src_nodes, last.counts, s.local_id);
+        launch_pdl(chained, frontier_release_kernel, dim3(grid_for(last.cap_src, T)), dim3(T), 0, st, last.src_nodes, last.counts,
+                   s.local_id);
     }
     if (side && (transpose || (pairs && n_hops < kMaxHops))) {
         if (flags & E2EGREC_SAMPLE_DEFER_TRANSPOSE) side->defer();
@@ -816,7 +822,8 @@ extern "C" int32_t e2egrec_blocks_transpose(int64_t n_nodes, int32_t n_hops, con
         const SortLane &l = s.lane[h];
         cudaStream_t ts = st;
         if (forked && ((n_hops - 1 - h) & 1)) ts = side->stream;
-        transpose_block(b.col, b.counts, b.cap_edges, l.edge_row, b.csc_col, b.csc_eid, b.csc_row, b.csc_ptr, sp, l, me < kChainEdges, ts);
+        transpose_block(b.col, b.counts, b.cap_edges, l.edge_row, b.csc_col, b.csc_eid, b.csc_row, b.csc_ptr, sp, l, me < kChainEdges,
+                        ts);
     }
     if (forked) side->join(st);
     return check_launch("blocks_transpose");

@@ -328,9 +328,9 @@ constexpr size_t seg_run_smem_bytes()
 // with the segment's first gathered row); 0 = neither, and those registers and branches disappear.
 // Four gathered rows per lane group are requested before any is added (latency hidden inside the thread: the streams of
 // a sampled block keep few warps resident).
-template <typename T, typename PtrT, int LPR, int CPL, bool kWeight, int kExtra>
+template <typename T, int LPR, int CPL, bool kWeight, int kExtra>
 __global__ void __launch_bounds__(kAggThreads)
-seg_run_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict__ ptr, const int32_t *__restrict__ idx,
+seg_run_kernel(const T *__restrict__ in, int64_t ld_in, const int32_t *__restrict__ ptr, const int32_t *__restrict__ idx,
                const int32_t *n_seg_dev, int64_t n_seg_host, const float *__restrict__ w, int run_len, int d,
                float *__restrict__ head2, float *__restrict__ tail2, int4 *__restrict__ win_info, int64_t cap_runs,
                const int32_t *__restrict__ seg_of, SegOut<T> o)
@@ -339,7 +339,6 @@ seg_run_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict__
     constexpr int U = CPL >= 4 ? 1 : 4 / CPL;
     constexpr int RB = kAggThreads / LPR;          // runs of this block = one window
     constexpr int ROW = LPR * CPL * E;             // floats per shared row (>= d)
-    constexpr int kFar = 1 << 30;
     extern __shared__ float4 seg_smem[];
     float *sh_head = reinterpret_cast<float *>(seg_smem);
     float *sh_tail = sh_head + RB * ROW;
@@ -367,7 +366,7 @@ seg_run_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict__
             if (ch < n_chunks) {
                 float r[E];
 #pragma unroll
-                for (int e = 0; e < E; ++e) r[e] = to_float<T>(from_float<T>(acc[q][e] * inv));   // inv = 1 without mean / scale
+                for (int e = 0; e < E; ++e) r[e] = to_float<T>(from_float<T>(acc[q][e] * inv));   // inv = 1 without scale
                 if (kExtra == 2 && o.mask) {
                     float m[E];
                     Chunk<T>::unpack(mrow[q], m);
@@ -390,8 +389,6 @@ seg_run_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict__
         int32_t ws = seg0[0];          // segment of the entry classified last
         const bool first_begins = k0 == 0 || seg0[-1] != ws;
         const bool last_ends = k0 + len == total || seg0[len] != seg0[len - 1];
-        // where the run's first segment begins (<= 0)
-        const int first_beg_rel = o.mean ? (int)max((int64_t)ptr[ws] - k0, (int64_t)-kFar) : 0;
 
         int32_t seg_n[U], id_n[U];
         bool start_n[U];
@@ -413,7 +410,6 @@ seg_run_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict__
         };
 
         int32_t cur_seg = -1;
-        int cur_beg_rel = 0;
         bool cur_begins = false;
         uint4 cur_mask[CPL];
         float acc[CPL][E];
@@ -424,10 +420,10 @@ seg_run_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict__
             for (int e = 0; e < E; ++e) acc[q][e] = 0.f;
         }
 
-        // closes the current segment, which ends at relative position end_rel, with the sum in acc
-        auto emit = [&](bool ended, int end_rel) {
+        // closes the current segment with the sum in acc
+        auto emit = [&](bool ended) {
             if (cur_begins && ended) {
-                const float inv = o.mean ? 1.0f / (float)(end_rel - cur_beg_rel) : (o.seg_scale ? o.seg_scale[cur_seg] : 1.0f);
+                const float inv = o.seg_scale ? o.seg_scale[cur_seg] : 1.0f;
                 finish(cur_seg, inv, acc, cur_mask);
             } else {
                 float *dst = (cur_begins ? sh_tail : sh_head) + rl * ROW;
@@ -480,10 +476,9 @@ seg_run_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict__
             for (int u = 0; u < U; ++u) {
                 if (r0 + u < len) {
                     if (start_c[u]) {
-                        if (cur_seg >= 0) emit(true, r0 + u);
+                        if (cur_seg >= 0) emit(true);
                         cur_seg = seg_c[u];
                         cur_begins = r0 + u != 0 || first_begins;
-                        cur_beg_rel = r0 + u != 0 ? r0 + u : first_beg_rel;
 #pragma unroll
                         for (int q = 0; q < CPL; ++q) {
                             if (kExtra) {
@@ -512,9 +507,9 @@ seg_run_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict__
                 }
             }
         }
-        emit(last_ends, len);
+        emit(last_ends);
     }
-    seg_join_window<T, PtrT, LPR, CPL, kExtra>(sh_head, sh_tail, sh_info, sh_win, rl, c, n_chunks, d, head_seg, head_ends, tail_seg, ptr,
+    seg_join_window<T, int32_t, LPR, CPL, kExtra>(sh_head, sh_tail, sh_info, sh_win, rl, c, n_chunks, d, head_seg, head_ends, tail_seg, ptr,
                                                head2, tail2, win_info, o);
 }
 
@@ -879,21 +874,22 @@ inline void launch_seg_final(const PtrT *ptr, const int32_t *n_seg_dev, int64_t 
     const int64_t empty_blocks = std::min<int64_t>(ceil_div(cap_seg > 0 ? cap_seg : 1, kAggThreads), 148 * 8);
     tap_begin(TAP_SEG_L3, st);
     note_launch();
-    launch_pdl(sc.chain && n_seg_dev && sc.cap_runs * run_len < kChainEdges, seg_final_kernel<T, PtrT>, dim3((unsigned)(window_blocks + empty_blocks)), dim3(kAggThreads), 0, st, ptr, n_seg_dev,
-               n_seg_host, run_len, sc.runs_per_window, d, (const float *)sc.head2, (const float *)sc.tail2, (const int4 *)sc.win_info,
-               sc.n_windows, window_blocks, o);
+    launch_pdl(sc.chain && n_seg_dev && sc.cap_runs * run_len < kChainEdges, seg_final_kernel<T, PtrT>,
+               dim3((unsigned)(window_blocks + empty_blocks)), dim3(kAggThreads), 0, st, ptr, n_seg_dev, n_seg_host, run_len,
+               sc.runs_per_window, d, (const float *)sc.head2, (const float *)sc.tail2, (const int4 *)sc.win_info, sc.n_windows,
+               window_blocks, o);
     tap_end(TAP_SEG_L3, st);
 }
 
-template <typename T, typename PtrT, int LPR, int CPL, bool kWeight>
-inline void launch_seg_reduce(const T *in, int64_t ld_in, const PtrT *ptr, const int32_t *idx, const int32_t *n_seg_dev,
+template <typename T, int LPR, int CPL, bool kWeight>
+inline void launch_seg_reduce(const T *in, int64_t ld_in, const int32_t *ptr, const int32_t *idx, const int32_t *n_seg_dev,
                               int64_t n_seg_host, int64_t cap_seg, const float *w, int run_len, int d,
                               const int32_t *seg_of, const SegScratch &sc, const SegOut<T> &o, cudaStream_t st)
 {
     constexpr size_t smem = seg_run_smem_bytes<LPR, CPL, Chunk<T>::kElems>();
     bool block_form = false;
-    if constexpr (CPL == 1 && !kWeight && sizeof(PtrT) == 4)
-        block_form = seg_of && n_seg_dev && o.self && !o.mean && !o.seg_scale && !seg_general_only();
+    if constexpr (CPL == 1 && !kWeight)
+        block_form = seg_of && n_seg_dev && o.self && !o.seg_scale && !seg_general_only();
     if (o.n_rhs > 1 && !(block_form && sc.chain_cnt)) {
         // the general kernels take one right-hand side per pass
         for (int r = 0; r < o.n_rhs; ++r) {
@@ -906,7 +902,7 @@ inline void launch_seg_reduce(const T *in, int64_t ld_in, const PtrT *ptr, const
             s1.tail2 = sc.tail2 + (size_t)r * sc.n_windows * d;
             s1.win_info = sc.win_info + (size_t)r * sc.n_windows;
             s1.chain_cnt = nullptr;
-            launch_seg_reduce<T, PtrT, LPR, CPL, kWeight>(in + r * o.rhs_in, ld_in, ptr, idx, n_seg_dev, n_seg_host, cap_seg, w,
+            launch_seg_reduce<T, LPR, CPL, kWeight>(in + r * o.rhs_in, ld_in, ptr, idx, n_seg_dev, n_seg_host, cap_seg, w,
                                                                      run_len, d, seg_of, s1, o1, st);
         }
         return;
@@ -915,17 +911,13 @@ inline void launch_seg_reduce(const T *in, int64_t ld_in, const PtrT *ptr, const
     tap_begin(TAP_SEG_L1, st);
     note_launch();
     const unsigned grid1 = (unsigned)sc.n_windows;
-    if constexpr (CPL == 1 && !kWeight && sizeof(PtrT) == 4) {
+    if constexpr (CPL == 1 && !kWeight) {
         // the transposed aggregation of a sampled block: the kernel written for that case
         if (block_form) {
-            block_form = true;
             const dim3 grid_b(grid1, (unsigned)(o.n_rhs > 1 && sc.chain_cnt ? o.n_rhs : 1));
-            if (o.mask)
-                launch_pdl(chain, seg_run_block_kernel<T, LPR, true>, grid_b, dim3(kAggThreads), smem, st, in, ld_in, ptr, idx, seg_of, n_seg_dev,
-                           run_len, d, sc.head2, sc.tail2, sc.win_info, sc.cap_runs, sc.chain_cnt, o);
-            else
-                launch_pdl(chain, seg_run_block_kernel<T, LPR, false>, grid_b, dim3(kAggThreads), smem, st, in, ld_in, ptr, idx, seg_of, n_seg_dev,
-                           run_len, d, sc.head2, sc.tail2, sc.win_info, sc.cap_runs, sc.chain_cnt, o);
+            auto kern = o.mask ? seg_run_block_kernel<T, LPR, true> : seg_run_block_kernel<T, LPR, false>;
+            launch_pdl(chain, kern, grid_b, dim3(kAggThreads), smem, st, in, ld_in, ptr, idx, seg_of, n_seg_dev, run_len, d, sc.head2,
+                       sc.tail2, sc.win_info, sc.cap_runs, sc.chain_cnt, o);
             if (sc.chain_cnt) {                   // chains, empty segments and padding were all done in that launch
                 tap_end(TAP_SEG_L1, st);
                 tap_begin(TAP_SEG_L3, st);        // (an armed tap of the second kernel reads zero)
@@ -934,22 +926,12 @@ inline void launch_seg_reduce(const T *in, int64_t ld_in, const PtrT *ptr, const
             }
         }
     }
-    if (block_form) {
-    } else if (o.mask) {
-        auto kern = seg_run_kernel<T, PtrT, LPR, CPL, kWeight, 2>;
+    if (!block_form) {
+        auto kern = o.mask ? seg_run_kernel<T, LPR, CPL, kWeight, 2>
+                    : o.self ? seg_run_kernel<T, LPR, CPL, kWeight, 1> : seg_run_kernel<T, LPR, CPL, kWeight, 0>;
         if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        launch_pdl(chain, kern, dim3(grid1), dim3(kAggThreads), smem, st, in, ld_in, ptr, idx, n_seg_dev, n_seg_host, w, run_len, d, sc.head2,
-                   sc.tail2, sc.win_info, sc.cap_runs, seg_of, o);
-    } else if (o.self) {
-        auto kern = seg_run_kernel<T, PtrT, LPR, CPL, kWeight, 1>;
-        if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        launch_pdl(chain, kern, dim3(grid1), dim3(kAggThreads), smem, st, in, ld_in, ptr, idx, n_seg_dev, n_seg_host, w, run_len, d, sc.head2,
-                   sc.tail2, sc.win_info, sc.cap_runs, seg_of, o);
-    } else {
-        auto kern = seg_run_kernel<T, PtrT, LPR, CPL, kWeight, 0>;
-        if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        launch_pdl(chain, kern, dim3(grid1), dim3(kAggThreads), smem, st, in, ld_in, ptr, idx, n_seg_dev, n_seg_host, w, run_len, d, sc.head2,
-                   sc.tail2, sc.win_info, sc.cap_runs, seg_of, o);
+        launch_pdl(chain, kern, dim3(grid1), dim3(kAggThreads), smem, st, in, ld_in, ptr, idx, n_seg_dev, n_seg_host, w, run_len, d,
+                   sc.head2, sc.tail2, sc.win_info, sc.cap_runs, seg_of, o);
     }
     tap_end(TAP_SEG_L1, st);
     launch_seg_final(ptr, n_seg_dev, n_seg_host, cap_seg, run_len, d, sc, o, st);
@@ -957,15 +939,15 @@ inline void launch_seg_reduce(const T *in, int64_t ld_in, const PtrT *ptr, const
 
 // Returns false (nothing enqueued) when no kernel is built for the row width; rows of up to 4096 bytes (kMaxDim fp32
 // values) are covered, so callers that checked dim <= kMaxDim never see it.
-template <typename T, typename PtrT, bool kWeight>
-inline bool dispatch_seg_reduce(const T *in, int64_t ld_in, const PtrT *ptr, const int32_t *idx, const int32_t *n_seg_dev,
+template <typename T, bool kWeight>
+inline bool dispatch_seg_reduce(const T *in, int64_t ld_in, const int32_t *ptr, const int32_t *idx, const int32_t *n_seg_dev,
                                 int64_t n_seg_host, int64_t cap_seg, const float *w, int run_len, int d, int32_t dtype,
                                 const int32_t *seg_of, const SegScratch &sc, const SegOut<T> &o, cudaStream_t st)
 {
     const RowShape rs = row_shape(d, dtype);
 #define E2E_CASE(L, C)                                                                                                \
     if (rs.lpr == L && rs.cpl == C) {                                                                                 \
-        launch_seg_reduce<T, PtrT, L, C, kWeight>(in, ld_in, ptr, idx, n_seg_dev, n_seg_host, cap_seg, w, run_len, \
+        launch_seg_reduce<T, L, C, kWeight>(in, ld_in, ptr, idx, n_seg_dev, n_seg_host, cap_seg, w, run_len, \
                                                          d, seg_of, sc, o, st);                                       \
         return true;                                                                                                  \
     }
