@@ -6,8 +6,9 @@
 // the kernel that joins them are those of segreduce.cuh; a window is cut into one stretch of consecutive entries per
 // warp of the block.
 //
-// What bounds it: the instructions per gathered row and per segment, then latency; DRAM and L2 are at 10 % (B200, 128-byte
-// rows).  With one lane group per run, 32 / LPR runs per warp each with its own segment ends, a 128-byte row took 22 warp
+// What bounds it: latency, of the gathered rows first and then of the barrier before the join (stalls per issue 4.6 and 3.4;
+// issue slots 57 % busy, L1 at 34 %, L2 and DRAM at 10 %: B200, 128-byte rows).  What it could be sped up by so far were
+// instructions per gathered row and per segment.  With one lane group per run, 32 / LPR runs per warp each with its own segment ends, a 128-byte row took 22 warp
 // instructions, most of them bookkeeping that the warp executes for all of its groups' different positions.  Here the
 // offsets come 32 segments at a time, one lane each, and the segments are handled by their length:
 //   - longer ones by the whole warp: 32 entry ids in one coalesced load (the next 32 and the entry weights on their way),
