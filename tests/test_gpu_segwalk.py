@@ -60,6 +60,7 @@ def test_walk(lengths, dtype, d):
 def test_as_many_segments_as_the_entry_point_takes():
     """2^31 - 1 segments, with entries in the first and the last ones: windows of 32 segments that begin among the last and
     reach beyond 2^31.  52 GB of offsets and rows."""
+    torch.cuda.empty_cache()
     if torch.cuda.mem_get_info()[0] < 70 << 30:
         pytest.skip("needs 70 GB of device memory")
     n, d = (1 << 31) - 1, 4
