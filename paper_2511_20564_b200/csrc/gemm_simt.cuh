@@ -11,15 +11,16 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 
 #include "common.cuh"
 
 namespace e2egrec {
 
-// At the sizes of a batch the time is the K loop's chain of loads, not its arithmetic: the next 64 x 32 tiles are loaded
-// into registers (four values at a time where rows are aligned) while the current ones are multiplied out of shared memory,
-// two buffers, one barrier per step.  Loading, storing and multiplying in turn with steps of 16 took 1.7 us a step; B200,
-// 10 k x 72 x 200 fp32 29 -> 22 us, 777 x 72 x 144 16 -> 12.
+// gemm_simt_kernel, for bf16 operands (fp32 ones: gemm_async_kernel below).  At the sizes of a batch the time is the K loop's
+// chain of loads, not its arithmetic: the next 64 x 32 tiles are loaded into registers (four values at a time where rows are
+// aligned) while the current ones are multiplied out of shared memory, two buffers, one barrier per step.  Loading, storing and
+// multiplying in turn with steps of 16 took 1.7 us a step.
 constexpr int kGemmBM = 64, kGemmBN = 64, kGemmBK = 32, kGemmThreads = 256;
 
 // four values from p on, `n` of them there
@@ -166,12 +167,167 @@ gemm_simt_kernel(const T *A, int64_t lda, const T *B, int64_t ldb, int64_t M_hos
         }
 }
 
+// The same product of fp32 operands, for batches whose few tiles leave most of an SM idle: the tiles are copied to shared memory
+// asynchronously, as they lie in memory (rows of k, or lines of k), kGemmStages - 1 K steps ahead, and two groups of 256
+// threads take half of every K step each; their sums are added at the end.  What bounds it is latency at 16 warps per SM.
+// B200, fp32 step of 777 seeds at fanouts 25, 15, 100 and 72 values, its six products together (us) and the step: loads through
+// registers one step ahead, one group 88, 163; copies, one group 74, 154; two groups 144; four groups (64 registers, spills) 166;
+// 128 threads of 8 x 4 values instead of 256 of 4 x 4 164.  No chain of additions is longer than in gemm_simt_kernel.
+constexpr int kGemmStages = 4, kGemmGroups = 2, kAsyncThreads = kGemmThreads * kGemmGroups;
+template <bool KM> struct AsyncTile {
+    static constexpr int kLd = KM ? 64 + 4 : kGemmBK + 4;        // floats per line: 64 values of a k, or kGemmBK of a row
+    static constexpr int kFloats = (KM ? kGemmBK : 64) * kLd;
+    // requests the tile of rows r0 .. r0 + 63 and k0 .. k0 + kGemmBK - 1; values beyond `rows` and `ke` read zero
+    static __device__ __forceinline__ void request(float *s, const float *__restrict__ p, int64_t ld, int64_t rows, int64_t r0, int64_t k0,
+                                                   int64_t ke, bool vec)
+    {
+#pragma unroll
+        for (int t = 0; t < (512 + kAsyncThreads - 1) / kAsyncThreads; ++t) {
+            const int id = threadIdx.x + t * kAsyncThreads;
+            if (512 % kAsyncThreads && id >= 512) break;
+            const int line = KM ? id >> 4 : id >> 3, col = (KM ? id & 15 : id & 7) * 4;
+            const int64_t l = (KM ? k0 : r0) + line, c = (KM ? r0 : k0) + col, l_end = KM ? ke : rows, c_end = KM ? rows : ke;
+            const int n = l < l_end ? (int)max((int64_t)0, min((int64_t)4, c_end - c)) : 0;
+            const float *src = n > 0 ? p + l * ld + c : p;
+            const uint32_t dst = (uint32_t)__cvta_generic_to_shared(s + line * kLd + col);
+            if (vec) {
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n * 4) : "memory");
+            } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + 4 * e), "l"(e < n ? src + e : p), "r"(e < n ? 4 : 0)
+                                 : "memory");
+            }
+        }
+    }
+};
+template <bool A_KM, bool B_KN> constexpr size_t gemm_async_smem() { return (size_t)kGemmStages * (AsyncTile<A_KM>::kFloats + AsyncTile<B_KN>::kFloats) * 4; }
+
+template <bool A_KM, bool B_KN, class Epi>
+__global__ void __launch_bounds__(kAsyncThreads)
+gemm_async_kernel(const float *A, int64_t lda, const float *B, int64_t ldb, int64_t M_host, int N, int64_t K_host, const int32_t *m_dev,
+                  const int32_t *k_dev, Epi epi)
+{
+    using TA = AsyncTile<A_KM>;
+    using TB = AsyncTile<B_KN>;
+    extern __shared__ __align__(16) float gemm_sm[];
+    pdl_wait();
+    const int64_t M = m_dev ? min((int64_t)__ldcg(m_dev), M_host) : M_host;
+    const int64_t K = k_dev ? min((int64_t)__ldcg(k_dev), K_host) : K_host;
+    const int64_t m0 = (int64_t)blockIdx.x * kGemmBM;
+    const int n0 = blockIdx.y * kGemmBN;
+    if (m0 >= M) return;
+    const int64_t k_per = ceil_div(ceil_div(K, (int64_t)gridDim.z), kGemmBK) * kGemmBK;
+    const int64_t kb = (int64_t)blockIdx.z * k_per;
+    const int64_t ke = min(K, kb + k_per);
+    const int steps = kb < ke ? (int)ceil_div(ke - kb, kGemmBK) : 0;
+    const int tx = threadIdx.x & 15, ty = (threadIdx.x & (kGemmThreads - 1)) >> 4, g = threadIdx.x / kGemmThreads;
+    constexpr bool kFold = A_KM && B_KN;                         // as in gemm_simt_kernel
+    float acc[4][4], total[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            acc[i][j] = 0.f;
+            if (kFold) total[i][j] = 0.f;
+        }
+    const bool vec_a = lda % 4 == 0 && reinterpret_cast<uintptr_t>(A) % 16 == 0, vec_b = ldb % 4 == 0 && reinterpret_cast<uintptr_t>(B) % 16 == 0;
+    auto request = [&](int step) {
+        if (step < steps) {
+            float *s = gemm_sm + (step % kGemmStages) * (TA::kFloats + TB::kFloats);
+            TA::request(s, A, lda, M, m0, kb + (int64_t)step * kGemmBK, ke, vec_a);
+            TB::request(s + TA::kFloats, B, ldb, N, n0, kb + (int64_t)step * kGemmBK, ke, vec_b);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+#pragma unroll
+    for (int i = 0; i < kGemmStages - 1; ++i) request(i);
+    for (int step = 0; step < steps; ++step) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(kGemmStages - 2) : "memory");
+        __syncthreads();                                         // step's tiles are there, and everybody has left the buffer that is filled next
+        request(step + kGemmStages - 1);
+        const float *sa = gemm_sm + (step % kGemmStages) * (TA::kFloats + TB::kFloats), *sb = sa + TA::kFloats;
+#pragma unroll
+        for (int q0 = 0; q0 < kGemmBK / 4 / kGemmGroups; ++q0) {
+            const int q = g * (kGemmBK / 4 / kGemmGroups) + q0;
+            // rows ty * 4 + i; columns tx + 16 j (rows of k: 16 lines side by side, no bank twice) or tx * 4 + j (lines of k)
+            float a[4][4], b[4][4];                              // [k][row], [k][column]
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float4 v = *reinterpret_cast<const float4 *>(A_KM ? sa + (4 * q + i) * TA::kLd + ty * 4 : sa + (ty * 4 + i) * TA::kLd + 4 * q);
+                const float x[4] = {v.x, v.y, v.z, v.w};
+                const float4 w = *reinterpret_cast<const float4 *>(B_KN ? sb + (4 * q + i) * TB::kLd + tx * 4 : sb + (tx + 16 * i) * TB::kLd + 4 * q);
+                const float y[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    a[A_KM ? i : e][A_KM ? e : i] = x[e];
+                    b[B_KN ? i : e][B_KN ? e : i] = y[e];
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[k][i], b[k][j], acc[i][j]);
+        }
+        if (kFold) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    total[i][j] += acc[i][j];
+                    acc[i][j] = 0.f;
+                }
+        }
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    // the groups' sums in the order of the groups
+    float (*sum)[4] = kFold ? total : acc;
+    __syncthreads();
+    if (g > 0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            *reinterpret_cast<float4 *>(gemm_sm + (((g - 1) * 4 + i) * kGemmThreads + (threadIdx.x & (kGemmThreads - 1))) * 4) =
+                make_float4(sum[i][0], sum[i][1], sum[i][2], sum[i][3]);
+    }
+    __syncthreads();
+    if (g > 0) return;
+#pragma unroll
+    for (int o = 0; o < kGemmGroups - 1; ++o)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float4 v = *reinterpret_cast<const float4 *>(gemm_sm + ((o * 4 + i) * kGemmThreads + threadIdx.x) * 4);
+            sum[i][0] += v.x; sum[i][1] += v.y; sum[i][2] += v.z; sum[i][3] += v.w;
+        }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int64_t m = m0 + ty * 4 + i;
+            const int n = n0 + (B_KN ? tx * 4 + j : tx + 16 * j);
+            if (m < M && n < N) epi(m, n, sum[i][j], blockIdx.z);
+        }
+}
+
 template <typename T, bool A_KM, bool B_KN, class Epi>
 inline void launch_gemm_simt(bool chain, dim3 grid, cudaStream_t st, const T *A, int64_t lda, const T *B, int64_t ldb, int64_t M, int N,
                              int64_t K, const int32_t *m_dev, const int32_t *k_dev, const Epi &epi)
 {
     note_launch();
-    launch_pdl(chain, gemm_simt_kernel<T, A_KM, B_KN, Epi>, grid, dim3(kGemmThreads), 0, st, A, lda, B, ldb, M, N, K, m_dev, k_dev, epi);
+    if constexpr (sizeof(T) == 4) {
+        constexpr size_t smem = gemm_async_smem<A_KM, B_KN>();
+        static std::atomic<bool> set[64] = {};                   // per device; two threads may both raise the limit
+        int dev = 0;
+        cudaGetDevice(&dev);
+        if (dev < 0 || dev >= 64 || !set[dev].load(std::memory_order_relaxed)) {
+            cudaFuncSetAttribute(gemm_async_kernel<A_KM, B_KN, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (dev >= 0 && dev < 64) set[dev].store(true, std::memory_order_relaxed);
+        }
+        launch_pdl(chain, gemm_async_kernel<A_KM, B_KN, Epi>, grid, dim3(kAsyncThreads), smem, st, A, lda, B, ldb, M, N, K, m_dev, k_dev, epi);
+    } else {
+        launch_pdl(chain, gemm_simt_kernel<T, A_KM, B_KN, Epi>, grid, dim3(kGemmThreads), 0, st, A, lda, B, ldb, M, N, K, m_dev, k_dev, epi);
+    }
 }
 
 // Splits over `rows` (a capacity) of an m x n weight gradient on this kernel, at most `most` (148): two blocks per SM over all
