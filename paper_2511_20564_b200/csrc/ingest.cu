@@ -5,7 +5,7 @@
 // The CSR is the (col, row) pairs sorted by column and then, key and value exchanged, by row: the other id travels as the
 // value, so nothing is gathered between the sorts (entries equal in both ids need no order).  The transpose sorts
 // (col, position) and looks up the row of every position afterwards.  B200, 10^7 interactions (2 * 10^7 entries, 500 k nodes),
-// CSR and CSC together: 3.23 -> 1.52 ms.
+// CSR and CSC together: 1.51 -> 1.19 ms.
 #include <algorithm>
 
 #include "radix.cuh"
@@ -16,13 +16,18 @@ namespace {
 
 struct IngestScratch {
     int32_t *counts;                 // int32[4]: CNT_STATUS is the status word of the run
-    int32_t *a, *k0, *v0, *k1, *v1;  // arrays of m
+    int32_t *a;                      // [m]
+    uint2 *pair[2];                  // [m]
     SortState sort[2];
     char *zero;                      // the part that has to be zero beforehand
     size_t zero_bytes, bytes;
 };
 
-IngestScratch carve_ingest(int64_t m, void *base)
+SortPlan plan_for(int64_t key_range) { return sort_plan((int32_t)std::min<int64_t>(std::max<int64_t>(key_range, 2), 0x7fffffff)); }
+
+// n_sorts sorts of m entries by `sp`: digit counts and scan state of what these will use lie together, to be zeroed at once
+// (for the larger tiles and both sorts whatever the call: 80 MB and 14 us at 2 * 10^7 entries).
+IngestScratch carve_ingest(int64_t m, const SortPlan &sp, int n_sorts, void *base)
 {
     IngestScratch s{};
     size_t off = 0;
@@ -33,14 +38,16 @@ IngestScratch carve_ingest(int64_t m, void *base)
     };
     const size_t mm = (size_t)(m > 0 ? m : 1);
     s.counts = (int32_t *)take(256);
-    for (int32_t **p : {&s.a, &s.k0, &s.v0, &s.k1, &s.v1}) *p = (int32_t *)take(mm * 4);
-    const int64_t tiles = ceil_div((int64_t)mm, kSortTile);
+    s.a = (int32_t *)take(mm * 4);
+    for (uint2 *&p : s.pair) p = (uint2 *)take(mm * 8);
+    const int64_t tiles = ceil_div((int64_t)mm, (int64_t)mm >= kSortWide ? kSortWideTile : kSortTile);
     const size_t begin = off;
     s.zero = base ? static_cast<char *>(base) + off : nullptr;
-    for (SortState &ss : s.sort) {
+    for (int i = 0; i < n_sorts; ++i) {
+        SortState &ss = s.sort[i];
         ss.ghist = (unsigned *)take(kSortCountWords * sizeof(unsigned));
         ss.tiles = tiles;
-        ss.state = (unsigned *)take(sort_state_bytes(tiles));
+        ss.state = (unsigned *)take(sizeof(unsigned) * (size_t)sp.passes * (size_t)tiles << sp.bits);
     }
     s.zero_bytes = off - begin;
     s.bytes = off;
@@ -56,69 +63,113 @@ __global__ void ingest_begin_kernel(int32_t *counts, int32_t m)
 }
 
 // Digit counts of one or two id arrays for every pass of their sorts.  Ids outside [0, n) are flagged here and count as
-// 0, which the first pass of a sort makes of them.
-__global__ void __launch_bounds__(256)
+// 0, which the first pass of a sort makes of them.  One block of 1024 threads per SM, and two copies of the counts, for even
+// and odd lanes: what the blocks add to the global counts at their ends (4096 each) and the lanes of a warp that meet in a
+// hub's digits were what it cost.
+constexpr int kHistThreads = 1024;
+__global__ void __launch_bounds__(kHistThreads)
 id_hist_kernel(const int32_t *__restrict__ ids0, const int32_t *__restrict__ ids1, int64_t m, int64_t n, int bits, int passes,
                unsigned *__restrict__ ghist0, unsigned *__restrict__ ghist1, int32_t *counts)
 {
-    extern __shared__ unsigned hist_sm[];                        // [arrays][passes][1 << bits]
+    extern __shared__ unsigned hist_sm[];                        // [2][arrays][passes][1 << bits]
     const int R = 1 << bits, per = passes * R;
     const int all = ids1 ? 2 * per : per;
-    for (int d = threadIdx.x; d < all; d += 256) hist_sm[d] = 0;
+    for (int d = threadIdx.x; d < 2 * all; d += kHistThreads) hist_sm[d] = 0;
     __syncthreads();
+    unsigned *h = hist_sm + (threadIdx.x & 1) * all;
     bool bad = false;
-    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < m; i += (int64_t)gridDim.x * 256) {
-        uint32_t v0 = (uint32_t)ids0[i], v1 = ids1 ? (uint32_t)ids1[i] : 0u;
-        if (v0 >= (uint64_t)n) { bad = true; v0 = 0; }
-        if (v1 >= (uint64_t)n) { bad = true; v1 = 0; }
-        for (int p = 0; p < passes; ++p) {
-            atomicAdd(&hist_sm[p * R + ((v0 >> (p * bits)) & (R - 1))], 1u);
-            if (ids1) atomicAdd(&hist_sm[per + p * R + ((v1 >> (p * bits)) & (R - 1))], 1u);
+    const int64_t step = (int64_t)gridDim.x * kHistThreads;
+    auto count = [&](uint32_t v, unsigned *hh) {
+        if (v >= (uint64_t)n) { bad = true; v = 0; }
+        for (int p = 0; p < passes; ++p) atomicAdd(&hh[p * R + ((v >> (p * bits)) & (R - 1))], 1u);
+    };
+    constexpr int U = 4;
+    int64_t i = (int64_t)blockIdx.x * kHistThreads + threadIdx.x;
+    for (; i + (U - 1) * step < m; i += U * step) {
+        uint32_t v0[U], v1[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            v0[u] = (uint32_t)__ldg(ids0 + i + u * step);
+            v1[u] = ids1 ? (uint32_t)__ldg(ids1 + i + u * step) : 0u;
         }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            count(v0[u], h);
+            if (ids1) count(v1[u], h + per);
+        }
+    }
+    for (; i < m; i += step) {
+        count((uint32_t)ids0[i], h);
+        if (ids1) count((uint32_t)ids1[i], h + per);
     }
     if (bad) atomicOr((unsigned *)&counts[CNT_STATUS], E2EGREC_DEV_RANGE);
     __syncthreads();
-    for (int d = threadIdx.x; d < all; d += 256) {
-        if (!hist_sm[d]) continue;
+    for (int d = threadIdx.x; d < all; d += kHistThreads) {
+        const unsigned c = hist_sm[d] + hist_sm[all + d];
+        if (!c) continue;
         const int e = d % per;
-        atomicAdd(&(d < per ? ghist0 : ghist1)[(e / R) * kMaxRadix + e % R], hist_sm[d]);
+        atomicAdd(&(d < per ? ghist0 : ghist1)[(e / R) * kMaxRadix + e % R], c);
     }
 }
 
-// row_of[e] = row of CSR position e.  A warp owns 1024 consecutive positions: it finds its first row by a search over the
-// offsets and then goes through them 32 rows at a time, lane i holding the end of row base + i; a position's row is the
-// number of ends at or before it, found by bisection across the lanes.
+// row_of[e] = row of CSR position e.  A warp owns kSpan consecutive positions: it finds its first row by a search over the
+// offsets, goes through the rows 32 at a time and notes every row with entries where it begins, in shared memory; a running
+// maximum over the span (each lane over 32 positions, then over the lanes) carries the rows on.  (A bisection across the lanes
+// for every 32 positions, as before, was 1100 instructions a span where this is 300: 2 * 10^7 positions 52 -> 26 us.)
 __global__ void __launch_bounds__(256)
 expand_rows_kernel(const int64_t *__restrict__ indptr, int64_t n_rows, int64_t m, int32_t *__restrict__ row_of)
 {
-    constexpr int kSpan = 1024;
+    constexpr int kSpan = 1024, kPad = 33;                       // position p lies at (p / 32) * kPad + p % 32
+    __shared__ int32_t sm[8][32 * kPad];
     const int lane = threadIdx.x & 31;
+    int32_t *mark = sm[threadIdx.x >> 5];
     const int64_t k0 = (((int64_t)blockIdx.x * 256 + threadIdx.x) >> 5) * kSpan;
     if (k0 >= m) return;
     const int len = (int)min((int64_t)kSpan, m - k0);
     int64_t base = warp_seg_containing(indptr, n_rows, k0);
-    auto load_ends = [&](int64_t b) -> int { return b + lane < n_rows ? (int)min(indptr[b + lane + 1] - k0, (int64_t)kSpan) : kSpan; };
-    int ends = load_ends(base);
-    int quiet = 0;
-    for (int e0 = 0; e0 < len;) {
-        const int last = __shfl_sync(0xffffffffu, ends, 31);     // positions before it belong to this window of rows
-        if (last > e0) {
-            quiet = 0;
-            const int e = e0 + lane;
-            int r = 0;
+    const int32_t first = (int32_t)max(min(base, n_rows - 1), (int64_t)0);
 #pragma unroll
-            for (int step = 16; step > 0; step >>= 1)
-                if (__shfl_sync(0xffffffffu, ends, r + step - 1) <= e) r += step;
-            if (e < last && e < len) row_of[k0 + e] = (int32_t)max(min(base + r, n_rows - 1), (int64_t)0);
-            e0 = min(e0 + 32, last);
-            if (e0 < last) continue;
-            if (e0 >= len) break;
-        } else {
-            ++quiet;
+    for (int c = 0; c < 32; ++c) mark[c * kPad + lane] = 0;
+    __syncwarp();
+    auto load_beg = [&](int64_t b) -> int { return b + lane <= n_rows ? (int)max(min(indptr[b + lane] - k0, (int64_t)kSpan), (int64_t)0) : kSpan; };
+    int beg = load_beg(base);
+    for (int quiet = 0;;) {
+        const int beg_n = load_beg(base + 32);                   // the window after this one, on its way
+        const int after = __shfl_sync(0xffffffffu, beg_n, 0);    // where the row behind the window begins
+        int end = __shfl_down_sync(0xffffffffu, beg, 1);
+        if (lane == 31) end = after;
+        if (beg > 0 && beg < end && beg < len) mark[(beg >> 5) * kPad + (beg & 31)] = (int32_t)(base + lane);
+        if (after >= len || base + 32 >= n_rows) break;
+        quiet = __any_sync(0xffffffffu, beg < end) ? 0 : quiet + 1;
+        if (quiet < kQuietWindows) {
+            base += 32;
+            beg = beg_n;
+        } else {                                                 // a long stretch of empty rows
+            base = window_found(base, warp_seg_containing(indptr, n_rows, k0 + after));
+            beg = load_beg(base);
+            quiet = 0;
         }
-        base = quiet < kQuietWindows ? base + 32 : window_found(base, warp_seg_containing(indptr, n_rows, k0 + e0));
-        ends = load_ends(base);
     }
+    __syncwarp();
+    int32_t run = 0;
+#pragma unroll
+    for (int j = 0; j < 32; ++j) run = max(run, mark[lane * kPad + j]);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t t = __shfl_up_sync(0xffffffffu, run, o);
+        if (lane >= o) run = max(run, t);
+    }
+    run = __shfl_up_sync(0xffffffffu, run, 1);
+    run = lane > 0 ? max(run, first) : first;
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+        run = max(run, mark[lane * kPad + j]);
+        mark[lane * kPad + j] = run;
+    }
+    __syncwarp();
+#pragma unroll
+    for (int c = 0; c < 32; ++c)
+        if (c * 32 + lane < len) row_of[k0 + c * 32 + lane] = mark[c * kPad + lane];
 }
 
 // csc_row[k] = row_of[csc_eid[k]], four scattered reads per thread in flight.  In a launch of its own row_of stays in L2
@@ -158,15 +209,13 @@ __global__ void offsets_kernel(const int32_t *__restrict__ sorted, int64_t m, in
 
 unsigned wide_grid(int64_t n) { return (unsigned)std::min<int64_t>(ceil_div(n > 0 ? n : 1, 256), 148 * 16); }
 
-SortPlan plan_for(int64_t key_range) { return sort_plan((int32_t)std::min<int64_t>(std::max<int64_t>(key_range, 2), 0x7fffffff)); }
-
 void id_hist(const int32_t *ids0, const int32_t *ids1, int64_t m, int64_t n, const SortPlan &sp, IngestScratch &s, cudaStream_t st)
 {
     cudaMemsetAsync(s.zero, 0, s.zero_bytes, st);
-    const size_t smem = (size_t)(ids1 ? 2 : 1) * sp.passes * (1 << sp.bits) * sizeof(unsigned);
+    const size_t smem = (size_t)(ids1 ? 4 : 2) * sp.passes * (1 << sp.bits) * sizeof(unsigned);      // at most 32 KB
     note_launch();
-    id_hist_kernel<<<(unsigned)std::min<int64_t>(ceil_div(m, 2048), 148 * 8), 256, smem, st>>>(ids0, ids1, m, n, sp.bits, sp.passes,
-                                                                                             s.sort[0].ghist, s.sort[1].ghist, s.counts);
+    id_hist_kernel<<<(unsigned)std::min<int64_t>(ceil_div(m, 4 * kHistThreads), 148), kHistThreads, smem, st>>>(
+        ids0, ids1, m, n, sp.bits, sp.passes, s.sort[0].ghist, s.sort[1].ghist, s.counts);
 }
 
 }  // namespace
@@ -181,7 +230,8 @@ extern "C" int32_t e2egrec_graph_from_coo(int64_t n_nodes, int64_t n_edges, cons
     if (!ws_bytes) return E2EGREC_ERR_NULL;
     if (n_nodes < 0 || n_edges < 0) return E2EGREC_ERR_ARG;
     if (n_nodes >= (1ll << 31) || n_edges >= (1ll << 31) - 1) return E2EGREC_ERR_UNSUPPORTED;
-    IngestScratch s = carve_ingest(n_edges, ws);
+    const SortPlan sp = plan_for(n_nodes);
+    IngestScratch s = carve_ingest(n_edges, sp, 2, ws);
     if (!ws) { *ws_bytes = s.bytes; return E2EGREC_OK; }
     if (*ws_bytes < s.bytes) { *ws_bytes = s.bytes; return E2EGREC_ERR_WORKSPACE; }
     if (reinterpret_cast<uintptr_t>(ws) % 256) return E2EGREC_ERR_ALIGN;
@@ -191,23 +241,28 @@ extern "C" int32_t e2egrec_graph_from_coo(int64_t n_nodes, int64_t n_edges, cons
     note_launch();
     ingest_begin_kernel<<<1, 1, 0, st>>>(s.counts, (int32_t)m);
     if (m > 0) {
-        const SortPlan sp = plan_for(n_nodes);
         const int32_t clamp = (int32_t)std::max<int64_t>(n_nodes, 1);
         id_hist(col, row, m, n_nodes, sp, s, st);
         // (col, row) by column, then (row, col) by row
-        const int32_t *k = col, *v = row;
-        int32_t *ka = s.k0, *va = s.v0, *kb = s.k1, *vb = s.v1;
+        SortIn in{col, row, nullptr, false, kRankAny};           // equal pairs are alike: the first pass needs no order
         for (int q = 0; q < 2 * sp.passes; ++q) {
             const int sort = q / sp.passes, pass = q % sp.passes;
-            if (q == sp.passes) std::swap(k, v);
             const bool last = q == 2 * sp.passes - 1;
-            sort_pass<int32_t>(sp, k, v, nullptr, m, q == 0 ? clamp : 0, q == 0 ? clamp : 0, pass, s.sort[sort], false, last ? s.a : ka,
-                               last ? indices : va, SortMap{}, &s.counts[CNT_STATUS], st);
-            k = ka;
-            v = va;
-            std::swap(ka, kb);
-            std::swap(va, vb);
-        }                                                        // s.a = rows sorted
+            if (q == sp.passes) {
+                in.swap = true;
+                in.rank = kRankSpread;
+            }
+            SortOut<int32_t> out{};
+            if (last) {
+                out.keys = s.a;                                  // the rows in order
+                out.vals = indices;
+            } else {
+                out.pairs = s.pair[q & 1];
+            }
+            sort_pass<int32_t>(sp, in, nullptr, m, q == 0 ? clamp : 0, q == 0 ? clamp : 0, pass, s.sort[sort], false, out,
+                               &s.counts[CNT_STATUS], st);
+            in = SortIn{nullptr, nullptr, s.pair[q & 1], false, kRankMatch};
+        }
     }
     note_launch();
     offsets_kernel<<<wide_grid(n_nodes + 1), 256, 0, st>>>(s.a, m, n_nodes, s.counts, indptr);
@@ -221,37 +276,36 @@ extern "C" int32_t e2egrec_csr_transpose(const e2egrec_csr *csr, int64_t n_cols,
     if (!ws_bytes || !csr) return E2EGREC_ERR_NULL;
     if (csr->n_nodes < 0 || csr->n_edges < 0 || n_cols < 0) return E2EGREC_ERR_ARG;
     if (csr->n_nodes >= (1ll << 31) || n_cols >= (1ll << 31) || csr->n_edges >= (1ll << 31) - 1) return E2EGREC_ERR_UNSUPPORTED;
-    IngestScratch s = carve_ingest(csr->n_edges, ws);
+    const SortPlan sp = plan_for(n_cols);
+    IngestScratch s = carve_ingest(csr->n_edges, sp, 1, ws);
     if (!ws) { *ws_bytes = s.bytes; return E2EGREC_OK; }
     if (*ws_bytes < s.bytes) { *ws_bytes = s.bytes; return E2EGREC_ERR_WORKSPACE; }
     if (reinterpret_cast<uintptr_t>(ws) % 256) return E2EGREC_ERR_ALIGN;
     if (!csr->indptr || !csc_ptr || (csr->n_edges > 0 && (!csr->indices || !csc_row || !csc_eid))) return E2EGREC_ERR_NULL;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int64_t m = csr->n_edges;
-    const int32_t *sorted = s.k0;
+    const int32_t *sorted = s.a;
     note_launch();
     ingest_begin_kernel<<<1, 1, 0, st>>>(s.counts, (int32_t)m);
     if (m > 0) {
-        const SortPlan sp = plan_for(n_cols);
         id_hist(csr->indices, nullptr, m, n_cols, sp, s, st);
         note_launch();
         expand_rows_kernel<<<(unsigned)ceil_div(m, 8 * 1024), 256, 0, st>>>(csr->indptr, csr->n_nodes, m, s.a);
-        const int32_t *k = csr->indices, *v = nullptr;           // value = CSR position
-        int32_t *ka = s.k0, *va = s.v0, *kb = s.k1, *vb = s.v1;
+        SortIn in{csr->indices, nullptr, nullptr, false, kRankMatch};        // value = CSR position
         for (int q = 0; q < sp.passes; ++q) {
             const int32_t clamp = q == 0 ? (int32_t)std::max<int64_t>(n_cols, 1) : 0;
-            if (q == sp.passes - 1)
-                sort_pass<int64_t>(sp, k, v, nullptr, m, clamp, (int32_t)m, q, s.sort[0], false, ka, csc_eid, SortMap{},
-                                   &s.counts[CNT_STATUS], st);
-            else
-                sort_pass<int32_t>(sp, k, v, nullptr, m, clamp, (int32_t)m, q, s.sort[0], false, ka, va, SortMap{},
-                                   &s.counts[CNT_STATUS], st);
-            k = ka;
-            v = va;
-            std::swap(ka, kb);
-            std::swap(va, vb);
+            if (q == sp.passes - 1) {
+                SortOut<int64_t> out{};
+                sorted = out.keys = reinterpret_cast<int32_t *>(s.pair[q & 1]);          // the columns in order
+                out.vals = csc_eid;
+                sort_pass<int64_t>(sp, in, nullptr, m, clamp, (int32_t)m, q, s.sort[0], false, out, &s.counts[CNT_STATUS], st);
+            } else {
+                SortOut<int32_t> out{};
+                out.pairs = s.pair[q & 1];
+                sort_pass<int32_t>(sp, in, nullptr, m, clamp, (int32_t)m, q, s.sort[0], false, out, &s.counts[CNT_STATUS], st);
+                in = SortIn{nullptr, nullptr, s.pair[q & 1], false, kRankMatch};
+            }
         }
-        sorted = k;                                              // the columns in order
         note_launch();
         rows_of_kernel<<<(unsigned)std::min<int64_t>(ceil_div(m, 1024), 148 * 16), 256, 0, st>>>(csc_eid, s.a, m, csc_row);
     }

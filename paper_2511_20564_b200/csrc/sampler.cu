@@ -61,7 +61,7 @@ static inline int dst_tile(int32_t cap_dst, int32_t fanout)
 // transposition of hop h can run beside the sampling of hop h+1.
 struct SortLane {
     int32_t  *edge_row;    // [max cap_edges]   destination of each block entry
-    int32_t  *key, *val;   // [max cap_edges]   the passes alternate between these and the block's arrays
+    uint2    *pair;        // [max cap_edges]   the passes alternate between these and the block's arrays
     SortState sort;        // counts and tickets zeroed before relabel, which zeroes the live tiles' scan state
 };
 
@@ -104,8 +104,7 @@ static SamplerScratch carve(int64_t n_nodes, int64_t max_dst, int64_t max_src, i
     for (int h = 0; h < kMaxHops; ++h) {
         SortLane &l = s.lane[h];
         l.edge_row = (int32_t *)take(sizeof(int32_t) * (size_t)(max_edges + 1));
-        l.key = (int32_t *)take(sizeof(int32_t) * (size_t)(max_edges + 1));
-        l.val = (int32_t *)take(sizeof(int32_t) * (size_t)(max_edges + 1));
+        l.pair = (uint2 *)take(sizeof(uint2) * (size_t)(max_edges + 1));
         l.sort.ghist = s.ghist[h];
         l.sort.tiles = sort_tiles;
         l.sort.state = (unsigned *)take(sort_state_bytes(sort_tiles));
@@ -528,14 +527,22 @@ static void transpose_block(const int32_t *col, int32_t *counts, int32_t cap_edg
                             const SortLane &l, bool chain, cudaStream_t st, const int32_t *release_nodes = nullptr,
                             int32_t *local_id = nullptr)
 {
-    const int32_t *k = col, *v = nullptr;
+    SortIn in{col, nullptr, nullptr, false, kRankSpread};
     for (int p = 0; p < sp.passes; ++p) {
         const bool last = p == sp.passes - 1, own = (sp.passes - 1 - p) % 2 == 0;       // the last pass ends in the block's arrays
-        int32_t *ko = own ? csc_col : l.key, *vo = own ? csc_eid : l.val;
-        sort_pass<int32_t>(sp, k, v, &counts[CNT_EDGES], cap_edges, 0, cap_edges, p, l.sort, chain, ko, vo,
-                           last ? SortMap{row_of, csc_row} : SortMap{}, &counts[CNT_STATUS], st);
-        k = ko;
-        v = vo;
+        SortOut<int32_t> out{};
+        if (own) {
+            out.keys = csc_col;
+            out.vals = csc_eid;
+        } else {
+            out.pairs = l.pair;
+        }
+        if (last) {
+            out.row_of = row_of;
+            out.row_out = csc_row;
+        }
+        sort_pass<int32_t>(sp, in, &counts[CNT_EDGES], cap_edges, 0, cap_edges, p, l.sort, chain, out, &counts[CNT_STATUS], st);
+        in = own ? SortIn{csc_col, csc_eid, nullptr, false, kRankMatch} : SortIn{nullptr, nullptr, l.pair, false, kRankMatch};
     }
     note_launch();
     launch_pdl(chain, csc_finalize_kernel, dim3((unsigned)std::min<int64_t>(ceil_div((int64_t)cap_edges + 1, 256), 148 * 8)), dim3(256),
