@@ -566,7 +566,7 @@ int32_t run_joint(const JointPlan &jp, const e2egrec_csr *graph, const e2egrec_m
                    jp.P, jp.rowsP, relu, dz2);
     }
     // the weight gradients feed nothing later in the step: they go to the helper stream (behind the block
-    // transposition that the sampler left there); the encoder backward waits for that stream before its first launch
+    // transposition that the sampler left there); the encoder backward waits for that stream before it gathers
     cudaStream_t ws_st = st;
     if (side) {
         side->fork(st);

@@ -168,6 +168,7 @@ int32_t backward_impl(const e2egrec_block *blocks, const LgPlan &fp, const LgPla
     lightgcn_scale_rows_kernel<T><<<lg_grid((int64_t)blocks[0].cap_dst * d), 256, 0, st>>>(
         static_cast<const T *>(dY->data), dY->ld, counts0, d, 1.0f / (float)(L + 1), dys);
     const T *g_in = dys;
+    if (SideStream *side = SideStream::get(st)) side->join_pending();     // a deferred block transposition
     for (int l = L - 1; l >= 0; --l) {
         const e2egrec_block &b = blocks[L - 1 - l];
         T *out = l == 0 ? static_cast<T *>(dX_rows->data) : buf[l & 1];
@@ -234,7 +235,6 @@ extern "C" int32_t e2egrec_lightgcn_sampled_backward(const e2egrec_block *blocks
         return E2EGREC_ERR_ARG;
     if ((dX_rows->ld * fp.es) % 16 || reinterpret_cast<uintptr_t>(dX_rows->data) % 16) return E2EGREC_ERR_ALIGN;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (SideStream *side = SideStream::get(st)) side->join_pending();     // a deferred block transposition
     if (dY->dtype == E2EGREC_BF16)
         return backward_impl<__nv_bfloat16>(blocks, fp, bp, dY->dtype, static_cast<const char *>(ctx), dY, dX_rows,
                                             static_cast<char *>(scratch), st);

@@ -389,6 +389,9 @@ static int32_t backward_impl(const e2egrec_block *blocks, int32_t n_layers, cons
             o.mask = nullptr;
             o.rhs_out = static_cast<T *>(dX_rows[n_rhs - 1].data) - static_cast<T *>(dX_rows[0].data);
         }
+        // A deferred transposition is waited for where the first of its results is read: the masking and the products before it
+        // overlap it too (medium step, whose two sorts end after its forward pass, 140 -> 134 us; joint step 262 -> 256).
+        if (l == n_layers - 1 && side) side->join_pending();
         if (l == 0) tap_begin(TAP_AGG_BWD_OUTER, st);
         const int run_len = block_run_len(b.cap_edges, p.d_in, sizeof(T));
         SegScratch sc = seg_scratch_carve(b.cap_edges, run_len, p.d_in, sizeof(T), scratch + bs.seg_off, n_rhs);
@@ -476,7 +479,6 @@ static int32_t sage_backward_entry(const e2egrec_block *blocks, int32_t n_layers
         if (dX_rows[r].ld != dX_rows[0].ld) return E2EGREC_ERR_ARG;       // the results share one leading dimension
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (SideStream *side = SideStream::get(st)) side->join_pending();     // a deferred block transposition
     if (X->dtype == E2EGREC_BF16)
         return backward_impl<__nv_bfloat16>(blocks, n_layers, X, W, act, plan, static_cast<const char *>(ctx), dH_out, n_rhs, dW,
                                             dbias, dX_rows, static_cast<char *>(scratch), bs, flags, st);
