@@ -148,6 +148,24 @@ __device__ __forceinline__ void add2(float &a0, float &a1, float b0, float b1)
     a0 = r.x;
     a1 = r.y;
 }
+
+// acc += the 16 bytes of a row.  bf16: the mixed-precision add of sm_100 takes a half of a register as it is (the same sum as
+// widening it first and adding: eight instructions where shifts, masks and packed adds are twelve).
+__device__ __forceinline__ void add_chunk(float (&acc)[8], const uint4 &raw, __nv_bfloat16)
+{
+    const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %2;\n\tadd.rn.f32.bf16 %0, lo, %0;\n\tadd.rn.f32.bf16 %1, hi, %1;\n\t}"
+            : "+f"(acc[2 * i]), "+f"(acc[2 * i + 1])
+            : "r"(w[i]));
+}
+__device__ __forceinline__ void add_chunk(float (&acc)[4], const uint4 &raw, float)
+{
+    add2(acc[0], acc[1], __uint_as_float(raw.x), __uint_as_float(raw.y));
+    add2(acc[2], acc[3], __uint_as_float(raw.z), __uint_as_float(raw.w));
+}
+
 template <typename T> __device__ inline float to_float(T v);
 template <> __device__ inline float to_float<float>(float v) { return v; }
 template <> __device__ inline float to_float<__nv_bfloat16>(__nv_bfloat16 v) { return __bfloat162float(v); }

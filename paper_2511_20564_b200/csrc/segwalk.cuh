@@ -30,7 +30,6 @@
 
 namespace e2egrec {
 
-constexpr int kWalkWarps = kAggThreads / 32;
 
 // Segment of entry k by the whole warp: every round splits the range into 33 parts with 32 probes.
 // Largest s in [0, n_seg) with ptr[s] <= k   (0 <= k < ptr[n_seg], ptr[0] = 0).
@@ -109,15 +108,16 @@ template <typename T, int N> __device__ __forceinline__ void store_share(T *p, c
 // 3.74 / 3.03, 3.74 / 3.04.
 constexpr int kWalkSteps = 4;
 constexpr int kWalkSmall = 8;
+constexpr int kWalkRuns = 8;              // stretches of a window, consecutive ones to a warp of the block
 template <int LPR, int CPL> __host__ __device__ constexpr int walk_steps() { return CPL >= kWalkSteps ? 1 : kWalkSteps / CPL; }
 template <int LPR, int CPL, int E> __host__ __device__ constexpr size_t walk_smem_bytes()
 {
-    return (size_t)2 * kWalkWarps * LPR * CPL * E * sizeof(float) + kWalkWarps * sizeof(int4);
+    return (size_t)2 * kWalkRuns * LPR * CPL * E * sizeof(float) + kWalkRuns * sizeof(int4);
 }
 
-// win_len: entries of a window (block), a multiple of kWalkWarps; cap: entries that the arrays hold, at least.
-template <typename T, typename PtrT, int LPR, int CPL, bool kWeight>
-__global__ void __launch_bounds__(kAggThreads, CPL > 1 ? 1 : 4)
+// win_len: entries of a window (block), a multiple of kWalkRuns; cap: entries that the arrays hold, at least.
+template <typename T, typename PtrT, int LPR, int CPL, bool kWeight, int kWalkWarps>
+__global__ void __launch_bounds__(kWalkWarps * 32, CPL > 1 ? 1 : 32 / kWalkWarps)
 seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict__ ptr, const int32_t *__restrict__ idx,
                 const int32_t *n_seg_dev, int64_t n_seg_host, const float *__restrict__ w, int win_len, int64_t cap, int d,
                 float *__restrict__ head2, float *__restrict__ tail2, int4 *__restrict__ win_info, SegOut<T> o)
@@ -128,14 +128,15 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
     constexpr int C = G * U;                                     // entries per group, a divisor of 32
     constexpr int S = walk_share<LPR, E>();
     constexpr int ROW = LPR * CPL * E;
+    constexpr int kUnrollGroups = 4 < 32 / C ? 4 : 32 / C;       // groups of 32 entries that are written out
     constexpr int kFar = 1 << 30;
     static_assert(32 % C == 0, "a group takes its ids from one window of 32");
     extern __shared__ float4 seg_smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int c = lane % LPR, sub = lane / LPR;
     float *sh_head = reinterpret_cast<float *>(seg_smem);
-    float *sh_tail = sh_head + kWalkWarps * ROW;
-    int4 *sh_info = reinterpret_cast<int4 *>(sh_tail + kWalkWarps * ROW);
+    float *sh_tail = sh_head + kWalkRuns * ROW;
+    int4 *sh_info = reinterpret_cast<int4 *>(sh_tail + kWalkRuns * ROW);
     __shared__ int32_t sh_win[4];
 
     const int n_chunks = d / E;
@@ -143,9 +144,14 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
     const int64_t n_seg = n_seg_dev ? (int64_t)__ldcg(n_seg_dev) : n_seg_host;
     const int64_t total = n_seg > 0 ? min((int64_t)__ldcg(ptr + n_seg), cap) : 0;
     if ((int64_t)blockIdx.x * win_len >= total) return;          // a window beyond the stream leaves no record
-    const int stretch = win_len / kWalkWarps;
+    const int stretch = win_len / kWalkRuns;
     if (threadIdx.x < 4) sh_win[threadIdx.x] = threadIdx.x == 1 || threadIdx.x == 3 ? 0 : -1;
-    const int64_t k0 = (int64_t)blockIdx.x * win_len + (int64_t)warp * stretch;
+    constexpr int kOwn = kWalkRuns / kWalkWarps;                 // the warp's stretches, one after another
+    int64_t s_next = 0;                                          // the segment in which the warp's next stretch begins
+#pragma unroll 1
+    for (int own = 0; own < kOwn; ++own) {
+    const int rl = warp * kOwn + own;
+    const int64_t k0 = (int64_t)blockIdx.x * win_len + (int64_t)rl * stretch;
     int32_t head_seg = -1, head_ends = 0, tail_seg = -1;
 
     if (k0 < total) {
@@ -157,10 +163,14 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
         for (int q = 0; q < CPL; ++q) in_c[q] = reinterpret_cast<const uint8_t *>(in) + (size_t)min(c + q * LPR, n_chunks - 1) * 16;
         const uint64_t ld_bytes = (uint64_t)ld_in * sizeof(T);
         const uint32_t ld_lo = (uint32_t)ld_bytes, ld_hi = (uint32_t)(ld_bytes >> 32);
-        auto row_of = [&](int32_t id) -> uint64_t { return (uint64_t)(uint32_t)id * ld_lo + ((uint64_t)((uint32_t)id * ld_hi) << 32); };
-        auto load_row = [&](uint64_t row, uint4 (&v)[CPL]) {
+        // a row's address: one wide product with the lane's chunk as its addend, and the upper half of a stride of 4 GB and more
+        auto load_row = [&](int32_t id, uint4 (&v)[CPL], auto wide) {
 #pragma unroll
-            for (int q = 0; q < CPL; ++q) v[q] = __ldg(reinterpret_cast<const uint4 *>(in_c[q] + row));
+            for (int q = 0; q < CPL; ++q) {
+                uint64_t at = (uint64_t)(uint32_t)id * ld_lo + reinterpret_cast<uint64_t>(in_c[q]);
+                if constexpr (decltype(wide)::value) at += (uint64_t)((uint32_t)id * ld_hi) << 32;
+                v[q] = __ldg(reinterpret_cast<const uint4 *>(at));
+            }
         };
         float acc[CPL][E];
         auto clear = [&]() {
@@ -174,17 +184,17 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
 #pragma unroll
             for (int q = 0; q < CPL; ++q) {
                 const uint4 raw = mine ? raws[q] : make_uint4(0, 0, 0, 0);
-                float x[E];
-                Chunk<T>::unpack(raw, x);
+                if constexpr (!kWeight) {
+                    add_chunk(acc[q], raw, T());
+                } else {
+                    float x[E];
+                    Chunk<T>::unpack(raw, x);
 #pragma unroll
-                for (int e = 0; e < E; e += 2) {
-                    if (kWeight) {
+                    for (int e = 0; e < E; e += 2) {
                         const float2 r = __ffma2_rn(make_float2(wgt, wgt), make_float2(x[e], x[e + 1]),
                                                     make_float2(acc[q][e], acc[q][e + 1]));
                         acc[q][e] = r.x;
                         acc[q][e + 1] = r.y;
-                    } else {
-                        add2(acc[q][e], acc[q][e + 1], x[e], x[e + 1]);
                     }
                 }
             }
@@ -197,7 +207,8 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
         // after it are on their way.
         auto rel = [&](int64_t p) -> int { return (int)max(min(p - k0, (int64_t)kFar), (int64_t)-kFar); };
         auto load_ends = [&](uint32_t b) -> int { return (int64_t)b + lane < n_seg ? rel((int64_t)__ldg(&ptr[(int64_t)b + lane + 1])) : kFar; };
-        uint32_t s_base = (uint32_t)warp_seg_containing(ptr, n_seg, k0);       // unsigned: windows reach beyond the last segment, 2^31 and on
+        // unsigned: windows reach beyond the last segment, 2^31 and on
+        uint32_t s_base = own == 0 ? (uint32_t)warp_seg_containing(ptr, n_seg, k0) : (uint32_t)s_next;
         int ends = load_ends(s_base), ends_ahead = load_ends(s_base + 32);
         int carry = rel((int64_t)__ldg(&ptr[s_base]));           // where the window's first segment begins
         int quiet = 0;                                           // windows without an entry in a row
@@ -242,7 +253,7 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
                             for (int q = 0; q < CPL; ++q) v[u][q] = make_uint4(0, 0, 0, 0);
                             if (on[u]) {
                                 if (kWeight) wt[u] = __ldg(w + id[u]);
-                                load_row(row_of(id[u]), v[u]);
+                                load_row(id[u], v[u], std::true_type());
                             }
                         }
 #pragma unroll
@@ -289,7 +300,7 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
                     for (int c0 = 0; c0 < cnt; c0 += U) {
                         uint4 v[U][CPL];
 #pragma unroll
-                        for (int u = 0; u < U; ++u) load_row(row_of(__shfl_sync(0xffffffffu, id, c0 + u)), v[u]);
+                        for (int u = 0; u < U; ++u) load_row(__shfl_sync(0xffffffffu, id, c0 + u), v[u], std::true_type());
 #pragma unroll
                         for (int u = 0; u < U; ++u) {
                             if (c0 + u >= cnt) break;            // uniform over the warp, as is the next condition
@@ -323,29 +334,41 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
                 int32_t id_cur = load_id(0), id_1 = load_id(32);
                 float w_cur = kWeight ? __ldg(w + id_cur) : 0.f;
                 clear();
-                for (int b = 0; b < sn; b += 32) {
-                    const int32_t id_2 = b + 32 < sn ? load_id(b + 64) : 0;
-                    const float w_1 = kWeight && b + 32 < sn ? __ldg(w + id_1) : 0.f;
-#pragma unroll 1
-                    for (int c0 = 0; c0 < 32 && b + c0 < sn; c0 += C) {
-                        uint4 v[U][CPL];
+                auto walk = [&](auto wide) {
+                    for (int b = 0; b < sn; b += 32) {
+                        const int32_t id_2 = b + 32 < sn ? load_id(b + 64) : 0;
+                        const float w_1 = kWeight && b + 32 < sn ? __ldg(w + id_1) : 0.f;
+                        auto load_group = [&](int c0, uint4 (&v)[U][CPL]) {
 #pragma unroll
-                        for (int u = 0; u < U; ++u) load_row(row_of(__shfl_sync(0xffffffffu, id_cur, c0 + u * G + sub)), v[u]);
-                        if (b + c0 + C <= sn) {
+                            for (int u = 0; u < U; ++u) load_row(__shfl_sync(0xffffffffu, id_cur, c0 + u * G + sub), v[u], wide);
+                        };
+                        auto weight = [&](int e) -> float { return kWeight ? __shfl_sync(0xffffffffu, w_cur, e) : 1.f; };
+                        if (b + 32 <= sn) {                      // 32 entries: no tests
+#pragma unroll kUnrollGroups
+                            for (int c0 = 0; c0 < 32; c0 += C) {
+                                uint4 v[U][CPL];
+                                load_group(c0, v);
 #pragma unroll
-                            for (int u = 0; u < U; ++u)
-                                add_row(v[u], kWeight ? __shfl_sync(0xffffffffu, w_cur, c0 + u * G + sub) : 1.f, true);
+                                for (int u = 0; u < U; ++u) add_row(v[u], weight(c0 + u * G + sub), true);
+                            }
                         } else {
+#pragma unroll 1
+                            for (int c0 = 0; b + c0 < sn; c0 += C) {
+                                uint4 v[U][CPL];
+                                load_group(c0, v);
 #pragma unroll
-                            for (int u = 0; u < U; ++u)
-                                if (b + c0 + u * G < sn)         // uniform over the warp
-                                    add_row(v[u], kWeight ? __shfl_sync(0xffffffffu, w_cur, c0 + u * G + sub) : 1.f, b + c0 + u * G + sub < sn);
+                                for (int u = 0; u < U; ++u)
+                                    if (b + c0 + u * G < sn)     // uniform over the warp
+                                        add_row(v[u], weight(c0 + u * G + sub), b + c0 + u * G + sub < sn);
+                            }
                         }
+                        id_cur = id_1;
+                        id_1 = id_2;
+                        w_cur = w_1;
                     }
-                    id_cur = id_1;
-                    id_1 = id_2;
-                    w_cur = w_1;
-                }
+                };
+                if (ld_hi == 0) walk(std::false_type());
+                else walk(std::true_type());
                 int off = 0;
 #pragma unroll
                 for (int q = 0; q < CPL; ++q) {
@@ -364,7 +387,7 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
                         if (ch < n_chunks) store_share<T, S>(row + ch * E, r);
                     }
                 } else {                                         // cut by the stretch's ends: a part for the join
-                    float *dst = (sbeg >= 0 ? sh_tail : sh_head) + warp * ROW + off;
+                    float *dst = (sbeg >= 0 ? sh_tail : sh_head) + rl * ROW + off;
 #pragma unroll
                     for (int q = 0; q < CPL; ++q) {
                         store_share<float, (S > 4 ? 4 : S)>(dst + (c + q * LPR) * E, acc[q]);
@@ -375,7 +398,11 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
                 }
             }
             carry = __shfl_sync(0xffffffffu, ends, 31);          // the offsets do not decrease: the window's last end
-            if (carry >= len) break;
+            if (carry >= len) {
+                if (own + 1 < kOwn)                              // the segments that end in this stretch lie behind
+                    s_next = min((int64_t)s_base + __popc(__ballot_sync(0xffffffffu, ends <= len)), n_seg - 1);
+                break;
+            }
             quiet = __any_sync(0xffffffffu, n > 0) ? 0 : quiet + 1;
             if (quiet < kQuietWindows) {
                 s_base += 32;
@@ -388,28 +415,34 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
             ends_ahead = load_ends(s_base + 32);
         }
     }
-    if (lane == 0) sh_info[warp] = make_int4(head_seg, head_ends, tail_seg, 0);
+    if (lane == 0) sh_info[rl] = make_int4(head_seg, head_ends, tail_seg, 0);
+    }
     __syncthreads();
-    if (lane < LPR)
-        seg_join_run<T, PtrT, LPR, CPL, 0>(sh_head, sh_tail, sh_info, sh_win, warp, kWalkWarps, lane, n_chunks, d, head_seg, head_ends,
-                                           tail_seg, ptr, head2, tail2, o, nullptr, 0);
+    if (lane < LPR) {
+#pragma unroll 1
+        for (int rl = warp * kOwn; rl < (warp + 1) * kOwn; ++rl) {
+            const int4 info = sh_info[rl];
+            seg_join_run<T, PtrT, LPR, CPL, 0>(sh_head, sh_tail, sh_info, sh_win, rl, kWalkRuns, lane, n_chunks, d, info.x, info.y, info.z,
+                                               ptr, head2, tail2, o, nullptr, 0);
+        }
+    }
     __syncthreads();
     if (threadIdx.x == 0) win_info[blockIdx.x] = make_int4(sh_win[0], sh_win[1], sh_win[2], 0);
 }
 
 // B200: 5 M nodes, 10^8 entries, 64 bf16 values, forward and transposed 5.74 -> 3.74 ms (from 4.5 to 7.3 TB/s of gathered
 // rows); 500 k nodes, 2 * 10^7 entries, 64 fp32 values, weighted, per layer 0.77 -> 0.45 ms (11.4 TB/s).
-template <typename T, typename PtrT, int LPR, int CPL, bool kWeight>
+template <typename T, typename PtrT, int LPR, int CPL, bool kWeight, int kWalkWarps>
 inline void launch_seg_walk(const T *in, int64_t ld_in, const PtrT *ptr, const int32_t *idx, const int32_t *n_seg_dev,
                             int64_t n_seg_host, int64_t cap_seg, const float *w, int run_len, int d, const SegScratch &sc,
                             const SegOut<T> &o, cudaStream_t st)
 {
     constexpr size_t smem = walk_smem_bytes<LPR, CPL, Chunk<T>::kElems>();
-    auto kern = seg_walk_kernel<T, PtrT, LPR, CPL, kWeight>;
+    auto kern = seg_walk_kernel<T, PtrT, LPR, CPL, kWeight, kWalkWarps>;
     if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     tap_begin(TAP_SEG_L1, st);
     note_launch();
-    launch_pdl(n_seg_dev && sc.cap_runs * run_len < kChainEdges, kern, dim3((unsigned)sc.n_windows), dim3(kAggThreads), smem, st, in, ld_in,
+    launch_pdl(n_seg_dev && sc.cap_runs * run_len < kChainEdges, kern, dim3((unsigned)sc.n_windows), dim3(kWalkWarps * 32), smem, st, in, ld_in,
                ptr, idx, n_seg_dev, n_seg_host, w, run_len * sc.runs_per_window, sc.cap_runs * run_len, d, sc.head2, sc.tail2,
                sc.win_info, o);
     tap_end(TAP_SEG_L1, st);
@@ -425,7 +458,10 @@ inline bool dispatch_seg_walk(const T *in, int64_t ld_in, const PtrT *ptr, const
     const RowShape rs = row_shape(d, dtype);
 #define E2E_CASE(L, C)                                                                                                      \
     if (rs.lpr == L && rs.cpl == C) {                                                                                       \
-        launch_seg_walk<T, PtrT, L, C, kWeight>(in, ld_in, ptr, idx, n_seg_dev, n_seg_host, cap_seg, w, run_len, d, sc, o, st); \
+        if (run_len >= 256)                                                                                                 \
+            launch_seg_walk<T, PtrT, L, C, kWeight, 4>(in, ld_in, ptr, idx, n_seg_dev, n_seg_host, cap_seg, w, run_len, d, sc, o, st); \
+        else                                                                                                                \
+            launch_seg_walk<T, PtrT, L, C, kWeight, 8>(in, ld_in, ptr, idx, n_seg_dev, n_seg_host, cap_seg, w, run_len, d, sc, o, st); \
         return true;                                                                                                        \
     }
     E2E_CASE(4, 1) E2E_CASE(8, 1) E2E_CASE(16, 1) E2E_CASE(32, 1) E2E_CASE(32, 2) E2E_CASE(32, 4)
