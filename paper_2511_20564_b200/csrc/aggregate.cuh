@@ -53,6 +53,12 @@ sage_aggregate_kernel(const T *__restrict__ Hsrc, int64_t ld, const int32_t *__r
         }
     };
     fetch(i, beg, end, mine, self_row);
+    // lanes beyond the row's chunks read its last one and store nothing
+    uint64_t chunk[CPL];
+#pragma unroll
+    for (int q = 0; q < CPL; ++q) chunk[q] = reinterpret_cast<uint64_t>(Hsrc + min(c + q * LPR, n_chunks - 1) * E);
+    const uint64_t ld_bytes = (uint64_t)ld * sizeof(T);
+    const uint32_t ld_lo = (uint32_t)ld_bytes, ld_hi = (uint32_t)(ld_bytes >> 32);
     while (i < pad_end) {
         const int64_t i_next = i + warps;
         int32_t beg_n, end_n, mine_n;
@@ -84,23 +90,18 @@ sage_aggregate_kernel(const T *__restrict__ Hsrc, int64_t ld, const int32_t *__r
                     for (int u = 0; u < U; ++u) {
                         const int j = (t + u) * G + g;
                         const int32_t id = __shfl_sync(0xffffffffu, mine, j & 31);
-                        const T *row = Hsrc + (int64_t)id * ld;
 #pragma unroll
                         for (int q = 0; q < CPL; ++q) {
-                            const int ch = c + q * LPR;
                             v[u][q] = make_uint4(0, 0, 0, 0);     // zero bits are 0.0 in both types
-                            if (j < m && ch < n_chunks) v[u][q] = Chunk<T>::load_raw(row + ch * E);
+                            if (j < m)
+                                v[u][q] = __ldg(reinterpret_cast<const uint4 *>((uint64_t)(uint32_t)id * ld_lo + chunk[q] +
+                                                                               ((uint64_t)((uint32_t)id * ld_hi) << 32)));
                         }
                     }
 #pragma unroll
                     for (int u = 0; u < U; ++u)
 #pragma unroll
-                        for (int q = 0; q < CPL; ++q) {
-                            float x[E];
-                            Chunk<T>::unpack(v[u][q], x);
-#pragma unroll
-                            for (int k = 0; k < E; k += 2) add2(acc[q][k], acc[q][k + 1], x[k], x[k + 1]);
-                        }
+                        for (int q = 0; q < CPL; ++q) add_chunk(acc[q], v[u][q], T());
                 }
             }
 #pragma unroll

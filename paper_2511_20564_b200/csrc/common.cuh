@@ -166,6 +166,12 @@ __device__ __forceinline__ void add_chunk(float (&acc)[4], const uint4 &raw, flo
     add2(acc[2], acc[3], __uint_as_float(raw.z), __uint_as_float(raw.w));
 }
 
+// 16 bytes of row `row` of a matrix whose rows are ld_bytes < 2^32 apart: one wide product with the chunk's address as addend.
+__device__ __forceinline__ uint4 load_row16(const void *chunk, int32_t row, uint32_t ld_bytes)
+{
+    return __ldg(reinterpret_cast<const uint4 *>((uint64_t)(uint32_t)row * ld_bytes + reinterpret_cast<uint64_t>(chunk)));
+}
+
 template <typename T> __device__ inline float to_float(T v);
 template <> __device__ inline float to_float<float>(float v) { return v; }
 template <> __device__ inline float to_float<__nv_bfloat16>(__nv_bfloat16 v) { return __bfloat162float(v); }

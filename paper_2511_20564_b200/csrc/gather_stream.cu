@@ -158,10 +158,7 @@ sage_aggregate_stream_kernel(const __grid_constant__ CUtensorMap map, const int3
         const int32_t k0 = b_w + 4 * q;
         auto add_row = [&](int r) {
             while (k0 + r >= end_i) finalize();     // the entry belongs to a later destination: close the ones before it
-            float x[8];
-            Chunk<__nv_bfloat16>::unpack(*reinterpret_cast<const uint4 *>(rows + r * kRowBytes), x);
-#pragma unroll
-            for (int kk = 0; kk < 8; kk += 2) add2(acc[kk], acc[kk + 1], x[kk], x[kk + 1]);
+            add_chunk(acc, *reinterpret_cast<const uint4 *>(rows + r * kRowBytes), __nv_bfloat16());
         };
         if (k0 + 4 <= e_w) {
 #pragma unroll

@@ -492,16 +492,13 @@ seg_run_kernel(const T *__restrict__ in, int64_t ld_in, const int32_t *__restric
                     }
 #pragma unroll
                     for (int q = 0; q < CPL; ++q) {
-                        float x[E];
-                        Chunk<T>::unpack(v[u][q], x);
+                        if constexpr (kWeight) {
+                            float x[E];
+                            Chunk<T>::unpack(v[u][q], x);
 #pragma unroll
-                        for (int e = 0; e < E; e += 2) {
-                            if (kWeight) {
-                                acc[q][e] = fmaf(wt[u], x[e], acc[q][e]);
-                                acc[q][e + 1] = fmaf(wt[u], x[e + 1], acc[q][e + 1]);
-                            } else {
-                                add2(acc[q][e], acc[q][e + 1], x[e], x[e + 1]);
-                            }
+                            for (int e = 0; e < E; ++e) acc[q][e] = fmaf(wt[u], x[e], acc[q][e]);
+                        } else {
+                            add_chunk(acc[q], v[u][q], T());
                         }
                     }
                 }
@@ -575,6 +572,9 @@ seg_run_block_kernel(const T *__restrict__ in, int64_t ld_in, const int32_t *__r
         const T *__restrict__ in_c = in + cc * E;
         const T *__restrict__ self_c = o.self + cc * E;
         const T *__restrict__ mask_c = kMask ? o.mask + cc * E : nullptr;
+        // row strides in bytes; the host sends wider ones to the general kernel
+        const uint32_t in_ld = (uint32_t)ld_in * (uint32_t)sizeof(T), self_ld = (uint32_t)o.ld_self * (uint32_t)sizeof(T),
+                       mask_ld = (uint32_t)o.ld_mask * (uint32_t)sizeof(T);
         const bool vec_ok = ((reinterpret_cast<uintptr_t>(idx0) | reinterpret_cast<uintptr_t>(seg0)) & 15u) == 0;
         const bool first_begins = k0 == 0 || seg0[-1] != seg0[0];
         const bool last_ends = k0 + len == total || seg0[len] != seg0[len - 1];
@@ -621,14 +621,14 @@ seg_run_block_kernel(const T *__restrict__ in, int64_t ld_in, const int32_t *__r
             uint4 v[U], sv[U], mv[kMask ? U : 1];
             bool start[U];
 #pragma unroll
-            for (int u = 0; u < U; ++u) v[u] = Chunk<T>::load_raw(in_c + row_offset(id[u], ld_in));
+            for (int u = 0; u < U; ++u) v[u] = load_row16(in_c, id[u], in_ld);
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 start[u] = r0 + u < len && sg[u] != (u == 0 ? last_sg : sg[u - 1]);      // entry 0 always starts (last_sg = -1)
                 sv[u] = make_uint4(0, 0, 0, 0);
                 if (start[u]) {
-                    if ((u > 0 || r0 > 0 || first_begins) && sg[u] < n_self) sv[u] = Chunk<T>::load_raw(self_c + row_offset(sg[u], o.ld_self));
-                    if (kMask) mv[u] = Chunk<T>::load_raw(mask_c + row_offset(sg[u], o.ld_mask));
+                    if ((u > 0 || r0 > 0 || first_begins) && sg[u] < n_self) sv[u] = load_row16(self_c, sg[u], self_ld);
+                    if (kMask) mv[u] = load_row16(mask_c, sg[u], mask_ld);
                 }
             }
             last_sg = sg[U - 1];
@@ -642,10 +642,7 @@ seg_run_block_kernel(const T *__restrict__ in, int64_t ld_in, const int32_t *__r
                         Chunk<T>::unpack(sv[u], acc[0]);                 // the self row (zeros if there is none)
                         if (kMask) cur_mask[0] = mv[u];
                     }
-                    float x[E];
-                    Chunk<T>::unpack(v[u], x);
-#pragma unroll
-                    for (int e = 0; e < E; e += 2) add2(acc[0][e], acc[0][e + 1], x[e], x[e + 1]);
+                    add_chunk(acc[0], v[u], T());
                 }
             }
         }
@@ -889,7 +886,8 @@ inline void launch_seg_reduce(const T *in, int64_t ld_in, const int32_t *ptr, co
     constexpr size_t smem = seg_run_smem_bytes<LPR, CPL, Chunk<T>::kElems>();
     bool block_form = false;
     if constexpr (CPL == 1 && !kWeight)
-        block_form = seg_of && n_seg_dev && o.self && !o.seg_scale && !seg_general_only();
+        block_form = seg_of && n_seg_dev && o.self && !o.seg_scale && !seg_general_only() &&
+                     (std::max({ld_in, o.ld_self, o.ld_mask}) * (int64_t)sizeof(T)) >> 32 == 0;
     if (o.n_rhs > 1 && !(block_form && sc.chain_cnt)) {
         // the general kernels take one right-hand side per pass
         for (int r = 0; r < o.n_rhs; ++r) {

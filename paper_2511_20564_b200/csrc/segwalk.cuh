@@ -6,10 +6,12 @@
 // the kernel that joins them are those of segreduce.cuh; a window is cut into one stretch of consecutive entries per
 // warp of the block.
 //
-// What bounds it: latency, of the gathered rows first and then of the barrier before the join (stalls per issue 4.6 and 3.4;
-// issue slots 57 % busy, L1 at 34 %, L2 and DRAM at 10 %: B200, 128-byte rows).  What it could be sped up by so far were
-// instructions per gathered row and per segment.  With one lane group per run, 32 / LPR runs per warp each with its own segment ends, a 128-byte row took 22 warp
-// instructions, most of them bookkeeping that the warp executes for all of its groups' different positions.  Here the
+// What bounds it: instructions (rows that L2 serves: issue slots 65 % busy, L1 hit 2 %) and, on power-law graphs, the barrier before the
+// join and the latency of rows that L2 does not hold (issue slots 54 %; B200, 128-byte rows).  A bf16 row is added without being
+// widened first and its address is one product: 10^8 entries of 64 bf16 values and the transpose, weighted, 3.75 -> 3.30 ms; 32 entries
+// of a long segment without tests 3.16, with stretches twice as long, whose longer sums however doubled the rounding error; with two
+// stretches per warp 3.26.  Before that, too, instructions were what it could be sped up by.  With one lane group per run, 32 / LPR
+// runs per warp each with its own segment ends, a 128-byte row took 22 warp instructions, most of them bookkeeping that the warp executes for all of its groups' different positions.  Here the
 // offsets come 32 segments at a time, one lane each, and the segments are handled by their length:
 //   - longer ones by the whole warp: 32 entry ids in one coalesced load (the next 32 and the entry weights on their way),
 //     steps of 32 / LPR rows with no test per entry, and one sum across the lane groups per segment that halves the row at
@@ -20,8 +22,9 @@
 //     2 M segments of two entries on average took 719 and, weighted, 857 us with 256 bf16 values, 824 with 100 fp32 values;
 //     now 578, 655 and 577).
 // Together 11 warp instructions per row.  Tried and slower: rows through a cp.async ring in shared memory (4.57 ms
-// against 3.74: the copies and the reads of the ring load the L1 path to 86 %), two groups of rows in registers (5.18),
-// all segments by the whole warp (4.57), stretches handed out by a counter (3.76 to 3.88: less waiting at the join's
+// against 3.74 at the time: the copies and the reads of the ring load the L1 path to 86 %), two groups of rows in registers (5.18),
+// all segments by the whole warp (4.57), a row's registers loaded again as soon as it has been added (3.70 against 3.55),
+// stretches handed out by a counter (3.76 to 3.88: less waiting at the join's
 // barrier, more stretches to begin and to join).
 #pragma once
 
@@ -430,8 +433,8 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
     if (threadIdx.x == 0) win_info[blockIdx.x] = make_int4(sh_win[0], sh_win[1], sh_win[2], 0);
 }
 
-// B200: 5 M nodes, 10^8 entries, 64 bf16 values, forward and transposed 5.74 -> 3.74 ms (from 4.5 to 7.3 TB/s of gathered
-// rows); 500 k nodes, 2 * 10^7 entries, 64 fp32 values, weighted, per layer 0.77 -> 0.45 ms (11.4 TB/s).
+// B200: 5 M nodes, 10^8 entries, 64 bf16 values, forward and transposed 3.73 -> 3.26 ms (8.6 TB/s of gathered rows);
+// 500 k nodes, 2 * 10^7 entries, 64 fp32 values, weighted, per layer 0.45 -> 0.41 ms (12.5 TB/s).
 template <typename T, typename PtrT, int LPR, int CPL, bool kWeight, int kWalkWarps>
 inline void launch_seg_walk(const T *in, int64_t ld_in, const PtrT *ptr, const int32_t *idx, const int32_t *n_seg_dev,
                             int64_t n_seg_host, int64_t cap_seg, const float *w, int run_len, int d, const SegScratch &sc,
@@ -449,6 +452,8 @@ inline void launch_seg_walk(const T *in, int64_t ld_in, const PtrT *ptr, const i
     launch_seg_final(ptr, n_seg_dev, n_seg_host, cap_seg, run_len, d, sc, o, st);
 }
 
+// Four warps with two stretches each for rows of up to 128 bytes of large inputs, eight with one otherwise: 10^8 entries of 128-byte
+// rows 3.29 and 3.41 ms, three layers of 2 * 10^7 entries of 256-byte rows 2.83 and 2.76.
 // Same contract as dispatch_seg_reduce, without an entry -> segment array, self rows or masks.
 template <typename T, typename PtrT, bool kWeight>
 inline bool dispatch_seg_walk(const T *in, int64_t ld_in, const PtrT *ptr, const int32_t *idx, const int32_t *n_seg_dev,
@@ -458,8 +463,8 @@ inline bool dispatch_seg_walk(const T *in, int64_t ld_in, const PtrT *ptr, const
     const RowShape rs = row_shape(d, dtype);
 #define E2E_CASE(L, C)                                                                                                      \
     if (rs.lpr == L && rs.cpl == C) {                                                                                       \
-        if (run_len >= 256)                                                                                                 \
-            launch_seg_walk<T, PtrT, L, C, kWeight, 4>(in, ld_in, ptr, idx, n_seg_dev, n_seg_host, cap_seg, w, run_len, d, sc, o, st); \
+        if (L <= 8 && run_len >= 256)                                                                                       \
+            launch_seg_walk<T, PtrT, L, C, kWeight, L <= 8 ? 4 : 8>(in, ld_in, ptr, idx, n_seg_dev, n_seg_host, cap_seg, w, run_len, d, sc, o, st); \
         else                                                                                                                \
             launch_seg_walk<T, PtrT, L, C, kWeight, 8>(in, ld_in, ptr, idx, n_seg_dev, n_seg_host, cap_seg, w, run_len, d, sc, o, st); \
         return true;                                                                                                        \
