@@ -220,8 +220,8 @@ __device__ __forceinline__ void seg_chain_arrive(int32_t sg, const int32_t *__re
 // the group).  n_runs: runs of the window.
 template <typename T, typename PtrT, int LPR, int CPL, int kExtra>
 __device__ __forceinline__ void seg_join_run(const float *sh_head, const float *sh_tail, const int4 *sh_info, int32_t *sh_win, int rl,
-                                             int n_runs, int c, int n_chunks, int d, int32_t head_seg, int32_t head_ends, int32_t tail_seg,
-                                             const PtrT *__restrict__ ptr, float *__restrict__ head2, float *__restrict__ tail2,
+                                             int n_runs, int64_t win, int c, int n_chunks, int d, int32_t head_seg, int32_t head_ends,
+                                             int32_t tail_seg, const PtrT *__restrict__ ptr, float *__restrict__ head2, float *__restrict__ tail2,
                                              const SegOut<T> &o, int32_t *chain_cnt, int run_len)
 {
     constexpr int E = Chunk<T>::kElems;
@@ -263,7 +263,7 @@ __device__ __forceinline__ void seg_join_run(const float *sh_head, const float *
                 seg_store_row<T, LPR, CPL, kExtra>(o, head_seg, inv, acc, mrow, c, n_chunks);
             } else {
                 // leaves the window: towards earlier windows (head2) or, begun here and still open, later ones (tail2)
-                float *dst = (first >= 0 ? tail2 : head2) + (int64_t)blockIdx.x * d;
+                float *dst = (first >= 0 ? tail2 : head2) + win * d;
 #pragma unroll
                 for (int q = 0; q < CPL; ++q) {
                     const int ch = c + q * LPR;
@@ -282,7 +282,7 @@ __device__ __forceinline__ void seg_join_run(const float *sh_head, const float *
             }
         }
         if (last_run && tail_seg >= 0) {           // a segment that begins in the window's last run and continues
-            float *dst = tail2 + (int64_t)blockIdx.x * d;
+            float *dst = tail2 + win * d;
 #pragma unroll
             for (int q = 0; q < CPL; ++q) {
                 const int ch = c + q * LPR;
@@ -300,7 +300,7 @@ __device__ __forceinline__ void seg_join_run(const float *sh_head, const float *
 }
 
 template <typename T, typename PtrT, int LPR, int CPL, int kExtra>
-__device__ __forceinline__ void seg_join_window(float *sh_head, float *sh_tail, int4 *sh_info, int32_t *sh_win, int rl, int c,
+__device__ __forceinline__ void seg_join_window(float *sh_head, float *sh_tail, int4 *sh_info, int32_t *sh_win, int64_t win, int rl, int c,
                                                 int n_chunks, int d, int32_t head_seg, int32_t head_ends, int32_t tail_seg,
                                                 const PtrT *__restrict__ ptr, float *__restrict__ head2, float *__restrict__ tail2,
                                                 int4 *__restrict__ win_info, const SegOut<T> &o, int32_t *chain_cnt = nullptr,
@@ -309,11 +309,11 @@ __device__ __forceinline__ void seg_join_window(float *sh_head, float *sh_tail, 
     if (c == 0) sh_info[rl] = make_int4(head_seg, head_ends, tail_seg, 0);
     if (threadIdx.x < 4) sh_win[threadIdx.x] = threadIdx.x == 1 || threadIdx.x == 3 ? 0 : -1;
     __syncthreads();
-    seg_join_run<T, PtrT, LPR, CPL, kExtra>(sh_head, sh_tail, sh_info, sh_win, rl, kAggThreads / LPR, c, n_chunks, d, head_seg, head_ends,
+    seg_join_run<T, PtrT, LPR, CPL, kExtra>(sh_head, sh_tail, sh_info, sh_win, rl, kAggThreads / LPR, win, c, n_chunks, d, head_seg, head_ends,
                                             tail_seg, ptr, head2, tail2, o, chain_cnt, run_len);
     if (chain_cnt) return;                        // no record: nobody reads it
     __syncthreads();
-    if (threadIdx.x == 0) win_info[blockIdx.x] = make_int4(sh_win[0], sh_win[1], sh_win[2], 0);
+    if (threadIdx.x == 0) win_info[win] = make_int4(sh_win[0], sh_win[1], sh_win[2], 0);
 }
 
 // Shared memory of seg_run_kernel (dynamic): head and tail rows of the block's runs, fp32, one row of
@@ -506,7 +506,7 @@ seg_run_kernel(const T *__restrict__ in, int64_t ld_in, const int32_t *__restric
         }
         emit(last_ends);
     }
-    seg_join_window<T, int32_t, LPR, CPL, kExtra>(sh_head, sh_tail, sh_info, sh_win, rl, c, n_chunks, d, head_seg, head_ends, tail_seg, ptr,
+    seg_join_window<T, int32_t, LPR, CPL, kExtra>(sh_head, sh_tail, sh_info, sh_win, blockIdx.x, rl, c, n_chunks, d, head_seg, head_ends, tail_seg, ptr,
                                                head2, tail2, win_info, o);
 }
 
@@ -521,7 +521,10 @@ seg_run_kernel(const T *__restrict__ in, int64_t ld_in, const int32_t *__restric
 // What is left is instructions: two entries per segment on average, so every second entry closes a segment, rounds and
 // stores a row.  Row addresses by two 32-bit products, loads without tests (ids beyond the run and lanes beyond the row
 // repeat the last ones) and a mask taken two values at a time took the outer blocks of the largest training step from 54,
-// 218 and 213 us to 41, 149 and 180 (bf16 rows of 512 bytes, B200).  A form whose rows came in through a TMA ring per warp
+// 218 and 213 us to 41, 149 and 180 (bf16 rows of 512 bytes, B200).  One wave of blocks goes over the windows: with a block per
+// window of the capacity nine tenths of the blocks found none, took two dependent loads to see it and looked after a few segments
+// without entries each; the segments without entries are looked for 32 to a warp (per pass: large step 1202 -> 1166 us, two-task
+// step 200 -> 188, joint step 253 -> 242, medium step 132.9 -> 130.1).  A form whose rows came in through a TMA ring per warp
 // was ahead before that (0.421 against 0.439 ms on a larger block) and is behind it: 253 and 226 us, the barrier waits and
 // the rows kept one group ahead being instructions too.
 template <typename T, int LPR, bool kMask, int U = 4, int kMinBlocks = (kMask ? 3 : 4)>
@@ -529,7 +532,7 @@ __global__ void __launch_bounds__(kAggThreads, kMinBlocks)
 seg_run_block_kernel(const T *__restrict__ in, int64_t ld_in, const int32_t *__restrict__ ptr, const int32_t *__restrict__ idx,
                      const int32_t *__restrict__ seg_of, const int32_t *__restrict__ n_seg_dev, int run_len, int d,
                      float *__restrict__ head2, float *__restrict__ tail2, int4 *__restrict__ win_info, int64_t cap_runs,
-                     int32_t *__restrict__ chain_cnt, SegOut<T> o)
+                     int64_t n_windows, int32_t *__restrict__ chain_cnt, SegOut<T> o)
 {
     constexpr int E = Chunk<T>::kElems;
     constexpr int RB = kAggThreads / LPR;
@@ -544,10 +547,9 @@ seg_run_block_kernel(const T *__restrict__ in, int64_t ld_in, const int32_t *__r
     const int c = threadIdx.x % LPR;
     const int rl = threadIdx.x / LPR;
     const int n_chunks = d / E;
-    const int64_t run = (int64_t)blockIdx.x * RB + rl;
     pdl_wait();                                    // the kernel before this one in the stream has completed
     if (blockIdx.y) {                              // the second right-hand side: other rows, same segments
-        const int64_t r = blockIdx.y, nw = gridDim.x;
+        const int64_t r = blockIdx.y, nw = n_windows;
         in += r * o.rhs_in;
         o.self += r * o.rhs_self;
         o.out += r * o.rhs_out;
@@ -557,11 +559,11 @@ seg_run_block_kernel(const T *__restrict__ in, int64_t ld_in, const int32_t *__r
     }
     const int32_t n_seg = __ldcg(n_seg_dev);
     const int32_t total = n_seg > 0 ? __ldcg(ptr + n_seg) : 0;
+    // the blocks go over the windows of the stream, of which the host knows only the capacity
+    for (int64_t win = blockIdx.x; win * RB * run_len < total; win += gridDim.x) {
+    const int64_t run = win * RB + rl;
     const int64_t k0 = run * run_len;
     int32_t head_seg = -1, head_ends = 0, tail_seg = -1;
-    // a window that lies wholly beyond the stream (grids are sized for capacities) has no run work and no join, but
-    // still takes its share of the segments without entries below
-    const bool live_window = (int64_t)blockIdx.x * RB * run_len < total;
 
     if (run < cap_runs && k0 < total) {
         const int len = (int)min((int64_t)run_len, (int64_t)total - k0);
@@ -648,28 +650,52 @@ seg_run_block_kernel(const T *__restrict__ in, int64_t ld_in, const int32_t *__r
         }
         emit(last_ends);
     }
-    if (live_window)
-        seg_join_window<T, int32_t, LPR, 1, kExtra>(sh_head, sh_tail, sh_info, sh_win, rl, c, n_chunks, d, head_seg, head_ends,
-                                                    tail_seg, ptr, head2, tail2, win_info, o, chain_cnt, run_len);
+    seg_join_window<T, int32_t, LPR, 1, kExtra>(sh_head, sh_tail, sh_info, sh_win, win, rl, c, n_chunks, d, head_seg, head_ends, tail_seg,
+                                                ptr, head2, tail2, win_info, o, chain_cnt, run_len);
+    __syncthreads();                               // the next window's parts go where this one's were
+    }
     if (!chain_cnt) return;                        // the two-kernel form: seg_final_kernel writes the rest
 
     // ---- segments without entries (their row is the self row, masked, or zero) and the zero rows up to the next
-    // multiple of 128: every block of the grid takes a slice, one lane group per segment
+    // multiple of 128: up to 32 segments per warp at a time, one lane each; the empty ones by one lane group each, four rows in flight
     {
+        constexpr int G = 32 / LPR, F = 4;
         const int32_t n_self = o.n_self ? __ldcg(o.n_self) : n_seg;
-        const int32_t per = (n_seg + (int32_t)gridDim.x - 1) / (int32_t)gridDim.x;
-        const int32_t s1 = min(n_seg, ((int32_t)blockIdx.x + 1) * per);
-        for (int32_t sg = (int32_t)blockIdx.x * per + rl; sg < s1; sg += RB) {
-            if (ptr[sg + 1] != ptr[sg]) continue;
-            float acc[1][E];
-            uint4 mrow[1] = {make_uint4(0, 0, 0, 0)};
-            uint4 raw = make_uint4(0, 0, 0, 0);
-            if (c < n_chunks) {
-                if (sg < n_self) raw = Chunk<T>::load_raw(o.self + (int64_t)sg * o.ld_self + c * E);
-                if (kMask) mrow[0] = Chunk<T>::load_raw(o.mask + (int64_t)sg * o.ld_mask + c * E);
+        const int lane = threadIdx.x & 31, sub = lane / LPR;
+        const int64_t warps = (int64_t)gridDim.x * (kAggThreads / 32);
+        const int take = (int)min((int64_t)32, max((int64_t)4, ceil_div(n_seg, warps)));
+        // from the last block on: the first ones have the windows
+        for (int64_t s0 = (((int64_t)gridDim.x - 1 - blockIdx.x) * (kAggThreads / 32) + threadIdx.x / 32) * take; s0 < n_seg; s0 += warps * take) {
+            const int64_t s = min(s0 + lane, (int64_t)n_seg - 1);
+            unsigned empty = __ballot_sync(0xffffffffu, lane < take && s0 + lane < n_seg && ptr[s] == ptr[s + 1]);
+            while (empty) {
+                int32_t sg[F];
+                uint4 raw[F], mrow[F];
+#pragma unroll
+                for (int f = 0; f < F; ++f) {
+                    sg[f] = -1;
+#pragma unroll
+                    for (int g = 0; g < G; ++g) {
+                        if (g == sub && empty) sg[f] = (int32_t)s0 + __ffs(empty) - 1;
+                        empty &= empty - 1;
+                    }
+                }
+#pragma unroll
+                for (int f = 0; f < F; ++f) {
+                    raw[f] = mrow[f] = make_uint4(0, 0, 0, 0);
+                    if (sg[f] < 0 || c >= n_chunks) continue;
+                    if (sg[f] < n_self) raw[f] = Chunk<T>::load_raw(o.self + (int64_t)sg[f] * o.ld_self + c * E);
+                    if (kMask && o.mask) mrow[f] = Chunk<T>::load_raw(o.mask + (int64_t)sg[f] * o.ld_mask + c * E);
+                }
+#pragma unroll
+                for (int f = 0; f < F; ++f) {
+                    if (sg[f] < 0) continue;
+                    float acc[1][E];
+                    const uint4 m1[1] = {mrow[f]};
+                    Chunk<T>::unpack(raw[f], acc[0]);
+                    seg_store_row<T, LPR, 1, kExtra>(o, sg[f], 1.0f, acc, m1, c, n_chunks);
+                }
             }
-            Chunk<T>::unpack(raw, acc[0]);
-            seg_store_row<T, LPR, 1, kExtra>(o, sg, 1.0f, acc, mrow, c, n_chunks);
         }
         if (o.pad_rows > 0) {
             const int64_t pad_end = min(((int64_t)n_seg + 127) / 128 * 128, o.pad_rows);
@@ -912,10 +938,12 @@ inline void launch_seg_reduce(const T *in, int64_t ld_in, const int32_t *ptr, co
     if constexpr (CPL == 1 && !kWeight) {
         // the transposed aggregation of a sampled block: the kernel written for that case
         if (block_form) {
-            const dim3 grid_b(grid1, (unsigned)(o.n_rhs > 1 && sc.chain_cnt ? o.n_rhs : 1));
+            // one wave of blocks, which go over the windows themselves
+            const int64_t rhs = o.n_rhs > 1 && sc.chain_cnt ? o.n_rhs : 1;
+            const dim3 grid_b((unsigned)std::min<int64_t>(sc.n_windows, ceil_div(148 * (o.mask ? 3 : 4), rhs)), (unsigned)rhs);
             auto kern = o.mask ? seg_run_block_kernel<T, LPR, true> : seg_run_block_kernel<T, LPR, false>;
             launch_pdl(chain, kern, grid_b, dim3(kAggThreads), smem, st, in, ld_in, ptr, idx, seg_of, n_seg_dev, run_len, d, sc.head2,
-                       sc.tail2, sc.win_info, sc.cap_runs, sc.chain_cnt, o);
+                       sc.tail2, sc.win_info, sc.cap_runs, sc.n_windows, sc.chain_cnt, o);
             if (sc.chain_cnt) {                   // chains, empty segments and padding were all done in that launch
                 tap_end(TAP_SEG_L1, st);
                 tap_begin(TAP_SEG_L3, st);        // (an armed tap of the second kernel reads zero)

@@ -425,7 +425,7 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
 #pragma unroll 1
         for (int rl = warp * kOwn; rl < (warp + 1) * kOwn; ++rl) {
             const int4 info = sh_info[rl];
-            seg_join_run<T, PtrT, LPR, CPL, 0>(sh_head, sh_tail, sh_info, sh_win, rl, kWalkRuns, lane, n_chunks, d, info.x, info.y, info.z,
+            seg_join_run<T, PtrT, LPR, CPL, 0>(sh_head, sh_tail, sh_info, sh_win, rl, kWalkRuns, blockIdx.x, lane, n_chunks, d, info.x, info.y, info.z,
                                                ptr, head2, tail2, o, nullptr, 0);
         }
     }
