@@ -274,18 +274,17 @@ static int32_t backward_impl(const e2egrec_block *blocks, int32_t n_layers, cons
     float *part = reinterpret_cast<float *>(scratch + bs.part_off);
     const bool chain = chain_blocks(blocks, n_layers);
 
-    // counters of the transposed aggregation (one per window of a block's entry stream); every launch leaves them zero
-    cudaMemsetAsync(scratch + bs.chain_off, 0, bs.chain_bytes, st);
-    // gradient entering the top layer, masked by its activation
+    // gradient entering the top layer, masked by its activation; and the counters of the transposed aggregation (one per window
+    // of a block's entry stream) cleared, which every launch of it leaves zero
     {
         const LayerPlan &p = plan[n_layers - 1];
         const e2egrec_block &b = blocks[p.block];
-        const int64_t total = p.rows * p.d_out;
+        const int64_t total = p.rows * (p.d_out / Chunk<T>::kElems);
         note_launch();
         launch_pdl(chain, relu_mask_kernel<T>, dim3((unsigned)std::max<int64_t>(1, ceil_div(total, 256)), (unsigned)n_rhs), dim3(256), 0, st,
-                   static_cast<const T *>(dH_out[0].data), dH_out[0].ld, reinterpret_cast<const T *>(ctx + p.h_off), (int64_t)p.d_out,
-                   &b.counts[CNT_DST], p.rows, p.d_out, act ? act[n_layers - 1] : 1, dz_buf[(n_layers - 1) & 1],
-                   static_cast<const T *>(dH_out[n_rhs - 1].data), dH_out[n_rhs - 1].ld);
+                   static_cast<const T *>(dH_out[0].data), dH_out[0].ld, reinterpret_cast<const T *>(ctx + p.h_off), &b.counts[CNT_DST],
+                   p.rows, p.d_out, act ? act[n_layers - 1] : 1, dz_buf[(n_layers - 1) & 1], static_cast<const T *>(dH_out[n_rhs - 1].data),
+                   dH_out[n_rhs - 1].ld, reinterpret_cast<uint4 *>(scratch + bs.chain_off), (int64_t)(bs.chain_bytes / 16));
     }
     SideStream *side = SideStream::get(st);
     cudaEvent_t dz_free[2] = {nullptr, nullptr};
