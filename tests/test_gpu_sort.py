@@ -125,3 +125,14 @@ def test_sample_whose_transposition_waits_run_out(impatient, monkeypatch):
         else:
             for k in ("csc_row", "csc_eid", "csc_col"):
                 assert torch.equal(got[k][:n_edges], ref[k][:n_edges])
+
+
+@pytest.mark.parametrize("m", [5000, 2 * 148 * 8192 + 100])
+def test_keys_that_neighbours_share(m):
+    """Warps that see one key, two keys in turn, and a hub in between others: what the ranking does with lanes of one digit."""
+    n, at = 70_000, np.arange(m)
+    rng = np.random.default_rng(m)
+    spread = rng.integers(0, n, m)
+    for row in (at // 40 % n, np.where(at % 2, 5, 66_000), np.where(rng.random(m) < 0.3, 1234, spread)):
+        check_ingest(n, row.astype(np.int32), spread.astype(np.int32))
+        check_ingest(n, spread.astype(np.int32), row.astype(np.int32))
