@@ -24,6 +24,7 @@
 // Together 11 warp instructions per row.  Tried and slower: rows through a cp.async ring in shared memory (4.57 ms
 // against 3.74 at the time: the copies and the reads of the ring load the L1 path to 86 %), two groups of rows in registers (5.18),
 // all segments by the whole warp (4.57), a row's registers loaded again as soon as it has been added (3.70 against 3.55),
+// the ids of the next short segments loaded before the rows of these (3.48 against 3.28: registers spilled),
 // stretches handed out by a counter (3.76 to 3.88: less waiting at the join's
 // barrier, more stretches to begin and to join).
 #pragma once
