@@ -287,7 +287,7 @@ static int32_t backward_impl(const e2egrec_block *blocks, int32_t n_layers, cons
                    dH_out[n_rhs - 1].ld, reinterpret_cast<uint4 *>(scratch + bs.chain_off), (int64_t)(bs.chain_bytes / 16));
     }
     SideStream *side = SideStream::get(st);
-    cudaEvent_t dz_free[2] = {nullptr, nullptr};
+    cudaEvent_t dz_free[2] = {nullptr, nullptr}, part_free = nullptr;
     for (int l = n_layers - 1; l >= 0; --l) {
         const LayerPlan &p = plan[l];
         const e2egrec_block &b = blocks[p.block];
@@ -297,12 +297,16 @@ static int32_t backward_impl(const e2egrec_block *blocks, int32_t n_layers, cons
         const int two_d = 2 * p.d_in;
         // dW_l = dZ^T [h | agg]   (split over the rows, partial sums added in a fixed order).  Nothing later in
         // this call reads dW, so it runs on the helper stream beside the dCat product and the transposed
-        // aggregation; `dz_free` holds the event after which the helper stream no longer reads a dZ buffer.
+        // aggregation; `dz_free` holds the event after which the helper stream no longer reads a dZ buffer, `part_free` the one
+        // after which it no longer uses the partial sums, of which there is one buffer.
         cudaStream_t ws = st;
         const bool dw_beside = side && (size_t)p.rows * (n_rhs * p.d_out + two_d) * sizeof(T) < dw_serial_bytes();
         if (dw_beside) {
             side->fork(st);
             ws = side->stream;
+        } else if (part_free) {                   // the layer above may still be adding up its partial sums
+            cudaStreamWaitEvent(st, part_free, 0);
+            part_free = nullptr;
         }
         if (l == 0) tap_begin(TAP_DW_OUTER, ws);
         bool dw_done = false;
@@ -341,6 +345,7 @@ static int32_t backward_impl(const e2egrec_block *blocks, int32_t n_layers, cons
         if (dw_beside) {
             dz_free[l & 1] = side->event();
             cudaEventRecord(dz_free[l & 1], side->stream);
+            part_free = dz_free[l & 1];
         }
         // dCat = dZ W_l, the agg half scaled by 1/|S|
         if (l == 0) tap_begin(TAP_DCAT_OUTER, st);

@@ -170,3 +170,39 @@ def test_without_helper_streams_the_results_are_the_same(tmp_path):
     want = [_joint_run(_joint_case(f, 200, torch.bfloat16), f, torch.bfloat16)[1] for f in ([5, 3], [3, 2, 2, 2])] + [_sage_run()]
     for a, b in zip(got, want):
         assert len(a) == len(b) and all(torch.equal(x, y.cpu()) for x, y in zip(a, b))
+
+
+@pytest.mark.parametrize("dtype,d", [(torch.bfloat16, 256), (torch.float32, 128)])
+def test_weight_gradients_on_two_streams_share_one_buffer_of_partial_sums(dtype, d):
+    """The bottom layer's product would move more than 256 MB by its block's capacity and stays on the caller's stream, the top
+    layer's runs on the helper stream behind the deferred transposition, and few rows are live: the bottom layer is soon there."""
+    n, batch, hidden = 250_000, 8192, 2 * d if dtype == torch.float32 else d
+    g = torch.Generator(device="cuda")
+    g.manual_seed(d)
+    ip, ix, _ = E.graph_from_coo(n, *(torch.randint(0, n, (n,), device="cuda", generator=g, dtype=torch.int32) for _ in range(2)))
+    X = torch.randn(n, d, device="cuda", generator=g).to(dtype)
+    Ws = [(0.1 * torch.randn(hidden, 2 * k, device="cuda", generator=g)).to(dtype) for k in (d, hidden)]
+    b = E.Blocks(n, batch, [25, 15], "cuda")
+    dH = torch.randn(batch, hidden, device="cuda", generator=g).to(dtype)
+    rows, es = b.caps[-1][0], X.element_size()
+    assert rows * (hidden + 2 * d) * es >= 256 << 20 > batch * 3 * hidden * es
+    H, ctx = E.sage_forward(_sampled(b, ip, ix, g, 0), X, Ws)
+    scratch = torch.empty(E.binding.sage_backward_scratch_bytes(b, X, Ws), dtype=torch.uint8, device="cuda")
+    dWs, dX = E.sage_backward(b, X, Ws, ctx, dH, scratch=scratch)
+    for step in range(1, 9):
+        _sampled(b, ip, ix, g, step)
+        E.sage_forward(b, X, Ws, ctx=ctx, H_out=H)
+        E.sage_backward(b, X, Ws, ctx, dH, dWs=dWs, dX_rows=dX, scratch=scratch)
+        torch.cuda.synchronize()
+        cat = E.binding.sage_ctx_views(b, X, Ws, ctx)[1][0][:batch].double()
+        dZ = dH.double() * (H > 0)
+        # no chain of additions is longer than the rows of a split and the splits: 8192 / 148 + 148, doubled for the tensor core's
+        # sums, which may truncate
+        bound = 512 * 2.0 ** -24 * (dZ.abs().T @ cat.abs())
+        assert bool(((dWs[1].double() - dZ.T @ cat).abs() <= bound).all()), step
+
+
+def _sampled(b, ip, ix, g, step):
+    seeds = torch.randperm(ip.numel() - 1, device="cuda", generator=g)[: b.caps[0][0]].to(torch.int32)
+    E.sample_khop(ip, ix, seeds, b, 77, step, defer_transpose=True)
+    return b
