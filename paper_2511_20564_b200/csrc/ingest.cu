@@ -138,8 +138,9 @@ expand_rows_kernel(const int64_t *__restrict__ indptr, int64_t n_rows, int64_t m
         const int after = __shfl_sync(0xffffffffu, beg_n, 0);    // where the row behind the window begins
         int end = __shfl_down_sync(0xffffffffu, beg, 1);
         if (lane == 31) end = after;
-        if (beg > 0 && beg < end && beg < len) mark[(beg >> 5) * kPad + (beg & 31)] = (int32_t)(base + lane);
-        if (after >= len || base + 32 >= n_rows) break;
+        const int32_t row = row_to_note(base + lane, n_rows, beg, end, len);
+        if (row >= 0) mark[(beg >> 5) * kPad + (beg & 31)] = row;
+        if (!more_rows(base, n_rows, after, len)) break;
         quiet = __any_sync(0xffffffffu, beg < end) ? 0 : quiet + 1;
         if (quiet < kQuietWindows) {
             base += 32;

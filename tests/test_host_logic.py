@@ -80,4 +80,40 @@ for (int64_t stuck : {int64_t(0), int64_t(40), n - 1}) {
 }
 if (window_found(int64_t(64), int64_t(500)) != 500) return 2;
 if (window_found(uint32_t(2147483647u), 0u) != 2147483679u) return 3;
-""", "stdint.h", "window.h")
+""", "window.h")
+
+
+def test_rows_of_entries_behind_the_last_offset(tmp_path):
+    """The row expansion's walk over 32 rows at a time, for offsets that end with the entries and for offsets that end before
+    them, with the last rows empty or not: every entry's row, and never one beyond the last."""
+    run_cpp(tmp_path, """
+for (int n_rows : {1, 31, 32, 33, 64, 100})
+    for (int tail : {0, 1, 40})                              // empty rows at the end
+        for (int extra : {0, 5, 200}) {                      // entries that the offsets do not cover
+            std::vector<int64_t> ptr(1, 0);
+            for (int r = 0; r < n_rows; ++r) ptr.push_back(ptr.back() + (r < n_rows - tail ? r % 4 : 0));
+            const int m = (int)ptr.back() + extra;
+            for (int k0 = 0; k0 < m; k0 += 48) {             // spans
+                const int len = std::min(48, m - k0);
+                int64_t base = 0;
+                while (base + 1 < n_rows && ptr[base + 1] <= k0) ++base;
+                std::vector<int32_t> row(len, -1);
+                row[0] = (int32_t)base;
+                auto begin = [&](int64_t r) { return r <= n_rows ? (int)std::max<int64_t>(std::min<int64_t>(ptr[r] - k0, 48), 0) : 48; };
+                for (;; base += 32) {
+                    for (int lane = 0; lane < 32; ++lane) {
+                        const int beg = begin(base + lane);
+                        const int32_t noted = row_to_note(base + lane, n_rows, beg, begin(base + lane + 1), len);
+                        if (noted >= 0) row[beg] = noted;
+                    }
+                    if (!more_rows(base, n_rows, begin(base + 32), len)) break;
+                }
+                for (int e = 0; e < len; ++e) {
+                    if (e && row[e] < 0) row[e] = row[e - 1];
+                    int64_t want = 0;
+                    while (want + 1 < n_rows && ptr[want + 1] <= k0 + e) ++want;
+                    if (row[e] != want) return 1;
+                }
+            }
+        }
+""", "algorithm", "vector", "window.h")
