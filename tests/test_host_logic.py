@@ -80,7 +80,7 @@ for (int64_t stuck : {int64_t(0), int64_t(40), n - 1}) {
 }
 if (window_found(int64_t(64), int64_t(500)) != 500) return 2;
 if (window_found(uint32_t(2147483647u), 0u) != 2147483679u) return 3;
-""", "window.h")
+""", "stdint.h", "window.h")
 
 
 def test_rows_of_entries_behind_the_last_offset(tmp_path):
