@@ -76,3 +76,29 @@ def test_host_side_argument_checks_of_the_newer_entry_points_need_no_gpu():
     assert L.e2egrec_blocks_transpose(0, 2, blocks, C.c_void_p(256), 1 << 20, None) == ERR_ARG
     assert L.e2egrec_blocks_transpose(5000, 2, blocks, C.c_void_p(264), 1 << 20, None) == -4         # scratch not 256-byte aligned
     assert L.e2egrec_blocks_transpose(5000, 2, blocks, C.c_void_p(256), 1 << 20, None) == ERR_NULL    # blocks without arrays
+
+
+def test_an_ingest_workspace_serves_shorter_edge_lists_any_ids_and_both_calls():
+    """A program keeps one workspace, made for its longest edge list, for all its ingest calls.  (A misaligned workspace of
+    sufficient size is refused for its alignment, before anything is enqueued: the size check let it pass.)"""
+    import paper_2511_20564_b200 as E
+    L = E.lib()
+    ws, n_ws = ctypes.c_void_p(8), ctypes.c_size_t
+
+    def coo(n, m, size=None):
+        b = n_ws(size or 0)
+        rc = L.e2egrec_graph_from_coo(n, m, None, None, None, None, None, ws if size else None, ctypes.byref(b), None)
+        return rc if size else b.value
+
+    def csc(n, m, size=None):
+        b, g = n_ws(size or 0), E.binding.Csr(7, m, None, None, None)
+        rc = L.e2egrec_csr_transpose(ctypes.byref(g), n, None, None, None, None, ws if size else None, ctypes.byref(b), None)
+        return rc if size else b.value
+
+    nodes = [1, 300, 1 << 10, 1 << 16, 1 << 20, 1 << 24, (1 << 24) + 1, (1 << 31) - 1]
+    entries = [0, 1, 5000, 2_424_831, 2_424_832, 4_000_000, 20_000_000, (1 << 31) - 2]
+    for i, m in enumerate(entries):
+        for size in {f(n, m) for n in nodes for f in (coo, csc)}:
+            for n in nodes:
+                for shorter in entries[: i + 1]:
+                    assert coo(n, shorter, size) == csc(n, shorter, size) == -4, (n, m, shorter, size)
