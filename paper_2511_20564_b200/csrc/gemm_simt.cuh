@@ -17,10 +17,10 @@
 
 namespace e2egrec {
 
-// gemm_simt_kernel, for bf16 operands (fp32 ones: gemm_async_kernel below).  At the sizes of a batch the time is the K loop's
-// chain of loads, not its arithmetic: the next 64 x 32 tiles are loaded into registers (four values at a time where rows are
-// aligned) while the current ones are multiplied out of shared memory, two buffers, one barrier per step.  Loading, storing and
-// multiplying in turn with steps of 16 took 1.7 us a step.
+// gemm_simt_kernel, for bf16 operands and large fp32 products (the others: gemm_async_kernel below).  At the sizes of a batch the
+// time is the K loop's chain of loads, not its arithmetic: the next 64 x 32 tiles are loaded into registers (four values at a
+// time where rows are aligned) while the current ones are multiplied out of shared memory, two buffers, one barrier per step.
+// Loading, storing and multiplying in turn with steps of 16 took 1.7 us a step.
 constexpr int kGemmBM = 64, kGemmBN = 64, kGemmBK = 32, kGemmThreads = 256;
 
 // four values from p on, `n` of them there
@@ -169,7 +169,8 @@ gemm_simt_kernel(const T *A, int64_t lda, const T *B, int64_t ldb, int64_t M_hos
 
 // The same product of fp32 operands, for batches whose few tiles leave most of an SM idle: the tiles are copied to shared memory
 // asynchronously, as they lie in memory (rows of k, or lines of k), kGemmStages - 1 K steps ahead, and two groups of 256
-// threads take half of every K step each; their sums are added at the end.  What bounds it is latency at 16 warps per SM.
+// threads take half of every K step each; their sums are added at the end.  What bounds it is latency at 16 warps per SM (products
+// of the forward pass, 86 registers) or 32 (the others, 64 registers).
 // B200, fp32 step of 777 seeds at fanouts 25, 15, 100 and 72 values, its six products together (us) and the step: loads through
 // registers one step ahead, one group 88, 163; copies, one group 74, 154; two groups 144; four groups (64 registers, spills) 166;
 // 128 threads of 8 x 4 values instead of 256 of 4 x 4 164.  No chain of additions is longer than in gemm_simt_kernel.
@@ -310,24 +311,32 @@ gemm_async_kernel(const float *A, int64_t lda, const float *B, int64_t ldb, int6
         }
 }
 
+// Which of the two takes an fp32 product.  The asynchronous one needs tiles that wait for their loads: up to 65536 rows of capacity
+// (as M or as K) and, in products over rows, 4096 tiles.  Beyond, tiles hide each other's loads, and most of them hold no live row
+// at all: one or two blocks of 512 threads per SM, four of the other kernel's 256, have to come and go for those.  B200, us by
+// the asynchronous / the other kernel: forward of 2048 and 8192 seeds of 256 values at fanouts 15, 10 (32768 and 131072 rows) 155 / 173
+// and 393 / 369, training step of 2048 and 8192 seeds of 128 values 169 / 188 and 377 / 348, of 4096 seeds of 64 at 25, 15 185 / 167.
+constexpr int64_t kAsyncRows = 65536, kAsyncTiles = 4096;
 template <typename T, bool A_KM, bool B_KN, class Epi>
 inline void launch_gemm_simt(bool chain, dim3 grid, cudaStream_t st, const T *A, int64_t lda, const T *B, int64_t ldb, int64_t M, int N,
                              int64_t K, const int32_t *m_dev, const int32_t *k_dev, const Epi &epi)
 {
     note_launch();
     if constexpr (sizeof(T) == 4) {
-        constexpr size_t smem = gemm_async_smem<A_KM, B_KN>();
-        static std::atomic<bool> set[64] = {};                   // per device; two threads may both raise the limit
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (dev < 0 || dev >= 64 || !set[dev].load(std::memory_order_relaxed)) {
-            cudaFuncSetAttribute(gemm_async_kernel<A_KM, B_KN, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (dev >= 0 && dev < 64) set[dev].store(true, std::memory_order_relaxed);
+        if (A_KM ? K <= kAsyncRows : M <= kAsyncRows && (int64_t)grid.x * grid.y <= kAsyncTiles) {
+            constexpr size_t smem = gemm_async_smem<A_KM, B_KN>();
+            static std::atomic<bool> set[64] = {};               // per device; two threads may both raise the limit
+            int dev = 0;
+            cudaGetDevice(&dev);
+            if (dev < 0 || dev >= 64 || !set[dev].load(std::memory_order_relaxed)) {
+                cudaFuncSetAttribute(gemm_async_kernel<A_KM, B_KN, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                if (dev >= 0 && dev < 64) set[dev].store(true, std::memory_order_relaxed);
+            }
+            launch_pdl(chain, gemm_async_kernel<A_KM, B_KN, Epi>, grid, dim3(kAsyncThreads), smem, st, A, lda, B, ldb, M, N, K, m_dev, k_dev, epi);
+            return;
         }
-        launch_pdl(chain, gemm_async_kernel<A_KM, B_KN, Epi>, grid, dim3(kAsyncThreads), smem, st, A, lda, B, ldb, M, N, K, m_dev, k_dev, epi);
-    } else {
-        launch_pdl(chain, gemm_simt_kernel<T, A_KM, B_KN, Epi>, grid, dim3(kGemmThreads), 0, st, A, lda, B, ldb, M, N, K, m_dev, k_dev, epi);
     }
+    launch_pdl(chain, gemm_simt_kernel<T, A_KM, B_KN, Epi>, grid, dim3(kGemmThreads), 0, st, A, lda, B, ldb, M, N, K, m_dev, k_dev, epi);
 }
 
 // Splits over `rows` (a capacity) of an m x n weight gradient on this kernel, at most `most` (148): two blocks per SM over all

@@ -55,3 +55,14 @@ def test_weight_gradients_over_many_rows(rows, d, hidden):
     want = dH.double().T @ cat.double()
     err = float((dWs[0].double() - want).norm() / want.norm())
     assert err <= 0.5 * EPS * (148 + rows / 148) ** 0.5 + EPS, err
+
+
+@pytest.mark.parametrize("rows,d", [(65_536, 256), (65_536, 257), (65_537, 33), (70_000, 4)])
+def test_gate_in_fp32_where_the_kernels_change(rows, d):
+    """The last products of the asynchronous kernel and the first of the other one, by rows and by tiles."""
+    test_gate_in_fp32(rows, d)
+
+
+@pytest.mark.parametrize("rows,d,hidden", [(65_536, 64, 128), (65_537, 64, 128), (90_000, 100, 72)])
+def test_weight_gradients_where_the_kernels_change(rows, d, hidden):
+    test_weight_gradients_over_many_rows(rows, d, hidden)
