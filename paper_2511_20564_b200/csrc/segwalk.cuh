@@ -119,9 +119,10 @@ template <int LPR, int CPL, int E> __host__ __device__ constexpr size_t walk_sme
     return (size_t)2 * kWalkRuns * LPR * CPL * E * sizeof(float) + kWalkRuns * sizeof(int4);
 }
 
-// win_len: entries of a window (block), a multiple of kWalkRuns; cap: entries that the arrays hold, at least.
-template <typename T, typename PtrT, int LPR, int CPL, bool kWeight, int kWalkWarps>
-__global__ void __launch_bounds__(kWalkWarps * 32, CPL > 1 ? 1 : 32 / kWalkWarps)
+// win_len: entries of a window (block), a multiple of kWalkRuns; cap: entries that the arrays hold, at least; kWide: rows lie
+// 4 GB or more apart.
+template <typename T, typename PtrT, int LPR, int CPL, bool kWeight, int kWalkWarps, bool kWide>
+__global__ void __launch_bounds__(kWalkWarps * 32, CPL > 4 ? 2 : CPL > 1 ? 1 : 32 / kWalkWarps)
 seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict__ ptr, const int32_t *__restrict__ idx,
                 const int32_t *n_seg_dev, int64_t n_seg_host, const float *__restrict__ w, int win_len, int64_t cap, int d,
                 float *__restrict__ head2, float *__restrict__ tail2, int4 *__restrict__ win_info, SegOut<T> o)
@@ -132,7 +133,10 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
     constexpr int C = G * U;                                     // entries per group, a divisor of 32
     constexpr int S = walk_share<LPR, E>();
     constexpr int ROW = LPR * CPL * E;
-    constexpr int kUnrollGroups = 4 < 32 / C ? 4 : 32 / C;       // groups of 32 entries that are written out
+    // Groups of 32 entries that are written out.  Rows that a lane reads in several parts have enough loads in flight with one: four
+    // took 141 instead of 80 registers, one block per SM instead of three (10^7 entries of 256 fp32 values and the transpose 2.68 ms,
+    // 1.76 with one; two blocks of the widest rows, up to 128 registers, 0.81 where one took 1.15 for 1.2 M entries of 1024).
+    constexpr int kUnrollGroups = CPL > 1 ? 1 : 4 < 32 / C ? 4 : 32 / C;
     constexpr int kFar = 1 << 30;
     static_assert(32 % C == 0, "a group takes its ids from one window of 32");
     extern __shared__ float4 seg_smem[];
@@ -167,12 +171,13 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
         for (int q = 0; q < CPL; ++q) in_c[q] = reinterpret_cast<const uint8_t *>(in) + (size_t)min(c + q * LPR, n_chunks - 1) * 16;
         const uint64_t ld_bytes = (uint64_t)ld_in * sizeof(T);
         const uint32_t ld_lo = (uint32_t)ld_bytes, ld_hi = (uint32_t)(ld_bytes >> 32);
-        // a row's address: one wide product with the lane's chunk as its addend, and the upper half of a stride of 4 GB and more
-        auto load_row = [&](int32_t id, uint4 (&v)[CPL], auto wide) {
+        // a row's address: one wide product with the lane's chunk as its addend (a stride of 4 GB and more has an upper half too: in
+        // kernels of their own, beside the others it cost registers)
+        auto load_row = [&](int32_t id, uint4 (&v)[CPL]) {
 #pragma unroll
             for (int q = 0; q < CPL; ++q) {
                 uint64_t at = (uint64_t)(uint32_t)id * ld_lo + reinterpret_cast<uint64_t>(in_c[q]);
-                if constexpr (decltype(wide)::value) at += (uint64_t)((uint32_t)id * ld_hi) << 32;
+                if constexpr (kWide) at += (uint64_t)((uint32_t)id * ld_hi) << 32;
                 v[q] = __ldg(reinterpret_cast<const uint4 *>(at));
             }
         };
@@ -257,7 +262,7 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
                             for (int q = 0; q < CPL; ++q) v[u][q] = make_uint4(0, 0, 0, 0);
                             if (on[u]) {
                                 if (kWeight) wt[u] = __ldg(w + id[u]);
-                                load_row(id[u], v[u], std::true_type());
+                                load_row(id[u], v[u]);
                             }
                         }
 #pragma unroll
@@ -304,7 +309,7 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
                     for (int c0 = 0; c0 < cnt; c0 += U) {
                         uint4 v[U][CPL];
 #pragma unroll
-                        for (int u = 0; u < U; ++u) load_row(__shfl_sync(0xffffffffu, id, c0 + u), v[u], std::true_type());
+                        for (int u = 0; u < U; ++u) load_row(__shfl_sync(0xffffffffu, id, c0 + u), v[u]);
 #pragma unroll
                         for (int u = 0; u < U; ++u) {
                             if (c0 + u >= cnt) break;            // uniform over the warp, as is the next condition
@@ -338,41 +343,45 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
                 int32_t id_cur = load_id(0), id_1 = load_id(32);
                 float w_cur = kWeight ? __ldg(w + id_cur) : 0.f;
                 clear();
-                auto walk = [&](auto wide) {
-                    for (int b = 0; b < sn; b += 32) {
-                        const int32_t id_2 = b + 32 < sn ? load_id(b + 64) : 0;
-                        const float w_1 = kWeight && b + 32 < sn ? __ldg(w + id_1) : 0.f;
-                        auto load_group = [&](int c0, uint4 (&v)[U][CPL]) {
+                for (int b = 0; b < sn; b += 32) {
+                    const int32_t id_2 = b + 32 < sn ? load_id(b + 64) : 0;
+                    const float w_1 = kWeight && b + 32 < sn ? __ldg(w + id_1) : 0.f;
+                    auto load_group = [&](int c0, uint4 (&v)[U][CPL]) {
 #pragma unroll
-                            for (int u = 0; u < U; ++u) load_row(__shfl_sync(0xffffffffu, id_cur, c0 + u * G + sub), v[u], wide);
-                        };
-                        auto weight = [&](int e) -> float { return kWeight ? __shfl_sync(0xffffffffu, w_cur, e) : 1.f; };
-                        if (b + 32 <= sn) {                      // 32 entries: no tests
+                        for (int u = 0; u < U; ++u) load_row(__shfl_sync(0xffffffffu, id_cur, c0 + u * G + sub), v[u]);
+                    };
+                    auto weight = [&](int e) -> float { return kWeight ? __shfl_sync(0xffffffffu, w_cur, e) : 1.f; };
+                    // 32 entries without tests; fewer, or where 32 are one group, a test per group first: segments of small inputs are
+                    // mostly cut within 32 (60 k nodes, 10^6 entries, 32 bf16 values, two layers and back 178 us with tests per
+                    // entry there, 172)
+                    if (C < 32 && b + 32 <= sn) {
 #pragma unroll kUnrollGroups
-                            for (int c0 = 0; c0 < 32; c0 += C) {
-                                uint4 v[U][CPL];
-                                load_group(c0, v);
+                        for (int c0 = 0; c0 < 32; c0 += C) {
+                            uint4 v[U][CPL];
+                            load_group(c0, v);
+#pragma unroll
+                            for (int u = 0; u < U; ++u) add_row(v[u], weight(c0 + u * G + sub), true);
+                        }
+                    } else {
+#pragma unroll 1
+                        for (int c0 = 0; c0 < 32 && b + c0 < sn; c0 += C) {
+                            uint4 v[U][CPL];
+                            load_group(c0, v);
+                            if (b + c0 + C <= sn) {
 #pragma unroll
                                 for (int u = 0; u < U; ++u) add_row(v[u], weight(c0 + u * G + sub), true);
-                            }
-                        } else {
-#pragma unroll 1
-                            for (int c0 = 0; b + c0 < sn; c0 += C) {
-                                uint4 v[U][CPL];
-                                load_group(c0, v);
+                            } else {
 #pragma unroll
                                 for (int u = 0; u < U; ++u)
                                     if (b + c0 + u * G < sn)     // uniform over the warp
                                         add_row(v[u], weight(c0 + u * G + sub), b + c0 + u * G + sub < sn);
                             }
                         }
-                        id_cur = id_1;
-                        id_1 = id_2;
-                        w_cur = w_1;
                     }
-                };
-                if (ld_hi == 0) walk(std::false_type());
-                else walk(std::true_type());
+                    id_cur = id_1;
+                    id_1 = id_2;
+                    w_cur = w_1;
+                }
                 int off = 0;
 #pragma unroll
                 for (int q = 0; q < CPL; ++q) {
@@ -436,13 +445,13 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
 
 // B200: 5 M nodes, 10^8 entries, 64 bf16 values, forward and transposed 3.73 -> 3.26 ms (8.6 TB/s of gathered rows);
 // 500 k nodes, 2 * 10^7 entries, 64 fp32 values, weighted, per layer 0.45 -> 0.41 ms (12.5 TB/s).
-template <typename T, typename PtrT, int LPR, int CPL, bool kWeight, int kWalkWarps>
+template <typename T, typename PtrT, int LPR, int CPL, bool kWeight, int kWalkWarps, bool kWide>
 inline void launch_seg_walk(const T *in, int64_t ld_in, const PtrT *ptr, const int32_t *idx, const int32_t *n_seg_dev,
                             int64_t n_seg_host, int64_t cap_seg, const float *w, int run_len, int d, const SegScratch &sc,
                             const SegOut<T> &o, cudaStream_t st)
 {
     constexpr size_t smem = walk_smem_bytes<LPR, CPL, Chunk<T>::kElems>();
-    auto kern = seg_walk_kernel<T, PtrT, LPR, CPL, kWeight, kWalkWarps>;
+    auto kern = seg_walk_kernel<T, PtrT, LPR, CPL, kWeight, kWalkWarps, kWide>;
     if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     tap_begin(TAP_SEG_L1, st);
     note_launch();
@@ -453,8 +462,8 @@ inline void launch_seg_walk(const T *in, int64_t ld_in, const PtrT *ptr, const i
     launch_seg_final(ptr, n_seg_dev, n_seg_host, cap_seg, run_len, d, sc, o, st);
 }
 
-// Four warps with two stretches each for rows of up to 128 bytes of large inputs, eight with one otherwise: 10^8 entries of 128-byte
-// rows 3.29 and 3.41 ms, three layers of 2 * 10^7 entries of 256-byte rows 2.83 and 2.76.
+// Four warps with two stretches each for rows of up to 128 bytes of large inputs (offsets of sampled blocks never are), eight
+// with one otherwise: 10^8 entries of 128-byte rows 3.29 and 3.41 ms, three layers of 2 * 10^7 entries of 256-byte rows 2.83 and 2.76.
 // Same contract as dispatch_seg_reduce, without an entry -> segment array, self rows or masks.
 template <typename T, typename PtrT, bool kWeight>
 inline bool dispatch_seg_walk(const T *in, int64_t ld_in, const PtrT *ptr, const int32_t *idx, const int32_t *n_seg_dev,
@@ -462,12 +471,21 @@ inline bool dispatch_seg_walk(const T *in, int64_t ld_in, const PtrT *ptr, const
                               const SegScratch &sc, const SegOut<T> &o, cudaStream_t st)
 {
     const RowShape rs = row_shape(d, dtype);
+    const bool wide = (uint64_t)ld_in * sizeof(T) >> 32 != 0;
+#define E2E_WALK(L, C, WARPS, WIDE)                                                                                         \
+    launch_seg_walk<T, PtrT, L, C, kWeight, WARPS, WIDE>(in, ld_in, ptr, idx, n_seg_dev, n_seg_host, cap_seg, w, run_len, d, sc, o, st)
 #define E2E_CASE(L, C)                                                                                                      \
     if (rs.lpr == L && rs.cpl == C) {                                                                                       \
-        if (L <= 8 && run_len >= 256)                                                                                       \
-            launch_seg_walk<T, PtrT, L, C, kWeight, L <= 8 ? 4 : 8>(in, ld_in, ptr, idx, n_seg_dev, n_seg_host, cap_seg, w, run_len, d, sc, o, st); \
-        else                                                                                                                \
-            launch_seg_walk<T, PtrT, L, C, kWeight, 8>(in, ld_in, ptr, idx, n_seg_dev, n_seg_host, cap_seg, w, run_len, d, sc, o, st); \
+        if (wide) {                                                                                                         \
+            E2E_WALK(L, C, 8, true);                                                                                        \
+            return true;                                                                                                    \
+        }                                                                                                                   \
+        if constexpr (L <= 8 && sizeof(PtrT) == 8)                                                                          \
+            if (run_len >= 256) {                                                                                           \
+                E2E_WALK(L, C, 4, false);                                                                                   \
+                return true;                                                                                                \
+            }                                                                                                               \
+        E2E_WALK(L, C, 8, false);                                                                                           \
         return true;                                                                                                        \
     }
     E2E_CASE(4, 1) E2E_CASE(8, 1) E2E_CASE(16, 1) E2E_CASE(32, 1) E2E_CASE(32, 2) E2E_CASE(32, 4)
@@ -475,6 +493,7 @@ inline bool dispatch_seg_walk(const T *in, int64_t ld_in, const PtrT *ptr, const
         E2E_CASE(32, 8)
     }
 #undef E2E_CASE
+#undef E2E_WALK
     return false;
 }
 
