@@ -462,8 +462,14 @@ inline void launch_seg_walk(const T *in, int64_t ld_in, const PtrT *ptr, const i
     launch_seg_final(ptr, n_seg_dev, n_seg_host, cap_seg, run_len, d, sc, o, st);
 }
 
-// Four warps with two stretches each for rows of up to 128 bytes of large inputs (offsets of sampled blocks never are), eight
-// with one otherwise: 10^8 entries of 128-byte rows 3.29 and 3.41 ms, three layers of 2 * 10^7 entries of 256-byte rows 2.83 and 2.76.
+// Four warps with two stretches each, of which fewer wait before the join, or eight with one.  Four pay for rows of 65 to 128 bytes
+// once so many windows follow one another that a block's begin and end count less than the wait.  B200, ms with four / eight, mean and
+// transpose, 64 bf16 values: 2 * 10^7 entries of 500 k rows 0.70 / 0.65, 2.5 * 10^7 of 2.5 M 1.23 / 1.17, 5 * 10^7 of 1, 2.5 and 5 M
+// 1.38 / 1.39, 1.73 / 1.74 and 2.15 / 2.20, 10^8 of 1, 5 and 10 M 2.26 / 2.37, 3.19 / 3.35 and 4.01 / 4.20; 32 fp32 values, 5 * 10^7 1.57 / 1.56,
+// 10^8 2.89 / 3.01.  Narrower rows, whose stretches hold fewer loads: 3 * 10^7 of 32 bf16 values 1.20 / 1.06, 10^8 2.44 / 2.43; wider ones,
+// three layers of 2 * 10^7 entries of 256 bytes, 2.83 / 2.76.
+constexpr int64_t kWalkPaired = 48'000'000;          // entries
+
 // Same contract as dispatch_seg_reduce, without an entry -> segment array, self rows or masks.
 template <typename T, typename PtrT, bool kWeight>
 inline bool dispatch_seg_walk(const T *in, int64_t ld_in, const PtrT *ptr, const int32_t *idx, const int32_t *n_seg_dev,
@@ -480,8 +486,8 @@ inline bool dispatch_seg_walk(const T *in, int64_t ld_in, const PtrT *ptr, const
             E2E_WALK(L, C, 8, true);                                                                                        \
             return true;                                                                                                    \
         }                                                                                                                   \
-        if constexpr (L <= 8 && sizeof(PtrT) == 8)                                                                          \
-            if (run_len >= 256) {                                                                                           \
+        if constexpr (L == 8 && sizeof(PtrT) == 8)                                                                          \
+            if (sc.cap_runs * run_len >= kWalkPaired) {                                                                     \
                 E2E_WALK(L, C, 4, false);                                                                                   \
                 return true;                                                                                                \
             }                                                                                                               \

@@ -112,3 +112,32 @@ def test_upstream_gradients_on_no_boundary(dtype, hidden):
     (dW2,), dX2 = E.sage_backward_multi(b, X, [W], ctx, [h.contiguous() for h in dHs])
     assert torch.equal(dW1, dW2) and all(torch.equal(p, q) for p, q in zip(dX1, dX2))
     assert not np.array_equal(dX1[0].float().cpu().numpy(), dX1[1].float().cpu().numpy())
+
+
+@pytest.mark.parametrize("dtype,d,m", [("bf16", 64, 48_000_000), ("bf16", 40, 50_000_001), ("f32", 20, 48_000_001), ("f32", 32, 47_999_000)])
+def test_windows_that_four_warps_share(dtype, d, m):
+    """As many entries as take two stretches per warp, and one window less: hubs, short and empty segments, exact sums."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(d)
+    n, n_rows = 1_200_000, 3000
+    lens = torch.randint(0, 30, (n,), device="cuda", generator=g)
+    lens[::7] = 0
+    lens[5::1000] = 4000
+    lens[[3, 77, n // 2]] = torch.tensor([2_000_000, 8191, 1025], device="cuda")
+    lens[n - 1] = 0
+    lens[n - 1] = m - lens.sum()
+    assert int(lens[n - 1]) > 1_000_000
+    ptr = torch.zeros(n + 1, dtype=torch.int64, device="cuda")
+    ptr[1:] = torch.cumsum(lens, 0)
+    idx = torch.randint(0, n_rows, (m,), device="cuda", generator=g, dtype=torch.int32)
+    X = torch.randint(-4, 5, (n_rows, d), device="cuda", generator=g).to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    w = torch.randint(1, 3, (n_rows,), device="cuda", generator=g).float()
+    # prefix sums of whole numbers of up to 8 are exact in 64 bits; sums below 2^24 are exact in 32, in any order
+    ids, run = idx.long(), torch.zeros(m + 1, dtype=torch.float64, device="cuda")
+    for scale, out in ((None, E.aggregate_forward(ptr, idx, X, sum_only=True)[0]), (w, E.aggregate_backward(ptr, idx, w, X)[0])):
+        for c in range(d):
+            column = X[:, c].double() if scale is None else X[:, c].double() * scale.double()
+            torch.cumsum(column[ids], 0, out=run[1:])
+            want = run[ptr[1:]] - run[ptr[:-1]]
+            assert float(want.abs().max()) < 2 ** 24
+            assert torch.equal(out[:, c].double(), want.to(out.dtype).double()), c
