@@ -26,8 +26,9 @@ struct IngestScratch {
 SortPlan plan_for(int64_t key_range) { return sort_plan((int32_t)std::min<int64_t>(std::max<int64_t>(key_range, 2), 0x7fffffff)); }
 
 // n_sorts sorts of m entries by `sp`: digit counts and scan state of what these will use lie together, to be zeroed at once
-// (all that the size provides for: 80 MB and 14 us at 2 * 10^7 entries).  The size goes by m alone and grows with it, so that a
-// workspace serves shorter lists, other id ranges and the other call: two sorts, state for any digits of the smaller tiles.
+// (zeroing the smaller tiles' state for two sorts, 80 MB, took 14 us at 2 * 10^7 entries).  The size goes by m alone and grows with
+// it, so that a workspace serves shorter lists, other id ranges and the other call: two sorts, state for any digits and for the tiles of
+// whichever list up to m has most.
 IngestScratch carve_ingest(int64_t m, const SortPlan &sp, int n_sorts, void *base)
 {
     IngestScratch s{};
@@ -51,8 +52,8 @@ IngestScratch carve_ingest(int64_t m, const SortPlan &sp, int n_sorts, void *bas
         ss.state = (unsigned *)take(sizeof(unsigned) * (size_t)sp.passes * (size_t)tiles << sp.bits);
     }
     s.zero_bytes = off - begin;
-    s.bytes = begin + 2 * (align_up(kSortCountWords * sizeof(unsigned), 256) +
-                           align_up(sort_state_bytes(ceil_div((int64_t)mm, (int64_t)kSortTile)), 256));
+    const int64_t most = std::max(ceil_div(std::min<int64_t>((int64_t)mm, kSortWide - 1), (int64_t)kSortTile), ceil_div((int64_t)mm, kSortWideTile));
+    s.bytes = begin + 2 * (align_up(kSortCountWords * sizeof(unsigned), 256) + align_up(sort_state_bytes(most), 256));
     return s;
 }
 
