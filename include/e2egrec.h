@@ -138,7 +138,8 @@ int32_t e2egrec_profile_tap(int32_t which, void *start_event, void *stop_event);
  * e2egrec_csr_transpose: the CSC of a CSR with n_cols columns: csc_ptr device int64[n_cols+1]; for every
  * transposed entry csc_row int32 (its row) and csc_eid int64 (its CSR position), entries of a column in
  * CSR order.  status: optional device int32, receives E2EGREC_DEV_RANGE if an id was out of range (such
- * ids are treated as 0) and E2EGREC_DEV_TIMEOUT if a wait of the sort ran out.  ws: scratch (size query with ws == NULL).  Limits: n_edges < 2^31 - 1. */
+ * ids are treated as 0) and E2EGREC_DEV_TIMEOUT if a wait of the sort ran out.  ws: scratch (size query with ws == NULL; the size
+ * goes by n_edges alone and grows with it: one buffer serves both calls and shorter lists).  Limits: n_edges < 2^31 - 1. */
 int32_t e2egrec_graph_from_coo(int64_t n_nodes, int64_t n_edges, const int32_t *row, const int32_t *col,
                                int64_t *indptr, int32_t *indices, int32_t *status, void *ws, size_t *ws_bytes,
                                void *stream);

@@ -90,7 +90,8 @@ __device__ inline int chain_ticket(unsigned *ticket, int *bcast)
 
 
 // ---------------------------------------------------------------------------------------
-// Stable LSD radix sort, one launch per digit.  A block takes a tile of consecutive elements, ranks the equal digits in
+// Stable LSD radix sort, one launch per digit (the published method of single-pass scans with decoupled look-back, Merrill and
+// Garland, applied to a pass's digits, Adinets and Merrill; the code is this file's own).  A block takes a tile of consecutive elements, ranks the equal digits in
 // element order (per warp, see kRank..., then across warps), publishes its digit counts and looks back over the tiles
 // before it, digit by digit, until it meets one whose full prefix is known -- the chained scan above with one chain per
 // digit.  The words of a chain tell their kind by themselves: 0 not there yet, count + 1 a tile's own count, top bit set
@@ -121,7 +122,8 @@ constexpr unsigned kPosFlag = 0x80000000u;
 // How the warp ranks equal digits.  kRankMatch: by match_any, whose time goes with the number of different digits in the
 // warp.  kRankSpread, for passes whose neighbouring elements mostly differ in their digits: counts by shared-memory atomics, and
 // a match only among the lanes whose digit was counted more than once.  kRankAny: elements of a digit may leave in any order, the
-// atomics' result is the rank.  B200, 2 * 10^7 pairs, 1024 digits, us a pass by match / spread / any: ids of random order 203 /
+// atomics' result is the rank.  Counters are words of two halves: the atomics work on words, which cannot carry (a tile has fewer
+// than 2^16 elements), everything else on halves, and between the two there is always a __syncwarp or a barrier.  B200, 2 * 10^7 pairs, 1024 digits, us a pass by match / spread / any: ids of random order 203 /
 // 158 / 137, the second digits of such a sort (hubs in runs: lanes that count the same digit wait for one another) 145 / 172.
 enum { kRankMatch, kRankSpread, kRankAny };
 

@@ -519,8 +519,8 @@ seg_run_kernel(const T *__restrict__ in, int64_t ld_in, const int32_t *__restric
 // offsets), which takes the instructions per entry from ~110 to ~35: with two entries per segment on average the
 // general kernel was bound by instruction issue, not by memory.
 // What is left is instructions: two entries per segment on average, so every second entry closes a segment, rounds and
-// stores a row.  Row addresses by two 32-bit products, loads without tests (ids beyond the run and lanes beyond the row
-// repeat the last ones) and a mask taken two values at a time took the outer blocks of the largest training step from 54,
+// stores a row.  Row addresses by two 32-bit products (one wide one now), loads without tests (ids beyond the run and lanes beyond
+// the row repeat the last ones) and a mask taken two values at a time took the outer blocks of the largest training step from 54,
 // 218 and 213 us to 41, 149 and 180 (bf16 rows of 512 bytes, B200).  One wave of blocks goes over the windows: with a block per
 // window of the capacity nine tenths of the blocks found none, took two dependent loads to see it and looked after a few segments
 // without entries each; the segments without entries are looked for 32 to a warp (per pass: large step 1202 -> 1166 us, two-task

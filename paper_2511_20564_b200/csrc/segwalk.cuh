@@ -6,13 +6,14 @@
 // the kernel that joins them are those of segreduce.cuh; a window is cut into one stretch of consecutive entries per
 // warp of the block.
 //
-// What bounds it: instructions (rows that L2 serves: issue slots 65 % busy, L1 hit 2 %) and, on power-law graphs, the barrier before the
-// join and the latency of rows that L2 does not hold (issue slots 54 %; B200, 128-byte rows).  A bf16 row is added without being
-// widened first and its address is one product: 10^8 entries of 64 bf16 values and the transpose, weighted, 3.75 -> 3.30 ms; 32 entries
-// of a long segment without tests 3.16, with stretches twice as long, whose longer sums however doubled the rounding error; with two
-// stretches per warp 3.26.  Before that, too, instructions were what it could be sped up by.  With one lane group per run, 32 / LPR
-// runs per warp each with its own segment ends, a 128-byte row took 22 warp instructions, most of them bookkeeping that the warp executes for all of its groups' different positions.  Here the
-// offsets come 32 segments at a time, one lane each, and the segments are handled by their length:
+// What bounds it: instructions and the latency of the rows (sources that L2 serves: issue slots 57 % busy, 7.6 warps waiting for loads
+// per issue) and, on power-law graphs, as much the barrier before the join (issue slots 50 %, 4.6 waiting for loads, 4.2 at the
+// barrier; 2 * 10^7 entries of 128-byte rows, B200).
+// A bf16 row is added without being widened first and its address is one product, and 32 entries of a long segment take no tests:
+// 10^8 entries of 64 bf16 values and the transpose, weighted, 3.75 -> 3.19 ms (with stretches twice as long 3.16 at the time, but
+// their longer sums doubled the rounding error).  With one lane group per run, 32 / LPR runs per warp each with its own
+// segment ends, a 128-byte row took 22 warp instructions, most of them bookkeeping that the warp executes for all of its groups'
+// different positions.  Here the offsets come 32 segments at a time, one lane each, and the segments are handled by their length:
 //   - longer ones by the whole warp: 32 entry ids in one coalesced load (the next 32 and the entry weights on their way),
 //     steps of 32 / LPR rows with no test per entry, and one sum across the lane groups per segment that halves the row at
 //     every exchange, so that every lane stores its own share of the finished row;
@@ -21,19 +22,18 @@
 //     ids and weights come 32 at a time and four rows are in flight whatever the segments' lengths (one after another,
 //     2 M segments of two entries on average took 719 and, weighted, 857 us with 256 bf16 values, 824 with 100 fp32 values;
 //     now 578, 655 and 577).
-// Together 11 warp instructions per row.  Tried and slower: rows through a cp.async ring in shared memory (4.57 ms
-// against 3.74 at the time: the copies and the reads of the ring load the L1 path to 86 %), two groups of rows in registers (5.18),
-// all segments by the whole warp (4.57), a row's registers loaded again as soon as it has been added (3.70 against 3.55),
-// the ids of the next short segments loaded before the rows of these (3.48 against 3.28: registers spilled),
-// stretches handed out by a counter (3.76 to 3.88: less waiting at the join's
-// barrier, more stretches to begin and to join).
+// Together 5.6 warp instructions per row where segments are long and 10 on a power-law graph with weights.  Tried and slower:
+// rows through a cp.async ring in shared memory (4.57 ms against 3.74 at the time: the copies and the reads of the ring load the L1
+// path to 86 %), two groups of rows in registers (5.18), all segments by the whole warp (4.57), a row's registers loaded again as
+// soon as it has been added (3.70 against 3.55), the ids of the next short segments loaded before the rows of these (3.48 against
+// 3.28: registers spilled), stretches handed out by a counter (3.76 to 3.88: less waiting at the join's barrier, more stretches to
+// begin and to join).
 #pragma once
 
 #include "segreduce.cuh"
 #include "window.h"
 
 namespace e2egrec {
-
 
 // Segment of entry k by the whole warp: every round splits the range into 33 parts with 32 probes.
 // Largest s in [0, n_seg) with ptr[s] <= k   (0 <= k < ptr[n_seg], ptr[0] = 0).
@@ -443,8 +443,8 @@ seg_walk_kernel(const T *__restrict__ in, int64_t ld_in, const PtrT *__restrict_
     if (threadIdx.x == 0) win_info[blockIdx.x] = make_int4(sh_win[0], sh_win[1], sh_win[2], 0);
 }
 
-// B200: 5 M nodes, 10^8 entries, 64 bf16 values, forward and transposed 3.73 -> 3.26 ms (8.6 TB/s of gathered rows);
-// 500 k nodes, 2 * 10^7 entries, 64 fp32 values, weighted, per layer 0.45 -> 0.41 ms (12.5 TB/s).
+// B200: 5 M nodes, 10^8 entries, 64 bf16 values, forward and transposed 3.74 -> 3.18 ms (8.8 TB/s of gathered rows);
+// 500 k nodes, 2 * 10^7 entries, 64 fp32 values, weighted, per layer 0.45 -> 0.40 ms (12.7 TB/s).
 template <typename T, typename PtrT, int LPR, int CPL, bool kWeight, int kWalkWarps, bool kWide>
 inline void launch_seg_walk(const T *in, int64_t ld_in, const PtrT *ptr, const int32_t *idx, const int32_t *n_seg_dev,
                             int64_t n_seg_host, int64_t cap_seg, const float *w, int run_len, int d, const SegScratch &sc,
