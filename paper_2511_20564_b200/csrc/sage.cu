@@ -227,18 +227,31 @@ static int32_t forward_impl(const e2egrec_block *blocks, int32_t n_layers, const
 
 // ------------------------------------------------------------------------------ backward
 struct BackwardScratch {
-    size_t dz_off[2], dcat_off, seg_off, seg_bytes, chain_off, chain_bytes, part_off, wt_off, bytes;
+    size_t dz_off[2], dcat_off, seg_off, seg_bytes, chain_off, chain_bytes, part_off[2], wt_off, bytes;
 };
+
+// Splits of a weight gradient on the caller's stream: at most these (tensor cores; fp32-FMA kernel).
+static int tc_serial_splits(const LayerPlan &p) { return std::max(1, kDwSplits / tc_weight_grad_tiles(p.d_out, 2 * p.d_in)); }
+static int serial_splits(const LayerPlan &p) { return std::max(tc_serial_splits(p), simt_splits(p.rows, p.d_out, 2 * p.d_in, kDwSplits)); }
+
+// Whether a layer's weight gradient stays on the caller's stream
+static bool dw_serial(const LayerPlan &p, int n_rhs, size_t es)
+{
+    return (size_t)p.rows * (n_rhs * p.d_out + 2 * p.d_in) * es >= dw_serial_bytes();
+}
 
 static BackwardScratch plan_backward(const e2egrec_block *blocks, int32_t n_layers, const LayerPlan *plan, size_t es, int n_rhs)
 {
     BackwardScratch s{};
-    size_t dz = 0, dcat = 0, part = 0, ht = 0, wt = 0, chain = 0;
+    size_t dz = 0, dcat = 0, part[2] = {0, 0}, ht = 0, wt = 0, chain = 0;
     for (int l = 0; l < n_layers; ++l) {
         const LayerPlan &p = plan[l];
         dz = std::max(dz, (size_t)n_rhs * p.rows * p.d_out * es);
         dcat = std::max(dcat, (size_t)n_rhs * p.rows * 2 * p.d_in * es);
-        part = std::max(part, (size_t)kDwSplits * p.d_out * 2 * p.d_in * sizeof(float));
+        // on the helper stream, on the caller's (whichever layers will be there: the size grows with the batch)
+        const size_t n_w = (size_t)p.d_out * 2 * p.d_in * sizeof(float);
+        part[0] = std::max(part[0], kDwSplits * n_w);
+        part[1] = std::max(part[1], (size_t)serial_splits(p) * n_w);
         wt = std::max(wt, (size_t)p.d_out * 2 * p.d_in * es);
         const int64_t edges = blocks[p.block].cap_edges;
         const int run_len = block_run_len(edges, p.d_in, es);
@@ -254,7 +267,8 @@ static BackwardScratch plan_backward(const e2egrec_block *blocks, int32_t n_laye
     s.seg_bytes = ht;
     s.chain_off = take(chain);
     s.chain_bytes = chain;
-    s.part_off = take(part);
+    s.part_off[0] = take(part[0]);
+    s.part_off[1] = take(part[1]);
     s.wt_off = take(wt);
     s.bytes = off;
     return s;
@@ -271,7 +285,6 @@ static int32_t backward_impl(const e2egrec_block *blocks, int32_t n_layers, cons
     const int accumulate = (flags & E2EGREC_ACCUMULATE_DW) ? 1 : 0;
     T *dz_buf[2] = {reinterpret_cast<T *>(scratch + bs.dz_off[0]), reinterpret_cast<T *>(scratch + bs.dz_off[1])};
     T *dcat = reinterpret_cast<T *>(scratch + bs.dcat_off);
-    float *part = reinterpret_cast<float *>(scratch + bs.part_off);
     const bool chain = chain_blocks(blocks, n_layers);
 
     // gradient entering the top layer, masked by its activation; and the counters of the transposed aggregation (one per window
@@ -287,7 +300,7 @@ static int32_t backward_impl(const e2egrec_block *blocks, int32_t n_layers, cons
                    dH_out[n_rhs - 1].ld, reinterpret_cast<uint4 *>(scratch + bs.chain_off), (int64_t)(bs.chain_bytes / 16));
     }
     SideStream *side = SideStream::get(st);
-    cudaEvent_t dz_free[2] = {nullptr, nullptr}, part_free = nullptr;
+    cudaEvent_t dz_free[2] = {nullptr, nullptr};
     for (int l = n_layers - 1; l >= 0; --l) {
         const LayerPlan &p = plan[l];
         const e2egrec_block &b = blocks[p.block];
@@ -297,16 +310,15 @@ static int32_t backward_impl(const e2egrec_block *blocks, int32_t n_layers, cons
         const int two_d = 2 * p.d_in;
         // dW_l = dZ^T [h | agg]   (split over the rows, partial sums added in a fixed order).  Nothing later in
         // this call reads dW, so it runs on the helper stream beside the dCat product and the transposed
-        // aggregation; `dz_free` holds the event after which the helper stream no longer reads a dZ buffer, `part_free` the one
-        // after which it no longer uses the partial sums, of which there is one buffer.
+        // aggregation; `dz_free` holds the event after which the helper stream no longer reads a dZ buffer.  The partial sums of
+        // layers that stay on the caller's stream have a buffer of their own: the helper may still be adding up those of the
+        // layer above.  (One buffer and a wait instead: 4096 seeds of 128 bf16 values at 20, 10, 5 314 -> 324 us.)
         cudaStream_t ws = st;
-        const bool dw_beside = side && (size_t)p.rows * (n_rhs * p.d_out + two_d) * sizeof(T) < dw_serial_bytes();
+        const bool serial = dw_serial(p, n_rhs, sizeof(T)), dw_beside = side && !serial;
+        float *part = reinterpret_cast<float *>(scratch + bs.part_off[serial]);
         if (dw_beside) {
             side->fork(st);
             ws = side->stream;
-        } else if (part_free) {                   // the layer above may still be adding up its partial sums
-            cudaStreamWaitEvent(st, part_free, 0);
-            part_free = nullptr;
         }
         if (l == 0) tap_begin(TAP_DW_OUTER, ws);
         bool dw_done = false;
@@ -314,7 +326,7 @@ static int32_t backward_impl(const e2egrec_block *blocks, int32_t n_layers, cons
         // whole machine), one wave of CTAs over all output tiles for a large one, where every further wave pays the set-up
         // of a CTA and another set of fp32 partials (2 * 10^9-entry workload, 256 x 512 weights: 0.191 ms with 148
         // splits in four waves, 0.153 ms with 37 in one).
-        const int tc_splits = dw_beside ? kDwSplits : std::max(1, kDwSplits / tc_weight_grad_tiles(p.d_out, two_d));
+        const int tc_splits = dw_beside ? kDwSplits : tc_serial_splits(p);
         if (X->dtype == E2EGREC_BF16)
             dw_done = tc_weight_grad(reinterpret_cast<const __nv_bfloat16 *>(dz), p.rows, p.d_out,
                                      reinterpret_cast<const __nv_bfloat16 *>(cat), two_d, n_dst, part, tc_splits,
@@ -345,7 +357,6 @@ static int32_t backward_impl(const e2egrec_block *blocks, int32_t n_layers, cons
         if (dw_beside) {
             dz_free[l & 1] = side->event();
             cudaEventRecord(dz_free[l & 1], side->stream);
-            part_free = dz_free[l & 1];
         }
         // dCat = dZ W_l, the agg half scaled by 1/|S|
         if (l == 0) tap_begin(TAP_DCAT_OUTER, st);
